@@ -174,44 +174,86 @@ __global__ void __launch_bounds__(128) mlp_gemm(const GemmArgs g) {
 
 namespace {
 
-__global__ void to_bf16_kernel(const float *x, size_t n, int fin, __nv_bfloat16 *X, size_t rows, int ld) {
-  const size_t total = rows * size_t(ld);
-  for (size_t e = blockIdx.x * size_t(blockDim.x) + threadIdx.x; e < total; e += size_t(gridDim.x) * blockDim.x) {
-    const size_t r = e / ld;
-    const int c = int(e % ld);
-    X[e] = __float2bfloat16_rn(r < n && c < fin ? x[r * fin + c] : 0.f);
+// Rows are padded to kRow = 64 columns (network inputs and outputs); a thread
+// takes eight columns of a row and stores them as 16 bytes.  (Indexing by
+// 64-bit division over single elements: 12.5 us for 65,536 rows; this: see
+// the launch list in profiles/.)
+constexpr int kRow = 64;
+
+__device__ __forceinline__ uint4 pack8(const float (&v)[8]) {
+  uint32_t w[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+    w[i] = *reinterpret_cast<const uint32_t *>(&h);
   }
+  return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
+__global__ void to_bf16_kernel(const float *x, size_t n, int fin, __nv_bfloat16 *X, size_t rows) {
+  const size_t e = blockIdx.x * size_t(blockDim.x) + threadIdx.x;
+  const size_t r = e >> 3;
+  const int c0 = int(e & 7) * 8;
+  if (r >= rows) return;
+  float v[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = r < n && c0 + i < fin ? x[r * fin + c0 + i] : 0.f;
+  *reinterpret_cast<uint4 *>(X + r * kRow + c0) = pack8(v);
+}
+
+// Eight threads a minibatch row (one thread a row held 64 dependent stores:
+// 15 us for 1,024 rows).
 __global__ void gather_kernel(const float *x, const float *t, size_t n_data, int fin, int fout,
                               const uint64_t *step, uint32_t s0, uint32_t s1, size_t batch,
-                              __nv_bfloat16 *X, int ldx, float *T) {
-  const size_t b = blockIdx.x * size_t(blockDim.x) + threadIdx.x;
+                              __nv_bfloat16 *X, float *T) {
+  const size_t e = blockIdx.x * size_t(blockDim.x) + threadIdx.x;
+  const size_t b = e >> 3;
+  const int q = int(e & 7), c0 = q * 8;
   if (b >= batch) return;
   const uint64_t st = *step;
   // the first word of Philox4x32-10 at counter (b, step), key (s0, s1)
   const uint32_t u = philox(make_uint4(uint32_t(b), uint32_t(b >> 32), uint32_t(st), uint32_t(st >> 32)), s0, s1).x;
   const size_t src = size_t(u) % n_data;
-  for (int c = 0; c < ldx; ++c) X[b * ldx + c] = __float2bfloat16_rn(c < fin ? x[src * fin + c] : 0.f);
-  for (int c = 0; c < fout; ++c) T[b * fout + c] = t[src * fout + c];
+  float v[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = c0 + i < fin ? x[src * fin + c0 + i] : 0.f;
+  *reinterpret_cast<uint4 *>(X + b * kRow + c0) = pack8(v);
+  for (int c = q; c < fout; c += 8) T[b * fout + c] = t[src * fout + c];
 }
 
-__global__ void loss_kernel(const float *Y, int ldy, const float *T, const float *w, size_t n, int fout,
-                            size_t rows, __nv_bfloat16 *dY, int ldd, float *part) {
+// Weighted squared error; rows of kRow columns, thread (tid / 64, tid % 64)
+// of block k takes rows 4 k + tid / 64, + 4 gridDim, ... of its column, four
+// at a time so that their loads overlap.
+__global__ void loss_kernel(const float *Y, const float *T, const float *w, size_t n, int fout,
+                            size_t rows, __nv_bfloat16 *dY, float *part) {
   __shared__ float red[32];
-  const size_t total = rows * size_t(ldd);
   float acc = 0.f;
   const float inv = 1.f / float(n);
-  for (size_t e = blockIdx.x * size_t(blockDim.x) + threadIdx.x; e < total; e += size_t(gridDim.x) * blockDim.x) {
-    const size_t r = e / ldd;
-    const int c = int(e % ldd);
-    float g = 0.f;
-    if (r < n && c < fout) {
-      const float diff = Y[r * ldy + c] - T[r * fout + c];
-      acc += w[c] * diff * diff * inv;
-      g = 2.f * w[c] * diff * inv;
+  const int c = int(threadIdx.x) & (kRow - 1);
+  const size_t step = size_t(gridDim.x) * (blockDim.x / kRow);
+  const bool col = c < fout;
+  const float wc = col ? w[c] : 0.f;
+  for (size_t r0 = blockIdx.x * size_t(blockDim.x / kRow) + threadIdx.x / kRow; r0 < rows; r0 += 4 * step) {
+    float y[4], t[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const size_t r = r0 + size_t(i) * step;
+      const bool in = col && r < n;
+      y[i] = in ? Y[r * kRow + c] : 0.f;
+      t[i] = in ? T[r * fout + c] : 0.f;
     }
-    dY[e] = __float2bfloat16_rn(g);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const size_t r = r0 + size_t(i) * step;
+      if (r >= rows) break;
+      float g = 0.f;
+      if (col && r < n) {
+        const float diff = y[i] - t[i];
+        acc += wc * diff * diff * inv;
+        g = 2.f * wc * diff * inv;
+      }
+      dY[r * kRow + c] = __float2bfloat16_rn(g);
+    }
   }
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
@@ -223,45 +265,121 @@ __global__ void loss_kernel(const float *Y, int ldy, const float *T, const float
   }
 }
 
-__global__ void split_sum_kernel(const float *part, int splits, size_t stride, size_t count, float *out) {
-  for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < count; i += size_t(gridDim.x) * blockDim.x) {
-    float s = 0.f;
-    for (int z = 0; z < splits; ++z) s += part[size_t(z) * stride + i];
-    out[i] = s;
+// Column sums of dZ over chunks of kColChunk rows, in row order: a block
+// brings its chunk's 64 columns to shared memory with every load in flight,
+// then one thread a column adds the rows (a thread a column straight from
+// memory waited on each of its 256 loads: 24 us whatever the row count; the
+// chunk's chain of 256 additions is the floor, about 0.6 us).
+constexpr int kColChunk = 256, kColStride = 64 + 8;
+
+__global__ void __launch_bounds__(256) colsum_kernel(const __nv_bfloat16 *dZ, size_t rows, int ld, int cols,
+                                                     float *scratch) {
+  __shared__ __align__(16) __nv_bfloat16 s[kColChunk * kColStride];
+  const int c0 = blockIdx.x * 64;
+  const size_t r0 = size_t(blockIdx.y) * kColChunk;
+  const int nr = int(min(rows - r0, size_t(kColChunk)));
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int v = threadIdx.x + 256 * j, r = v >> 3, q = (v & 7) * 8;
+    if (r < nr)
+      *reinterpret_cast<uint4 *>(s + r * kColStride + q) =
+          *reinterpret_cast<const uint4 *>(dZ + (r0 + r) * size_t(ld) + c0 + q);
   }
+  __syncthreads();
+  if (threadIdx.x >= 64) return;
+  float a = 0.f;
+#pragma unroll 16
+  for (int r = 0; r < nr; ++r) a += __bfloat162float(s[r * kColStride + threadIdx.x]);
+  scratch[size_t(blockIdx.y) * cols + c0 + threadIdx.x] = a;
 }
 
-constexpr int kColChunk = 256;
-
-__global__ void colsum_kernel(const __nv_bfloat16 *dZ, size_t rows, int ld, int cols, float *scratch) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= cols) return;
-  const size_t r0 = size_t(blockIdx.y) * kColChunk, r1 = min(rows, r0 + kColChunk);
-  float s = 0.f;
-  for (size_t r = r0; r < r1; ++r) s += __bfloat162float(dZ[r * ld + c]);
-  scratch[size_t(blockIdx.y) * cols + c] = s;
-}
-
-__global__ void adam_kernel(float *p, const float *g, float *m, float *v, __nv_bfloat16 *pb, size_t n,
-                            const uint64_t *step, float lr, float b1, float b2, float eps) {
+// Bias corrections of Adam for step *step + 1, once per step (two FP64
+// powers in every thread of the update were 66 of a step's 237 us).
+__global__ void adam_consts_kernel(const uint64_t *step, float b1, float b2, float *c) {
   const double t = double(*step + 1);
-  const float c1 = float(1.0 - pow(double(b1), t)), c2 = float(1.0 - pow(double(b2), t));
-  for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x) {
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    const float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-    p[i] = pi;
-    pb[i] = __float2bfloat16_rn(pi);
-  }
+  if (threadIdx.x == 0) c[0] = float(1.0 - pow(double(b1), t));
+  if (threadIdx.x == 32) c[1] = float(1.0 - pow(double(b2), t));
 }
 
+// Ordered sum of `n` values `stride` apart, kAhead loads in flight (one at a
+// time waited a memory latency each).
+constexpr int kAhead = 16;
+__device__ __forceinline__ float ordered_sum(const float *p, int n, size_t stride) {
+  float s = 0.f;
+  int z = 0;
+  for (; z + kAhead <= n; z += kAhead) {
+    float v[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) v[u] = p[size_t(z + u) * stride];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) s += v[u];
+  }
+  float v[kAhead];
+#pragma unroll
+  for (int u = 0; u < kAhead; ++u) v[u] = z + u < n ? p[size_t(z + u) * stride] : 0.f;
+#pragma unroll
+  for (int u = 0; u < kAhead; ++u)
+    if (z + u < n) s += v[u];
+  return s;
+}
+
+// A layer's gradient from its partials, in one launch: the weight elements
+// (sums over the k splits, in order) by blocks 0 .. wb - 1, then the biases
+// (sums over the row chunks of colsum_kernel, in order) 32 columns a block,
+// their chunk values staged in shared memory.  With ADAM the parameters are
+// updated from the sum in hand and the gradient is not stored.
+template <bool ADAM>
+__global__ void __launch_bounds__(256) layer_grad_kernel(const LayerGrad g, const AdamStep a) {
+  __shared__ float sh[256][33];
+  size_t i;
+  float s;
+  if (blockIdx.x < g.w_blocks) {
+    i = blockIdx.x * size_t(256) + threadIdx.x;
+    if (i >= g.count) return;
+    s = ordered_sum(g.part + i, g.splits, g.count);
+  } else {
+    const int c = int(threadIdx.x) & 31, q = int(threadIdx.x) >> 5;
+    const int col = int(blockIdx.x - g.w_blocks) * 32 + c;
+    s = 0.f;
+    for (int z0 = 0; z0 < g.chunks; z0 += 256) {
+#pragma unroll
+      for (int u = 0; u < 32; ++u) {
+        const int z = z0 + q + 8 * u;
+        if (z < g.chunks) sh[q + 8 * u][c] = g.colpart[size_t(z) * g.cols + col];
+      }
+      __syncthreads();
+      if (q == 0) {
+        const int nz = min(256, g.chunks - z0);
+#pragma unroll 16
+        for (int z = 0; z < nz; ++z) s += sh[z][c];
+      }
+      __syncthreads();
+    }
+    if (q) return;
+    i = g.count + size_t(col);
+  }
+  if (!ADAM) {
+    g.out[i] = s;
+    return;
+  }
+  const float b1 = a.b1, b2 = a.b2, c1 = a.consts[0], c2 = a.consts[1];
+  const float mi = b1 * a.m[i] + (1.f - b1) * s;
+  const float vi = b2 * a.v[i] + (1.f - b2) * s * s;
+  a.m[i] = mi;
+  a.v[i] = vi;
+  const float pi = a.p[i] - a.lr * (mi / c1) / (sqrtf(vi / c2) + a.eps);
+  a.p[i] = pi;
+  a.pb[i] = __float2bfloat16_rn(pi);
+}
+
+// The block partials' total in FP64: 32 lanes' strided sums, then a fixed
+// shuffle tree (one thread's chain of dependent loads was 43 us for 512).
 __global__ void loss_total_kernel(const float *part, int blocks, double *loss, uint64_t *step) {
-  if (threadIdx.x != 0) return;
   double s = 0.0;
-  for (int i = 0; i < blocks; ++i) s += double(part[i]);
+#pragma unroll 4
+  for (int i = threadIdx.x; i < blocks; i += 32) s += double(part[i]);
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (threadIdx.x != 0) return;
   *loss = s;
   if (step) *step += 1;
 }
@@ -305,44 +423,49 @@ cudaError_t launch_gemm(GemmKind kind, int epi, const GemmArgs &g, int splits, c
 
 cudaError_t launch_to_bf16(const float *x, size_t n, int fin, __nv_bfloat16 *X, size_t rows, int ld,
                            cudaStream_t s) {
-  to_bf16_kernel<<<grid_for(rows * ld, 256), 256, 0, s>>>(x, n, fin, X, rows, ld);
+  if (ld != kRow) return cudaErrorInvalidValue;
+  to_bf16_kernel<<<unsigned((rows * 8 + 255) / 256), 256, 0, s>>>(x, n, fin, X, rows);
   return cudaGetLastError();
 }
 
 cudaError_t launch_gather(const float *x, const float *t, size_t n_data, int fin, int fout,
                           const uint64_t *step, uint32_t s0, uint32_t s1, size_t batch,
                           __nv_bfloat16 *X, int ldx, float *T, cudaStream_t s) {
-  gather_kernel<<<unsigned((batch + 127) / 128), 128, 0, s>>>(x, t, n_data, fin, fout, step, s0, s1, batch,
-                                                              X, ldx, T);
+  if (ldx != kRow) return cudaErrorInvalidValue;
+  gather_kernel<<<unsigned((batch * 8 + 127) / 128), 128, 0, s>>>(x, t, n_data, fin, fout, step, s0, s1, batch, X, T);
   return cudaGetLastError();
 }
 
-int loss_blocks(size_t rows) { return int(grid_for(rows * 64, 256, 512)); }
+int loss_blocks(size_t rows) { return int(grid_for(rows * kRow, 256, 512)); }
 
 cudaError_t launch_loss(const float *Y, int ldy, const float *T, const float *w, size_t n, int fout,
                         size_t rows, __nv_bfloat16 *dY, int ldd, float *part, int blocks, cudaStream_t s) {
-  loss_kernel<<<blocks, 256, 0, s>>>(Y, ldy, T, w, n, fout, rows, dY, ldd, part);
+  if (ldy != kRow || ldd != kRow) return cudaErrorInvalidValue;
+  loss_kernel<<<blocks, 256, 0, s>>>(Y, T, w, n, fout, rows, dY, part);
   return cudaGetLastError();
 }
 
-cudaError_t launch_split_sum(const float *part, int splits, size_t stride, size_t count, float *out,
-                             cudaStream_t s) {
-  split_sum_kernel<<<grid_for(count, 256), 256, 0, s>>>(part, splits, stride, count, out);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_colsum(const __nv_bfloat16 *dZ, size_t rows, int ld, int cols, float *scratch,
-                          float *out, cudaStream_t s) {
+cudaError_t launch_colsum(const __nv_bfloat16 *dZ, size_t rows, int ld, int cols, float *scratch, cudaStream_t s) {
+  if (cols % 64 || ld % 8) return cudaErrorInvalidValue;
   const unsigned chunks = unsigned((rows + kColChunk - 1) / kColChunk);
-  colsum_kernel<<<dim3(unsigned((cols + 127) / 128), chunks), 128, 0, s>>>(dZ, rows, ld, cols, scratch);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  return launch_split_sum(scratch, int(chunks), size_t(cols), size_t(cols), out, s);
+  colsum_kernel<<<dim3(unsigned(cols / 64), chunks), 256, 0, s>>>(dZ, rows, ld, cols, scratch);
+  return cudaGetLastError();
 }
 
-cudaError_t launch_adam(float *p, const float *g, float *m, float *v, __nv_bfloat16 *pb, size_t n,
-                        uint64_t *step, float lr, float b1, float b2, float eps, cudaStream_t s) {
-  adam_kernel<<<grid_for(n, 256, 1024), 256, 0, s>>>(p, g, m, v, pb, n, step, lr, b1, b2, eps);
+cudaError_t launch_layer_grad(LayerGrad g, size_t rows, const AdamStep *adam, cudaStream_t s) {
+  if (g.cols % 32) return cudaErrorInvalidValue;
+  g.chunks = int((rows + kColChunk - 1) / kColChunk);
+  g.w_blocks = unsigned((g.count + 255) / 256);
+  const unsigned grid = g.w_blocks + unsigned(g.cols / 32);
+  if (adam)
+    layer_grad_kernel<true><<<grid, 256, 0, s>>>(g, *adam);
+  else
+    layer_grad_kernel<false><<<grid, 256, 0, s>>>(g, AdamStep{});
+  return cudaGetLastError();
+}
+
+cudaError_t launch_adam_consts(const uint64_t *step, float b1, float b2, float *consts, cudaStream_t s) {
+  adam_consts_kernel<<<1, 64, 0, s>>>(step, b1, b2, consts);
   return cudaGetLastError();
 }
 

@@ -119,18 +119,37 @@ cudaError_t launch_loss(const float *Y, int ldy, const float *T, const float *w,
                         size_t rows, __nv_bfloat16 *dY, int ldd, float *part, int blocks,
                         cudaStream_t s);
 int loss_blocks(size_t rows);
-// out[i] = sum_s part[s * stride + i], s < splits, in order; i < count.
-cudaError_t launch_split_sum(const float *part, int splits, size_t stride, size_t count, float *out,
-                             cudaStream_t s);
-// Column sums of dZ [rows, ld] (BF16) for columns < cols into out (FP32),
-// in a fixed order (row chunks, then the chunk partials).
-cudaError_t launch_colsum(const __nv_bfloat16 *dZ, size_t rows, int ld, int cols, float *scratch,
-                          float *out, cudaStream_t s);
-// Adam over flat parameters p (FP32) with gradient g; moments m, v; bf16
-// copy pb; bias corrections for step *step + 1.
-cudaError_t launch_adam(float *p, const float *g, float *m, float *v, __nv_bfloat16 *pb, size_t n,
-                        uint64_t *step, float lr, float b1, float b2, float eps, cudaStream_t s);
-// Sum of part[0..blocks) into *loss (FP64) in order; then ++*step if step.
+// Column sums of dZ [rows, ld] (BF16), columns < cols (a multiple of 64), over
+// chunks of 256 rows in row order: scratch[chunk][cols].
+cudaError_t launch_colsum(const __nv_bfloat16 *dZ, size_t rows, int ld, int cols, float *scratch, cudaStream_t s);
+// A layer's gradient from its partials: out[i] = sum_z part[z * count + i] in
+// order (z < splits, i < count: the weights), then out[count + c] = the sum
+// of colpart[chunk][c] in order (c < cols: the biases; a multiple of 32).
+struct LayerGrad {
+  const float *part;
+  int splits;
+  size_t count;
+  const float *colpart;
+  int cols;
+  float *out;
+  int chunks;                   // set by the launcher, as w_blocks
+  unsigned w_blocks;
+};
+// Adam's update of the layer's parameters (flat arrays from the layer's
+// first weight: p and moments m, v FP32, pb the BF16 copy) by the gradient
+// as it is summed; consts: the step's bias corrections 1 - b1^t, 1 - b2^t.
+struct AdamStep {
+  float *p, *m, *v;
+  __nv_bfloat16 *pb;
+  const float *consts;
+  float lr, b1, b2, eps;
+};
+// rows: the batch's padded rows (the chunks of launch_colsum).  With adam,
+// out is not written.
+cudaError_t launch_layer_grad(LayerGrad g, size_t rows, const AdamStep *adam, cudaStream_t s);
+// consts[0..1] = 1 - b1^t, 1 - b2^t for t = *step + 1 (in FP64, rounded).
+cudaError_t launch_adam_consts(const uint64_t *step, float b1, float b2, float *consts, cudaStream_t s);
+// Sum of part[0..blocks) into *loss (FP64, a fixed order); then ++*step if step.
 cudaError_t launch_loss_total(const float *part, int blocks, double *loss, uint64_t *step, cudaStream_t s);
 // y [n, fout] FP32 from Y [rows, ldy].
 cudaError_t launch_unpad(const float *Y, int ldy, size_t n, int fout, float *y, cudaStream_t s);

@@ -45,7 +45,8 @@ struct pc_mlp {
   std::vector<__nv_bfloat16 *> H;   // hidden activations, layers 0..L-2
   __nv_bfloat16 *dZ[2] = {nullptr, nullptr};
   float *Y = nullptr, *T = nullptr, *wts = nullptr;
-  float *part = nullptr, *colscr = nullptr, *loss_part = nullptr;
+  float *part[2] = {nullptr, nullptr};  // weight-gradient partials of consecutive layers in turn
+  float *colscr = nullptr, *loss_part = nullptr, *adam_c = nullptr;
   size_t part_cap = 0;
   double *loss = nullptr;
   uint64_t *step = nullptr;
@@ -171,8 +172,9 @@ size_t layout(pc_mlp *N, size_t rows) {
   N->Y = c.take<float>(rows * N->wp[N->L]);
   N->T = c.take<float>(rows * N->wp[N->L]);
   N->wts = c.take<float>(kPad);
-  N->part = c.take<float>(part);
+  for (float *&q : N->part) q = c.take<float>(part);
   N->colscr = c.take<float>(chunks * widest);
+  N->adam_c = c.take<float>(2);
   N->loss_part = c.take<float>(512);
   N->loss = c.take<double>(1);
   N->step = c.take<uint64_t>(1);
@@ -241,17 +243,50 @@ cudaError_t forward(pc_mlp *N, size_t rows, cudaStream_t s) {
   return cudaSuccess;
 }
 
-// Loss on the first n of `rows` rows (targets in T), gradients into g.
-cudaError_t backward(pc_mlp *N, size_t n, size_t rows, cudaStream_t s) {
+// A training step's branches beside the main one, under stream capture: `w`
+// the weight-gradient products, `c` the bias sums and each layer's gradient
+// sums with the update.  The main branch is the chain forward -> loss ->
+// data gradients.  The events order the branches (backward); the caller
+// destroys them after the capture.
+struct Branches {
+  cudaStream_t w = nullptr, c = nullptr;
+  cudaEvent_t dz[kMaxLayers] = {}, wgrad[kMaxLayers] = {}, colsum[kMaxLayers] = {}, dgrad[kMaxLayers] = {},
+              sums[kMaxLayers] = {};
+  cudaEvent_t start = nullptr;
+};
+
+cudaError_t signal(cudaEvent_t ev, cudaStream_t from, cudaStream_t to) {
+  cudaError_t e = cudaEventRecord(ev, from);
+  return e == cudaSuccess ? cudaStreamWaitEvent(to, ev, 0) : e;
+}
+
+// Loss on the first n of `rows` rows (targets t, [n][outputs]), gradients into
+// g; with `adam` (p, m, v, pb at the flat arrays' starts) the parameters are
+// updated instead.  With branches a layer's weight gradient, and the sums
+// and update of the layer before, run beside its data gradient, so a step's
+// critical path is one product a layer.  Layer l's update waits for its data
+// gradient, which reads the weights; the data gradient that reuses a signal
+// buffer waits for the reads of its former contents.
+cudaError_t backward(pc_mlp *N, const float *t, size_t n, size_t rows, cudaStream_t s, const AdamStep *adam = nullptr,
+                     const Branches *br = nullptr) {
   const int fout = N->w[N->L];
   const int lb = loss_blocks(rows);
-  cudaError_t e = launch_loss(N->Y, N->wp[N->L], N->T, N->wts, n, fout, rows, N->dZ[0], N->wp[N->L],
+  cudaError_t e = launch_loss(N->Y, N->wp[N->L], t, N->wts, n, fout, rows, N->dZ[0], N->wp[N->L],
                               N->loss_part, lb, s);
   if (e != cudaSuccess) return e;
+  const cudaStream_t sw = br ? br->w : s, sc = br ? br->c : s;
   int cur = 0;
   for (int l = N->L - 1; l >= 0; --l) {
     const __nv_bfloat16 *in = l == 0 ? N->X : N->H[l - 1];
     const int out_w = N->wp[l + 1], in_w = N->wp[l];
+    if (br) {
+      e = signal(br->dz[l], s, sw);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(sc, br->dz[l], 0);
+      if (e == cudaSuccess && l + 2 < N->L) e = cudaStreamWaitEvent(sw, br->sums[l + 2], 0);  // part[l & 1] read
+      if (e == cudaSuccess && l == N->L - 1)  // the loss, and the step count: its readers precede it
+        e = launch_loss_total(N->loss_part, lb, N->loss, N->step, sc);
+      if (e != cudaSuccess) return e;
+    }
     // dW_l = dZ^T in
     GemmArgs a = gemm0();
     a.A = N->dZ[cur];
@@ -264,17 +299,21 @@ cudaError_t backward(pc_mlp *N, size_t n, size_t rows, cudaStream_t s) {
     int splits = grad_splits(N, out_w, in_w, rows, a.k_split);
     int tc_ks = 0;
     const int tc_splits = rows % 64 == 0 ? tc_grad_splits(N, out_w, in_w, rows, tc_ks) : 0;
-    a.Cf = N->part;
+    a.Cf = N->part[l & 1];
     a.ldc = in_w;
-    e = product(N, kGemmWeightGrad, kEpiPartial, l, rows, a, splits, tc_ks, tc_splits, s, &splits);
+    e = product(N, kGemmWeightGrad, kEpiPartial, l, rows, a, splits, tc_ks, tc_splits, sw, &splits);
     if (e != cudaSuccess) return e;
-    const size_t cnt = size_t(out_w) * in_w;
-    e = launch_split_sum(N->part, splits, cnt, cnt, N->g + N->offW[l], s);
-    if (e != cudaSuccess) return e;
-    e = launch_colsum(N->dZ[cur], rows, out_w, out_w, N->colscr, N->g + N->offB[l], s);
+    e = launch_colsum(N->dZ[cur], rows, out_w, out_w, N->colscr, sc);
+    if (e == cudaSuccess && br) e = cudaEventRecord(br->colsum[l], sc);
+    if (e == cudaSuccess && br) e = signal(br->wgrad[l], sw, sc);
     if (e != cudaSuccess) return e;
     if (l > 0) {
       // dZ_{l-1} = (dZ_l W_l) * softplus'(z_{l-1})
+      if (br && l + 1 < N->L) {  // the buffer it writes: read by layer l + 1's gradients
+        e = cudaStreamWaitEvent(s, br->wgrad[l + 1], 0);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(s, br->colsum[l + 1], 0);
+        if (e != cudaSuccess) return e;
+      }
       GemmArgs b = gemm0();
       b.A = N->dZ[cur];
       b.lda = out_w;
@@ -290,8 +329,28 @@ cudaError_t backward(pc_mlp *N, size_t n, size_t rows, cudaStream_t s) {
       b.ldc = in_w;
       e = product(N, kGemmDataGrad, kEpiDSoftplus, l, rows, b, 1, 0, 1, s);
       if (e != cudaSuccess) return e;
+      if (br && (e = signal(br->dgrad[l], s, sc)) != cudaSuccess) return e;
       cur ^= 1;
     }
+    LayerGrad lg{};
+    lg.part = N->part[l & 1];
+    lg.splits = splits;
+    lg.count = size_t(out_w) * in_w;
+    lg.colpart = N->colscr;
+    lg.cols = out_w;
+    lg.out = N->g + N->offW[l];
+    AdamStep step{};
+    if (adam) {
+      step = *adam;
+      const size_t o = N->offW[l];
+      step.p += o;
+      step.m += o;
+      step.v += o;
+      step.pb += o;
+    }
+    e = launch_layer_grad(lg, rows, adam ? &step : nullptr, sc);
+    if (e == cudaSuccess && br) e = cudaEventRecord(br->sums[l], sc);
+    if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
@@ -515,9 +574,8 @@ pc_status pc_mlp_gradients(pc_mlp *N, const float *d_x, const float *d_t, const 
   pc_status st = set_weights(N, w);
   if (st != PC_OK) return st;
   CU(launch_to_bf16(d_x, n, N->w[0], N->X, rows, N->wp[0], s), "input");
-  CU(cudaMemcpyAsync(N->T, d_t, n * N->w[N->L] * sizeof(float), cudaMemcpyDeviceToDevice, s), "targets");
   CU(forward(N, rows, s), "forward");
-  CU(backward(N, n, rows, s), "backward");
+  CU(backward(N, d_t, n, rows, s), "backward");
   CU(launch_loss_total(N->loss_part, loss_blocks(rows), N->loss, nullptr, s), "loss");
   if (d_grads) {
     st = copy_unpadded(N, N->g, d_grads, cudaMemcpyDeviceToDevice);
@@ -546,26 +604,39 @@ pc_status pc_mlp_train(pc_mlp *N, const float *d_x, const float *d_t, size_t n_d
     st = wait_stream(c);
     if (st != PC_OK) return st;
     cudaStream_t cap = nullptr;
-    CU(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking), "capture stream");
+    Branches br;
     const size_t rows = rows_for(batch);
-    cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
+    cudaError_t e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&br.w, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&br.c, cudaStreamNonBlocking);
+    std::vector<cudaEvent_t *> evs = {&br.start};
+    for (int l = 0; l < N->L; ++l)
+      for (cudaEvent_t *v : {&br.dz[l], &br.wgrad[l], &br.colsum[l], &br.dgrad[l], &br.sums[l]}) evs.push_back(v);
+    for (cudaEvent_t *v : evs)
+      if (e == cudaSuccess) e = cudaEventCreateWithFlags(v, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-      if (rows > batch) e = cudaMemsetAsync(N->X, 0, rows * N->wp[0] * sizeof(__nv_bfloat16), cap);
+      AdamStep adam{N->p, N->m, N->v, N->pb, N->adam_c, lr, 0.9f, 0.999f, 1e-8f};
+      // the bias corrections of this step, beside the forward products
+      e = signal(br.start, cap, br.c);
+      if (e == cudaSuccess) e = launch_adam_consts(N->step, adam.b1, adam.b2, N->adam_c, br.c);
+      if (e == cudaSuccess && rows > batch) e = cudaMemsetAsync(N->X, 0, rows * N->wp[0] * sizeof(__nv_bfloat16), cap);
       if (e == cudaSuccess)
         e = launch_gather(d_x, d_t, n_data, N->w[0], N->w[N->L], N->step, uint32_t(seed), uint32_t(seed >> 32),
                           batch, N->X, N->wp[0], N->T, cap);
       if (e == cudaSuccess) e = forward(N, rows, cap);
-      if (e == cudaSuccess) e = backward(N, batch, rows, cap);
-      if (e == cudaSuccess)
-        e = launch_adam(N->p, N->g, N->m, N->v, N->pb, N->n_flat, N->step, lr, 0.9f, 0.999f, 1e-8f, cap);
-      if (e == cudaSuccess) e = launch_loss_total(N->loss_part, loss_blocks(rows), N->loss, N->step, cap);
+      if (e == cudaSuccess) e = backward(N, N->T, batch, rows, cap, &adam, &br);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(cap, br.sums[0], 0);  // joins both branches
       cudaGraph_t graph = nullptr;
       const cudaError_t e2 = cudaStreamEndCapture(cap, &graph);
       if (e == cudaSuccess) e = e2;
       if (e == cudaSuccess) e = cudaGraphInstantiate(&N->exec, graph, 0);
       if (graph) cudaGraphDestroy(graph);
     }
-    cudaStreamDestroy(cap);
+    for (cudaEvent_t *v : evs)
+      if (*v) cudaEventDestroy(*v);
+    for (cudaStream_t q : {cap, br.w, br.c})
+      if (q) cudaStreamDestroy(q);
     if (e != cudaSuccess) {
       N->exec = nullptr;
       return cuda_fail(e, "training graph");

@@ -334,3 +334,51 @@ def test_adam_step_matches_oracle(ctx):
         assert moved.mean() > 0.9
     finally:
         pc.pc_mlp_destroy(net)
+
+
+@pytest.mark.parametrize("widths,batch", [([16, 5], 1), ([16, 64, 5], 255), ([3, 64, 128, 64, 1], 257),
+                                          ([16] + [64] * 7 + [5], 1023), (WIDTHS, 4096)])
+def test_training_sums_at_the_edges_of_their_chunks(ctx, widths, batch):
+    """One to eight layers and row counts around the 64-row and 256-row
+    chunks of the gradient sums: a training step (its branches: weight
+    gradients, bias sums and updates beside the data gradients) equals Adam
+    on pc_mlp_gradients of the same rows to FP32 rounding (the tolerance of
+    test_adam_step_matches_oracle), the gradients match the oracle (the
+    tolerance of test_gradients_match_oracle), and three replays equal three
+    calls bit for bit."""
+    from oracle.paths import philox4x32_10, split_seed
+    rng = np.random.default_rng(batch)
+    params = mlp.init(widths, rng)
+    n_data, seed, lr = 5000, 77, 1e-3
+    x = rng.normal(size=(n_data, widths[0])).astype(np.float32)
+    t = rng.normal(size=(n_data, widths[-1])).astype(np.float32)
+    w = np.linspace(0.5, 1.5, widths[-1]).astype(np.float32)
+    idx = (philox4x32_10([np.arange(batch, dtype=np.uint64), np.uint64(0), np.uint64(0), np.uint64(0)],
+                         split_seed(seed))[0] % np.uint64(n_data)).astype(np.int64)
+    net = pc.pc_mlp_create(ctx, widths, batch)
+    try:
+        p0 = flat(params)
+        pc.pc_mlp_set_params(net, p0)
+        xg, tg = torch.tensor(x[idx], device="cuda"), torch.tensor(t[idx], device="cuda")
+        dg = torch.full((p0.size,), float("nan"), dtype=torch.float32, device="cuda")
+        loss = pc.pc_mlp_gradients(net, xg.data_ptr(), tg.data_ptr(), w, batch, dg.data_ptr())
+        g = unflat(dg.double().cpu().numpy(), widths)
+        L, grads = mlp.backward(rounded(params), bf16(x[idx]), t[idx].astype(np.float64), w.astype(np.float64))
+        assert loss == pytest.approx(L, rel=1e-2)
+        for l, ((gW, gb), (rW, rb)) in enumerate(zip(g, grads)):
+            assert_close_el(gW, rW, 8.0, np.sqrt(np.mean(rW ** 2)), f"dW{l}")
+            assert_close_el(gb, rb, 8.0, np.sqrt(np.mean(rb ** 2)), f"db{l}")
+        dx, dt = torch.tensor(x, device="cuda"), torch.tensor(t, device="cuda")
+        got = []
+        for calls, steps in ((3, 1), (1, 3)):
+            pc.pc_mlp_set_params(net, p0)
+            for i in range(calls):
+                pc.pc_mlp_train(net, dx.data_ptr(), dt.data_ptr(), n_data, w, batch, steps, lr, seed)
+                if calls == 3 and i == 0:
+                    one = pc.pc_mlp_get_params(net).astype(np.float64)
+            got.append(pc.pc_mlp_get_params(net))
+        np.testing.assert_array_equal(got[0], got[1])
+        want = flat(mlp.adam(unflat(p0.astype(np.float64), widths), g, {}, lr)).astype(np.float64)
+        assert np.max(np.abs(one - want) - (2e-6 * lr + 2.0 ** -22 * np.abs(want))) <= 0
+    finally:
+        pc.pc_mlp_destroy(net)
