@@ -20,7 +20,7 @@ float *mlp_scratch(struct ::pc_mlp *net, size_t floats);
 bool mlp_cv_tables_tc(struct ::pc_mlp *net, size_t rows, float *tables, float *delta0, CvTablesTc &t);
 // Waits for the context's stream; PC_ETIMEOUT (and the status cleared) if a
 // tensor-core product of the network reported an expired wait.
-pc_status mlp_status(struct ::pc_mlp *net);
+pc_status mlp_status(struct ::pc_mlp *net, double *loss = nullptr);
 // The network's forward on a given stream (capturable), and what a
 // captured table build needs: the slot of its graph by key (created empty),
 // the network's pinned read-back buffer [8] (null if none), its status word.

@@ -224,7 +224,7 @@ __global__ void gather_kernel(const float *x, const float *t, size_t n_data, int
 // Weighted squared error; rows of kRow columns, thread (tid / 64, tid % 64)
 // of block k takes rows 4 k + tid / 64, + 4 gridDim, ... of its column, four
 // at a time so that their loads overlap.
-__global__ void loss_kernel(const float *Y, const float *T, const float *w, size_t n, int fout,
+__global__ void loss_kernel(const float *Y, const float *T, const LossWeights w, size_t n, int fout,
                             size_t rows, __nv_bfloat16 *dY, float *part) {
   __shared__ float red[32];
   float acc = 0.f;
@@ -232,7 +232,7 @@ __global__ void loss_kernel(const float *Y, const float *T, const float *w, size
   const int c = int(threadIdx.x) & (kRow - 1);
   const size_t step = size_t(gridDim.x) * (blockDim.x / kRow);
   const bool col = c < fout;
-  const float wc = col ? w[c] : 0.f;
+  const float wc = w.w[c];
   for (size_t r0 = blockIdx.x * size_t(blockDim.x / kRow) + threadIdx.x / kRow; r0 < rows; r0 += 4 * step) {
     float y[4], t[4];
 #pragma unroll
@@ -359,7 +359,12 @@ __global__ void __launch_bounds__(256) layer_grad_kernel(const LayerGrad g, cons
     i = g.count + size_t(col);
   }
   if (!ADAM) {
-    g.out[i] = s;
+    if (i < g.count) {
+      const unsigned r = unsigned(i) / unsigned(g.in_w), c = unsigned(i) % unsigned(g.in_w);
+      if (r < unsigned(g.w_out) && c < unsigned(g.w_in)) g.out[size_t(r) * g.w_in + c] = s;
+    } else if (i - g.count < size_t(g.w_out)) {
+      g.out[size_t(g.w_out) * g.w_in + (i - g.count)] = s;
+    }
     return;
   }
   const float b1 = a.b1, b2 = a.b2, c1 = a.consts[0], c2 = a.consts[1];
@@ -438,7 +443,7 @@ cudaError_t launch_gather(const float *x, const float *t, size_t n_data, int fin
 
 int loss_blocks(size_t rows) { return int(grid_for(rows * kRow, 256, 512)); }
 
-cudaError_t launch_loss(const float *Y, int ldy, const float *T, const float *w, size_t n, int fout,
+cudaError_t launch_loss(const float *Y, int ldy, const float *T, const LossWeights &w, size_t n, int fout,
                         size_t rows, __nv_bfloat16 *dY, int ldd, float *part, int blocks, cudaStream_t s) {
   if (ldy != kRow || ldd != kRow) return cudaErrorInvalidValue;
   loss_kernel<<<blocks, 256, 0, s>>>(Y, T, w, n, fout, rows, dY, part);

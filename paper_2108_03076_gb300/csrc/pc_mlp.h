@@ -115,22 +115,28 @@ cudaError_t launch_gather(const float *x, const float *t, size_t n_data, int fin
 // Weighted squared-error loss of Y [rows, ldy] (FP32) against T [n, fout]:
 // dY = (2 / n) w (Y - T) as BF16 [rows, ldd] (zero beyond n rows / fout
 // columns), per-block loss partials into part[blocks].
-cudaError_t launch_loss(const float *Y, int ldy, const float *T, const float *w, size_t n, int fout,
+struct LossWeights {
+  float w[64];
+};
+cudaError_t launch_loss(const float *Y, int ldy, const float *T, const LossWeights &w, size_t n, int fout,
                         size_t rows, __nv_bfloat16 *dY, int ldd, float *part, int blocks,
                         cudaStream_t s);
 int loss_blocks(size_t rows);
 // Column sums of dZ [rows, ld] (BF16), columns < cols (a multiple of 64), over
 // chunks of 256 rows in row order: scratch[chunk][cols].
 cudaError_t launch_colsum(const __nv_bfloat16 *dZ, size_t rows, int ld, int cols, float *scratch, cudaStream_t s);
-// A layer's gradient from its partials: out[i] = sum_z part[z * count + i] in
-// order (z < splits, i < count: the weights), then out[count + c] = the sum
-// of colpart[chunk][c] in order (c < cols: the biases; a multiple of 32).
+// A layer's gradient from its partials: element i = sum_z part[z * count + i]
+// in order (z < splits; the weights, i < count = cols * in_w, row-major),
+// then the sums of colpart[chunk][c] in order (c < cols: the biases; a
+// multiple of 32), written to `out` without the padding: w_out rows of w_in
+// weights, then w_out biases.
 struct LayerGrad {
   const float *part;
   int splits;
   size_t count;
   const float *colpart;
   int cols;
+  int in_w, w_in, w_out;
   float *out;
   int chunks;                   // set by the launcher, as w_blocks
   unsigned w_blocks;

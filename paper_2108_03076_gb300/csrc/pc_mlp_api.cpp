@@ -44,7 +44,7 @@ struct pc_mlp {
   __nv_bfloat16 *X = nullptr;
   std::vector<__nv_bfloat16 *> H;   // hidden activations, layers 0..L-2
   __nv_bfloat16 *dZ[2] = {nullptr, nullptr};
-  float *Y = nullptr, *T = nullptr, *wts = nullptr;
+  float *Y = nullptr, *T = nullptr;
   float *part[2] = {nullptr, nullptr};  // weight-gradient partials of consecutive layers in turn
   float *colscr = nullptr, *loss_part = nullptr, *adam_c = nullptr;
   size_t part_cap = 0;
@@ -63,7 +63,7 @@ struct pc_mlp {
   int32_t gemm = PC_MLP_GEMM_AUTO;  // product kernel choice (pc_mlp_set_gemm)
   bool tc_ok = false;               // tcgen05 products available on this device
   std::map<uint64_t, TcMaps> tc_maps;  // operand descriptors by (product kind, layer, rows)
-  float *h_pin = nullptr;             // pinned [8]: read-back of captured table builds
+  float *h_pin = nullptr;             // pinned [12]: read-back of captured table builds [8], loss and status [4]
   std::vector<std::pair<std::vector<uint8_t>, cudaGraphExec_t>> graphs;  // captured table builds
 };
 
@@ -82,11 +82,16 @@ float *mlp_scratch(pc_mlp *N, size_t floats) {
   return N->scratch;
 }
 
-pc_status mlp_status(pc_mlp *N) {
-  int32_t st = 0;
-  CU(cudaMemcpyAsync(&st, N->dstatus, sizeof(st), cudaMemcpyDeviceToHost, N->ctx->stream), "status copy");
+// Waits for the stream's work; the loss (when wanted) and the products'
+// status come back in one copy to pinned memory.
+pc_status mlp_status(pc_mlp *N, double *loss) {
+  double own[2], *h = N->h_pin ? reinterpret_cast<double *>(N->h_pin + 8) : own;
+  CU(cudaMemcpyAsync(h, N->loss, sizeof(own), cudaMemcpyDeviceToHost, N->ctx->stream), "status copy");
   pc_status r = wait_stream(N->ctx);
   if (r != PC_OK) return r;
+  int32_t st = 0;
+  std::memcpy(&st, h + 1, sizeof(st));
+  if (loss) *loss = h[0];
   if (st == 0) return PC_OK;
   CU(cudaMemsetAsync(N->dstatus, 0, sizeof(st), N->ctx->stream), "status reset");
   wait_stream(N->ctx);
@@ -171,14 +176,13 @@ size_t layout(pc_mlp *N, size_t rows) {
   N->dZ[1] = c.take<__nv_bfloat16>(rows * widest);
   N->Y = c.take<float>(rows * N->wp[N->L]);
   N->T = c.take<float>(rows * N->wp[N->L]);
-  N->wts = c.take<float>(kPad);
   for (float *&q : N->part) q = c.take<float>(part);
   N->colscr = c.take<float>(chunks * widest);
   N->adam_c = c.take<float>(2);
   N->loss_part = c.take<float>(512);
-  N->loss = c.take<double>(1);
+  N->loss = c.take<double>(2);  // the loss, then the products' status word
   N->step = c.take<uint64_t>(1);
-  N->dstatus = c.take<int32_t>(1);
+  N->dstatus = reinterpret_cast<int32_t *>(N->loss + 1);
   return c.off;
 }
 
@@ -243,6 +247,13 @@ cudaError_t forward(pc_mlp *N, size_t rows, cudaStream_t s) {
   return cudaSuccess;
 }
 
+// First parameter of layer l in the unpadded layout.
+size_t real_offset(const pc_mlp *N, int l) {
+  size_t k = 0;
+  for (int j = 0; j < l; ++j) k += size_t(N->w[j + 1]) * (N->w[j] + 1);
+  return k;
+}
+
 // A training step's branches beside the main one, under stream capture: `w`
 // the weight-gradient products, `c` the bias sums and each layer's gradient
 // sums with the update.  The main branch is the chain forward -> loss ->
@@ -261,17 +272,17 @@ cudaError_t signal(cudaEvent_t ev, cudaStream_t from, cudaStream_t to) {
 }
 
 // Loss on the first n of `rows` rows (targets t, [n][outputs]), gradients into
-// g; with `adam` (p, m, v, pb at the flat arrays' starts) the parameters are
+// `grads` (the unpadded layout); with `adam` (p, m, v, pb at the flat arrays' starts) the parameters are
 // updated instead.  With branches a layer's weight gradient, and the sums
 // and update of the layer before, run beside its data gradient, so a step's
 // critical path is one product a layer.  Layer l's update waits for its data
 // gradient, which reads the weights; the data gradient that reuses a signal
 // buffer waits for the reads of its former contents.
-cudaError_t backward(pc_mlp *N, const float *t, size_t n, size_t rows, cudaStream_t s, const AdamStep *adam = nullptr,
-                     const Branches *br = nullptr) {
+cudaError_t backward(pc_mlp *N, const float *t, const LossWeights &lw, size_t n, size_t rows, cudaStream_t s,
+                     float *grads, const AdamStep *adam = nullptr, const Branches *br = nullptr) {
   const int fout = N->w[N->L];
   const int lb = loss_blocks(rows);
-  cudaError_t e = launch_loss(N->Y, N->wp[N->L], t, N->wts, n, fout, rows, N->dZ[0], N->wp[N->L],
+  cudaError_t e = launch_loss(N->Y, N->wp[N->L], t, lw, n, fout, rows, N->dZ[0], N->wp[N->L],
                               N->loss_part, lb, s);
   if (e != cudaSuccess) return e;
   const cudaStream_t sw = br ? br->w : s, sc = br ? br->c : s;
@@ -338,7 +349,10 @@ cudaError_t backward(pc_mlp *N, const float *t, size_t n, size_t rows, cudaStrea
     lg.count = size_t(out_w) * in_w;
     lg.colpart = N->colscr;
     lg.cols = out_w;
-    lg.out = N->g + N->offW[l];
+    lg.in_w = in_w;
+    lg.w_in = N->w[l];
+    lg.w_out = N->w[l + 1];
+    if (!adam) lg.out = grads + real_offset(N, l);
     AdamStep step{};
     if (adam) {
       step = *adam;
@@ -392,11 +406,10 @@ pc_status copy_unpadded(pc_mlp *N, const float *src, float *dst, cudaMemcpyKind 
   return PC_OK;
 }
 
-pc_status set_weights(pc_mlp *N, const float *w) {
-  float h[kPad] = {0};
-  for (int j = 0; j < N->w[N->L]; ++j) h[j] = w[j];
-  CU(cudaMemcpyAsync(N->wts, h, sizeof(h), cudaMemcpyHostToDevice, N->ctx->stream), "loss weights");
-  return PC_OK;
+LossWeights loss_weights(const pc_mlp *N, const float *w) {
+  LossWeights lw{};
+  for (int j = 0; j < N->w[N->L]; ++j) lw.w[j] = w[j];
+  return lw;
 }
 
 }  // namespace
@@ -503,7 +516,7 @@ pc_status pc_mlp_create(pc_ctx *c, const int32_t *widths, int32_t n_widths, uint
   cudaMemsetAsync(N->mem, 0, bytes, c->stream);
   N->tc_ok = gemm_tc_init() == cudaSuccess;
   cudaGetLastError();
-  if (cudaHostAlloc(reinterpret_cast<void **>(&N->h_pin), 8 * sizeof(float), 0) != cudaSuccess) {
+  if (cudaHostAlloc(reinterpret_cast<void **>(&N->h_pin), 12 * sizeof(float), 0) != cudaSuccess) {
     N->h_pin = nullptr;
     cudaGetLastError();
   }
@@ -571,18 +584,14 @@ pc_status pc_mlp_gradients(pc_mlp *N, const float *d_x, const float *d_t, const 
   cudaStream_t s = N->ctx->stream;
   CU(cudaSetDevice(N->ctx->device), "cudaSetDevice");
   const size_t rows = rows_for(n);
-  pc_status st = set_weights(N, w);
-  if (st != PC_OK) return st;
   CU(launch_to_bf16(d_x, n, N->w[0], N->X, rows, N->wp[0], s), "input");
   CU(forward(N, rows, s), "forward");
-  CU(backward(N, d_t, n, rows, s), "backward");
+  CU(backward(N, d_t, loss_weights(N, w), n, rows, s, d_grads ? d_grads : N->g), "backward");
   CU(launch_loss_total(N->loss_part, loss_blocks(rows), N->loss, nullptr, s), "loss");
-  if (d_grads) {
-    st = copy_unpadded(N, N->g, d_grads, cudaMemcpyDeviceToDevice);
-    if (st != PC_OK) return st;
-  }
-  CU(cudaMemcpyAsync(out_loss, N->loss, sizeof(double), cudaMemcpyDeviceToHost, s), "loss copy");
-  return mlp_status(N);
+  double loss = 0.0;
+  const pc_status st = mlp_status(N, &loss);
+  if (st == PC_OK) *out_loss = loss;
+  return st;
 }
 
 pc_status pc_mlp_train(pc_mlp *N, const float *d_x, const float *d_t, size_t n_data, const float *w,
@@ -599,9 +608,7 @@ pc_status pc_mlp_train(pc_mlp *N, const float *d_x, const float *d_t, size_t n_d
   if (!same) {
     if (N->exec) cudaGraphExecDestroy(N->exec);
     N->exec = nullptr;
-    pc_status st = set_weights(N, w);
-    if (st != PC_OK) return st;
-    st = wait_stream(c);
+    pc_status st = wait_stream(c);
     if (st != PC_OK) return st;
     cudaStream_t cap = nullptr;
     Branches br;
@@ -625,7 +632,7 @@ pc_status pc_mlp_train(pc_mlp *N, const float *d_x, const float *d_t, size_t n_d
         e = launch_gather(d_x, d_t, n_data, N->w[0], N->w[N->L], N->step, uint32_t(seed), uint32_t(seed >> 32),
                           batch, N->X, N->wp[0], N->T, cap);
       if (e == cudaSuccess) e = forward(N, rows, cap);
-      if (e == cudaSuccess) e = backward(N, N->T, batch, rows, cap, &adam, &br);
+      if (e == cudaSuccess) e = backward(N, N->T, loss_weights(N, w), batch, rows, cap, nullptr, &adam, &br);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(cap, br.sums[0], 0);  // joins both branches
       cudaGraph_t graph = nullptr;
       const cudaError_t e2 = cudaStreamEndCapture(cap, &graph);
@@ -650,9 +657,10 @@ pc_status pc_mlp_train(pc_mlp *N, const float *d_x, const float *d_t, size_t n_d
     N->g_w = wv;
   }
   for (int32_t i = 0; i < steps; ++i) CU(cudaGraphLaunch(N->exec, c->stream), "training step");
-  CU(cudaMemcpyAsync(out_loss, N->loss, sizeof(double), cudaMemcpyDeviceToHost, c->stream), "loss copy");
-  pc_status st = mlp_status(N);
+  double loss = 0.0;
+  pc_status st = mlp_status(N, &loss);
   if (st != PC_OK) return st;
+  *out_loss = loss;
   N->steps += uint64_t(steps);
   return PC_OK;
 }
