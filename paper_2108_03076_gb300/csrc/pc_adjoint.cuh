@@ -89,12 +89,16 @@ __device__ float2 eval_adjoint(const uint4 *P, const float *pool, float2 *R, con
                                const Rng2 &g, bool live0, bool live1, const float (&Bm)[D * D],
                                const float (&S0)[D], const float (&Lm)[D * D], Tape &T, int &res) {
 #include "pc_adjoint_state.inc"
+#define ENSURE(o) ensure(o)
+#define NEXT_INSN P[pc + 1]
   for (;;) {
     const uint4 I = P[pc];
     const uint32_t op = I.x & 0xffu;
     const float kk = __uint_as_float(I.y);
 #include "pc_adjoint_ops.inc"
   }
+#undef ENSURE
+#undef NEXT_INSN
 }
 
 // Reverse sweep of one tile's tape: the per-path derivatives of the result
@@ -144,13 +148,10 @@ __device__ __forceinline__ void adjoint_tiles(const PriceArgs &a, const TapeArgs
   constexpr int V = 1 + 2 * D, W = 2 * V;
   extern __shared__ __align__(16) uint32_t smem[];
   __shared__ int last_block;
-  uint4 *P = reinterpret_cast<uint4 *>(smem);
-  const int prog_words = a.n_insn * 4 + a.n_pool;
-  const uint32_t *src = reinterpret_cast<const uint32_t *>(a.prog);
-  for (int i = threadIdx.x; i < prog_words; i += blockDim.x) smem[i] = src[i];
-  __syncthreads();
-  const float *pool = reinterpret_cast<const float *>(smem + a.n_insn * 4);
-  float2 *R = reinterpret_cast<float2 *>(smem + prog_words) + threadIdx.x;
+  const Staged st = stage_program(a, smem);
+  const uint4 *P = st.P;
+  const float *pool = st.pool;
+  float2 *R = warp_region(st.regions, layout_of(a).words);
   const float(&Bm)[D * D] = *reinterpret_cast<const float(*)[D * D]>(a.m.Bv);
   const float(&S0)[D] = *reinterpret_cast<const float(*)[D]>(a.m.S0v);
   float Lm[D * D];
@@ -167,9 +168,7 @@ __device__ __forceinline__ void adjoint_tiles(const PriceArgs &a, const TapeArgs
   T.status = a.status;
   unsigned long long *ctr = reinterpret_cast<unsigned long long *>(a.control);
   Rng2 g;
-  g.stream = a.stream;
-#pragma unroll
-  for (int i = 0; i < 20; ++i) g.rk[i] = a.rk[i];
+  rng_init(g, a.rk, a.stream, a.path_offset);
   for (;;) {
     unsigned long long tile = 0;
     if (lane == 0) tile = atomicAdd(ctr, 1ull);
@@ -178,10 +177,8 @@ __device__ __forceinline__ void adjoint_tiles(const PriceArgs &a, const TapeArgs
     const uint64_t i0 = tile * kTilePaths + lane, i1 = i0 + 32;
     const bool live0 = i0 < a.n_paths, live1 = i1 < a.n_paths;
     const uint64_t p0 = a.path_offset + i0, p1 = a.path_offset + i1;
-    g.plo[0] = uint32_t(p0);
-    g.phi[0] = uint32_t(p0 >> 32);
-    g.plo[1] = uint32_t(p1);
-    g.phi[1] = uint32_t(p1 >> 32);
+    rng_path(g, 0, p0, a.path_offset);
+    rng_path(g, 1, p1, a.path_offset);
     T.n = 0;
     int res = -1;
     const float2 x = eval(P, pool, R, g, live0, live1, Bm, S0, Lm, T, res);

@@ -93,12 +93,7 @@ pc_status run_adjoint(const pc_model *m, const pc_contract *k, uint64_t n_paths,
   PriceArgs a = L.args;
   a.lay = lay;
   a.width = width;
-  reduction_chunks(a.n_tiles, a.chunk_tiles, a.n_chunks);
-  const uint32_t max_chunks = uint32_t(kMaxChunks * 8 / width);
-  if (a.n_chunks > max_chunks) {
-    a.chunk_tiles = uint32_t((a.n_tiles + max_chunks - 1) / max_chunks);
-    a.n_chunks = uint32_t((a.n_tiles + a.chunk_tiles - 1) / a.chunk_tiles);
-  }
+  reduction_chunks(a, uint32_t(kMaxChunks * 8 / width));
   s = ensure_partials(c, size_t(a.n_tiles) * size_t(width));
   if (s != PC_OK) return s;
   a.tile_partials = c->d_partials;
@@ -110,14 +105,18 @@ pc_status run_adjoint(const pc_model *m, const pc_contract *k, uint64_t n_paths,
     // the program's run-time specialised adjoint kernel (same arguments,
     // block and tape regions; at most the interpreter's grid)
     cudaKernel_t jk = nullptr;
-    s = jit_kernel(k, d, kJitAdjoint + (d_paths ? 1 : 0), block, jk);
+    PriceArgs ja = a;
+    if (!L.walk->empty()) drop_bridge_stack(ja.lay);
+    s = jit_kernel(k, jit_spec(k, ja, kJitAdjoint + (d_paths ? 1 : 0), 0, *L.walk), jk);
     if (s != PC_OK) return s;
     const void *kern = reinterpret_cast<const void *>(jk);
     int nb = 0;
+    smem = price_smem_bytes(0, 0, ja.lay.words, block);
     CU(jit_occupancy(c, kern, block, smem, nb), "jit occupancy");
     if (nb >= 1) {
       const int jgrid = std::min(grid, c->sm_count * nb);
-      void *args[] = {&a, &t};
+      StaticGrid sg = static_grid(H, *L.walk);
+      void *args[] = {&ja, &t, &sg};
       CU(cudaLaunchKernel(kern, dim3(jgrid), dim3(block), args, smem, c->stream), "specialised adjoint kernel");
       return PC_OK;
     }

@@ -76,6 +76,7 @@ struct pc_batch {
     int grid = 0, block = 0;
     size_t smem = 0;
     PriceArgs args{};
+    StaticGrid sg{};
   };
   std::vector<JitItem> jit;
   std::vector<char> is_jit;
@@ -243,7 +244,6 @@ pc_status choose_jit(pc_batch *B, const pc_model *const *models, const pc_contra
     Launch L;
     int wk;
     size_t smem;
-    int min_blocks;
   };
   std::vector<Cand> cand;
   std::vector<JitRequest> reqs;
@@ -257,9 +257,8 @@ pc_status choose_jit(pc_batch *B, const pc_model *const *models, const pc_contra
     if (s != PC_OK) return s;
     cd.wk = jit_window_kind(c, cd.L);
     if (cd.wk & kJitHbm) continue;
-    cd.smem = jit_layout(c, contracts[i], cd.L, cd.wk);
-    cd.min_blocks = jit_min_blocks(c, cd.smem, cd.L.block);
-    reqs.push_back({contracts[i], models[i]->H.d, kJitPrice | cd.wk, cd.L.block, cd.min_blocks});
+    cd.smem = jit_layout(c, cd.L, cd.wk);
+    reqs.push_back({contracts[i], jit_price_spec(c, contracts[i], cd.L, kJitPrice | cd.wk, cd.smem)});
     cand.push_back(cd);
     est += cost(i);
   }
@@ -271,7 +270,7 @@ pc_status choose_jit(pc_batch *B, const pc_model *const *models, const pc_contra
     const int wk = cd.wk;
     const size_t smem = cd.smem;
     cudaKernel_t jk = nullptr;
-    pc_status s = jit_kernel(contracts[i], models[i]->H.d, kJitPrice | wk, L.block, jk, cd.min_blocks);
+    pc_status s = jit_kernel(contracts[i], jit_price_spec(c, contracts[i], L, kJitPrice | wk, smem), jk);
     if (s != PC_OK) return s;
     int nb = 0;
     CU(jit_occupancy(c, reinterpret_cast<const void *>(jk), L.block, smem, nb), "jit occupancy");
@@ -286,6 +285,7 @@ pc_status choose_jit(pc_batch *B, const pc_model *const *models, const pc_contra
     J.grid = int(std::max<uint64_t>(1, std::min<uint64_t>(uint64_t(c->sm_count) * nb, (units + wpb - 1) / wpb)));
     J.args = B->items[i];
     J.args.lay = L.args.lay;
+    J.sg = static_grid(models[i]->H, *L.walk);
     B->jit.push_back(J);
     B->is_jit[i] = 1;
   }
@@ -304,7 +304,8 @@ pc_status choose_jit(pc_batch *B, const pc_model *const *models, const pc_contra
 // One specialised contract's launch (its PriceArgs by value).
 cudaError_t launch_jit_item(const pc_batch::JitItem &J, cudaStream_t st) {
   PriceArgs a = J.args;
-  void *args[] = {&a};
+  StaticGrid sg = J.sg;
+  void *args[] = {&a, &sg};
   return cudaLaunchKernel(reinterpret_cast<const void *>(J.kern), dim3(J.grid), dim3(J.block), args, J.smem, st);
 }
 
@@ -332,6 +333,7 @@ pc_status capture(pc_batch *B) {
     a.units = B->d_units + g.u0;
     a.n_units = g.n_units;
     a.slot_bytes = uint32_t(g.slot);
+    a.words = g.words;
     a.counter = reinterpret_cast<unsigned long long *>(B->d_zero) + gi;
     e = cudaStreamWaitEvent(B->aux[gi], B->fork, 0);
     if (e == cudaSuccess) e = launch_batch(a, g.d, g.grid, g.block, g.smem, B->aux[gi]);
@@ -390,6 +392,7 @@ pc_status launch_direct(pc_batch *B) {
     a.units = B->d_units + g.u0;
     a.n_units = g.n_units;
     a.slot_bytes = uint32_t(g.slot);
+    a.words = g.words;
     a.counter = reinterpret_cast<unsigned long long *>(B->d_zero) + gi;
     CU(cudaStreamWaitEvent(c->batch_aux[gi], c->batch_fork, 0), "fork wait");
     CU(launch_batch(a, g.d, g.grid, g.block, g.smem, c->batch_aux[gi]), "batch kernel");
@@ -443,7 +446,7 @@ pc_status create(size_t n, const pc_model *const *models, const pc_contract *con
     if (s != PC_OK) return fail(s, "contract " + std::to_string(i) + ": " + pc_last_error(nullptr));
     PriceArgs &a = L.args;
     a.width = 2;
-    reduction_chunks(a.n_tiles, a.chunk_tiles, a.n_chunks);
+    reduction_chunks(a);
     B->d[i] = models[i]->H.d;
     B->words[i] = a.lay.words;
     B->tile_cost[i] = estimate_tile_cost(a, B->d[i]);

@@ -151,22 +151,54 @@ int32_t max_label(const Program &p) {
   return top;
 }
 
-pc_status window_for(const pc_model *m, const pc_contract *k, int32_t &win) {
+// The contract's window and static walks on the model (kept by the contract;
+// `out` stays valid as long as it does).
+pc_status window_for(const pc_model *m, const pc_contract *k, const pc_contract::Window *&out) {
   auto *kc = const_cast<pc_contract *>(k);
   std::lock_guard<std::mutex> g(kc->mu);
-  auto key = std::make_pair(m->id, uint64_t(0));
-  auto it = kc->win_cache.find(key);
-  if (it != kc->win_cache.end()) { win = it->second; return PC_OK; }
+  auto it = kc->win_cache.find(m->id);
+  if (it != kc->win_cache.end() && (it->second.with_walks || !k->ctx->jit)) {
+    out = &it->second;
+    return PC_OK;
+  }
   // labels must exist in the model
   const int32_t top = max_label(k->prog);
   if (top >= m->H.d)
     return fail(PC_ERANGE, "program observes label " + std::to_string(top) + " but the model has " +
                                std::to_string(m->H.d) + " underlyings");
   std::string err;
-  pc_status s = analyse_program(k->prog, m->H.t_now, m->H.n, m->H.n_hist, win, err);
+  pc_contract::Window w;
+  std::vector<uint8_t> reads;
+  pc_status s = analyse_program(k->prog, m->H.t_now, m->H.n, m->H.n_hist, w.win, reads, err);
   if (s != PC_OK) return fail(s, err);
-  kc->win_cache[key] = win;
+  if (k->ctx->jit && walk_jit_eligible(k->prog)) {
+    w.walk = static_walk(m->H, reads);
+    if (m->H.n <= kStaticOps) w.walk_all = static_walk(m->H, std::vector<uint8_t>(size_t(m->H.n) + 1, 1));
+    if (!w.walk.empty() && !admit_walk(k->ctx, k->prog, m->H, w.walk)) {
+      w.walk.clear();
+      w.walk_all.clear();
+    }
+  }
+  w.with_walks = k->ctx->jit != 0;
+  out = &(kc->win_cache[m->id] = std::move(w));
   return PC_OK;
+}
+
+StaticGrid static_grid(const ModelHost &H, const std::vector<int32_t> &walk) {
+  StaticGrid g{};
+  int step = 0, idx = 0;
+  for (size_t i = 0; i < walk.size(); ++step) {
+    const int date = walk[i], ops = walk[i + 2];
+    i += 3;
+    for (int l = 0; l < H.d; ++l) g.A[step][l] = H.A[size_t(date) * H.d + l].x;
+    for (int j = 0; j < ops; ++j, ++i, ++idx) {
+      const BridgeOp &op = H.ops[size_t(walk[i])];
+      g.wl[idx] = make_float2(op.wl, op.wl);
+      g.wr[idx] = make_float2(op.wr, op.wr);
+      g.sd[idx] = make_float2(op.sd, op.sd);
+    }
+  }
+  return g;
 }
 
 // Block size (128, 64 or 32 threads) that keeps the most warps resident per
@@ -195,9 +227,12 @@ pc_status prepare(const pc_model *m, const pc_contract *k, uint64_t n_paths, uin
   if (m->ctx != k->ctx) return fail(PC_EINVAL, "model and contract belong to different contexts");
   if (n_paths == 0) return fail(PC_EINVAL, "n_paths must be >= 1");
   if (n_paths > (uint64_t(1) << 40)) return fail(PC_ELIMIT, "n_paths exceeds 2^40");
-  int32_t win = 1;
-  pc_status s = window_for(m, k, win);
+  const pc_contract::Window *w = nullptr;
+  pc_status s = window_for(m, k, w);
   if (s != PC_OK) return s;
+  const int32_t win = w->win;
+  L.walk = &w->walk;
+  L.walk_all = &w->walk_all;
   pc_ctx *c = m->ctx;
   const int mode = allow_hbm ? c->window_mode : PC_WINDOW_SHARED;
   Layout lay = make_layout(k->prog, m->H, win);
@@ -270,6 +305,16 @@ pc_status bind_hbm_window(pc_ctx *c, Launch &L, int d) {
   return PC_OK;
 }
 
+// A static walk keeps the bridge stack in registers: its slots leave the
+// per-thread region.
+void drop_bridge_stack(Layout &lay) {
+  const int n = lay.off_cache - lay.off_bstack;
+  lay.off_cache -= n;
+  lay.off_win -= n;
+  lay.off_xwin -= n;
+  lay.words -= n;
+}
+
 // Sensitivity launch for underlying `label`: the pricing launch set-up with
 // three physical slots per program value and an extra window of X = L W.
 pc_status run_greeks(const pc_model *m, const pc_contract *k, uint64_t n_paths, uint64_t offset,
@@ -300,7 +345,7 @@ pc_status run_greeks(const pc_model *m, const pc_contract *k, uint64_t n_paths, 
   PriceArgs a = L.args;
   a.lay = lay;
   a.width = 6;
-  reduction_chunks(a.n_tiles, a.chunk_tiles, a.n_chunks);
+  reduction_chunks(a);
   a.tile_partials = c->d_partials;
   a.control = c->d_control;
   a.out = d_out;
@@ -312,14 +357,17 @@ pc_status run_greeks(const pc_model *m, const pc_contract *k, uint64_t n_paths, 
     // the contract's run-time specialised tangent kernel (same arguments,
     // shared-memory layout and block)
     cudaKernel_t jk = nullptr;
-    s = jit_kernel(k, d, kJitGreeks + (d_paths != nullptr ? 1 : 0), block, jk);
+    if (!L.walk->empty()) drop_bridge_stack(a.lay);
+    s = jit_kernel(k, jit_spec(k, a, kJitGreeks + (d_paths != nullptr ? 1 : 0), 0, *L.walk), jk);
     if (s != PC_OK) return s;
     const void *kern = reinterpret_cast<const void *>(jk);
     int nb = 0;
+    smem = price_smem_bytes(0, 0, a.lay.words, block);
     CU(jit_occupancy(c, kern, block, smem, nb), "jit occupancy");
     if (nb < 1) return fail(PC_ELIMIT, "specialised sensitivity kernel cannot be resident");
     const int jgrid = int(std::min<uint64_t>(uint64_t(c->sm_count) * nb, need));
-    void *args[] = {&a};
+    StaticGrid sg = static_grid(m->H, *L.walk);
+    void *args[] = {&a, &sg};
     CU(cudaLaunchKernel(kern, dim3(jgrid), dim3(block), args, smem, c->stream), "specialised sensitivity kernel");
     return PC_OK;
   }
@@ -338,7 +386,7 @@ int jit_window_kind(const pc_ctx *c, const Launch &L) {
   // automatic: two pairs where a path walks many dates (the daily barrier's
   // 365: 6.84 -> 6.49 ms at 2^22 paths); a few dates gain nothing (5 dates:
   // 0.069 ms either way), the tile loop and the reduction dominate there
-  const bool two = c->jit_pairs == 2 || (c->jit_pairs == 0 && L.args.m.n >= kJitPairsMinDates);
+  const bool two = c->jit_pairs == 2 || (c->jit_pairs == 0 && L.args.m.n >= kJitPairsMinDates && L.walk->empty());
   return kJitWinRegs | (two ? kJitPairs2 : 0);
 }
 
@@ -348,7 +396,7 @@ int jit_window_kind(const pc_ctx *c, const Launch &L) {
 // With two path pairs a lane the bridge stack holds both pairs' values per
 // level (twice the words), and the block is re-chosen for the most resident
 // warps that shared memory allows.
-size_t jit_layout(const pc_ctx *c, const pc_contract *k, Launch &L, int bits) {
+size_t jit_layout(const pc_ctx *c, Launch &L, int bits) {
   Layout &lay = L.args.lay;
   const int shift = lay.off_bstack;
   lay.stack = 0;
@@ -357,11 +405,16 @@ size_t jit_layout(const pc_ctx *c, const pc_contract *k, Launch &L, int bits) {
   lay.off_win -= shift;
   lay.words -= shift;
   if (bits & kJitWinRegs) lay.words = lay.off_win;
-  if (bits & kJitPairs2) {
+  if (!L.walk->empty()) {
+    drop_bridge_stack(lay);
+    L.block = kBlock;
+    while (L.block > 32 && price_smem_bytes(0, 0, lay.words, L.block) + kStaticSmemReserve > size_t(c->max_smem))
+      L.block /= 2;
+  } else if (bits & kJitPairs2) {
     lay.words = lay.off_bstack + 2 * (lay.off_cache - lay.off_bstack);
     int best = 0, best_warps = 0;
     for (int b = kBlock; b >= 32; b /= 2) {
-      const size_t sm = price_smem_bytes(k->prog.code.size(), pool_padded(k->prog), lay.words, b);
+      const size_t sm = price_smem_bytes(0, 0, lay.words, b);
       if (sm + kStaticSmemReserve > size_t(c->max_smem)) continue;
       const size_t per = sm + kJitStaticSmem + size_t(c->smem_reserve);
       const int blocks = c->sm_smem > 0 ? std::min<int>(32, int(size_t(c->sm_smem) / per)) : 1;
@@ -372,7 +425,12 @@ size_t jit_layout(const pc_ctx *c, const pc_contract *k, Launch &L, int bits) {
     }
     if (best) L.block = best;
   }
-  return price_smem_bytes(k->prog.code.size(), pool_padded(k->prog), lay.words, L.block);
+  return price_smem_bytes(0, 0, lay.words, L.block);
+}
+
+JitSpec jit_price_spec(const pc_ctx *c, const pc_contract *k, const Launch &L, int kind, size_t smem) {
+  const int bound = L.walk->empty() ? jit_min_blocks(c, smem, L.block) : kWalkMinBlocks;
+  return jit_spec(k, L.args, kind, bound, *L.walk);
 }
 
 // Resident blocks per SM (of kBlock threads, the block the kernel's bound
@@ -396,7 +454,7 @@ pc_status run_price(const pc_model *m, const pc_contract *k, uint64_t n_paths, u
   s = ensure_partials(c, size_t(L.args.n_tiles) * 2);
   if (s != PC_OK) return s;
   L.args.width = 2;
-  reduction_chunks(L.args.n_tiles, L.args.chunk_tiles, L.args.n_chunks);
+  reduction_chunks(L.args);
   L.args.tile_partials = c->d_partials;
   L.args.control = c->d_control;
   L.args.out = d_out;
@@ -406,9 +464,8 @@ pc_status run_price(const pc_model *m, const pc_contract *k, uint64_t n_paths, u
     // the contract's run-time specialised kernel (same arguments and shape)
     cudaKernel_t jk = nullptr;
     const int wk = jit_window_kind(c, L);
-    const size_t smem = jit_layout(c, k, L, wk);
-    s = jit_kernel(k, m->H.d, (d_payoffs != nullptr ? kJitPriceWrite : kJitPrice) | wk, L.block, jk,
-                   jit_min_blocks(c, smem, L.block));
+    const size_t smem = jit_layout(c, L, wk);
+    s = jit_kernel(k, jit_price_spec(c, k, L, (d_payoffs != nullptr ? kJitPriceWrite : kJitPrice) | wk, smem), jk);
     if (s != PC_OK) return s;
     const void *kern = reinterpret_cast<const void *>(jk);
     int nb = 0;
@@ -424,7 +481,8 @@ pc_status run_price(const pc_model *m, const pc_contract *k, uint64_t n_paths, u
       s = bind_hbm_window(c, L, m->H.d);
       if (s != PC_OK) return s;
     }
-    void *args[] = {&L.args};
+    StaticGrid sg = static_grid(m->H, *L.walk);
+    void *args[] = {&L.args, &sg};
     CU(cudaLaunchKernel(kern, dim3(grid), dim3(L.block), args, smem, c->stream), "specialised price kernel");
     return PC_OK;
   }
@@ -467,9 +525,9 @@ pc_status pc_price_noalloc(const pc_model *m, const pc_contract *k, uint64_t n_p
   {
     auto *kc = const_cast<pc_contract *>(k);
     std::lock_guard<std::mutex> g(kc->mu);
-    const auto it = kc->win_cache.find(std::make_pair(m->id, uint64_t(0)));
+    const auto it = kc->win_cache.find(m->id);
     if (it != kc->win_cache.end()) {
-      win = it->second;
+      win = it->second.win;
     } else {
       const char *why = "";
       auto on_fail = [&](pc_status st, int64_t, int64_t) {
@@ -511,7 +569,7 @@ pc_status pc_price_noalloc(const pc_model *m, const pc_contract *k, uint64_t n_p
   a.stream = stream;
   a.n_tiles = n_tiles;
   a.width = 2;
-  reduction_chunks(n_tiles, a.chunk_tiles, a.n_chunks);
+  reduction_chunks(a);
   a.control = static_cast<unsigned char *>(scratch);
   a.tile_partials = reinterpret_cast<double *>(static_cast<char *>(scratch) + kNoAllocCounterBytes);
   a.out = d_out;
@@ -663,7 +721,7 @@ pc_status pc_model_create(pc_ctx *c, const pc_model_desc *desc, pc_model **out) 
       return fail(s, err);
     }
     const ModelHost &H = m->H;
-    size_t bytes = padded(H.date_ops) + padded(H.ops) + padded(H.A) + padded(H.B) +
+    size_t bytes = padded(H.date_ops) + padded(H.ops) + padded(H.nodes) + padded(H.A) + padded(H.B) +
                    padded(H.disc) + padded(H.sval) + padded(H.tau) + padded(H.Lf) +
                    padded(H.sig) + 256;
     CU(cudaSetDevice(c->device), "cudaSetDevice");
@@ -678,6 +736,7 @@ pc_status pc_model_create(pc_ctx *c, const pc_model_desc *desc, pc_model **out) 
     pc_status u = PC_OK;
     if (u == PC_OK) u = upload(H.date_ops, base, off, D.date_ops, c->stream);
     if (u == PC_OK) u = upload(H.ops, base, off, D.ops, c->stream);
+    if (u == PC_OK) u = upload(H.nodes, base, off, D.nodes, c->stream);
     if (u == PC_OK) u = upload(H.A, base, off, D.A, c->stream);
     if (u == PC_OK) u = upload(H.B, base, off, D.B, c->stream);
     if (u == PC_OK) u = upload(H.disc, base, off, D.disc, c->stream);
@@ -1025,8 +1084,8 @@ pc_status pc_jit_compile(const pc_model *m, const pc_contract *k) {
   CU(cudaSetDevice(m->ctx->device), "cudaSetDevice");
   cudaKernel_t jk = nullptr;
   const int wk = jit_window_kind(m->ctx, L);
-  const size_t smem = jit_layout(m->ctx, k, L, wk);
-  return jit_kernel(k, m->H.d, kJitPrice | wk, L.block, jk, jit_min_blocks(m->ctx, smem, L.block));
+  const size_t smem = jit_layout(m->ctx, L, wk);
+  return jit_kernel(k, jit_price_spec(m->ctx, k, L, kJitPrice | wk, smem), jk);
 }
 
 pc_status pc_price_info(const pc_model *m, const pc_contract *k, uint64_t n_paths, pc_launch_info *info) {

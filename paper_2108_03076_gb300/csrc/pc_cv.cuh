@@ -200,21 +200,16 @@ __device__ __forceinline__ void cv_tiles(const PriceArgs &a, const CvArgs &c, EV
                  PILOT = (MODE & kCvPilot) != 0;
   extern __shared__ __align__(16) uint32_t smem[];
   __shared__ int last_block;
-  uint4 *P = reinterpret_cast<uint4 *>(smem);
-  const int prog_words = a.n_insn * 4 + a.n_pool;
-  const uint32_t *src = reinterpret_cast<const uint32_t *>(a.prog);
-  for (int i = threadIdx.x; i < prog_words; i += blockDim.x) smem[i] = src[i];
-  __syncthreads();
-  const float *pool = reinterpret_cast<const float *>(smem + a.n_insn * 4);
-  float2 *R = reinterpret_cast<float2 *>(smem + prog_words) + threadIdx.x;
+  const Staged st = stage_program(a, smem);
+  const uint4 *P = st.P;
+  const float *pool = st.pool;
+  float2 *R = warp_region(st.regions, layout_of(a).words);
   const float(&Bm)[D * D] = *reinterpret_cast<const float(*)[D * D]>(a.m.Bv);
   const float(&S0)[D] = *reinterpret_cast<const float(*)[D]>(a.m.S0v);
   const int lane = threadIdx.x & 31;
   unsigned long long *ctr = reinterpret_cast<unsigned long long *>(a.control);
   Rng2 g;
-  g.stream = a.stream;
-#pragma unroll
-  for (int i = 0; i < 20; ++i) g.rk[i] = a.rk[i];
+  rng_init(g, a.rk, a.stream, a.path_offset);
   for (;;) {
     unsigned long long tile = 0;
     if (lane == 0) tile = atomicAdd(ctr, 1ull);
@@ -223,10 +218,8 @@ __device__ __forceinline__ void cv_tiles(const PriceArgs &a, const CvArgs &c, EV
     const uint64_t i0 = tile * kTilePaths + lane, i1 = i0 + 32;
     const bool live0 = i0 < a.n_paths, live1 = i1 < a.n_paths;
     const uint64_t p0 = a.path_offset + i0, p1 = a.path_offset + i1;
-    g.plo[0] = uint32_t(p0);
-    g.phi[0] = uint32_t(p0 >> 32);
-    g.plo[1] = uint32_t(p1);
-    g.phi[1] = uint32_t(p1 >> 32);
+    rng_path(g, 0, p0, a.path_offset);
+    rng_path(g, 1, p1, a.path_offset);
     CvOnline<D, GAMMA> hg(c, a.m, S0);
     const float2 x = eval(P, pool, R, g, live0, live1, Bm, S0, &hg);
     const float(&Mv)[2] = hg.M;

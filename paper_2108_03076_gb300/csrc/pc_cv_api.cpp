@@ -107,7 +107,7 @@ pc_status cv_launch(const pc_model *m, const pc_contract *k, const pc_cv_desc *c
   PriceArgs a = L.args;
   a.lay = lay;
   a.width = pilot ? 8 : 4;
-  reduction_chunks(a.n_tiles, a.chunk_tiles, a.n_chunks);
+  reduction_chunks(a);
   s = ensure_partials(ctx, size_t(a.n_tiles) * size_t(a.width));
   if (s != PC_OK) return s;
   a.tile_partials = ctx->d_partials;
@@ -125,10 +125,6 @@ pc_status cv_launch(const pc_model *m, const pc_contract *k, const pc_cv_desc *c
     // register bound: 5 resident blocks by default (measured at 2^22 paths
     // of the autocall: 4 / 5 / 6 blocks 0.428 / 0.396 / 0.392 ms first
     // order, 0.490 / 0.466 / 0.552 ms with the second-order term)
-    s = jit_kernel(k, m->H.d, kJitCv + cv_mode(d_xm != nullptr, ca) + (win_regs ? kCvWinRegs : 0), kBlock, jk,
-                   ctx->cv_min_blocks > 0 ? ctx->cv_min_blocks : kJitCvMinBlocks);
-    if (s != PC_OK) return s;
-    const void *kern = reinterpret_cast<const void *>(jk);
     Layout &jl = a.lay;
     const int shift = jl.off_bstack;
     jl.stack = 0;
@@ -137,14 +133,20 @@ pc_status cv_launch(const pc_model *m, const pc_contract *k, const pc_cv_desc *c
     jl.off_win -= shift;
     jl.words -= shift;
     if (win_regs) jl.words = jl.off_win;  // the frontier's S in registers: no window words
-    const size_t jsm = price_smem_bytes(k->prog.code.size(), pool, jl.words, kBlock);
+    if (!L.walk_all->empty()) drop_bridge_stack(jl);
+    s = jit_kernel(k, jit_spec(k, a, kJitCv + cv_mode(d_xm != nullptr, ca) + (win_regs ? kCvWinRegs : 0),
+                               ctx->cv_min_blocks > 0 ? ctx->cv_min_blocks : kJitCvMinBlocks, *L.walk_all), jk);
+    if (s != PC_OK) return s;
+    const void *kern = reinterpret_cast<const void *>(jk);
+    const size_t jsm = price_smem_bytes(0, 0, jl.words, kBlock);
     int nb = 0;
     CU(jit_occupancy(ctx, kern, kBlock, jsm, nb), "jit occupancy");
     if (nb < 1) return fail(PC_ELIMIT, "specialised control-variate kernel cannot be resident");
     const uint64_t jneed = (a.n_tiles + kBlock / 32 - 1) / (kBlock / 32);
     const int jgrid = int(std::min<uint64_t>(uint64_t(ctx->sm_count) * nb, jneed));
     CvArgs cv = ca;
-    void *args[] = {&a, &cv};
+    StaticGrid sg = static_grid(m->H, *L.walk_all);
+    void *args[] = {&a, &cv, &sg};
     CU(cudaLaunchKernel(kern, dim3(jgrid), dim3(kBlock), args, jsm, ctx->stream),
        "specialised control-variate kernel");
     return PC_OK;

@@ -5,9 +5,11 @@
 // correlated GBM, the fused multi-asset reads, and the deterministic
 // reduction (float-pair tile sums, FP64 chunk sums).
 //
-// Per-thread state lives in shared memory as word-interleaved slots: slot s
-// of thread t is at region[s * blockDim.x + t] (float2: two paths per lane),
-// so the warp-uniform slot indices give conflict-free accesses.
+// Per-thread state lives in shared memory as lane-interleaved slots of the
+// warp's own region: slot s of lane l is at region[s * 32 + l] (float2: two
+// paths per lane), so the warp-uniform slot indices give conflict-free
+// accesses and the stride is a constant (a stride of the block size cost a
+// multiply per slot in the interpreting kernels).
 #pragma once
 
 #include "pc_types.h"
@@ -66,6 +68,18 @@ __device__ __forceinline__ float2 mul_x2(float2 a, float2 b) {
       : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
   return d;
 }
+__device__ __forceinline__ float2 add_x2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
+      "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+      "add.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+__device__ __forceinline__ float2 sub_x2(float2 a, float2 b) {
+  return fma_x2(b, make_float2(-1.f, -1.f), a);  // exact product: rounds as a - b
+}
 __device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
 
 // Philox4x32-10: ten rounds of two 32x32->64 multiplies, the key bumped by
@@ -80,19 +94,6 @@ __device__ __forceinline__ uint4 philox(uint4 c, uint32_t k0, uint32_t k1) {
     const uint32_t hi0 = __umulhi(kPhiloxM0, c.x), lo0 = kPhiloxM0 * c.x;
     const uint32_t hi1 = __umulhi(kPhiloxM1, c.z), lo1 = kPhiloxM1 * c.z;
     c = make_uint4(hi1 ^ c.y ^ k0, lo1, hi0 ^ c.w ^ k1, lo0);
-  }
-  return c;
-}
-
-// The same with the round keys precomputed (rk[2r], rk[2r + 1]: PriceArgs):
-// no key arithmetic, and in a kernel parameter the keys come from the
-// constant bank.
-__device__ __forceinline__ uint4 philox_rk(uint4 c, const uint32_t *rk) {
-#pragma unroll
-  for (int r = 0; r < 10; ++r) {
-    const uint32_t hi0 = __umulhi(kPhiloxM0, c.x), lo0 = kPhiloxM0 * c.x;
-    const uint32_t hi1 = __umulhi(kPhiloxM1, c.z), lo1 = kPhiloxM1 * c.z;
-    c = make_uint4(hi1 ^ c.y ^ rk[2 * r], lo1, hi0 ^ c.w ^ rk[2 * r + 1], lo0);
   }
   return c;
 }
@@ -135,46 +136,157 @@ __device__ __forceinline__ void box_muller2(uint32_t a0, uint32_t b0, uint32_t a
 // instruction does the work of two paths and the two independent dependency
 // chains (Philox rounds, Box-Muller, bridge) overlap in the pipeline.
 // A lane with H pairs of paths (H = 2 in a specialised kernel with four
-// paths per lane) keeps the counters of its 2H paths.
+// paths per lane) keeps the generator state of its 2H paths.
+//
+// Philox at counter (b, p_lo, p_hi, stream), block after block of one path:
+// only b changes.  Round 1 multiplies b and p_hi, so its first word,
+// mulhi(M1, p_hi) ^ p_lo ^ key, does not depend on b: with PC_ONE_PHI (every
+// path of the launch has the same p_hi: the specialised kernels, unless the
+// launch's paths cross a multiple of 2^32) round 2's product of it is kept
+// per path (hi, lo) in place of the counter words.  Every other word of
+// rounds 1 and 2, and one of round 3's two products, then depends on b
+// alone and is shared by the lane's paths: a block costs a path 32
+// instructions instead of 40.  (The interpreting kernels keep the counter:
+// with a third word per path for p_hi they measured 2-6 % slower.)
 template <int H>
 struct RngH {
+#ifdef PC_ONE_PHI
+  uint32_t hi[2 * H], lo[2 * H], y;
+#else
   uint32_t plo[2 * H], phi[2 * H];
+#endif
   uint32_t stream;
   uint32_t rk[20];  // Philox round keys (PriceArgs::rk), copied: the compiler keeps them uniform
 };
 using Rng2 = RngH<1>;
 
-// The four normals of Philox block b of both paths.
-__device__ __forceinline__ void block_normals2(uint32_t b, const Rng2 &g, float2 (&e)[4]) {
-  const uint4 x0 = philox_rk(make_uint4(b, g.plo[0], g.phi[0], g.stream), g.rk);
-  const uint4 x1 = philox_rk(make_uint4(b, g.plo[1], g.phi[1], g.stream), g.rk);
-  box_muller2(x0.x, x0.y, x1.x, x1.y, e[0], e[1]);
-  box_muller2(x0.z, x0.w, x1.z, x1.w, e[2], e[3]);
+// Launch-wide state, then path p as the lane's path q.
+template <int H>
+__device__ __forceinline__ void rng_init(RngH<H> &g, const uint32_t *rk, uint32_t stream, uint64_t path_offset) {
+  g.stream = stream;
+#pragma unroll
+  for (int i = 0; i < 20; ++i) g.rk[i] = rk[i];
+#ifdef PC_ONE_PHI
+  g.y = kPhiloxM1 * uint32_t(path_offset >> 32);
+#else
+  (void)path_offset;
+#endif
+}
+template <int H>
+__device__ __forceinline__ void rng_path(RngH<H> &g, int q, uint64_t p, uint64_t path_offset) {
+#ifdef PC_ONE_PHI
+  const uint32_t x = __umulhi(kPhiloxM1, uint32_t(path_offset >> 32)) ^ uint32_t(p) ^ g.rk[0];
+  g.hi[q] = __umulhi(kPhiloxM0, x);
+  g.lo[q] = kPhiloxM0 * x;
+#else
+  (void)path_offset;
+  g.plo[q] = uint32_t(p);
+  g.phi[q] = uint32_t(p >> 32);
+#endif
 }
 
-// The same for each pair h of a lane's 2H paths.
+// Philox block b of the lane's path q (round keys precomputed: no key
+// arithmetic, and in a kernel parameter they come from the constant bank).
+template <int H>
+__device__ __forceinline__ uint4 philox_path(uint32_t b, const RngH<H> &g, int q) {
+#ifdef PC_ONE_PHI
+  const uint32_t z1 = __umulhi(kPhiloxM0, b) ^ g.stream ^ g.rk[1];
+  uint4 c = make_uint4(__umulhi(kPhiloxM1, z1) ^ g.y ^ g.rk[2], kPhiloxM1 * z1,
+                       g.hi[q] ^ ((kPhiloxM0 * b) ^ g.rk[3]), g.lo[q]);
+  constexpr int kFirst = 2;
+#else
+  uint4 c = make_uint4(b, g.plo[q], g.phi[q], g.stream);
+  constexpr int kFirst = 0;
+#endif
+#pragma unroll
+  for (int r = kFirst; r < 10; ++r) {
+    const uint32_t hi0 = __umulhi(kPhiloxM0, c.x), lo0 = kPhiloxM0 * c.x;
+    const uint32_t hi1 = __umulhi(kPhiloxM1, c.z), lo1 = kPhiloxM1 * c.z;
+    c = make_uint4(hi1 ^ c.y ^ g.rk[2 * r], lo1, hi0 ^ c.w ^ g.rk[2 * r + 1], lo0);
+  }
+  return c;
+}
+
+// The four normals of Philox block b for each pair h of a lane's 2H paths.
 template <int H>
 __device__ __forceinline__ void block_normals_h(uint32_t b, const RngH<H> &g, float2 (&e)[H][4]) {
 #pragma unroll
   for (int h = 0; h < H; ++h) {
-    const uint4 x0 = philox_rk(make_uint4(b, g.plo[2 * h], g.phi[2 * h], g.stream), g.rk);
-    const uint4 x1 = philox_rk(make_uint4(b, g.plo[2 * h + 1], g.phi[2 * h + 1], g.stream), g.rk);
+    const uint4 x0 = philox_path<H>(b, g, 2 * h), x1 = philox_path<H>(b, g, 2 * h + 1);
     box_muller2(x0.x, x0.y, x1.x, x1.y, e[h][0], e[h][1]);
     box_muller2(x0.z, x0.w, x1.z, x1.w, e[h][2], e[h][3]);
   }
 }
 
-// Slot s of this thread in the word-interleaved per-thread region (the
-// stride is the block size, 32..kBlock threads; a run-time specialised
-// kernel is compiled for its block size, so its slot offsets are constants).
-#ifdef PC_SLOT_STRIDE
-#define SL(s) R[(s) * PC_SLOT_STRIDE]
+// Slot s of this lane in its warp's region (warp_region).
+#define SL(s) R[(s) * 32]
+
+// A specialised kernel's layout is a constant (PC_LAYOUT), and with a static
+// walk the model's grid too (PC_GRID): slot addresses become immediate
+// offsets, and grid checks and ordinals fold.
+#if defined(PC_LAYOUT)
+__device__ __forceinline__ Layout layout_of(const PriceArgs &a) {
+  constexpr int32_t v[] = {PC_LAYOUT};
+  Layout l = a.lay;
+  l.stack = v[0];
+  l.off_bstack = v[1];
+  l.off_cache = v[2];
+  l.off_win = v[3];
+  l.off_xwin = v[4];
+  l.words = v[5];
+  l.win = v[6];
+  return l;
+}
 #else
-#define SL(s) R[(s) * blockDim.x]
+__device__ __forceinline__ const Layout &layout_of(const PriceArgs &a) { return a.lay; }
+#endif
+#if defined(PC_GRID)
+__device__ __forceinline__ ModelDev model_of(const PriceArgs &a) {
+  constexpr int32_t v[] = {PC_GRID};
+  ModelDev m = a.m;
+  m.n = v[0];
+  m.n_hist = v[1];
+  m.t_now = v[2];
+  return m;
+}
+#else
+__device__ __forceinline__ const ModelDev &model_of(const PriceArgs &a) { return a.m; }
 #endif
 
+// This lane's slot 0 in the warp's region of `words` slots, the regions of
+// the block's warps one after the other from `base`.  The offset is opaque
+// to the compiler, which otherwise recomputes it from the thread index at
+// the accesses (76 S2R and as many shifts and adds per tile of the autocall).
+__device__ __forceinline__ float2 *warp_region(uint32_t *base, int words) {
+  int off = int(threadIdx.x >> 5) * words * 32 + int(threadIdx.x & 31);
+  asm volatile("" : "+r"(off));
+  return reinterpret_cast<float2 *>(base) + off;
+}
+
+// The launch's program and constant pool, staged in shared memory once per
+// block; the per-thread regions follow.  A specialised kernel has both in its
+// code, and its regions start at once.
+struct Staged {
+  const uint4 *P;
+  const float *pool;
+  uint32_t *regions;
+};
+__device__ __forceinline__ Staged stage_program(const PriceArgs &a, uint32_t *smem) {
+#ifdef PC_JIT
+  (void)a;
+  return {nullptr, nullptr, smem};
+#else
+  const int prog_words = a.n_insn * 4 + a.n_pool;
+  const uint32_t *src = reinterpret_cast<const uint32_t *>(a.prog);
+  for (int i = threadIdx.x; i < prog_words; i += blockDim.x) smem[i] = src[i];
+  __syncthreads();
+  return {reinterpret_cast<const uint4 *>(smem), reinterpret_cast<const float *>(smem + a.n_insn * 4),
+          smem + prog_words};
+#endif
+}
+
 // Window slot w (0 .. win * d - 1) of this thread: in the shared region
-// (word-interleaved after lay.off_win) or, with GW, in the thread's column
+// (lane-interleaved after lay.off_win) or, with GW, in the thread's column
 // of the HBM window (coalesced across the warp for a uniform slot).
 template <bool GW>
 __device__ __forceinline__ float2 win_load(const float2 *R, const Layout &lay, int w) {
@@ -196,10 +308,17 @@ __device__ __forceinline__ void win_store(float2 *R, const Layout &lay, int w, f
 template <int D, int H = 1>
 struct PathState {
   float2 w[H][D];               // W at the last produced date
-  float2 zc[H][3];              // words 1..3 of the last Philox block (d < 4)
   int f;                        // last produced ordinal (frontier), warp-uniform
+#ifdef PC_STATIC_DEPTH
+  // a static walk (pc_jit.cpp): stack and normals in registers, every index a constant
+  float2 bst[PC_STATIC_DEPTH][H][D];
+  float2 e[H][4];               // the last Philox block's normals
+  int step;                     // steps run so far, warp-uniform
+#else
+  float2 zc[H][3];              // words 1..3 of the last Philox block (d < 4)
   int bsp;                      // bridge stack size, warp-uniform
   int k;                        // ops run so far (the next op's number), warp-uniform
+#endif
 #ifdef PC_WIN_REGS
   float2 s[H][D];               // S at the frontier date: the whole window of a program
                                 // that reads no date behind the frontier
@@ -211,18 +330,118 @@ struct PathState {
 template <int D, int H>
 __device__ __forceinline__ void path_state_init(PathState<D, H> &ps, float2 *R, const Layout &lay) {
 #pragma unroll
+  for (int h = 0; h < H; ++h)
+#pragma unroll
+    for (int i = 0; i < D; ++i) ps.w[h][i] = make_float2(0.f, 0.f);
+  ps.f = 0;
+#ifdef PC_STATIC_DEPTH
+  ps.step = 0;
+#else
+#pragma unroll
   for (int i = 0; i < D * H; ++i) SL(lay.off_bstack + i) = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int h = 0; h < H; ++h)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) ps.zc[h][i] = make_float2(0.f, 0.f);
+  ps.bsp = 0;
+  ps.k = 0;
+#endif
+}
+
+// GBM at date t from W at the frontier into the window slot of t.  With XW
+// the correlated Brownian values X = L W of the date are also kept (window
+// at lay.off_xwin), which the pathwise sensitivities need.
+template <int D, bool XW, bool GW, int H>
+__device__ __forceinline__ void date_values(int t, PathState<D, H> &ps, const Layout &lay,
+                                            float2 *R, const float (&Bm)[D * D], const float (&S0)[D],
+                                            const float *Lm, const float2 (&drift)[D]) {
+  static_assert(H == 1 || (!XW && !GW), "several path pairs a lane: no X window, no HBM window");
+  const int ws = (t & (lay.win - 1)) * D;
 #pragma unroll
   for (int h = 0; h < H; ++h) {
 #pragma unroll
-    for (int i = 0; i < D; ++i) ps.w[h][i] = make_float2(0.f, 0.f);
+    for (int i = 0; i < D; ++i) {
+      float2 x = drift[i];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) ps.zc[h][i] = make_float2(0.f, 0.f);
+      for (int k = 0; k <= i; ++k)
+        x = make_float2(fmaf(Bm[i * D + k], ps.w[h][k].x, x.x), fmaf(Bm[i * D + k], ps.w[h][k].y, x.y));
+#ifdef PC_WIN_REGS
+      ps.s[h][i] = make_float2(S0[i] * ex2_approx(x.x), S0[i] * ex2_approx(x.y));
+      (void)ws;
+#else
+      win_store<GW>(R, lay, ws + i, make_float2(S0[i] * ex2_approx(x.x), S0[i] * ex2_approx(x.y)));
+#endif
+    }
   }
-  ps.f = 0;
-  ps.bsp = 0;
-  ps.k = 0;
+  if constexpr (XW) {
+    const int xs = lay.off_xwin + (t & (lay.win - 1)) * D;
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      float2 x = mul_x2(dup2(Lm[i * D]), ps.w[0][0]);
+#pragma unroll
+      for (int k = 1; k <= i; ++k) x = fma_x2(dup2(Lm[i * D + k]), ps.w[0][k], x);
+      SL(xs + i) = x;
+    }
+  }
 }
+
+#ifdef PC_STATIC_DEPTH
+// One op of a static walk: op number K (its normals D K .. D K + D - 1; the
+// Philox block computed last is CUR), weights at IDX of the launch's table,
+// stack size BSP before it.  The first op is the root.  Everything but the
+// values is known to the compiler: no op loads, no phase of the normals, no
+// stack in shared memory, no loop.
+template <int D, int H, int K, int IDX, int BSP, int CUR>
+__device__ __forceinline__ void static_op(PathState<D, H> &ps, const RngH<H> &g, const StaticGrid &sg) {
+  constexpr int B0 = (D * K) >> 2, B1 = (D * K + D - 1) >> 2;
+  float2 z[H][D];
+  if constexpr (B0 != CUR) block_normals_h<H>(B0, g, ps.e);
+#pragma unroll
+  for (int h = 0; h < H; ++h)
+#pragma unroll
+    for (int i = 0; i < D; ++i)
+      if (((D * K + i) >> 2) == B0) z[h][i] = ps.e[h][(D * K + i) & 3];
+  if constexpr (B1 != B0) {
+    block_normals_h<H>(B1, g, ps.e);
+#pragma unroll
+    for (int h = 0; h < H; ++h)
+#pragma unroll
+      for (int i = 0; i < D; ++i)
+        if (((D * K + i) >> 2) == B1) z[h][i] = ps.e[h][(D * K + i) & 3];
+  }
+#pragma unroll
+  for (int h = 0; h < H; ++h)
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      const float2 v = mul_x2(sg.sd[IDX], z[h][i]);
+      if constexpr (BSP == 0) ps.bst[0][h][i] = v;
+      else ps.bst[BSP][h][i] = fma_x2(sg.wl[IDX], ps.w[h][i], fma_x2(sg.wr[IDX], ps.bst[BSP - 1][h][i], v));
+    }
+}
+
+// The end of step STEP of a static walk: date t popped (stack level BSP) as
+// the frontier, its values formed when the program reads it.
+template <int D, int H, bool XW, bool GW, int STEP, int BSP, bool READ>
+__device__ __forceinline__ void static_date(int t, PathState<D, H> &ps, const Layout &lay, const StaticGrid &sg,
+                                            float2 *R, const float (&Bm)[D * D], const float (&S0)[D],
+                                            const float *Lm) {
+#pragma unroll
+  for (int h = 0; h < H; ++h)
+#pragma unroll
+    for (int i = 0; i < D; ++i) ps.w[h][i] = ps.bst[BSP][h][i];
+  if constexpr (READ) {
+    float2 drift[D];
+#pragma unroll
+    for (int i = 0; i < D; ++i) drift[i] = dup2(sg.A[STEP][i]);
+    date_values<D, XW, GW, H>(t, ps, lay, R, Bm, S0, Lm, drift);
+  }
+  ps.f = t;
+  ps.step = STEP + 1;
+}
+// the generated source defines PC_STEP: a switch on ps.step over the steps
+#define NEXT_DATE(XW_, GW_, LM_) PC_STEP(XW_, GW_, LM_)
+#else
+#define NEXT_DATE(XW_, GW_, LM_) gen_date<D, XW_, GW_>(ps.f + 1, ps, m, lay, g, R, Bm, S0, LM_)
 
 // The normals of op k for every path of the lane: normals D k .. D k + D - 1
 // of the path (Philox block m >> 2, word m & 3).  Ops run in order, so the
@@ -309,9 +528,11 @@ __device__ __forceinline__ void node_normals(uint32_t k, const RngH<H> &g, float
 }
 
 // A bridge op's weights as packed pairs (two 16-byte loads through the
-// read-only path: the address is the same in every lane).
+// read-only path: the address is the same in every lane), and in the by-date
+// table the op's number and the right end of its interval.
 struct OpRegs {
   float2 wl, wr, sd;
+  uint32_t j, m;
 };
 __device__ __forceinline__ OpRegs load_op(const BridgeOp *p) {
   const float4 *q = reinterpret_cast<const float4 *>(p);
@@ -320,78 +541,136 @@ __device__ __forceinline__ OpRegs load_op(const BridgeOp *p) {
   o.wl = make_float2(a.x, a.y);
   o.wr = make_float2(a.z, a.w);
   o.sd = make_float2(b.x, b.y);
+  o.j = __float_as_uint(b.z);
+  o.m = __float_as_uint(b.w) >> 16;
   return o;
 }
 
-// Produce date t (= frontier + 1) for the lane's paths: bridge ops of t,
-// then GBM into the window slot of t.  With XW the correlated Brownian
-// values X = L W of the date are also kept (window at lay.off_xwin), which
-// the pathwise sensitivities need.  The bridge, correlation and GBM products
-// run on packed pairs (two paths of the lane); with H pairs a lane, each op's
-// schedule and control serve all 2H paths.
-template <int D, bool XW = false, bool GW = false, int H = 1>
-__device__ __forceinline__ void gen_date(int t, PathState<D, H> &ps, const ModelDev &m,
-                                         const Layout &lay, const RngH<H> &g, float2 *R,
-                                         const float (&Bm)[D * D], const float (&S0)[D],
-                                         const float *Lm = nullptr) {
-  static_assert(H == 1 || (!XW && !GW), "several path pairs a lane: no X window, no HBM window");
-  const int k1 = __ldg(m.date_ops + t + 1);  // ops of date t: [ps.k, k1)
-  // Every op pushes its node; the date's own value (the last node, or one
-  // pushed on an earlier date when t has no op) is then popped as the new
-  // frontier value.  The root op has wl = wr = 0 and reads the bottom level,
-  // zeroed at the path's start, as its right end.  (Branch-free: a push or
-  // keep decision per op, and a root test, cost register moves at the joins.)
-  for (; ps.k < k1; ++ps.k) {
-    const OpRegs op = load_op(m.ops + ps.k);
-    float2 z[H][D];
-    node_normals<D, H>(uint32_t(ps.k), g, ps.zc, z);
-    const int top = lay.off_bstack + max(ps.bsp - 1, 0) * D * H;
-    const int nxt = lay.off_bstack + ps.bsp * D * H;
+// One bridge op: node from W at the frontier and the top of the stack (the
+// right end of its interval), pushed.  The root op has wl = wr = 0 and reads
+// the bottom level, zeroed at the path's start, as its right end.
+// (Branch-free: a push or keep decision per op, and a root test, cost
+// register moves at the joins.)
+template <int D, int H>
+__device__ __forceinline__ void push_node(const OpRegs &op, const float2 (&z)[H][D], PathState<D, H> &ps,
+                                          const Layout &lay, float2 *R) {
+  const int top = lay.off_bstack + max(ps.bsp - 1, 0) * D * H;
+  const int nxt = lay.off_bstack + ps.bsp * D * H;
 #pragma unroll
-    for (int h = 0; h < H; ++h) {
-      float2 nw[D];
+  for (int h = 0; h < H; ++h) {
+    float2 nw[D];
 #pragma unroll
-      for (int i = 0; i < D; ++i)
-        nw[i] = fma_x2(op.wl, ps.w[h][i], fma_x2(op.wr, SL(top + h * D + i), mul_x2(op.sd, z[h][i])));
+    for (int i = 0; i < D; ++i)
+      nw[i] = fma_x2(op.wl, ps.w[h][i], fma_x2(op.wr, SL(top + h * D + i), mul_x2(op.sd, z[h][i])));
 #pragma unroll
-      for (int i = 0; i < D; ++i) SL(nxt + h * D + i) = nw[i];
-    }
-    ++ps.bsp;
+    for (int i = 0; i < D; ++i) SL(nxt + h * D + i) = nw[i];
   }
+  ++ps.bsp;
+}
+
+// The stack's top popped as W of the new frontier date.
+template <int D, int H>
+__device__ __forceinline__ void pop_date(PathState<D, H> &ps, const Layout &lay, float2 *R) {
   --ps.bsp;
 #pragma unroll
   for (int h = 0; h < H; ++h)
 #pragma unroll
     for (int i = 0; i < D; ++i) ps.w[h][i] = SL(lay.off_bstack + ps.bsp * D * H + h * D + i);
-  const int ws = (t & (lay.win - 1)) * D;
-#pragma unroll
-  for (int h = 0; h < H; ++h) {
-#pragma unroll
-    for (int i = 0; i < D; ++i) {
-      float2 x = __ldg(m.A + t * D + i);
-#pragma unroll
-      for (int k = 0; k <= i; ++k)
-        x = make_float2(fmaf(Bm[i * D + k], ps.w[h][k].x, x.x), fmaf(Bm[i * D + k], ps.w[h][k].y, x.y));
-#ifdef PC_WIN_REGS
-      ps.s[h][i] = make_float2(S0[i] * ex2_approx(x.x), S0[i] * ex2_approx(x.y));
-      (void)ws;
-#else
-      win_store<GW>(R, lay, ws + i, make_float2(S0[i] * ex2_approx(x.x), S0[i] * ex2_approx(x.y)));
-#endif
-    }
+}
+
+// Produce date t (= frontier + 1) for the lane's paths: the bridge ops of t
+// (every op pushes its node; the date's own value, the last node or one
+// pushed on an earlier date, is popped), then its values.  The bridge,
+// correlation and GBM products run on packed pairs (two paths of the lane);
+// with H pairs a lane, each op's schedule and control serve all 2H paths.
+template <int D, bool XW = false, bool GW = false, int H = 1>
+__device__ __forceinline__ void gen_date(int t, PathState<D, H> &ps, const ModelDev &m,
+                                         const Layout &lay, const RngH<H> &g, float2 *R,
+                                         const float (&Bm)[D * D], const float (&S0)[D],
+                                         const float *Lm = nullptr) {
+  const int k1 = __ldg(m.date_ops + t + 1);  // ops of date t: [ps.k, k1)
+  for (; ps.k < k1; ++ps.k) {
+    const OpRegs op = load_op(m.ops + ps.k);
+    float2 z[H][D];
+    node_normals<D, H>(uint32_t(ps.k), g, ps.zc, z);
+    push_node<D, H>(op, z, ps, lay, R);
   }
-  if constexpr (XW) {
-    const int xs = lay.off_xwin + (t & (lay.win - 1)) * D;
+  pop_date<D, H>(ps, lay, R);
+  float2 drift[D];
 #pragma unroll
-    for (int i = 0; i < D; ++i) {
-      float2 x = mul_x2(dup2(Lm[i * D]), ps.w[0][0]);
-#pragma unroll
-      for (int k = 1; k <= i; ++k) x = fma_x2(dup2(Lm[i * D + k]), ps.w[0][k], x);
-      SL(xs + i) = x;
-    }
-  }
+  for (int i = 0; i < D; ++i) drift[i] = __ldg(m.A + t * D + i);
+  date_values<D, XW, GW, H>(t, ps, lay, R, Bm, S0, Lm, drift);
   ps.f = t;
 }
+#endif
+
+#ifndef PC_JIT
+// The frontier moved past dates that no read needs, straight to date t: from
+// the interval that the frontier opens (its right end from the by-date
+// table) bisect while t lies inside, pop the right end, and again until t is
+// popped.  Only the nodes above t in the bisection tree are computed, each
+// from its own normals (its Philox blocks anew, one or two), so the values
+// at t are those of the full walk: a contract that reads the last of 365
+// dates runs one op instead of 365.  Afterwards the state is as the full walk
+// leaves it (next op, the words kept of its block).  Called rarely and by
+// copy, so that the state stays in registers around the call.
+template <int D, bool XW, bool GW>
+__device__ __noinline__ void skip_to(int t, PathState<D, 1> &ps, const ModelDev &m, const Layout &lay,
+                                     const Rng2 &g, float2 *R, const float (&Bm)[D * D], const float (&S0)[D],
+                                     const float *Lm) {
+  while (ps.f < t) {
+    int r = int(__ldg(reinterpret_cast<const uint32_t *>(m.nodes + ps.f) + 7) >> 16);
+    while (t < r) {
+      r = (ps.f + r) >> 1;
+      const OpRegs op = load_op(m.nodes + r);
+      const uint32_t first = D * op.j;  // normals first .. first + D - 1
+      float2 z[1][D], e[1][4];
+      uint32_t blk = first >> 2;
+      block_normals_h<1>(blk, g, e);
+#pragma unroll
+      for (int i = 0; i < D; ++i) {
+        if (((first + i) >> 2) != blk) {
+          blk = (first + i) >> 2;
+          block_normals_h<1>(blk, g, e);
+        }
+        const uint32_t w = (first + i) & 3;
+        z[0][i] = w == 0 ? e[0][0] : w == 1 ? e[0][1] : w == 2 ? e[0][2] : e[0][3];
+      }
+      push_node<D, 1>(op, z, ps, lay, R);
+    }
+    pop_date<D, 1>(ps, lay, R);
+    ps.f = r;
+  }
+  float2 drift[D];
+#pragma unroll
+  for (int i = 0; i < D; ++i) drift[i] = __ldg(m.A + t * D + i);
+  date_values<D, XW, GW, 1>(t, ps, lay, R, Bm, S0, Lm, drift);
+  ps.k = __ldg(m.date_ops + t + 1);
+  if (t < m.n && ((D * ps.k) & 3)) {
+    float2 e[1][4];
+    block_normals_h<1>(uint32_t(D * ps.k) >> 2, g, e);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) ps.zc[0][i] = e[0][1 + i];
+  }
+}
+#endif
+
+// The frontier to date o_ (> frontier).  An interpreted program that reads no
+// date behind the frontier (a window of one date) skips the dates between.
+#if defined(PC_JIT)
+#define TO_DATE(o_, XW_, GW_, LM_)                                                     \
+  while (ps.f < (o_)) NEXT_DATE(XW_, GW_, LM_)
+#else
+#define TO_DATE(o_, XW_, GW_, LM_)                                                     \
+  do {                                                                                 \
+    if (lay.win == 1 && (o_) > ps.f + 1) {                                             \
+      PathState<D> skip_ = ps;                                                         \
+      skip_to<D, XW_, GW_>((o_), skip_, m, lay, g, R, Bm, S0, LM_);                    \
+      ps = skip_;                                                                      \
+    }                                                                                  \
+    while (ps.f < (o_)) NEXT_DATE(XW_, GW_, LM_);                                       \
+  } while (0)
+#endif
 
 // The evaluators' per-date hook: called after each generated date t with
 // the evaluator's reader (read(t, i): S_i at ordinal t of the lane's paths).
@@ -403,6 +682,7 @@ struct NoDateHook {
   __device__ __forceinline__ void on_date(int, RD &) {}
 };
 
+#if defined(PC_JIT) && !defined(PC_STATIC_DEPTH)
 // Dates ps.f + 1 .. o, out of line (the specialised evaluator calls it from
 // every instruction that reads a date, so it is not inlined there).
 template <int D, bool GW, int H>
@@ -411,6 +691,7 @@ __device__ __noinline__ void advance_dates(int o, PathState<D, H> &ps, const Mod
                                            const float (&S0)[D]) {
   while (ps.f < o) gen_date<D, false, GW>(ps.f + 1, ps, m, lay, g, R, Bm, S0);
 }
+#endif
 
 template <int D>
 __device__ __forceinline__ void load_model_regs(const ModelDev &m, float (&Bm)[D * D],
@@ -635,18 +916,25 @@ struct Moments {
     lo[v] = __fadd_rn(lo[v], __fmaf_rn(x, y, -p));
   }
   // warp totals (identical in every lane: the butterfly's additions are
-  // commutative) as doubles
+  // commutative) as doubles; two values at a time on packed pairs, each half
+  // rounding as the scalar two-sum
   __device__ __forceinline__ void warp_total(double (&tp)[W]) {
+    static_assert(W % 2 == 0, "values in pairs");
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
-      for (int v = 0; v < W; ++v) {
-        const float h = __shfl_xor_sync(kFull, hi[v], o), l = __shfl_xor_sync(kFull, lo[v], o);
-        const float s = __fadd_rn(hi[v], h);
-        const float b = __fsub_rn(s, hi[v]);
-        const float e = __fadd_rn(__fsub_rn(hi[v], __fsub_rn(s, b)), __fsub_rn(h, b));
-        hi[v] = s;
-        lo[v] = __fadd_rn(__fadd_rn(lo[v], l), e);
+      for (int v = 0; v < W; v += 2) {
+        const float2 a = make_float2(hi[v], hi[v + 1]), c = make_float2(lo[v], lo[v + 1]);
+        const float2 h = make_float2(__shfl_xor_sync(kFull, a.x, o), __shfl_xor_sync(kFull, a.y, o));
+        const float2 l = make_float2(__shfl_xor_sync(kFull, c.x, o), __shfl_xor_sync(kFull, c.y, o));
+        const float2 s = add_x2(a, h);
+        const float2 b = sub_x2(s, a);
+        const float2 e = add_x2(sub_x2(a, sub_x2(s, b)), sub_x2(h, b));
+        const float2 t = add_x2(add_x2(c, l), e);
+        hi[v] = s.x;
+        hi[v + 1] = s.y;
+        lo[v] = t.x;
+        lo[v + 1] = t.y;
       }
     }
 #pragma unroll
@@ -681,7 +969,7 @@ __device__ __noinline__ void finish_tile(const PriceArgs &a, uint64_t tile, cons
   unsigned long long *ctr = reinterpret_cast<unsigned long long *>(a.control);
   uint32_t *chunk_cnt = reinterpret_cast<uint32_t *>(a.control + kChunkCountOff);
   double *chunk_part = reinterpret_cast<double *>(a.control + kChunkPartOff);
-  const uint32_t chunk = uint32_t(tile / a.chunk_tiles);
+  const uint32_t chunk = uint32_t(__umul64hi(tile, a.chunk_magic));  // tile / chunk_tiles
   const uint64_t first = uint64_t(chunk) * a.chunk_tiles;
   const uint64_t rest = a.n_tiles - first;
   const uint32_t size = rest < a.chunk_tiles ? uint32_t(rest) : a.chunk_tiles;

@@ -54,7 +54,7 @@ __device__ float2 eval_path(const uint4 *P, const float *pool, float2 *R, const 
 #undef BINF
 #undef BINI
 #undef IMM
-#undef GEN_DATE
+#undef EACH_DATE
 #undef FUSED_VALUE
 #undef FUSED_TEST
 }

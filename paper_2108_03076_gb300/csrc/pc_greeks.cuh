@@ -72,15 +72,6 @@ __device__ __forceinline__ TV model_read(int o, int l, int g, const float2 *R, c
   return r;
 }
 
-// Dates up to o with the window of X = L W beside S, out of line (for a
-// specialised evaluator with many reading instructions).
-template <int D>
-__device__ __noinline__ void advance_dates_x(int o, PathState<D> &ps, const ModelDev &m, const Layout &lay,
-                                             const Rng2 &g, float2 *R, const float (&Bm)[D * D],
-                                             const float (&S0)[D], const float (&Lm)[D * D]) {
-  while (ps.f < o) gen_date<D, true>(ps.f + 1, ps, m, lay, g, R, Bm, S0, Lm);
-}
-
 // X_LRED / X_LANY with tangents (comparisons give zero tangents; min and
 // max carry the tangent of the operand they select, the first on ties).
 template <int D>
@@ -130,12 +121,16 @@ __device__ TV eval_greeks(const uint4 *P, const float *pool, float2 *R, const Pr
                           const Rng2 &g, bool live0, bool live1, const float (&Bm)[D * D],
                           const float (&S0)[D], const float (&Lm)[D * D], int gl, float sig_g) {
 #include "pc_greeks_state.inc"
+#define ENSURE(o) ensure(o)
+#define NEXT_INSN P[pc + 1]
   for (;;) {
     const uint4 I = P[pc];
     const uint32_t op = I.x & 0xffu;
     const float kk = __uint_as_float(I.y);
 #include "pc_greeks_ops.inc"
   }
+#undef ENSURE
+#undef NEXT_INSN
 }
 
 // The sensitivity launch for underlying g = a.greek_label, generic in the
@@ -148,13 +143,10 @@ template <int D, bool WRITE, typename EVAL>
 __device__ __forceinline__ void greeks_tiles(const PriceArgs &a, EVAL eval) {
   extern __shared__ __align__(16) uint32_t smem[];
   __shared__ int last_block;
-  uint4 *P = reinterpret_cast<uint4 *>(smem);
-  const int prog_words = a.n_insn * 4 + a.n_pool;
-  const uint32_t *src = reinterpret_cast<const uint32_t *>(a.prog);
-  for (int i = threadIdx.x; i < prog_words; i += blockDim.x) smem[i] = src[i];
-  __syncthreads();
-  const float *pool = reinterpret_cast<const float *>(smem + a.n_insn * 4);
-  float2 *R = reinterpret_cast<float2 *>(smem + prog_words) + threadIdx.x;
+  const Staged st = stage_program(a, smem);
+  const uint4 *P = st.P;
+  const float *pool = st.pool;
+  float2 *R = warp_region(st.regions, layout_of(a).words);
   const float(&Bm)[D * D] = *reinterpret_cast<const float(*)[D * D]>(a.m.Bv);
   const float(&S0)[D] = *reinterpret_cast<const float(*)[D]>(a.m.S0v);
   float Lm[D * D];
@@ -165,9 +157,7 @@ __device__ __forceinline__ void greeks_tiles(const PriceArgs &a, EVAL eval) {
   const int lane = threadIdx.x & 31;
   unsigned long long *ctr = reinterpret_cast<unsigned long long *>(a.control);
   Rng2 g;
-  g.stream = a.stream;
-#pragma unroll
-  for (int i = 0; i < 20; ++i) g.rk[i] = a.rk[i];
+  rng_init(g, a.rk, a.stream, a.path_offset);
   for (;;) {
     unsigned long long tile = 0;
     if (lane == 0) tile = atomicAdd(ctr, 1ull);
@@ -176,10 +166,8 @@ __device__ __forceinline__ void greeks_tiles(const PriceArgs &a, EVAL eval) {
     const uint64_t i0 = tile * kTilePaths + lane, i1 = i0 + 32;
     const bool live0 = i0 < a.n_paths, live1 = i1 < a.n_paths;
     const uint64_t p0 = a.path_offset + i0, p1 = a.path_offset + i1;
-    g.plo[0] = uint32_t(p0);
-    g.phi[0] = uint32_t(p0 >> 32);
-    g.plo[1] = uint32_t(p1);
-    g.phi[1] = uint32_t(p1 >> 32);
+    rng_path(g, 0, p0, a.path_offset);
+    rng_path(g, 1, p1, a.path_offset);
     const TV x = eval(P, pool, R, g, live0, live1, Bm, S0, Lm, gl, sig_g);
     Moments<6> mo;
     const float q0[3] = {x.v.x, x.a.x, x.b.x}, q1[3] = {x.v.y, x.a.y, x.b.y};

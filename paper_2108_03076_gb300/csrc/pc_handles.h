@@ -29,18 +29,37 @@ constexpr int kJitPrice = 0, kJitPriceWrite = 1, kJitHbm = 2, kJitWinRegs = 4, k
 // resident blocks per SM the specialised pricing kernel's register bound is
 // set for by default (<= 72 registers at 128 threads: the fastest measured)
 constexpr int kJitMinBlocks = 7;
+// the same with a static walk, whose bridge stack and normals are registers
+// (autocall, 3 underlyings, 5 dates, 2^20 paths: 5 / 6 / 7 / 8 blocks 52.5 / 51.4 / 52.1 / 52.1 us a call)
+constexpr int kWalkMinBlocks = 6;
 // resident blocks per SM the specialised control-variate kernel's register bound is set for
 constexpr int kJitCvMinBlocks = 5;
 // dates of the model from which a one-date-window kernel takes two path pairs a lane
 constexpr int kJitPairsMinDates = 64;
 constexpr size_t kJitStaticSmem = 256;  // bound on price_tiles' static shared memory
 
-struct JitEntry {
-  std::vector<uint32_t> program;
+// What a specialised kernel is compiled for beside its program.
+struct JitSpec {
   int d = 0;
   int kind = kJitPrice;
-  int block = 0;  // the launch block the kernel is compiled for (its slot stride)
   int min_blocks = 0;  // its launch bound's resident blocks per SM (0: the kernel's own)
+  // a static walk over the dates that the program reads (see static_walk in
+  // pc_capi.cpp): per step the date, 1 if it is read, the number of bridge
+  // ops and their numbers; empty: the general walk
+  std::vector<int32_t> walk;
+  // the launch's layout as constants (jit_layout_constants; empty: read from
+  // the arguments) and with a walk the model's n, n_hist and t_now
+  std::vector<int32_t> lay, grid;
+  bool one_phi = false;  // every path of the launch has the same upper 32 index bits
+  bool operator==(const JitSpec &o) const {
+    return d == o.d && kind == o.kind && min_blocks == o.min_blocks && one_phi == o.one_phi && walk == o.walk &&
+           lay == o.lay && grid == o.grid;
+  }
+};
+
+struct JitEntry {
+  std::vector<uint32_t> program;
+  JitSpec spec;
   cudaLibrary_t lib = nullptr;
   cudaKernel_t kernel = nullptr;
 };
@@ -73,6 +92,7 @@ struct pc_ctx {
   int32_t jit_pairs = 0;         // path pairs a lane of a specialised kernel with a one-date window (0 automatic, 1 or 2)
   std::mutex jit_mu;
   std::multimap<uint64_t, JitEntry> jit_cache;  // program hash -> compiled kernels
+  std::map<uint64_t, std::vector<std::vector<int32_t>>> jit_walks;  // program hash -> its static walks (admit_walk)
   std::map<std::pair<const void *, size_t>, int> jit_occ;  // (kernel, smem) -> resident blocks
   cudaMemPool_t pool = nullptr;  // stream-ordered allocations of contracts (null: cudaMalloc)
   double *h_res = nullptr;       // pinned [16]: results read back by the blocking calls
@@ -109,7 +129,14 @@ struct pc_contract {
   bool pooled = false;            // d_code came from the context's memory pool
   std::vector<uint32_t> image;    // program then padded pool: the uploaded words
   std::mutex mu;
-  std::map<std::pair<uint64_t, uint64_t>, int32_t> win_cache;  // (model id, layout key) -> window
+  struct Window {
+    int32_t win = 1;
+    bool with_walks = false;  // computed with the context's specialised kernels on
+    // static walks over the dates the program reads, and over every date
+    // up to its last (a per-date hook); empty where they are too long
+    std::vector<int32_t> walk, walk_all;
+  };
+  std::map<uint64_t, Window> win_cache;  // by model id
 };
 
 namespace pc {
@@ -153,6 +180,7 @@ struct Launch {
   int grid = 0;
   int block = kBlock;
   size_t smem = 0;
+  const std::vector<int32_t> *walk = nullptr, *walk_all = nullptr;  // the contract's static walks on the model
   bool hbm_window = false;  // window in HBM (args.lay.gwin set by the launcher)
 };
 
@@ -169,32 +197,48 @@ pc_status prepare(const pc_model *m, const pc_contract *k, uint64_t n_paths, uin
 pc_status ensure_partials(pc_ctx *c, size_t doubles);
 
 // The run-time specialised kernel of the contract's program for d
-// underlyings, a kernel kind (kJit*) and the launch's block size (the
-// per-thread slot stride, a constant in the compiled code); compiled on
-// first use, cached on the context by program content.
-// min_blocks: for pc_jit_price, the resident blocks per SM its launch bound
-// asks for (0: the default, 7); other kinds fix their own bound.
-pc_status jit_kernel(const pc_contract *k, int d, int kind, int block, cudaKernel_t &out, int min_blocks = 0);
+// underlyings, a kernel kind (kJit*), a register bound and a walk; compiled
+// on first use, cached on the context by program content.
+pc_status jit_kernel(const pc_contract *k, const JitSpec &spec, cudaKernel_t &out);
 // Programs of at most PC_JIT_MAX_INSNS instructions are specialised; the
 // launches of longer ones interpret them.
 bool jit_eligible(const pc_contract *k);
-// A program the specialised adjoint kernel takes (its date generator is
-// inlined at each reading instruction: a few of them at most).
+// A program the specialised adjoint kernel takes (at most the reading
+// instructions that the shared date generator's re-entry switch is kept to).
 bool adjoint_jit_eligible(const pc_contract *k);
+// A program whose evaluator can take a static walk: one copy of it, or two.
+bool walk_jit_eligible(const pc::Program &p);
+// A static walk's kernel is compiled for the grid too, so a program priced on
+// models of ever new grids would compile each time: whether this walk on this
+// model is one of the context's first kWalksPerProgram of the program (the
+// others take the general kernel, compiled once).
+constexpr size_t kWalksPerProgram = 8;
+bool admit_walk(pc_ctx *c, const Program &p, const ModelHost &H, const std::vector<int32_t> &walk);
+// The launch argument of a static walk on a model.
+StaticGrid static_grid(const ModelHost &H, const std::vector<int32_t> &walk);
+// Whether every path of offset .. offset + n_tiles tiles has the same p_hi.
+inline bool one_phi(uint64_t offset, uint64_t n_tiles) {
+  return (offset >> 32) == ((offset + n_tiles * kTilePaths - 1) >> 32);
+}
 // Compile the specialised kernels of many requests into the context's cache
 // (those not there yet), NVRTC on the host's cores in parallel; jit_kernel
 // then finds them.
 struct JitRequest {
   const pc_contract *k;
-  int d, kind, block, min_blocks;
+  JitSpec spec;
 };
 pc_status jit_compile_many(pc_ctx *c, const std::vector<JitRequest> &reqs);
 // The specialised pricing kernel's variant for a prepared launch (window in
 // registers, path pairs a lane, HBM window), its layout (the launch's shared
 // memory; may re-choose the block) and the register bound it is compiled for.
 int jit_window_kind(const pc_ctx *c, const Launch &L);
-size_t jit_layout(const pc_ctx *c, const pc_contract *k, Launch &L, int bits);
+size_t jit_layout(const pc_ctx *c, Launch &L, int bits);
 int jit_min_blocks(const pc_ctx *c, size_t smem, int block);
+// What the contract's specialised kernel of `kind` is compiled for: the
+// launch's arguments (layout final) and a walk (may be empty).
+JitSpec jit_spec(const pc_contract *k, const PriceArgs &a, int kind, int min_blocks, const std::vector<int32_t> &walk);
+JitSpec jit_price_spec(const pc_ctx *c, const pc_contract *k, const Launch &L, int kind, size_t smem);
+void drop_bridge_stack(Layout &lay);
 void jit_release(pc_ctx *c);
 
 // Turn a raised device status word into PC_EDEVICE (and clear it).

@@ -41,6 +41,7 @@ struct BatchArgs {
   const BatchUnit *units;       // this group's units (device)
   uint32_t n_units;
   uint32_t slot_bytes;          // per-warp slot: arguments + program + pool
+  int32_t words;                // per-thread slots of the group's largest footprint
   unsigned long long *counter;  // next unit; zero before the launch
 };
 // Per-warp slot in shared memory (a contract's arguments, then its program
@@ -117,6 +118,7 @@ struct TimeWalk {
   int64_t t_now, n_dates, n_hist;
   OnFail on_fail;
   int64_t frontier = 0, lookback = 0, steps = 0, entries = 0;
+  uint8_t *reads = nullptr;  // optional [n_dates + 1]: set to 1 for every simulated date read
   pc_status st = PC_OK;
 
   static int64_t entry_count(const XInsn &I) {
@@ -154,6 +156,7 @@ struct TimeWalk {
           return;
         }
         if (op != X_PAYOFF && o > 0) {
+          if (reads) reads[o] = 1;
           if (o > frontier) frontier = o;
           else if (frontier - o > lookback) lookback = frontier - o;
         }
@@ -206,9 +209,10 @@ struct TimeWalk {
 // Static analysis of a program against a model's time layout (TimeWalk):
 // every model and payoff time within [-n_hist, n] as ordinals; `win`
 // receives the window size needed (power of two, <= 2 * PC_MAX_DATES:
-// callers decide where such a window can live).
+// callers decide where such a window can live), `reads` [n + 1] marks the
+// dates read.
 pc_status analyse_program(const Program &p, int32_t t_now, int32_t n_dates, int32_t n_hist,
-                          int32_t &win, std::string &err);
+                          int32_t &win, std::vector<uint8_t> &reads, std::string &err);
 
 // cutPayoff (Sec. 4.1) on bytecode: every payoff(t, p1', p2') becomes
 // if(t < now, 0, payoff(t, p1', p2')); the literal 0.0 is appended to the
@@ -230,12 +234,21 @@ struct ModelHost {
   std::vector<double> history;
   // device tables, host copies
   std::vector<int32_t> date_ops;
-  std::vector<BridgeOp> ops;
+  std::vector<BridgeOp> ops, nodes;  // in op order; by date
   std::vector<float2> A;  // drift exponents, each twice (packed pairs)
   std::vector<float> B, disc, sval, tau, Lf, sig;
   int32_t n_levels = 0, bstack = 0;
 };
 
 pc_status build_model(const pc_model_desc &desc, ModelHost &out, std::string &err);
+
+// The walk over a model's dates that computes only the bridge nodes needed
+// for the dates marked in reads [n + 1]: those whose bisection interval has a
+// read date inside (each from the same normals and weights as in the full
+// walk, so every date read has the full walk's value).  Per step: the date
+// popped, 1 if it is read, the number of ops before it, their numbers.  Ends
+// with the last date read; empty when no date is read or it takes more than
+// kStaticOps ops.
+std::vector<int32_t> static_walk(const ModelHost &H, const std::vector<uint8_t> &reads);
 
 }  // namespace pc

@@ -53,10 +53,8 @@ constexpr int kInlineDateSites = 12;
 // generator makes NVRTC's time grow faster than the program (100 terms of
 // a two-asset average: 13 s shared, 3.2 s out of line): call it out of line.
 constexpr int kSharedDateSites = 64;
-// The tangent date generator (S and X windows) is about twice the size of
-// the pricing one: inlined at up to this many reading instructions.
-constexpr int kInlineTangentDateSites = 6;
-
+// The adjoint evaluator's code grows by its tape writes at every operation.
+constexpr int kAdjointDateSites = 6;
 // Instructions that read simulated dates (and may have to generate them).
 bool reads_dates(const XInsn &I) {
   const uint32_t op = I.opa & 0xffu;
@@ -144,30 +142,193 @@ bool stack_depths(const Program &p, std::vector<int> &sp_at) {
   return ok;
 }
 
-// Straight-line tangent evaluator (pc_jit_greeks around greeks_tiles; the
-// per-path triples written out with kJitGreeks + 1): each instruction is
-// the interpreter's case for its constant opcode and fields, followed by a
-// jump to whichever of its possible successors the case left in pc.  The
-// operand stack of value-with-tangents stays in shared memory, as in the
-// interpreter.  Beyond kInlineTangentDateSites reading instructions they
-// call one out-of-line copy of the date generator.
-// The adjoint evaluator straight-line over the program (each instruction's
-// block includes pc_adjoint_ops.inc with the instruction as a constant),
-// and pc_jit_adjoint: adjoint_tiles around it.  The date generator (with
-// the X window) is inlined at each reading instruction: programs with more
-// than kInlineTangentDateSites of them are not specialised (adjoint_eligible).
-std::string generate_adjoint(const Program &p, int d, bool write) {
-  std::ostringstream o;
+// A price or control-variate evaluator without re-entry points: many reading
+// instructions call one out-of-line copy of the generator instead of
+// inlining it at each.
+bool outlined_dates(const Program &p) {
+  std::vector<int> sp_at;
+  const bool shared = date_sites(p) >= 2 && date_sites(p) <= kSharedDateSites && stack_depths(p, sp_at);
+  return !shared && date_sites(p) > kInlineDateSites;
+}
+
+// A static walk as source: PC_STEP runs step ps.step (its ops, then its date).
+// Defined before the device headers, whose state it sizes.
+void define_walk(std::ostringstream &o, const JitSpec &sp) {
+  auto ints = [&](const char *name, const std::vector<int32_t> &v) {
+    if (v.empty()) return;
+    o << "#define " << name;
+    for (size_t i = 0; i < v.size(); ++i) o << (i ? ", " : " ") << v[i];
+    o << "\n";
+  };
+  ints("PC_LAYOUT", sp.lay);
+  ints("PC_GRID", sp.grid);
+  if (sp.walk.empty()) return;
+  int depth = 1, bsp = 0, idx = 0, cur = -1;
+  size_t steps = 0;
+  for (size_t i = 0; i < sp.walk.size(); ++steps) {
+    const int date = sp.walk[i], read = sp.walk[i + 1], ops = sp.walk[i + 2];
+    i += 3;
+    o << "#define PC_STEP_" << steps << "(XW_, GW_, LM_) { \\\n";
+    for (int j = 0; j < ops; ++j, ++i, ++idx, ++bsp) {
+      const int k = sp.walk[i];
+      o << "      static_op<D, PC_PAIRS, " << k << ", " << idx << ", " << bsp << ", " << cur << ">(ps, g, sg); \\\n";
+      cur = (sp.d * k + sp.d - 1) / 4;
+    }
+    depth = std::max(depth, bsp);
+    --bsp;
+    o << "      static_date<D, PC_PAIRS, XW_, GW_, " << steps << ", " << bsp << ", " << (read ? "true" : "false")
+      << ">(" << date << ", ps, lay, sg, R, Bm, S0, LM_); }\n";
+  }
+  o << "#define PC_STATIC_DEPTH " << depth << "\n"
+    << "#define PC_STEP(XW_, GW_, LM_) switch (ps.step) { \\\n";
+  for (size_t i = 0; i < steps; ++i) o << "    case " << i << ": PC_STEP_" << i << "(XW_, GW_, LM_) break; \\\n";
+  o << "    default: ps.f = 0x7fffffff; }\n";
+}
+
+// With a static walk: what every run has at an instruction, by data flow over
+// the program -- the loop offset t0 and the frontier (the last date produced),
+// each known or not (kUnknown) where paths of different history meet or a
+// loop is under way.  A reading instruction with both known runs exactly the
+// steps from its frontier to its date in line: no test, no jump, one copy in
+// programs that read each date first at one place.
+constexpr int kUnknown = -(1 << 30);
+struct FlowState {
+  int t0 = 0, f = 0;
+  bool reached = false;
+};
+std::vector<FlowState> flow_states(const Program &p, const JitSpec &sp) {
+  const int n = int(p.code.size()), t_now = sp.grid[2];
+  std::vector<FlowState> at(static_cast<size_t>(n));
+  std::vector<int> lend_t0(static_cast<size_t>(n), kUnknown), work;
+  auto flow = [&](uint32_t t, int t0, int f) {
+    if (t >= uint32_t(n)) return;
+    FlowState &x = at[t];
+    const int nt0 = !x.reached || x.t0 == t0 ? t0 : kUnknown, nf = !x.reached || x.f == f ? f : kUnknown;
+    if (x.reached && nt0 == x.t0 && nf == x.f) return;
+    x = {nt0, nf, true};
+    work.push_back(int(t));
+  };
+  flow(0, 0, 0);
+  while (!work.empty()) {
+    const int i = work.back();
+    work.pop_back();
+    const XInsn &I = p.code[size_t(i)];
+    const int t0 = at[size_t(i)].t0;
+    int f = at[size_t(i)].f;
+    const uint32_t nx = uint32_t(i + 1), op = I.opa & 0xffu;
+    if (reads_dates(I)) {
+      if (t0 == kUnknown) f = kUnknown;
+      else if (f != kUnknown) f = std::max(f, int(I.b) + t0 - t_now);
+      flow(nx, t0, f);
+      continue;
+    }
+    switch (op) {
+      case X_END: break;
+      case X_IF: case X_ELSE:
+        flow(nx, t0, f);
+        flow(I.c, t0, f);
+        break;
+      case X_LOOPANY: {
+        const int last = t0 == kUnknown ? kUnknown : int(p.code[size_t(i) + 1].b) + t0 + int(I.b) - t_now;
+        lend_t0[I.e - 1] = t0;
+        flow(I.e, t0, kUnknown);  // every path latched, at any of its dates
+        flow(uint32_t(i + 2), t0 == kUnknown ? kUnknown : t0 + int(I.b),
+             f == kUnknown || last == kUnknown ? kUnknown : std::max(f, last));
+        break;
+      }
+      case X_LEND: flow(nx, lend_t0[size_t(i)], f); break;
+      case X_LOOP: case X_LTEST: case X_LLATCH: case X_LNEXT: case X_LSTEPK:
+        flow(nx, kUnknown, kUnknown);
+        flow(I.c, kUnknown, kUnknown);
+        flow(I.e, kUnknown, kUnknown);
+        break;
+      default: flow(nx, t0, f); break;
+    }
+  }
+  return at;
+}
+// The ENSURE of a reading instruction whose state is known (false if it is
+// not): the steps to its date.
+bool known_ensure(const XInsn &I, const FlowState &st, const JitSpec &sp, const char *args, std::string &text) {
+  if (!st.reached || st.t0 == kUnknown || st.f == kUnknown) return false;
+  const int target = int(I.b) + st.t0 - sp.grid[2];
+  text = "#define ENSURE(o) {";
+  int step = 0;
+  for (size_t i = 0; i < sp.walk.size(); i += 3 + size_t(sp.walk[i + 2]), ++step)
+    if (sp.walk[i] > st.f && sp.walk[i] <= target) {
+      text += " PC_STEP_" + std::to_string(step) + args;
+      if (sp.kind >= kJitCv && sp.kind < kJitGreeks) text += " hook_->on_date(" + std::to_string(sp.walk[i]) + ", read);";
+    }
+  text += " }\n";
+  return true;
+}
+
+// A static walk's launch argument, as a kernel and as an evaluator parameter.
+const char *walk_kernel_param(const JitSpec &sp) { return sp.walk.empty() ? "" : ", const __grid_constant__ pc::StaticGrid sg"; }
+const char *walk_eval_param(const JitSpec &sp) { return sp.walk.empty() ? "" : ", const StaticGrid &sg"; }
+const char *walk_arg(const JitSpec &sp) { return sp.walk.empty() ? "" : ", sg"; }
+
+// The program's constant pool as literals.
+void define_pool(std::ostringstream &o, const Program &p) {
+  o << "__device__ constexpr float kPool[] = {0.f";
+  char b[40];
+  for (float f : p.pool) {
+    if (f - f == 0.f) std::snprintf(b, sizeof(b), ", %af", double(f));
+    else std::snprintf(b, sizeof(b), ", %s", f != f ? "__builtin_nanf(\"\")" : f > 0 ? "__builtin_huge_valf()" : "-__builtin_huge_valf()");
+    o << b;
+  }
+  o << "};\n#define pool (kPool + 1)\n";
+}
+
+// One copy of the date generator for the program's reading instructions: a
+// reading instruction that needs dates jumps to PC_GEN and it jumps back to
+// the top of that instruction (`resume` restores its static state).
+template <typename RESUME>
+void shared_generator(std::ostringstream &o, const Program &p, const std::vector<std::string> &known,
+                      const char *advance, RESUME resume) {
+  bool any = false;
+  for (size_t i = 0; i < p.code.size(); ++i) any = any || (reads_dates(p.code[i]) && known[i].empty());
+  if (!any) return;
+  o << "  int need_ = 0, resume_ = -1;\n"
+    << "  goto L0;\n"
+    << "PC_GEN:\n"
+    << "  " << advance << "\n"
+    << "  switch (resume_) {\n";
+  for (size_t i = 0; i < p.code.size(); ++i)
+    if (reads_dates(p.code[i]) && known[i].empty()) resume(i);
+  o << "    default: return tos;\n"
+    << "  }\n";
+}
+// Per instruction the ENSURE text of a reading instruction whose state is
+// known; empty for the others (and without a walk).
+std::vector<std::string> known_sites(const Program &p, const JitSpec &sp, const char *args) {
+  std::vector<std::string> known(p.code.size());
+  if (sp.walk.empty()) return known;
+  const std::vector<FlowState> at = flow_states(p, sp);
+  for (size_t i = 0; i < p.code.size(); ++i)
+    if (reads_dates(p.code[i])) known_ensure(p.code[i], at[i], sp, args, known[i]);
+  return known;
+}
+std::string shared_ensure(size_t i) {
+  return "#define ENSURE(o) { if ((o) > m.n || (o) < -m.n_hist) { atomicOr(a.status, 1); "
+         "(o) = (o) > m.n ? m.n : -m.n_hist; } if (ps.f < (o)) { need_ = (o); resume_ = " +
+         std::to_string(i) + "; goto PC_GEN; } }\n";
+}
+
+// The sensitivity evaluators straight-line over the program: each
+// instruction is the interpreter's case for its constant opcode and fields
+// (ops_inc), followed by a jump to whichever of its possible successors the
+// case left in pc.  The operand stack stays in shared memory, as in the
+// interpreter, so the shared date generator needs no stack depths.
+void sensitivity_blocks(std::ostringstream &o, const Program &p, const JitSpec &sp, const char *ops_inc,
+                        const char *end) {
   const size_t n = p.code.size();
-  o << "#include \"pc_adjoint.cuh\"\n"
-    << "namespace pc {\n"
-    << "namespace {\n"
-    << "constexpr int D = " << d << ";\n"
-    << "__device__ __forceinline__ float2 jit_eval_adjoint(const uint4 *P, const float *pool, float2 *R,\n"
-    << "    const PriceArgs &a, const Rng2 &g, bool live0, bool live1, const float (&Bm)[D * D],\n"
-    << "    const float (&S0)[D], const float (&Lm)[D * D], Tape &T, int &res) {\n"
-    << "#include \"pc_adjoint_state.inc\"\n"
-    << "  goto L0;\n";
+  const bool shared = date_sites(p) >= 2;
+  const std::vector<std::string> known = known_sites(p, sp, "(true, false, Lm)");
+  if (shared)
+    shared_generator(o, p, known, "while (ps.f < need_) NEXT_DATE(true, false, Lm);",
+                     [&](size_t i) { o << "    case " << i << ": goto L" << i << ";\n"; });
+  o << "  goto L0;\n";
   for (size_t i = 0; i < n; ++i) {
     const XInsn &I = p.code[i];
     o << "L" << i << ": {\n"
@@ -175,68 +336,75 @@ std::string generate_adjoint(const Program &p, int d, bool write) {
       << "  const uint4 I = " << insn_literal(I) << ";\n"
       << "  const uint32_t op = " << hex(I.opa & 0xffu) << ";\n"
       << "  const float kk = __uint_as_float(" << hex(I.b) << ");\n"
-      << "#include \"pc_adjoint_ops.inc\"\n";
+      << "#define NEXT_INSN " << insn_literal(i + 1 < n ? p.code[i + 1] : I) << "\n"
+      << (!known[i].empty() ? known[i]
+          : shared && reads_dates(I) ? shared_ensure(i) : std::string("#define ENSURE(o) ensure(o)\n"))
+      << "#include \"" << ops_inc << "\"\n"
+      << "#undef ENSURE\n#undef NEXT_INSN\n";
     std::vector<uint32_t> next = {uint32_t(i + 1), I.c, I.e, uint32_t(i + 2)};
     for (size_t j = 0; j < next.size(); ++j) {
       bool seen = false;
       for (size_t q = 0; q < j; ++q) seen = seen || next[q] == next[j];
       if (!seen && next[j] < n) o << "  if (pc == " << next[j] << ") goto L" << next[j] << ";\n";
     }
-    o << "  res = tid;\n"
-      << "  return tos;\n"
+    o << end << "  return tos;\n"
       << "}\n";
   }
+}
+
+// pc_jit_adjoint: adjoint_tiles around the specialised adjoint evaluator.
+std::string generate_adjoint(const Program &p, const JitSpec &sp, bool write) {
+  std::ostringstream o;
+  define_walk(o, sp);
+  o << "#include \"pc_adjoint.cuh\"\n"
+    << "namespace pc {\n"
+    << "namespace {\n"
+    << "constexpr int D = " << sp.d << ";\n";
+  define_pool(o, p);
+  o << "__device__ __forceinline__ float2 jit_eval_adjoint(const uint4 *P, float2 *R,\n"
+    << "    const PriceArgs &a, const Rng2 &g, bool live0, bool live1, const float (&Bm)[D * D],\n"
+    << "    const float (&S0)[D], const float (&Lm)[D * D], Tape &T, int &res" << walk_eval_param(sp) << ") {\n"
+    << "#include \"pc_adjoint_state.inc\"\n";
+  sensitivity_blocks(o, p, sp, "pc_adjoint_ops.inc", "  res = tid;\n");
   o << "}\n"
+    << "#undef pool\n"
     << "}  // namespace\n"
     << "}  // namespace pc\n"
     << "extern \"C\" __global__ void __launch_bounds__(" << kBlock
-    << ") pc_jit_adjoint(const __grid_constant__ pc::PriceArgs a, const pc::TapeArgs t) {\n"
-    << "  pc::adjoint_tiles<pc::D, " << (write ? "true" : "false") << ">(a, t, [&](const uint4 *P, const float *pool,\n"
+    << ") pc_jit_adjoint(const __grid_constant__ pc::PriceArgs a, const pc::TapeArgs t" << walk_kernel_param(sp) << ") {\n"
+    << "  pc::adjoint_tiles<pc::D, " << (write ? "true" : "false") << ">(a, t, [&](const uint4 *P, const float *,\n"
     << "      float2 *R, const pc::Rng2 &g, bool live0, bool live1, const float (&Bm)[pc::D * pc::D],\n"
     << "      const float (&S0)[pc::D], const float (&Lm)[pc::D * pc::D], pc::Tape &T, int &res) {\n"
-    << "    return pc::jit_eval_adjoint(P, pool, R, a, g, live0, live1, Bm, S0, Lm, T, res); });\n"
+    << "    return pc::jit_eval_adjoint(P, R, a, g, live0, live1, Bm, S0, Lm, T, res" << walk_arg(sp) << "); });\n"
     << "}\n";
   return o.str();
 }
 
-std::string generate_greeks(const Program &p, int d, bool write) {
+// pc_jit_greeks: greeks_tiles around the specialised tangent evaluator (the
+// per-path triples written out with kJitGreeks + 1).
+std::string generate_greeks(const Program &p, const JitSpec &sp, bool write) {
   std::ostringstream o;
-  const size_t n = p.code.size();
-  if (date_sites(p) > kInlineTangentDateSites) o << "#define PC_JIT_OUTLINE_DATES 1\n";
+  define_walk(o, sp);
   o << "#include \"pc_greeks.cuh\"\n"
     << "namespace pc {\n"
     << "namespace {\n"
-    << "constexpr int D = " << d << ";\n"
-    << "__device__ __forceinline__ TV jit_eval_greeks(const uint4 *P, const float *pool, float2 *R,\n"
+    << "constexpr int D = " << sp.d << ";\n";
+  define_pool(o, p);
+  o << "__device__ __forceinline__ TV jit_eval_greeks(const uint4 *P, float2 *R,\n"
     << "    const PriceArgs &a, const Rng2 &g, bool live0, bool live1, const float (&Bm)[D * D],\n"
-    << "    const float (&S0)[D], const float (&Lm)[D * D], int gl, float sig_g) {\n"
-    << "#include \"pc_greeks_state.inc\"\n"
-    << "  goto L0;\n";
-  for (size_t i = 0; i < n; ++i) {
-    const XInsn &I = p.code[i];
-    o << "L" << i << ": {\n"
-      << "  pc = " << i << ";\n"
-      << "  const uint4 I = " << insn_literal(I) << ";\n"
-      << "  const uint32_t op = " << hex(I.opa & 0xffu) << ";\n"
-      << "  const float kk = __uint_as_float(" << hex(I.b) << ");\n"
-      << "#include \"pc_greeks_ops.inc\"\n";
-    std::vector<uint32_t> next = {uint32_t(i + 1), I.c, I.e, uint32_t(i + 2)};
-    for (size_t j = 0; j < next.size(); ++j) {
-      bool seen = false;
-      for (size_t q = 0; q < j; ++q) seen = seen || next[q] == next[j];
-      if (!seen && next[j] < n) o << "  if (pc == " << next[j] << ") goto L" << next[j] << ";\n";
-    }
-    o << "  return tos;\n"
-      << "}\n";
-  }
+    << "    const float (&S0)[D], const float (&Lm)[D * D], int gl, float sig_g" << walk_eval_param(sp) << ") {\n"
+    << "#include \"pc_greeks_state.inc\"\n";
+  sensitivity_blocks(o, p, sp, "pc_greeks_ops.inc", "");
   o << "}\n"
+    << "#undef pool\n"
     << "}  // namespace\n"
     << "}  // namespace pc\n"
-    << "extern \"C\" __global__ void __launch_bounds__(" << kBlock << ") pc_jit_greeks(const __grid_constant__ pc::PriceArgs a) {\n"
-    << "  pc::greeks_tiles<pc::D, " << (write ? "true" : "false") << ">(a, [&](const uint4 *P, const float *pool,\n"
+    << "extern \"C\" __global__ void __launch_bounds__(" << kBlock
+    << ") pc_jit_greeks(const __grid_constant__ pc::PriceArgs a" << walk_kernel_param(sp) << ") {\n"
+    << "  pc::greeks_tiles<pc::D, " << (write ? "true" : "false") << ">(a, [&](const uint4 *P, const float *,\n"
     << "      float2 *R, const pc::Rng2 &g, bool live0, bool live1, const float (&Bm)[pc::D * pc::D],\n"
     << "      const float (&S0)[pc::D], const float (&Lm)[pc::D * pc::D], int gl, float sig_g) {\n"
-    << "    return pc::jit_eval_greeks(P, pool, R, a, g, live0, live1, Bm, S0, Lm, gl, sig_g); });\n"
+    << "    return pc::jit_eval_greeks(P, R, a, g, live0, live1, Bm, S0, Lm, gl, sig_g" << walk_arg(sp) << "); });\n"
     << "}\n";
   return o.str();
 }
@@ -251,16 +419,16 @@ std::string generate_greeks(const Program &p, int d, bool write) {
 // static stack pointer there (so the operand stack stays in registers).
 // Otherwise the generator is inlined at each reading instruction (out of
 // line beyond kInlineDateSites of them).
-std::string generate(const Program &p, int d, int kind) {
-  if (kind >= kJitAdjoint) return generate_adjoint(p, d, (kind & 1) != 0);
-  if (kind >= kJitGreeks) return generate_greeks(p, d, (kind & 1) != 0);
+std::string generate(const Program &p, const JitSpec &spec) {
+  const int d = spec.d, kind = spec.kind;
+  if (kind >= kJitAdjoint) return generate_adjoint(p, spec, (kind & 1) != 0);
+  if (kind >= kJitGreeks) return generate_greeks(p, spec, (kind & 1) != 0);
   std::ostringstream o;
   const size_t n = p.code.size();
   std::vector<int> sp_at;
   const bool shared = date_sites(p) >= 2 && date_sites(p) <= kSharedDateSites && stack_depths(p, sp_at);
-  // without re-entry points, many reading instructions call one
-  // out-of-line copy instead of inlining the generator at each
-  if (!shared && date_sites(p) > kInlineDateSites) o << "#define PC_JIT_OUTLINE_DATES 1\n";
+  if (outlined_dates(p)) o << "#define PC_JIT_OUTLINE_DATES 1\n";
+  define_walk(o, spec);
   // a program that reads no date behind the frontier keeps that date's S in
   // registers instead of a shared-memory window
   if ((kind < kJitCv && (kind & kJitWinRegs)) || (kind >= kJitCv && ((kind - kJitCv) & kCvWinRegs)))
@@ -276,26 +444,21 @@ std::string generate(const Program &p, int d, int kind) {
     << "namespace {\n"
     << "constexpr int D = " << d << ";\n"
     << "constexpr bool GW = " << (kind < kJitCv && (kind & kJitHbm) ? "true" : "false") << ";\n"
-    << "#define PC_JIT_STACK_SLOTS " << std::max(1, int(p.frame_slots)) << "\n"
-    << "template <class PcHook = NoDateHook>\n"
-    << "__device__ __forceinline__ PV jit_eval(const uint4 *P, const float *pool, float2 *R,\n"
+    << "#define PC_JIT_STACK_SLOTS " << std::max(1, int(p.frame_slots)) << "\n";
+  define_pool(o, p);
+  o << "template <class PcHook = NoDateHook>\n"
+    << "__device__ __forceinline__ PV jit_eval(const uint4 *P, float2 *R,\n"
     << (pairs2 ? "    const PriceArgs &a, const RngH<2> &g, const bool (&live_)[kPL], const float (&Bm)[D * D],\n"
                : "    const PriceArgs &a, const Rng2 &g, bool live0, bool live1, const float (&Bm)[D * D],\n")
-    << "    const float (&S0)[D], int *frontier = nullptr, PcHook *hook_ = nullptr) {\n"
+    << "    const float (&S0)[D]" << walk_eval_param(spec) << ", int *frontier = nullptr, PcHook *hook_ = nullptr) {\n"
     << "#include \"pc_eval_state.inc\"\n"
     << "  (void)pc;\n";
-  if (shared) {
-    o << "  int need_ = 0, resume_ = -1;\n"
-      << "  goto L0;\n"
-      << "PC_GEN:\n"
-      << "  while (ps.f < need_) GEN_DATE(ps.f + 1);\n"
-      << "  switch (resume_) {\n";
-    for (size_t i = 0; i < n; ++i)
-      if (reads_dates(p.code[i]) && sp_at[i] >= 0)
-        o << "    case " << i << ": sp = " << sp_at[i] << "; goto L" << i << ";\n";
-    o << "    default: return tos;\n"
-      << "  }\n";
-  }
+  const std::vector<std::string> known =
+      known_sites(p, spec, kind < kJitCv && (kind & kJitHbm) ? "(false, true, nullptr)" : "(false, false, nullptr)");
+  if (shared)
+    shared_generator(o, p, known, "EACH_DATE(need_)", [&](size_t i) {
+      if (sp_at[i] >= 0) o << "    case " << i << ": sp = " << sp_at[i] << "; goto L" << i << ";\n";
+    });
   for (size_t i = 0; i < n; ++i) {
     const XInsn &I = p.code[i];
     const size_t nx = i + 1 < n ? i + 1 : i;
@@ -306,10 +469,10 @@ std::string generate(const Program &p, int d, int kind) {
       << "#define JUMP_W { goto " << lbl(I.e) << "; }\n"
       << "#define JUMP_2 { goto " << lbl(i + 2) << "; }\n"
       << "#define NEXT_INSN " << (i + 1 < n ? insn_literal(p.code[i + 1]) : insn_literal(I)) << "\n";
-    if (shared && reads_dates(I) && sp_at[i] >= 0)
-      o << "#define ENSURE(o) { if ((o) > m.n || (o) < -m.n_hist) { atomicOr(a.status, 1); "
-           "(o) = (o) > m.n ? m.n : -m.n_hist; } if (ps.f < (o)) { need_ = (o); resume_ = "
-        << i << "; goto PC_GEN; } }\n";
+    if (!known[i].empty())
+      o << known[i];
+    else if (shared && reads_dates(I) && sp_at[i] >= 0)
+      o << shared_ensure(i);
     else
       o << "#define ENSURE(o) ensure(o)\n";
     o << "  const uint4 I = " << insn_literal(I) << ";\n"
@@ -318,7 +481,7 @@ std::string generate(const Program &p, int d, int kind) {
       << "}\n";
   }
   o << "  return tos;\n"
-    << "#undef PUSH\n#undef STK\n#undef BINF\n#undef BINI\n#undef IMM\n#undef GEN_DATE\n"
+    << "#undef PUSH\n#undef STK\n#undef BINF\n#undef BINI\n#undef IMM\n#undef EACH_DATE\n#undef pool\n"
     << "}\n"
     << "}  // namespace\n"
     << "}  // namespace pc\n";
@@ -329,12 +492,12 @@ std::string generate(const Program &p, int d, int kind) {
     o << "#ifndef PC_MIN_BLOCKS\n#define PC_MIN_BLOCKS " << kJitCvMinBlocks << "\n#endif\n"
       << "extern \"C\" __global__ void __launch_bounds__(" << kBlock
       << ", PC_MIN_BLOCKS) pc_jit_cv(const __grid_constant__ pc::PriceArgs a,\n"
-      << "    const __grid_constant__ pc::CvArgs c) {\n"
+      << "    const __grid_constant__ pc::CvArgs c" << walk_kernel_param(spec) << ") {\n"
       << "  using Hook = pc::CvOnline<pc::D, " << (gamma ? "true" : "false") << ">;\n"
-      << "  pc::cv_tiles<pc::D, " << ((kind - kJitCv) & 7) << ">(a, c, [&](const uint4 *P, const float *pool, float2 *R,\n"
+      << "  pc::cv_tiles<pc::D, " << ((kind - kJitCv) & 7) << ">(a, c, [&](const uint4 *P, const float *, float2 *R,\n"
       << "      const pc::Rng2 &g, bool live0, bool live1, const float (&Bm)[pc::D * pc::D],\n"
       << "      const float (&S0)[pc::D], Hook *hook) {\n"
-      << "    return pc::jit_eval<Hook>(P, pool, R, a, g, live0, live1, Bm, S0, nullptr, hook); });\n"
+      << "    return pc::jit_eval<Hook>(P, R, a, g, live0, live1, Bm, S0" << walk_arg(spec) << ", nullptr, hook); });\n"
       << "}\n";
     return o.str();
   }
@@ -343,15 +506,15 @@ std::string generate(const Program &p, int d, int kind) {
   // launch's shared memory already allows fewer, whose bound then leaves the
   // kernel the registers those blocks can have)
   o << "#ifndef PC_MIN_BLOCKS\n#define PC_MIN_BLOCKS " << kJitMinBlocks << "\n#endif\n"
-    << "extern \"C\" __global__ void __launch_bounds__(" << kBlock << ", PC_MIN_BLOCKS) pc_jit_price(const __grid_constant__ pc::PriceArgs a) {\n";
+    << "extern \"C\" __global__ void __launch_bounds__(" << kBlock << ", PC_MIN_BLOCKS) pc_jit_price(const __grid_constant__ pc::PriceArgs a" << walk_kernel_param(spec) << ") {\n";
   if (pairs2)
-    o << "  pc::price_tiles2<pc::D, " << (kind & kJitPriceWrite ? "true" : "false") << ">(a, [&](const uint4 *P, const float *pool,\n"
+    o << "  pc::price_tiles2<pc::D, " << (kind & kJitPriceWrite ? "true" : "false") << ">(a, [&](const uint4 *P, const float *,\n"
       << "      float2 *R, const pc::RngH<2> &g, const bool (&live)[4], const float (&Bm)[pc::D * pc::D],\n"
-      << "      const float (&S0)[pc::D]) { return pc::jit_eval(P, pool, R, a, g, live, Bm, S0); });\n";
+      << "      const float (&S0)[pc::D]) { return pc::jit_eval(P, R, a, g, live, Bm, S0" << walk_arg(spec) << "); });\n";
   else
-    o << "  pc::price_tiles<pc::D, " << (kind & kJitPriceWrite ? "true" : "false") << ">(a, [&](const uint4 *P, const float *pool,\n"
+    o << "  pc::price_tiles<pc::D, " << (kind & kJitPriceWrite ? "true" : "false") << ">(a, [&](const uint4 *P, const float *,\n"
       << "      float2 *R, const pc::Rng2 &g, bool live0, bool live1, const float (&Bm)[pc::D * pc::D],\n"
-      << "      const float (&S0)[pc::D]) { return pc::jit_eval(P, pool, R, a, g, live0, live1, Bm, S0); });\n";
+      << "      const float (&S0)[pc::D]) { return pc::jit_eval(P, R, a, g, live0, live1, Bm, S0" << walk_arg(spec) << "); });\n";
   o << "}\n";
   return o.str();
 }
@@ -369,18 +532,16 @@ pc_status nvrtc_fail(nvrtcResult r, nvrtcProgram prog, const char *what) {
 
 // NVRTC: the generated source and the embedded device headers to a cubin
 // for `arch` (e.g. "sm_103a").
-pc_status to_cubin(const Program &p, int d, int kind, int block, int min_blocks, const std::string &arch,
-                   std::vector<char> &cubin) {
-  const std::string src = generate(p, d, kind);
+pc_status to_cubin(const Program &p, const JitSpec &spec, const std::string &arch, std::vector<char> &cubin) {
+  const std::string src = generate(p, spec);
   nvrtcProgram prog = nullptr;
   nvrtcResult r = nvrtcCreateProgram(&prog, src.c_str(), "pc_jit.cu", kJitHeaderCount, kJitHeaderSrcs,
                                      kJitHeaderNames);
   if (r != NVRTC_SUCCESS) return nvrtc_fail(r, nullptr, "run-time compiler");
   const std::string a = "-arch=" + arch;
-  const std::string stride = "-DPC_SLOT_STRIDE=" + std::to_string(block);
-  const std::string bound = "-DPC_MIN_BLOCKS=" + std::to_string(min_blocks > 0 ? min_blocks : kJitMinBlocks);
-  const char *opts[] = {a.c_str(), "-std=c++17", "-default-device", "-DPC_JIT", stride.c_str(), bound.c_str()};
-  r = nvrtcCompileProgram(prog, 6, opts);
+  const std::string bound = "-DPC_MIN_BLOCKS=" + std::to_string(spec.min_blocks > 0 ? spec.min_blocks : kJitMinBlocks);
+  const char *opts[] = {a.c_str(), "-std=c++17", "-default-device", "-DPC_JIT", bound.c_str(), "-DPC_ONE_PHI"};
+  r = nvrtcCompileProgram(prog, spec.one_phi ? 6 : 5, opts);
   if (r != NVRTC_SUCCESS) {
     pc_status s = nvrtc_fail(r, prog, "run-time compilation");
     nvrtcDestroyProgram(&prog);
@@ -395,18 +556,19 @@ pc_status to_cubin(const Program &p, int d, int kind, int block, int min_blocks,
   return PC_OK;
 }
 
-pc_status compile(const Program &p, int d, int kind, int block, int min_blocks, int device, cudaLibrary_t &lib,
-                  cudaKernel_t &kern) {
+const char *jit_entry_name(int kind) {
+  return kind >= kJitAdjoint ? "pc_jit_adjoint" : kind >= kJitGreeks ? "pc_jit_greeks"
+         : kind >= kJitCv ? "pc_jit_cv" : "pc_jit_price";
+}
+
+pc_status compile(const Program &p, const JitSpec &spec, int device, cudaLibrary_t &lib, cudaKernel_t &kern) {
   cudaDeviceProp prop{};
   CU(cudaGetDeviceProperties(&prop, device), "device properties");
   std::vector<char> cubin;
-  pc_status s = to_cubin(p, d, kind, block, min_blocks,
-                         "sm_" + std::to_string(prop.major) + std::to_string(prop.minor) + "a", cubin);
+  pc_status s = to_cubin(p, spec, "sm_" + std::to_string(prop.major) + std::to_string(prop.minor) + "a", cubin);
   if (s != PC_OK) return s;
   CU(cudaLibraryLoadData(&lib, cubin.data(), nullptr, nullptr, 0, nullptr, nullptr, 0), "module load");
-  cudaError_t e = cudaLibraryGetKernel(&kern, lib, kind >= kJitAdjoint ? "pc_jit_adjoint"
-                                                    : kind >= kJitGreeks ? "pc_jit_greeks"
-                                                    : kind >= kJitCv ? "pc_jit_cv" : "pc_jit_price");
+  cudaError_t e = cudaLibraryGetKernel(&kern, lib, jit_entry_name(spec.kind));
   if (e != cudaSuccess) {
     cudaLibraryUnload(lib);
     lib = nullptr;
@@ -423,56 +585,30 @@ namespace pc {
 bool jit_eligible(const pc_contract *k) { return k->prog.code.size() <= size_t(PC_JIT_MAX_INSNS); }
 
 bool adjoint_jit_eligible(const pc_contract *k) {
-  return jit_eligible(k) && date_sites(k->prog) <= kInlineTangentDateSites;
+  return jit_eligible(k) && date_sites(k->prog) <= kAdjointDateSites;
 }
 
-pc_status jit_kernel(const pc_contract *k, int d, int kind, int block, cudaKernel_t &out, int min_blocks) {
-  // the program's words: code, then pool bits
-  std::vector<uint32_t> words;
-  words.reserve(k->prog.code.size() * 4 + k->prog.pool.size());
-  for (const XInsn &I : k->prog.code) {
-    words.push_back(I.opa);
-    words.push_back(I.b);
-    words.push_back(I.c);
-    words.push_back(I.e);
-  }
-  for (float f : k->prog.pool) {
-    uint32_t u;
-    std::memcpy(&u, &f, 4);
-    words.push_back(u);
-  }
-  uint64_t h = 1469598103934665603ull;  // FNV-1a
-  for (uint32_t w : words)
-    for (int b = 0; b < 4; ++b) h = (h ^ ((w >> (8 * b)) & 0xffu)) * 1099511628211ull;
-  pc_ctx *c = k->ctx;
-  std::lock_guard<std::mutex> g(c->jit_mu);
-  auto range = c->jit_cache.equal_range(h);
-  for (auto it = range.first; it != range.second; ++it) {
-    const JitEntry &E = it->second;
-    if (E.d == d && E.kind == kind && E.block == block && E.min_blocks == min_blocks && E.program == words) {
-      out = E.kernel;
-      return PC_OK;
-    }
-  }
-  JitEntry E;
-  E.program = words;
-  E.d = d;
-  E.kind = kind;
-  E.block = block;
-  E.min_blocks = min_blocks;
-  pc_status s = compile(k->prog, d, kind, block, min_blocks, c->device, E.lib, E.kernel);
-  if (s != PC_OK) return s;
-  out = E.kernel;
-  c->jit_cache.emplace(h, std::move(E));
-  return PC_OK;
+JitSpec jit_spec(const pc_contract *k, const PriceArgs &a, int kind, int min_blocks, const std::vector<int32_t> &walk) {
+  JitSpec sp;
+  sp.d = a.m.d;
+  sp.kind = kind;
+  sp.min_blocks = min_blocks;
+  sp.walk = walk;
+  sp.one_phi = one_phi(a.path_offset, a.n_tiles);
+  // constants by value, unless an out-of-line date generator takes them by reference
+  if (kind >= kJitCv || !outlined_dates(k->prog))
+    sp.lay = {a.lay.stack, a.lay.off_bstack, a.lay.off_cache, a.lay.off_win, a.lay.off_xwin, a.lay.words, a.lay.win};
+  if (!walk.empty()) sp.grid = {a.m.n, a.m.n_hist, a.m.t_now};
+  return sp;
+}
+
+bool walk_jit_eligible(const Program &p) {
+  std::vector<int> sp_at;
+  return date_sites(p) <= 2 || (date_sites(p) <= kSharedDateSites && stack_depths(p, sp_at));
 }
 
 namespace {
-const char *jit_entry_name(int kind) {
-  return kind >= kJitAdjoint ? "pc_jit_adjoint" : kind >= kJitGreeks ? "pc_jit_greeks"
-         : kind >= kJitCv ? "pc_jit_cv" : "pc_jit_price";
-}
-
+// The program's words: code, then pool bits.
 std::vector<uint32_t> program_words(const Program &p) {
   std::vector<uint32_t> words;
   words.reserve(p.code.size() * 4 + p.pool.size());
@@ -489,7 +625,48 @@ std::vector<uint32_t> program_words(const Program &p) {
   }
   return words;
 }
+uint64_t words_hash(const std::vector<uint32_t> &words) {
+  uint64_t h = 1469598103934665603ull;  // FNV-1a
+  for (uint32_t w : words)
+    for (int b = 0; b < 4; ++b) h = (h ^ ((w >> (8 * b)) & 0xffu)) * 1099511628211ull;
+  return h;
+}
+// The cached kernel of these words and this spec (jit_mu held); null if none.
+cudaKernel_t cached(pc_ctx *c, uint64_t h, const std::vector<uint32_t> &words, const JitSpec &spec) {
+  auto range = c->jit_cache.equal_range(h);
+  for (auto it = range.first; it != range.second; ++it)
+    if (it->second.spec == spec && it->second.program == words) return it->second.kernel;
+  return nullptr;
+}
 }  // namespace
+
+bool admit_walk(pc_ctx *c, const Program &p, const ModelHost &H, const std::vector<int32_t> &walk) {
+  std::vector<int32_t> key = {H.d, H.n, H.n_hist, H.t_now};
+  key.insert(key.end(), walk.begin(), walk.end());
+  const uint64_t h = words_hash(program_words(p));
+  std::lock_guard<std::mutex> g(c->jit_mu);
+  auto &known = c->jit_walks[h];
+  if (std::find(known.begin(), known.end(), key) != known.end()) return true;
+  if (known.size() >= kWalksPerProgram) return false;
+  known.push_back(std::move(key));
+  return true;
+}
+
+pc_status jit_kernel(const pc_contract *k, const JitSpec &spec, cudaKernel_t &out) {
+  JitEntry E;
+  E.program = program_words(k->prog);
+  E.spec = spec;
+  const uint64_t h = words_hash(E.program);
+  pc_ctx *c = k->ctx;
+  std::lock_guard<std::mutex> g(c->jit_mu);
+  out = cached(c, h, E.program, spec);
+  if (out) return PC_OK;
+  pc_status s = compile(k->prog, spec, c->device, E.lib, E.kernel);
+  if (s != PC_OK) return s;
+  out = E.kernel;
+  c->jit_cache.emplace(h, std::move(E));
+  return PC_OK;
+}
 
 pc_status jit_compile_many(pc_ctx *c, const std::vector<JitRequest> &reqs) {
   // the requests not yet in the context's cache (each once)
@@ -507,20 +684,9 @@ pc_status jit_compile_many(pc_ctx *c, const std::vector<JitRequest> &reqs) {
       Miss m;
       m.r = &r;
       m.words = program_words(r.k->prog);
-      uint64_t h = 1469598103934665603ull;  // FNV-1a, as jit_kernel
-      for (uint32_t w : m.words)
-        for (int b = 0; b < 4; ++b) h = (h ^ ((w >> (8 * b)) & 0xffu)) * 1099511628211ull;
-      m.h = h;
-      bool have = false;
-      auto range = c->jit_cache.equal_range(h);
-      for (auto it = range.first; it != range.second && !have; ++it) {
-        const JitEntry &E = it->second;
-        have = E.d == r.d && E.kind == r.kind && E.block == r.block && E.min_blocks == r.min_blocks &&
-               E.program == m.words;
-      }
-      for (const Miss &o : miss)
-        have = have || (o.h == h && o.r->d == r.d && o.r->kind == r.kind && o.r->block == r.block &&
-                         o.r->min_blocks == r.min_blocks && o.words == m.words);
+      m.h = words_hash(m.words);
+      bool have = cached(c, m.h, m.words, r.spec) != nullptr;
+      for (const Miss &o : miss) have = have || (o.h == m.h && o.r->spec == r.spec && o.words == m.words);
       if (!have) miss.push_back(std::move(m));
     }
   }
@@ -533,7 +699,7 @@ pc_status jit_compile_many(pc_ctx *c, const std::vector<JitRequest> &reqs) {
   auto work = [&]() {
     for (size_t i = next++; i < miss.size(); i = next++) {
       const JitRequest &r = *miss[i].r;
-      miss[i].s = to_cubin(r.k->prog, r.d, r.kind, r.block, r.min_blocks, arch, miss[i].cubin);
+      miss[i].s = to_cubin(r.k->prog, r.spec, arch, miss[i].cubin);
     }
   };
   const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
@@ -547,12 +713,9 @@ pc_status jit_compile_many(pc_ctx *c, const std::vector<JitRequest> &reqs) {
     if (m.s != PC_OK) return m.s;
     JitEntry E;
     E.program = m.words;
-    E.d = m.r->d;
-    E.kind = m.r->kind;
-    E.block = m.r->block;
-    E.min_blocks = m.r->min_blocks;
+    E.spec = m.r->spec;
     CU(cudaLibraryLoadData(&E.lib, m.cubin.data(), nullptr, nullptr, 0, nullptr, nullptr, 0), "module load");
-    cudaError_t e = cudaLibraryGetKernel(&E.kernel, E.lib, jit_entry_name(E.kind));
+    cudaError_t e = cudaLibraryGetKernel(&E.kernel, E.lib, jit_entry_name(E.spec.kind));
     if (e != cudaSuccess) {
       cudaLibraryUnload(E.lib);
       return cuda_fail(e, "kernel lookup");
@@ -592,7 +755,7 @@ extern "C" pc_status pc_debug_jit_compile(const uint32_t *bytecode, size_t n_wor
   pc_status s = compile_program(bytecode, n_words, consts, n_consts, tparams, n_params, p1, p2, true, p, err);
   if (s != PC_OK) return fail(s, err);
   std::vector<char> cubin;
-  s = to_cubin(p, d, kind, kBlock, 0, "sm_103a", cubin);
+  s = to_cubin(p, JitSpec{d, kind}, "sm_103a", cubin);
   if (s != PC_OK) return s;
   *cubin_bytes = cubin.size();
   return PC_OK;
@@ -613,7 +776,7 @@ extern "C" pc_status pc_debug_jit_source(const uint32_t *bytecode, size_t n_word
   std::string err;
   pc_status s = compile_program(bytecode, n_words, consts, n_consts, tparams, n_params, p1, p2, true, p, err);
   if (s != PC_OK) return fail(s, err);
-  const std::string src = generate(p, d, kind);
+  const std::string src = generate(p, JitSpec{d, kind});
   *len = src.size();
   if (out && cap > src.size()) std::memcpy(out, src.c_str(), src.size() + 1);
   return PC_OK;

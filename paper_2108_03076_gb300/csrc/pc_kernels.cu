@@ -59,18 +59,14 @@ __device__ __forceinline__ void batch_unit(const PriceArgs &a, const BatchUnit &
   float Bm[D * D], S0[D];
   load_model_regs<D>(a.m, Bm, S0);
   Rng2 g;
-  g.stream = a.stream;
-#pragma unroll
-  for (int i = 0; i < 20; ++i) g.rk[i] = a.rk[i];
+  rng_init(g, a.rk, a.stream, a.path_offset);
   for (uint32_t k = 0; k < U.n_tiles; ++k) {
     const uint64_t tile = U.tile0 + k;
     const uint64_t i0 = tile * kTilePaths + lane, i1 = i0 + 32;
     const bool live0 = i0 < a.n_paths, live1 = i1 < a.n_paths;
     const uint64_t p0 = a.path_offset + i0, p1 = a.path_offset + i1;
-    g.plo[0] = uint32_t(p0);
-    g.phi[0] = uint32_t(p0 >> 32);
-    g.plo[1] = uint32_t(p1);
-    g.phi[1] = uint32_t(p1 >> 32);
+    rng_path(g, 0, p0, a.path_offset);
+    rng_path(g, 1, p1, a.path_offset);
     const float2 x = eval_path<D>(P, pool, R, a, g, live0, live1, Bm, S0);
     Moments<2> mo;
     if (live0) {
@@ -93,7 +89,7 @@ __device__ __forceinline__ void batch_units(const BatchArgs &b, RUN run) {
   extern __shared__ __align__(16) uint32_t smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t *slot = smem + (b.slot_bytes / 4) * warp;
-  float2 *R = reinterpret_cast<float2 *>(smem + (b.slot_bytes / 4) * (blockDim.x >> 5)) + threadIdx.x;
+  float2 *R = warp_region(smem + (b.slot_bytes / 4) * (blockDim.x >> 5), b.words);
   const PriceArgs &a = *reinterpret_cast<const PriceArgs *>(slot);
   uint32_t cur = 0xffffffffu;
   for (;;) {
@@ -147,19 +143,15 @@ __global__ void __launch_bounds__(kBlock) debug_paths_kernel(const __grid_consta
                                                              const __grid_constant__ RoundKeys rk,
                                                              uint32_t stream, float *out) {
   extern __shared__ __align__(16) uint32_t smem[];
-  float2 *R = reinterpret_cast<float2 *>(smem) + threadIdx.x;
+  float2 *R = warp_region(smem, lay.words);
   const uint64_t i0 = 2 * (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x), i1 = i0 + 1;
   if (i0 >= n_paths) return;
   float Bm[D * D], S0[D];
   load_model_regs<D>(m, Bm, S0);
   Rng2 g;
-  g.plo[0] = uint32_t(offset + i0);
-  g.phi[0] = uint32_t((offset + i0) >> 32);
-  g.plo[1] = uint32_t(offset + i1);
-  g.phi[1] = uint32_t((offset + i1) >> 32);
-  g.stream = stream;
-#pragma unroll
-  for (int i = 0; i < 20; ++i) g.rk[i] = rk.k[i];
+  rng_init(g, rk.k, stream, offset);
+  rng_path(g, 0, offset + i0, offset);
+  rng_path(g, 1, offset + i1, offset);
   PathState<D> ps;
   path_state_init<D>(ps, R, lay);
   const size_t row = size_t(m.n) + 1;

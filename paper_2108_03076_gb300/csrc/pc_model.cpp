@@ -166,6 +166,16 @@ pc_status build_model(const pc_model_desc &desc, ModelHost &M, std::string &err)
   M.date_ops[n + 1] = int(M.ops.size());
   M.n_levels = n_levels;
   M.bstack = std::max(depth_max, 1);
+  // the same ops by date, for the walk that skips unread dates
+  M.nodes.assign(size_t(n) + 1, BridgeOp{});
+  M.nodes[0].m = uint16_t(2 * n);
+  for (size_t k = 0; k < M.ops.size(); ++k) {
+    BridgeOp op = M.ops[k];
+    const int date = op.m, right = nodes[op.j].r;
+    op.j = uint32_t(k);
+    op.m = uint16_t(right < 0 ? n : right);
+    M.nodes[date] = op;
+  }
 
   // Tables.
   const double log2e = 1.4426950408889634;
@@ -193,6 +203,38 @@ pc_status build_model(const pc_model_desc &desc, ModelHost &M, std::string &err)
   M.Lf.assign(M.L.begin(), M.L.end());
   M.sig.assign(M.sigma.begin(), M.sigma.end());
   return PC_OK;
+}
+
+std::vector<int32_t> static_walk(const ModelHost &H, const std::vector<uint8_t> &reads) {
+  const int n = H.n;
+  std::vector<int32_t> before(size_t(n) + 2, 0);  // dates read below o
+  for (int o = 0; o <= n; ++o) before[o + 1] = before[o] + (o > 0 && reads[o] ? 1 : 0);
+  const int total = before[n + 1];
+  std::vector<int32_t> walk;
+  if (total == 0) return walk;
+  std::vector<int> right = {n};  // right ends of the open intervals, the nearest last
+  int left = 0, ops = 0;
+  while (before[left + 1] < total) {  // a date right of `left` is read
+    const size_t at = walk.size();
+    walk.insert(walk.end(), {0, 0, 0});
+    auto op = [&](int date) {
+      walk.push_back(int32_t(H.nodes[date].j));
+      ++walk[at + 2];
+      ++ops;
+    };
+    if (left == 0) op(n);  // the root
+    while (right.back() - left >= 2 && before[right.back()] > before[left + 1]) {
+      const int m = (left + right.back()) / 2;
+      op(m);
+      right.push_back(m);
+    }
+    if (ops > kStaticOps) return {};
+    left = right.back();
+    right.pop_back();
+    walk[at] = left;
+    walk[at + 1] = reads[left] ? 1 : 0;
+  }
+  return walk;
 }
 
 }  // namespace pc

@@ -575,7 +575,7 @@ pc_status compile_program(const uint32_t *words, size_t n_words, const double *c
 }
 
 pc_status analyse_program(const Program &p, int32_t t_now, int32_t n_dates, int32_t n_hist,
-                          int32_t &win, std::string &err) {
+                          int32_t &win, std::vector<uint8_t> &reads, std::string &err) {
   auto on_fail = [&](pc_status st, int64_t t, int64_t o) {
     if (st == PC_ELIMIT)
       err = "program too long to analyse (loop trip counts)";
@@ -584,6 +584,8 @@ pc_status analyse_program(const Program &p, int32_t t_now, int32_t n_dates, int3
             ", grid " + std::to_string(-n_hist) + ".." + std::to_string(n_dates) + ")";
   };
   TimeWalk<decltype(on_fail)> walk{p.code.data(), t_now, n_dates, n_hist, on_fail};
+  reads.assign(size_t(n_dates) + 1, 0);
+  walk.reads = reads.data();
   walk.run(0, p.code.size(), 0);
   if (walk.st != PC_OK) return walk.st;
   win = walk.window();

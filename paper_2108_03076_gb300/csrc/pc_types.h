@@ -130,7 +130,9 @@ enum : uint16_t {
 // Device image of a model (one allocation, offsets in bytes).
 struct ModelDev {
   const int32_t *date_ops;  // [n+2] op range of date t: [date_ops[t], date_ops[t+1])
-  const BridgeOp *ops;      // [n]
+  const BridgeOp *ops;      // [n] in op order
+  const BridgeOp *nodes;    // [n+1] by date: the op of the date's node, its number in j, the right end of its
+                            // bisection interval in m; date 0: m = 2n, so that the first midpoint is the root
   const float2 *A;          // [(n+1)*d] log2(e)(r - sigma^2/2) tau_o (S = S0 2^(A + B W)), each twice
   const float *B;           // [d*d]     log2(e) sigma_i L_ik
   const float *disc;        // [n_hist+n+1] disc of ordinal o at index o + n_hist
@@ -148,8 +150,9 @@ struct ModelDev {
   float S0v[4];             // S0 of each underlying
 };
 
-// Per-thread shared-memory region: 32-bit words, word w of thread t at
-// region[w * BLOCK + t] (uniform w -> conflict-free).
+// Per-thread shared-memory region: float2 slots, slot s of lane l at
+// region[s * 32 + l] of the warp's own part (`words` slots): a uniform s is
+// conflict-free, and the stride is a constant whatever the block size.
 struct Layout {
   int32_t stack;      // operand stack words
   int32_t off_bstack; // bridge stack (bstack * d)
@@ -180,6 +183,15 @@ struct RoundKeys {
   uint32_t k[20];
 };
 
+// A specialised kernel's launch argument for a static walk (pc_jit.cpp): the
+// walk's at most kStaticOps ops' weights, each twice (the packed operand of
+// the lane's two paths), and its steps' drifts (ModelDev::A).
+constexpr int kStaticOps = 16;
+struct StaticGrid {
+  float2 wl[kStaticOps], wr[kStaticOps], sd[kStaticOps];
+  float A[kStaticOps][4];
+};
+
 // Philox4x32-10 round keys of a 64-bit seed: round r XORs (key0 + r W0,
 // key1 + r W1), the key bumped by the Weyl constants between rounds.
 inline void philox_round_keys(uint64_t seed, uint32_t *rk) {
@@ -203,8 +215,10 @@ struct PriceArgs {
   uint32_t rk[20];          // Philox round keys: (key0 + r W0, key1 + r W1) for r = 0..9
   uint64_t n_tiles;
   int32_t width;            // doubles per tile partial (2 for prices)
-  uint32_t chunk_tiles;     // tiles per reduction chunk
+  uint32_t chunk_tiles;     // tiles per reduction chunk (>= 2)
   uint32_t n_chunks;        // ceil(n_tiles / chunk_tiles) <= kMaxChunks
+  uint64_t chunk_magic;     // ceil(2^64 / chunk_tiles): tile / chunk_tiles = its high product with tile,
+                            // exact for tile * chunk_tiles < 2^64 (a 64-bit division per tile otherwise)
   double *tile_partials;    // [n_tiles * width] scratch
   unsigned char *control;   // kControlBytes of scratch, zero between launches (see below)
   double *out;              // [width + 1]: sums over all paths, then n_paths
@@ -230,11 +244,13 @@ constexpr int kMaxChunks = 256;
 constexpr size_t kChunkCountOff = 256;
 constexpr size_t kChunkPartOff = 2048;
 constexpr size_t kControlBytes = kChunkPartOff + size_t(kMaxChunks) * 8 * sizeof(double);
-inline void reduction_chunks(uint64_t n_tiles, uint32_t &chunk_tiles, uint32_t &n_chunks) {
-  uint64_t c = (n_tiles + kMaxChunks - 1) / kMaxChunks;
+inline void reduction_chunks(PriceArgs &a, uint32_t max_chunks = kMaxChunks) {
+  uint64_t c = (a.n_tiles + kMaxChunks - 1) / kMaxChunks;
   if (c < 64) c = 64;
-  chunk_tiles = uint32_t(c);
-  n_chunks = uint32_t((n_tiles + c - 1) / c);
+  if ((a.n_tiles + c - 1) / c > max_chunks) c = (a.n_tiles + max_chunks - 1) / max_chunks;
+  a.chunk_tiles = uint32_t(c);
+  a.n_chunks = uint32_t((a.n_tiles + c - 1) / c);
+  a.chunk_magic = ~uint64_t(0) / c + 1;
 }
 
 }  // namespace pc
