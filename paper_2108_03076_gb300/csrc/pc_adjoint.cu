@@ -9,7 +9,7 @@ namespace pc {
 namespace {
 
 template <int D, bool WRITE>
-__global__ void __launch_bounds__(kBlock) adjoint_kernel(const __grid_constant__ PriceArgs a, const TapeArgs t) {
+__global__ void __launch_bounds__(kBlock, D == 4 ? 4 : 5) adjoint_kernel(const __grid_constant__ PriceArgs a, const TapeArgs t) {
   adjoint_tiles<D, WRITE>(a, t, [&](const uint4 *P, const float *pool, float2 *R, const Rng2 &g, bool live0,
                                    bool live1, const float (&Bm)[D * D], const float (&S0)[D],
                                    const float (&Lm)[D * D], Tape &T, int &res) {

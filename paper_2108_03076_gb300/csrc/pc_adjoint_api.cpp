@@ -106,8 +106,8 @@ pc_status run_adjoint(const pc_model *m, const pc_contract *k, uint64_t n_paths,
     // block and tape regions; at most the interpreter's grid)
     cudaKernel_t jk = nullptr;
     PriceArgs ja = a;
-    if (!L.walk->empty()) drop_bridge_stack(ja.lay);
-    s = jit_kernel(k, jit_spec(k, ja, kJitAdjoint + (d_paths ? 1 : 0), 0, *L.walk), jk);
+    if (!L.w->walk.empty()) drop_bridge_stack(ja.lay);
+    s = jit_pair_kernel(k, L.w, ja, kJitAdjoint + (d_paths ? 1 : 0), 0, L.w->walk, jk);
     if (s != PC_OK) return s;
     const void *kern = reinterpret_cast<const void *>(jk);
     int nb = 0;
@@ -115,8 +115,7 @@ pc_status run_adjoint(const pc_model *m, const pc_contract *k, uint64_t n_paths,
     CU(jit_occupancy(c, kern, block, smem, nb), "jit occupancy");
     if (nb >= 1) {
       const int jgrid = std::min(grid, c->sm_count * nb);
-      StaticGrid sg = static_grid(H, *L.walk);
-      void *args[] = {&ja, &t, &sg};
+      void *args[] = {&ja, &t, &L.w->grid};
       CU(cudaLaunchKernel(kern, dim3(jgrid), dim3(block), args, smem, c->stream), "specialised adjoint kernel");
       return PC_OK;
     }

@@ -87,8 +87,10 @@ namespace {
 // Estimated cost of one tile: generation of every model date for every
 // underlying (normals, bridge, correlation, exponentials) plus one pass
 // over the program; only the order of units and their lengths depend on it.
+// A program that reads no date before lay.skip starts there (a few ops).
 double estimate_tile_cost(const PriceArgs &a, int d) {
-  return double(a.m.n) * (4.0 * d + 2.0) + double(a.n_insn) + 8.0;
+  const int dates = a.lay.skip > 1 ? std::min(a.m.n, a.m.n - a.lay.skip + 8) : a.m.n;
+  return double(dates) * (4.0 * d + 2.0) + double(a.n_insn) + 8.0;
 }
 
 int words_class(int words) {
@@ -285,7 +287,7 @@ pc_status choose_jit(pc_batch *B, const pc_model *const *models, const pc_contra
     J.grid = int(std::max<uint64_t>(1, std::min<uint64_t>(uint64_t(c->sm_count) * nb, (units + wpb - 1) / wpb)));
     J.args = B->items[i];
     J.args.lay = L.args.lay;
-    J.sg = static_grid(models[i]->H, *L.walk);
+    J.sg = L.w->grid;
     B->jit.push_back(J);
     B->is_jit[i] = 1;
   }

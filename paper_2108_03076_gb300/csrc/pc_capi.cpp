@@ -108,13 +108,14 @@ pc_status upload(const std::vector<T> &v, char *base, size_t &off, const T *&dst
 template <typename T>
 size_t padded(const std::vector<T> &v) { return ((v.size() * sizeof(T)) + 255) & ~size_t(255); }
 
-Layout make_layout(const Program &p, const ModelHost &H, int32_t win) {
+Layout make_layout(const Program &p, const ModelHost &H, int32_t win, int32_t skip) {
   Layout L{};
   L.stack = p.frame_slots;
   L.off_bstack = L.stack;
   L.off_cache = L.off_bstack + H.bstack * H.d;  // caches are in registers: no words
   L.off_win = L.off_cache;
   L.win = win;
+  L.skip = skip;
   // slot of ordinal o is o & (win - 1); when the whole grid fits (n < win)
   // that is o itself, so only slots 0..n are ever touched
   L.words = L.off_win + std::min(win, H.n + 1) * H.d;
@@ -153,7 +154,7 @@ int32_t max_label(const Program &p) {
 
 // The contract's window and static walks on the model (kept by the contract;
 // `out` stays valid as long as it does).
-pc_status window_for(const pc_model *m, const pc_contract *k, const pc_contract::Window *&out) {
+pc_status window_for(const pc_model *m, const pc_contract *k, pc_contract::Window *&out) {
   auto *kc = const_cast<pc_contract *>(k);
   std::lock_guard<std::mutex> g(kc->mu);
   auto it = kc->win_cache.find(m->id);
@@ -169,7 +170,7 @@ pc_status window_for(const pc_model *m, const pc_contract *k, const pc_contract:
   std::string err;
   pc_contract::Window w;
   std::vector<uint8_t> reads;
-  pc_status s = analyse_program(k->prog, m->H.t_now, m->H.n, m->H.n_hist, w.win, reads, err);
+  pc_status s = analyse_program(k->prog, m->H.t_now, m->H.n, m->H.n_hist, w.win, w.skip, reads, err);
   if (s != PC_OK) return fail(s, err);
   if (k->ctx->jit && walk_jit_eligible(k->prog)) {
     w.walk = static_walk(m->H, reads);
@@ -180,6 +181,8 @@ pc_status window_for(const pc_model *m, const pc_contract *k, const pc_contract:
     }
   }
   w.with_walks = k->ctx->jit != 0;
+  w.grid = static_grid(m->H, w.walk);
+  w.grid_all = static_grid(m->H, w.walk_all);
   out = &(kc->win_cache[m->id] = std::move(w));
   return PC_OK;
 }
@@ -227,15 +230,14 @@ pc_status prepare(const pc_model *m, const pc_contract *k, uint64_t n_paths, uin
   if (m->ctx != k->ctx) return fail(PC_EINVAL, "model and contract belong to different contexts");
   if (n_paths == 0) return fail(PC_EINVAL, "n_paths must be >= 1");
   if (n_paths > (uint64_t(1) << 40)) return fail(PC_ELIMIT, "n_paths exceeds 2^40");
-  const pc_contract::Window *w = nullptr;
+  pc_contract::Window *w = nullptr;
   pc_status s = window_for(m, k, w);
   if (s != PC_OK) return s;
   const int32_t win = w->win;
-  L.walk = &w->walk;
-  L.walk_all = &w->walk_all;
+  L.w = w;
   pc_ctx *c = m->ctx;
   const int mode = allow_hbm ? c->window_mode : PC_WINDOW_SHARED;
-  Layout lay = make_layout(k->prog, m->H, win);
+  Layout lay = make_layout(k->prog, m->H, win, w->skip);
   int bpsm = 0;
   bool hbm = mode == PC_WINDOW_HBM;
   if (!hbm) {
@@ -357,8 +359,8 @@ pc_status run_greeks(const pc_model *m, const pc_contract *k, uint64_t n_paths, 
     // the contract's run-time specialised tangent kernel (same arguments,
     // shared-memory layout and block)
     cudaKernel_t jk = nullptr;
-    if (!L.walk->empty()) drop_bridge_stack(a.lay);
-    s = jit_kernel(k, jit_spec(k, a, kJitGreeks + (d_paths != nullptr ? 1 : 0), 0, *L.walk), jk);
+    if (!L.w->walk.empty()) drop_bridge_stack(a.lay);
+    s = jit_pair_kernel(k, L.w, a, kJitGreeks + (d_paths != nullptr ? 1 : 0), 0, L.w->walk, jk);
     if (s != PC_OK) return s;
     const void *kern = reinterpret_cast<const void *>(jk);
     int nb = 0;
@@ -366,8 +368,7 @@ pc_status run_greeks(const pc_model *m, const pc_contract *k, uint64_t n_paths, 
     CU(jit_occupancy(c, kern, block, smem, nb), "jit occupancy");
     if (nb < 1) return fail(PC_ELIMIT, "specialised sensitivity kernel cannot be resident");
     const int jgrid = int(std::min<uint64_t>(uint64_t(c->sm_count) * nb, need));
-    StaticGrid sg = static_grid(m->H, *L.walk);
-    void *args[] = {&a, &sg};
+    void *args[] = {&a, &L.w->grid};
     CU(cudaLaunchKernel(kern, dim3(jgrid), dim3(block), args, smem, c->stream), "specialised sensitivity kernel");
     return PC_OK;
   }
@@ -386,7 +387,7 @@ int jit_window_kind(const pc_ctx *c, const Launch &L) {
   // automatic: two pairs where a path walks many dates (the daily barrier's
   // 365: 6.84 -> 6.49 ms at 2^22 paths); a few dates gain nothing (5 dates:
   // 0.069 ms either way), the tile loop and the reduction dominate there
-  const bool two = c->jit_pairs == 2 || (c->jit_pairs == 0 && L.args.m.n >= kJitPairsMinDates && L.walk->empty());
+  const bool two = c->jit_pairs == 2 || (c->jit_pairs == 0 && L.args.m.n >= kJitPairsMinDates && L.w->walk.empty());
   return kJitWinRegs | (two ? kJitPairs2 : 0);
 }
 
@@ -405,7 +406,7 @@ size_t jit_layout(const pc_ctx *c, Launch &L, int bits) {
   lay.off_win -= shift;
   lay.words -= shift;
   if (bits & kJitWinRegs) lay.words = lay.off_win;
-  if (!L.walk->empty()) {
+  if (!L.w->walk.empty()) {
     drop_bridge_stack(lay);
     L.block = kBlock;
     while (L.block > 32 && price_smem_bytes(0, 0, lay.words, L.block) + kStaticSmemReserve > size_t(c->max_smem))
@@ -428,9 +429,13 @@ size_t jit_layout(const pc_ctx *c, Launch &L, int bits) {
   return price_smem_bytes(0, 0, lay.words, L.block);
 }
 
+int jit_price_bound(const pc_ctx *c, const Launch &L, size_t smem) {
+  return L.w->walk.empty() ? jit_min_blocks(c, smem, L.block) : kWalkMinBlocks;
+}
+
 JitSpec jit_price_spec(const pc_ctx *c, const pc_contract *k, const Launch &L, int kind, size_t smem) {
-  const int bound = L.walk->empty() ? jit_min_blocks(c, smem, L.block) : kWalkMinBlocks;
-  return jit_spec(k, L.args, kind, bound, *L.walk);
+  const int bound = jit_price_bound(c, L, smem);
+  return jit_spec(k, L.args, kind, bound, L.w->walk);
 }
 
 // Resident blocks per SM (of kBlock threads, the block the kernel's bound
@@ -465,7 +470,8 @@ pc_status run_price(const pc_model *m, const pc_contract *k, uint64_t n_paths, u
     cudaKernel_t jk = nullptr;
     const int wk = jit_window_kind(c, L);
     const size_t smem = jit_layout(c, L, wk);
-    s = jit_kernel(k, jit_price_spec(c, k, L, (d_payoffs != nullptr ? kJitPriceWrite : kJitPrice) | wk, smem), jk);
+    s = jit_pair_kernel(k, L.w, L.args, (d_payoffs != nullptr ? kJitPriceWrite : kJitPrice) | wk,
+                        jit_price_bound(c, L, smem), L.w->walk, jk);
     if (s != PC_OK) return s;
     const void *kern = reinterpret_cast<const void *>(jk);
     int nb = 0;
@@ -481,8 +487,7 @@ pc_status run_price(const pc_model *m, const pc_contract *k, uint64_t n_paths, u
       s = bind_hbm_window(c, L, m->H.d);
       if (s != PC_OK) return s;
     }
-    StaticGrid sg = static_grid(m->H, *L.walk);
-    void *args[] = {&L.args, &sg};
+    void *args[] = {&L.args, &L.w->grid};
     CU(cudaLaunchKernel(kern, dim3(grid), dim3(L.block), args, smem, c->stream), "specialised price kernel");
     return PC_OK;
   }
@@ -521,13 +526,14 @@ pc_status pc_price_noalloc(const pc_model *m, const pc_contract *k, uint64_t n_p
   // the window: from the contract's cache when an allocating call resolved
   // it for this model already (a lookup, no insertion), else by the same
   // analysis without storing it
-  int32_t win = 0;
+  int32_t win = 0, skip = 0;
   {
     auto *kc = const_cast<pc_contract *>(k);
     std::lock_guard<std::mutex> g(kc->mu);
     const auto it = kc->win_cache.find(m->id);
     if (it != kc->win_cache.end()) {
       win = it->second.win;
+      skip = it->second.skip;
     } else {
       const char *why = "";
       auto on_fail = [&](pc_status st, int64_t, int64_t) {
@@ -538,12 +544,13 @@ pc_status pc_price_noalloc(const pc_model *m, const pc_contract *k, uint64_t n_p
       walk.run(0, k->prog.code.size(), 0);
       if (walk.st != PC_OK) return fail(walk.st, why);
       win = walk.window();
+      skip = walk.skip();
     }
   }
   if (win > PC_MAX_WINDOW)
     return fail(PC_ERANGE, "program looks back further than PC_MAX_WINDOW dates; pc_price_noalloc keeps "
                            "the window of dates in shared memory only");
-  const Layout lay = make_layout(k->prog, H, win);
+  const Layout lay = make_layout(k->prog, H, win, skip);
   size_t smem = 0;
   const int block = pick_block(k->prog, lay.words, c->max_smem, H.d, smem, false);
   if (!block) return fail(PC_ELIMIT, "program + per-path state exceed the device's shared memory per block");
@@ -1159,7 +1166,7 @@ pc_status pc_debug_paths(const pc_model *m, uint64_t n_paths, uint64_t path_offs
   if (!m || !d_S) return fail(PC_EINVAL, "null argument");
   if (n_paths > (uint64_t(1) << 24)) return fail(PC_ELIMIT, "n_paths too large for the probe");
   Program empty;
-  Layout lay = make_layout(empty, m->H, 1);
+  Layout lay = make_layout(empty, m->H, 1, 0);
   lay.stack = 0;
   lay.off_bstack = 0;
   lay.off_cache = m->H.bstack * m->H.d;

@@ -14,7 +14,7 @@ namespace {
 
 
 template <int D, int MODE>
-__global__ void __launch_bounds__(kBlock) cv_kernel(const __grid_constant__ PriceArgs a,
+__global__ void __launch_bounds__(kBlock, 4) cv_kernel(const __grid_constant__ PriceArgs a,
                                                     const __grid_constant__ CvArgs c) {
   using Hook = CvOnline<D, (MODE & kCvGamma) != 0>;
   cv_tiles<D, MODE>(a, c, [&](const uint4 *P, const float *pool, float2 *R, const Rng2 &g, bool live0,

@@ -133,9 +133,9 @@ pc_status cv_launch(const pc_model *m, const pc_contract *k, const pc_cv_desc *c
     jl.off_win -= shift;
     jl.words -= shift;
     if (win_regs) jl.words = jl.off_win;  // the frontier's S in registers: no window words
-    if (!L.walk_all->empty()) drop_bridge_stack(jl);
-    s = jit_kernel(k, jit_spec(k, a, kJitCv + cv_mode(d_xm != nullptr, ca) + (win_regs ? kCvWinRegs : 0),
-                               ctx->cv_min_blocks > 0 ? ctx->cv_min_blocks : kJitCvMinBlocks, *L.walk_all), jk);
+    if (!L.w->walk_all.empty()) drop_bridge_stack(jl);
+    s = jit_pair_kernel(k, L.w, a, kJitCv + cv_mode(d_xm != nullptr, ca) + (win_regs ? kCvWinRegs : 0),
+                        ctx->cv_min_blocks > 0 ? ctx->cv_min_blocks : kJitCvMinBlocks, L.w->walk_all, jk);
     if (s != PC_OK) return s;
     const void *kern = reinterpret_cast<const void *>(jk);
     const size_t jsm = price_smem_bytes(0, 0, jl.words, kBlock);
@@ -145,8 +145,7 @@ pc_status cv_launch(const pc_model *m, const pc_contract *k, const pc_cv_desc *c
     const uint64_t jneed = (a.n_tiles + kBlock / 32 - 1) / (kBlock / 32);
     const int jgrid = int(std::min<uint64_t>(uint64_t(ctx->sm_count) * nb, jneed));
     CvArgs cv = ca;
-    StaticGrid sg = static_grid(m->H, *L.walk_all);
-    void *args[] = {&a, &cv, &sg};
+    void *args[] = {&a, &cv, &L.w->grid_all};
     CU(cudaLaunchKernel(kern, dim3(jgrid), dim3(kBlock), args, jsm, ctx->stream),
        "specialised control-variate kernel");
     return PC_OK;

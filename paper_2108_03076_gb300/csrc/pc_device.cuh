@@ -319,10 +319,8 @@ struct PathState {
   int bsp;                      // bridge stack size, warp-uniform
   int k;                        // ops run so far (the next op's number), warp-uniform
 #endif
-#ifdef PC_WIN_REGS
-  float2 s[H][D];               // S at the frontier date: the whole window of a program
-                                // that reads no date behind the frontier
-#endif
+  float2 s[H][D];               // S at the last date whose values were formed: with PC_WIN_REGS (a
+                                // program that reads no date behind the frontier) the whole window
 };
 
 // A path's state at its start; the bottom level of the bridge stack is
@@ -365,11 +363,11 @@ __device__ __forceinline__ void date_values(int t, PathState<D, H> &ps, const La
 #pragma unroll
       for (int k = 0; k <= i; ++k)
         x = make_float2(fmaf(Bm[i * D + k], ps.w[h][k].x, x.x), fmaf(Bm[i * D + k], ps.w[h][k].y, x.y));
-#ifdef PC_WIN_REGS
       ps.s[h][i] = make_float2(S0[i] * ex2_approx(x.x), S0[i] * ex2_approx(x.y));
+#ifdef PC_WIN_REGS
       (void)ws;
 #else
-      win_store<GW>(R, lay, ws + i, make_float2(S0[i] * ex2_approx(x.x), S0[i] * ex2_approx(x.y)));
+      win_store<GW>(R, lay, ws + i, ps.s[h][i]);
 #endif
     }
   }
@@ -605,19 +603,29 @@ __device__ __forceinline__ void gen_date(int t, PathState<D, H> &ps, const Model
 #endif
 
 #ifndef PC_JIT
-// The frontier moved past dates that no read needs, straight to date t: from
-// the interval that the frontier opens (its right end from the by-date
-// table) bisect while t lies inside, pop the right end, and again until t is
-// popped.  Only the nodes above t in the bisection tree are computed, each
-// from its own normals (its Philox blocks anew, one or two), so the values
-// at t are those of the full walk: a contract that reads the last of 365
-// dates runs one op instead of 365.  Afterwards the state is as the full walk
-// leaves it (next op, the words kept of its block).  Called rarely and by
-// copy, so that the state stays in registers around the call.
-template <int D, bool XW, bool GW>
-__device__ __noinline__ void skip_to(int t, PathState<D, 1> &ps, const ModelDev &m, const Layout &lay,
-                                     const Rng2 &g, float2 *R, const float (&Bm)[D * D], const float (&S0)[D],
-                                     const float *Lm) {
+// A path's start for an interpreted program that reads no date before t
+// (Layout::skip): the frontier straight to t.  From the interval that the
+// frontier opens (its right end from the by-date table) bisect while t lies
+// inside, pop the right end, and again until t is popped.  Only the nodes
+// above t in the bisection tree are computed, each from its own normals (its
+// Philox blocks anew, one or two), so the values at t are those of the full
+// walk: a contract that reads the last of 365 dates runs one op instead of
+// 365.  Afterwards the state is as the full walk leaves it (next op, the words
+// kept of its block).  Out of line, at the one place where little else is
+// live (called from the reading instructions it cost every program 2-5 % in
+// registers and spills).
+template <int D, bool XW>
+__device__ __noinline__ void skip_to(int t, PathState<D, 1> &ps, const PriceArgs &a, uint4 ids, float2 *R) {
+  const ModelDev &m = a.m;
+  const Layout &lay = a.lay;
+  const float(&Bm)[D * D] = *reinterpret_cast<const float(*)[D * D]>(m.Bv);
+  const float(&S0)[D] = *reinterpret_cast<const float(*)[D]>(m.S0v);
+  Rng2 g;
+  rng_init(g, a.rk, a.stream, 0);
+  g.plo[0] = ids.x;
+  g.phi[0] = ids.y;
+  g.plo[1] = ids.z;
+  g.phi[1] = ids.w;
   while (ps.f < t) {
     int r = int(__ldg(reinterpret_cast<const uint32_t *>(m.nodes + ps.f) + 7) >> 16);
     while (t < r) {
@@ -644,7 +652,7 @@ __device__ __noinline__ void skip_to(int t, PathState<D, 1> &ps, const ModelDev 
   float2 drift[D];
 #pragma unroll
   for (int i = 0; i < D; ++i) drift[i] = __ldg(m.A + t * D + i);
-  date_values<D, XW, GW, 1>(t, ps, lay, R, Bm, S0, Lm, drift);
+  date_values<D, XW, false, 1>(t, ps, lay, R, Bm, S0, m.L, drift);
   ps.k = __ldg(m.date_ops + t + 1);
   if (t < m.n && ((D * ps.k) & 3)) {
     float2 e[1][4];
@@ -653,23 +661,6 @@ __device__ __noinline__ void skip_to(int t, PathState<D, 1> &ps, const ModelDev 
     for (int i = 0; i < 3; ++i) ps.zc[0][i] = e[0][1 + i];
   }
 }
-#endif
-
-// The frontier to date o_ (> frontier).  An interpreted program that reads no
-// date behind the frontier (a window of one date) skips the dates between.
-#if defined(PC_JIT)
-#define TO_DATE(o_, XW_, GW_, LM_)                                                     \
-  while (ps.f < (o_)) NEXT_DATE(XW_, GW_, LM_)
-#else
-#define TO_DATE(o_, XW_, GW_, LM_)                                                     \
-  do {                                                                                 \
-    if (lay.win == 1 && (o_) > ps.f + 1) {                                             \
-      PathState<D> skip_ = ps;                                                         \
-      skip_to<D, XW_, GW_>((o_), skip_, m, lay, g, R, Bm, S0, LM_);                    \
-      ps = skip_;                                                                      \
-    }                                                                                  \
-    while (ps.f < (o_)) NEXT_DATE(XW_, GW_, LM_);                                       \
-  } while (0)
 #endif
 
 // The evaluators' per-date hook: called after each generated date t with
@@ -760,10 +751,97 @@ __device__ __forceinline__ float2 fused_value_rd(const uint4 &I, int o, const fl
   return v;
 }
 
+#ifndef PC_JIT
+// The interpreter's short form of a plain fused op (kPlainBit): leaf i is
+// underlying i, unscaled.  An or of tests v < k (or v <= k) is the test of the
+// smallest value, of k < v of the largest (a NaN takes part in neither), so
+// every plain op is one min, max or sum and at most one comparison.  The
+// general form decodes each leaf's label, scale and comparison: about 185
+// instructions for a worst-of test of three against 45.
+template <int D, typename RD>
+__device__ __forceinline__ float2 fused_plain(const uint4 &I, int o, const ModelDev &m, RD rd) {
+  const uint32_t A = I.x >> 8;
+  const int n = int((A >> 8) & 3u) + 1, code = int((A >> 4) & 7u);
+  const int rop = (I.x & 0xffu) == X_LANY ? (code <= 2 ? 0 : 1) : int(A & 3u);
+  float2 s[D];
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    if (i >= n) break;
+    if (o > 0) {
+      s[i] = rd(i);
+    } else {
+      const float sv = __ldg(m.sval + (o + m.n_hist) * D + i);
+      s[i] = make_float2(sv, sv);
+    }
+  }
+  float2 v = s[0];
+  if (rop == 0) {
+#pragma unroll
+    for (int i = 1; i < D; ++i)
+      if (i < n) v = make_float2(fminf(v.x, s[i].x), fminf(v.y, s[i].y));
+  } else if (rop == 1) {
+#pragma unroll
+    for (int i = 1; i < D; ++i)
+      if (i < n) v = make_float2(fmaxf(v.x, s[i].x), fmaxf(v.y, s[i].y));
+  } else {
+#pragma unroll
+    for (int i = 1; i < D; ++i)
+      if (i < n) v = make_float2(__fadd_rn(v.x, s[i].x), __fadd_rn(v.y, s[i].y));
+  }
+  if (code) {
+    const float k = __uint_as_float(I.w);
+    const bool less = code <= 2, strict = (code & 1) != 0;
+    const float ax = less ? v.x : k, bx = less ? k : v.x, ay = less ? v.y : k, by = less ? k : v.y;
+    v = make_float2(fl(int(strict ? ax < bx : ax <= bx)), fl(int(strict ? ay < by : ay <= by)));
+  }
+  return v;
+}
+
+// A whole-loop barrier's test on the S just produced, decoded once before the
+// loop: path value v of any watched underlying with sgn v < lim.  v <= k is
+// v < the next float above k; an unwatched underlying's limit is -inf.  Only
+// for plain ops with a finite k that reduce to an or (a min against an upper
+// bound, a max against a lower one).
+template <int D>
+struct LoopTest {
+  float lim[D], sgn;
+  bool use;
+  __device__ __forceinline__ explicit LoopTest(const uint4 &I) {
+    const uint32_t A = I.x >> 8;
+    const int n = int((A >> 8) & 3u) + 1, code = int((A >> 4) & 7u), rop = int(A & 3u);
+    const float k = __uint_as_float(I.w);
+    const bool less = code <= 2;
+    use = (A >> kPlainBit) & 1u;
+    use = use && ((I.x & 0xffu) == X_LANY || n == 1 || (rop == 0 && less) || (rop == 1 && !less));
+    use = use && (I.w & 0x7f800000u) != 0x7f800000u;
+    sgn = less ? 1.f : -1.f;
+    float l = sgn * k;
+    if (!(code & 1)) {  // the next float above
+      const int b = __float_as_int(l);
+      l = l == 0.f ? __int_as_float(1) : __int_as_float(b > 0 ? b + 1 : b - 1);
+    }
+#pragma unroll
+    for (int i = 0; i < D; ++i) lim[i] = i < n ? l : __int_as_float(int(0xff800000u));
+  }
+  __device__ __forceinline__ void test(const float2 (&s)[D], bool &c0, bool &c1) const {
+    c0 = c1 = false;
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      c0 = c0 || sgn * s[i].x < lim[i];
+      c1 = c1 || sgn * s[i].y < lim[i];
+    }
+  }
+};
+#endif
+
 template <int D, bool GW = false>
 __device__ __forceinline__ float2 fused_value(const uint4 &I, int o, const float *pool, const float2 *R,
                                               const ModelDev &m, const Layout &lay) {
   const int base = (o & (lay.win - 1)) * D;
+#ifndef PC_JIT
+  if ((I.x >> (8 + kPlainBit)) & 1u)
+    return fused_plain<D>(I, o, m, [&](int l) { return win_load<GW>(R, lay, base + l); });
+#endif
   return fused_value_rd<D>(I, o, pool, m, [&](int l) { return win_load<GW>(R, lay, base + l); });
 }
 // The same with the frontier date's S in registers (cur; a window of one date).

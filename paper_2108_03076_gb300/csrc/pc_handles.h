@@ -130,11 +130,21 @@ struct pc_contract {
   std::vector<uint32_t> image;    // program then padded pool: the uploaded words
   std::mutex mu;
   struct Window {
-    int32_t win = 1;
+    int32_t win = 1, skip = 0;
     bool with_walks = false;  // computed with the context's specialised kernels on
     // static walks over the dates the program reads, and over every date
-    // up to its last (a per-date hook); empty where they are too long
+    // of the model (a per-date hook); empty where they are too long; and
+    // their launch arguments
     std::vector<int32_t> walk, walk_all;
+    pc::StaticGrid grid{}, grid_all{};
+    // the specialised kernels found for this pair so far (jit_kernel's
+    // answers: looking one up by its program costs a microsecond or two)
+    struct Kernel {
+      int kind, min_blocks, words;
+      bool one_phi;
+      cudaKernel_t kernel;
+    };
+    std::vector<Kernel> kernels;
   };
   std::map<uint64_t, Window> win_cache;  // by model id
 };
@@ -180,7 +190,7 @@ struct Launch {
   int grid = 0;
   int block = kBlock;
   size_t smem = 0;
-  const std::vector<int32_t> *walk = nullptr, *walk_all = nullptr;  // the contract's static walks on the model
+  pc_contract::Window *w = nullptr;  // the contract on the model: its static walks and kernels
   bool hbm_window = false;  // window in HBM (args.lay.gwin set by the launcher)
 };
 
@@ -238,6 +248,9 @@ int jit_min_blocks(const pc_ctx *c, size_t smem, int block);
 // launch's arguments (layout final) and a walk (may be empty).
 JitSpec jit_spec(const pc_contract *k, const PriceArgs &a, int kind, int min_blocks, const std::vector<int32_t> &walk);
 JitSpec jit_price_spec(const pc_ctx *c, const pc_contract *k, const Launch &L, int kind, size_t smem);
+// jit_kernel of jit_spec, or the pair's earlier answer for the same launch.
+pc_status jit_pair_kernel(const pc_contract *k, pc_contract::Window *w, const PriceArgs &a, int kind, int min_blocks,
+                          const std::vector<int32_t> &walk, cudaKernel_t &out);
 void drop_bridge_stack(Layout &lay);
 void jit_release(pc_ctx *c);
 

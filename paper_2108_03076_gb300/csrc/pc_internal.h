@@ -118,6 +118,7 @@ struct TimeWalk {
   int64_t t_now, n_dates, n_hist;
   OnFail on_fail;
   int64_t frontier = 0, lookback = 0, steps = 0, entries = 0;
+  int64_t first = 0;         // the earliest simulated date read (0: none)
   uint8_t *reads = nullptr;  // optional [n_dates + 1]: set to 1 for every simulated date read
   pc_status st = PC_OK;
 
@@ -157,6 +158,7 @@ struct TimeWalk {
         }
         if (op != X_PAYOFF && o > 0) {
           if (reads) reads[o] = 1;
+          if (first == 0 || o < first) first = o;
           if (o > frontier) frontier = o;
           else if (frontier - o > lookback) lookback = frontier - o;
         }
@@ -198,6 +200,8 @@ struct TimeWalk {
     }
   }
 
+  // Layout::skip
+  int32_t skip() const { return lookback == 0 ? int32_t(first) : 0; }
   // the window (power of two) that holds the largest lookback
   int32_t window() const {
     int32_t w = 1;
@@ -210,9 +214,9 @@ struct TimeWalk {
 // every model and payoff time within [-n_hist, n] as ordinals; `win`
 // receives the window size needed (power of two, <= 2 * PC_MAX_DATES:
 // callers decide where such a window can live), `reads` [n + 1] marks the
-// dates read.
+// dates read, `skip` = TimeWalk::skip.
 pc_status analyse_program(const Program &p, int32_t t_now, int32_t n_dates, int32_t n_hist,
-                          int32_t &win, std::vector<uint8_t> &reads, std::string &err);
+                          int32_t &win, int32_t &skip, std::vector<uint8_t> &reads, std::string &err);
 
 // cutPayoff (Sec. 4.1) on bytecode: every payoff(t, p1', p2') becomes
 // if(t < now, 0, payoff(t, p1', p2')); the literal 0.0 is appended to the

@@ -602,6 +602,19 @@ JitSpec jit_spec(const pc_contract *k, const PriceArgs &a, int kind, int min_blo
   return sp;
 }
 
+pc_status jit_pair_kernel(const pc_contract *k, pc_contract::Window *w, const PriceArgs &a, int kind, int min_blocks,
+                          const std::vector<int32_t> &walk, cudaKernel_t &out) {
+  const bool phi = one_phi(a.path_offset, a.n_tiles);
+  for (const pc_contract::Window::Kernel &e : w->kernels)
+    if (e.kind == kind && e.min_blocks == min_blocks && e.words == a.lay.words && e.one_phi == phi) {
+      out = e.kernel;
+      return PC_OK;
+    }
+  const pc_status s = jit_kernel(k, jit_spec(k, a, kind, min_blocks, walk), out);
+  if (s == PC_OK) w->kernels.push_back({kind, min_blocks, a.lay.words, phi, out});
+  return s;
+}
+
 bool walk_jit_eligible(const Program &p) {
   std::vector<int> sp_at;
   return date_sites(p) <= 2 || (date_sites(p) <= kSharedDateSites && stack_depths(p, sp_at));

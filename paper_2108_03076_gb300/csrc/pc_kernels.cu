@@ -32,7 +32,7 @@ namespace {
 // HBM (lay.gwin) instead of shared memory, for programs that look back
 // further than shared memory holds.
 template <int D, bool WRITE, bool GW = false>
-__global__ void __launch_bounds__(kBlock) price_kernel(const __grid_constant__ PriceArgs a) {
+__global__ void __launch_bounds__(kBlock, D == 1 ? 7 : D == 2 ? 6 : 5) price_kernel(const __grid_constant__ PriceArgs a) {
   price_tiles<D, WRITE>(a, [&](const uint4 *P, const float *pool, float2 *R, const Rng2 &g, bool live0,
                                bool live1, const float(&Bm)[D * D], const float(&S0)[D]) {
     return eval_path<D, GW>(P, pool, R, a, g, live0, live1, Bm, S0);

@@ -190,6 +190,12 @@ struct Emitter {
     for (size_t i = 0; i < ts.size(); ++i) f |= uint32_t(ts[i].label) << (10 + 2 * i);
     return f;
   }
+  // kPlainBit of a fused op's A
+  static uint32_t plain_field(const std::vector<STerm> &ts, int kind) {
+    for (size_t i = 0; i < ts.size(); ++i)
+      if (kind || ts[i].label != int(i)) return 0;
+    return 1u << kPlainBit;
+  }
   // chain of min/max/add over S-terms (1..4 leaves; 1 leaf only with a compare)
   bool red_terms(int idx, uint32_t &rop, std::vector<STerm> &ts) const {
     const TNode &x = T[idx];
@@ -232,7 +238,7 @@ struct Emitter {
       const int kind = terms_kind(ts);
       if (kind < 0) return false;
       const uint32_t off = pool_terms(ts, kind);
-      emit(X_LRED, rop | (uint32_t(kind) << 2) | (uint32_t(ts.size() - 1) << 8) | labels_field(ts),
+      emit(X_LRED, rop | (uint32_t(kind) << 2) | (uint32_t(ts.size() - 1) << 8) | labels_field(ts) | plain_field(ts, kind),
            uint32_t(int32_t(ts[0].time)), off, 0);
       push();
       return true;
@@ -245,7 +251,7 @@ struct Emitter {
       if (kind < 0) return false;
       const uint32_t off = pool_terms(ts, kind);
       emit(X_LRED, rop | (uint32_t(kind) << 2) | (uint32_t(code) << 4) |
-                       (uint32_t(ts.size() - 1) << 8) | labels_field(ts),
+                       (uint32_t(ts.size() - 1) << 8) | labels_field(ts) | plain_field(ts, kind),
            uint32_t(int32_t(ts[0].time)), off, fbits_(k));
       push();
       return true;
@@ -270,7 +276,8 @@ struct Emitter {
       if (kind < 0) return false;
       const uint32_t off = pool_terms(ts, kind);
       emit(X_LANY, (x.op == PC_OP_AND ? 1u : 0u) | (uint32_t(kind) << 2) | (uint32_t(code0) << 4) |
-                       (uint32_t(ts.size() - 1) << 8) | labels_field(ts),
+                       (uint32_t(ts.size() - 1) << 8) | labels_field(ts) |
+                       (x.op == PC_OP_OR ? plain_field(ts, kind) : 0u),
            uint32_t(int32_t(ts[0].time)), off, fbits_(k0));
       push();
       return true;
@@ -575,7 +582,7 @@ pc_status compile_program(const uint32_t *words, size_t n_words, const double *c
 }
 
 pc_status analyse_program(const Program &p, int32_t t_now, int32_t n_dates, int32_t n_hist,
-                          int32_t &win, std::vector<uint8_t> &reads, std::string &err) {
+                          int32_t &win, int32_t &skip, std::vector<uint8_t> &reads, std::string &err) {
   auto on_fail = [&](pc_status st, int64_t t, int64_t o) {
     if (st == PC_ELIMIT)
       err = "program too long to analyse (loop trip counts)";
@@ -589,6 +596,7 @@ pc_status analyse_program(const Program &p, int32_t t_now, int32_t n_dates, int3
   walk.run(0, p.code.size(), 0);
   if (walk.st != PC_OK) return walk.st;
   win = walk.window();
+  skip = walk.skip();
   return PC_OK;
 }
 

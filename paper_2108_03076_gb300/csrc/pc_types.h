@@ -42,6 +42,8 @@ struct XInsn {
 };
 static_assert(sizeof(XInsn) == 16, "XInsn is one 16-byte shared-memory load");
 
+constexpr uint32_t kPlainBit = 18;  // of A, X_LRED and X_LANY
+
 enum XOp : uint32_t {
   X_END = 0,
   X_CONST,      // push bits b
@@ -72,11 +74,13 @@ enum XOp : uint32_t {
   //   add; leaf_i = S_{l_i} [* or / pool[c + i]]; optionally compared with
   //   the immediate e.  A: bits 0-1 op (0 min, 1 max, 2 add), 2-3 scale
   //   (0 none, 1 mult, 2 div), 4-6 compare (0 none, 1 v<k, 2 v<=k, 3 k<v,
-  //   4 k<=v), 8-9 leaves-1, 10-17 labels (2 bits each).
+  //   4 k<=v), 8-9 leaves-1, 10-17 labels (2 bits each), 18 plain (labels
+  //   0, 1, ... in order, no scales: the interpreter's short forms).
   X_LRED,
   // X_LANY: p = cmp(leaf_0, k) or/and cmp(leaf_1, k) ...  A: bit 0 combine
   //   (0 or, 1 and), 2-3 scale, 4-6 compare (1..4 as X_LRED), 8-9 leaves-1,
-  //   10-17 labels; c = pool offset of the scales; e = immediate k.
+  //   10-17 labels, 18 plain and combined by or; c = pool offset of the
+  //   scales; e = immediate k.
   X_LANY,
   // X_LSTEPK: one loopif iteration whose then-branch is the literal
   //   pool[A >> 8]: pop the condition, latch the literal on newly true lanes,
@@ -161,6 +165,7 @@ struct Layout {
   int32_t off_xwin;   // window of X = L W (win * d), sensitivity kernel only
   int32_t words;      // total words per thread in shared memory
   int32_t win;        // window size (power of two)
+  int32_t skip;       // with a window of one date: the first date the program reads (else 0)
   // HBM window (programs whose lookback does not fit shared memory): the
   // window of thread t of the launch is column t of gwin, slot s at
   // gwin[s * gstride + t] (gstride = grid * block); null for the shared window.
