@@ -27,7 +27,7 @@ size_t tape_region_bytes(int64_t emax) {
 constexpr size_t kTapeCapBytes = size_t(8) << 30;
 
 pc_status run_adjoint(const pc_model *m, const pc_contract *k, uint64_t n_paths, uint64_t offset,
-                      uint64_t seed, uint32_t stream, double *d_out, float *d_paths) {
+                      uint64_t seed, uint32_t stream, double *d_out, float *d_paths, bool report = false) {
   Launch L;
   pc_status s = prepare(m, k, n_paths, offset, seed, stream, L, false);
   if (s != PC_OK) return s;
@@ -100,6 +100,7 @@ pc_status run_adjoint(const pc_model *m, const pc_contract *k, uint64_t n_paths,
   a.control = c->d_control;
   a.out = d_out;
   a.out_paths = d_paths;
+  if (report) report_to_host(c, a);
   CU(cudaSetDevice(c->device), "cudaSetDevice");
   if (c->jit && adjoint_jit_eligible(k)) {
     // the program's run-time specialised adjoint kernel (same arguments,
@@ -115,11 +116,13 @@ pc_status run_adjoint(const pc_model *m, const pc_contract *k, uint64_t n_paths,
     CU(jit_occupancy(c, kern, block, smem, nb), "jit occupancy");
     if (nb >= 1) {
       const int jgrid = std::min(grid, c->sm_count * nb);
+      ja.one_pass = uint64_t(jgrid) * wpb >= a.n_tiles;
       void *args[] = {&ja, &t, &L.w->grid};
       CU(cudaLaunchKernel(kern, dim3(jgrid), dim3(block), args, smem, c->stream), "specialised adjoint kernel");
       return PC_OK;
     }
   }
+  a.one_pass = uint64_t(grid) * wpb >= a.n_tiles;
   CU(launch_adjoint(a, t, grid, block, smem, c->stream), "adjoint kernel");
   return PC_OK;
 }
@@ -140,19 +143,10 @@ pc_status pc_greeks_adjoint(const pc_model *m, const pc_contract *k, uint64_t n_
   if (n_paths < 2) return fail(PC_EINVAL, "n_paths must be >= 2 for a standard error");
   pc_ctx *c = m->ctx;
   const int d = m->H.d;
-  pc_status s = run_adjoint(m, k, n_paths, 0, seed, 0, c->d_gout, nullptr);
+  pc_status s = run_adjoint(m, k, n_paths, 0, seed, 0, c->h_res, nullptr, true);
+  if (s == PC_OK) s = wait_report(c);
   if (s != PC_OK) return s;
-  const int width = 2 * (1 + 2 * d);
-  double h[PC_MAX_UNDERLYINGS * 8], st[5];
-  CU(cudaMemcpyAsync(h, c->d_gout, size_t(width + 1) * sizeof(double), cudaMemcpyDeviceToHost, c->stream),
-     "result copy");
-  CU(cudaMemcpyAsync(st, c->d_res, 5 * sizeof(double), cudaMemcpyDeviceToHost, c->stream), "status copy");
-  s = wait_stream(c);
-  if (s != PC_OK) return s;
-  int32_t status;
-  std::memcpy(&status, &st[4], 4);
-  s = check_status(c, status);
-  if (s != PC_OK) return s;
+  const double *h = c->h_res;
   const double n = double(n_paths);
   auto mean_se = [&](int j, double &mean, double &se) {
     mean = h[2 * j] / n;

@@ -287,6 +287,7 @@ pc_status choose_jit(pc_batch *B, const pc_model *const *models, const pc_contra
     J.grid = int(std::max<uint64_t>(1, std::min<uint64_t>(uint64_t(c->sm_count) * nb, (units + wpb - 1) / wpb)));
     J.args = B->items[i];
     J.args.lay = L.args.lay;
+    J.args.one_pass = uint64_t(J.grid) * wpb >= units;
     J.sg = L.w->grid;
     B->jit.push_back(J);
     B->is_jit[i] = 1;

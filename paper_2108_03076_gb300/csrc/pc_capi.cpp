@@ -51,6 +51,32 @@ pc_status wait_stream(pc_ctx *c) {
   }
 }
 
+void report_to_host(pc_ctx *c, PriceArgs &a) {
+  a.done = c->h_done;
+  a.ticket = ++c->ticket;
+}
+
+pc_status wait_report(pc_ctx *c) {
+  const auto t_start = std::chrono::steady_clock::now();
+  const volatile uint64_t *done = c->h_done;
+  uint64_t v = 0;
+  for (uint32_t spins = 1;; ++spins) {
+    v = *done;
+    if (uint32_t(v >> 32) == c->ticket) break;
+    if (spins % 256) continue;
+    const cudaError_t e = cudaStreamQuery(c->stream);
+    if (e != cudaSuccess && e != cudaErrorNotReady) return cuda_fail(e, "stream");
+    v = *done;  // a drained stream has written it
+    if (uint32_t(v >> 32) == c->ticket) break;
+    if (e == cudaSuccess) return fail(PC_ECUDA, "the launch finished without its report");
+    const double el = std::chrono::duration<double>(std::chrono::steady_clock::now() - t_start).count();
+    if (el > c->timeout_s) return fail(PC_ETIMEOUT, "device did not finish within the context's limit");
+    if (el > 2e-3) std::this_thread::sleep_for(std::chrono::microseconds(50));
+  }
+  std::atomic_thread_fence(std::memory_order_acquire);
+  return check_status(c, int32_t(uint32_t(v)));
+}
+
 cudaError_t ctx_malloc(pc_ctx *c, void **p, size_t bytes) {
   if (c->fail_allocs > 0) {
     --c->fail_allocs;
@@ -320,7 +346,7 @@ void drop_bridge_stack(Layout &lay) {
 // Sensitivity launch for underlying `label`: the pricing launch set-up with
 // three physical slots per program value and an extra window of X = L W.
 pc_status run_greeks(const pc_model *m, const pc_contract *k, uint64_t n_paths, uint64_t offset,
-                     uint64_t seed, int label, double *d_out, float *d_paths) {
+                     uint64_t seed, int label, double *d_out, float *d_paths, bool report = false) {
   Launch L;
   pc_status s = prepare(m, k, n_paths, offset, seed, 0, L);
   if (s != PC_OK) return s;
@@ -353,6 +379,7 @@ pc_status run_greeks(const pc_model *m, const pc_contract *k, uint64_t n_paths, 
   a.out = d_out;
   a.out_paths = d_paths;
   a.greek_label = label;
+  if (report) report_to_host(c, a);
   const uint64_t need = (a.n_tiles + block / 32 - 1) / (block / 32);
   CU(cudaSetDevice(c->device), "cudaSetDevice");
   if (c->jit && jit_eligible(k)) {
@@ -368,11 +395,13 @@ pc_status run_greeks(const pc_model *m, const pc_contract *k, uint64_t n_paths, 
     CU(jit_occupancy(c, kern, block, smem, nb), "jit occupancy");
     if (nb < 1) return fail(PC_ELIMIT, "specialised sensitivity kernel cannot be resident");
     const int jgrid = int(std::min<uint64_t>(uint64_t(c->sm_count) * nb, need));
+    a.one_pass = uint64_t(jgrid) * (block / 32) >= a.n_tiles;
     void *args[] = {&a, &L.w->grid};
     CU(cudaLaunchKernel(kern, dim3(jgrid), dim3(block), args, smem, c->stream), "specialised sensitivity kernel");
     return PC_OK;
   }
   const int grid = int(std::min<uint64_t>(uint64_t(c->sm_count) * best_warps / (block / 32), need));
+  a.one_pass = uint64_t(grid) * (block / 32) >= a.n_tiles;
   CU(launch_greeks(a, grid, block, smem, c->stream), "sensitivity kernel");
   return PC_OK;
 }
@@ -430,7 +459,7 @@ size_t jit_layout(const pc_ctx *c, Launch &L, int bits) {
 }
 
 int jit_price_bound(const pc_ctx *c, const Launch &L, size_t smem) {
-  return L.w->walk.empty() ? jit_min_blocks(c, smem, L.block) : kWalkMinBlocks;
+  return L.w->walk.empty() ? jit_min_blocks(c, smem, L.block, L.args.m.d) : kWalkMinBlocks;
 }
 
 JitSpec jit_price_spec(const pc_ctx *c, const pc_contract *k, const Launch &L, int kind, size_t smem) {
@@ -443,15 +472,16 @@ JitSpec jit_price_spec(const pc_ctx *c, const pc_contract *k, const Launch &L, i
 // for: the default, or fewer when the launch's shared memory allows no more
 // warps (the kernel may then use the registers those blocks leave).  The
 // kernel's own static shared memory is a few words (kJitStaticSmem bounds it).
-int jit_min_blocks(const pc_ctx *c, size_t smem, int block) {
-  if (c->sm_smem <= 0) return kJitMinBlocks;
+int jit_min_blocks(const pc_ctx *c, size_t smem, int block, int d) {
+  const int most = d == 1 ? kJitMinBlocks1 : kJitMinBlocks;
+  if (c->sm_smem <= 0) return most;
   const size_t per = smem + kJitStaticSmem + size_t(c->smem_reserve);
   const int warps = int(size_t(c->sm_smem) / per) * (block / 32);
-  return std::max(1, std::min(kJitMinBlocks, warps / (kBlock / 32)));
+  return std::max(1, std::min(most, warps / (kBlock / 32)));
 }
 
 pc_status run_price(const pc_model *m, const pc_contract *k, uint64_t n_paths, uint64_t offset,
-                    uint64_t seed, uint32_t stream, double *d_out, float *d_payoffs) {
+                    uint64_t seed, uint32_t stream, double *d_out, float *d_payoffs, bool report = false) {
   Launch L;
   pc_status s = prepare(m, k, n_paths, offset, seed, stream, L, true);
   if (s != PC_OK) return s;
@@ -464,6 +494,7 @@ pc_status run_price(const pc_model *m, const pc_contract *k, uint64_t n_paths, u
   L.args.control = c->d_control;
   L.args.out = d_out;
   L.args.out_paths = d_payoffs;
+  if (report) report_to_host(c, L.args);
   CU(cudaSetDevice(c->device), "cudaSetDevice");
   if (c->jit && jit_eligible(k)) {
     // the contract's run-time specialised kernel (same arguments and shape)
@@ -481,6 +512,7 @@ pc_status run_price(const pc_model *m, const pc_contract *k, uint64_t n_paths, u
     // a warp takes a tile, or a pair of tiles with two path pairs a lane
     const uint64_t units = (wk & kJitPairs2) ? (L.args.n_tiles + 1) / 2 : L.args.n_tiles;
     const int grid = int(std::min<uint64_t>(uint64_t(c->sm_count) * nb, (units + wpb - 1) / wpb));
+    L.args.one_pass = uint64_t(grid) * wpb >= units;
     if (L.hbm_window) {
       // the HBM window holds a column per thread of this launch's grid
       L.grid = grid;
@@ -495,6 +527,7 @@ pc_status run_price(const pc_model *m, const pc_contract *k, uint64_t n_paths, u
     s = bind_hbm_window(c, L, m->H.d);
     if (s != PC_OK) return s;
   }
+  L.args.one_pass = uint64_t(L.grid) * (L.block / 32) >= L.args.n_tiles;
   CU(launch_price(L.args, L.grid, L.block, L.smem, c->stream), "price kernel");
   return PC_OK;
 }
@@ -584,6 +617,7 @@ pc_status pc_price_noalloc(const pc_model *m, const pc_contract *k, uint64_t n_p
   a.status = reinterpret_cast<int32_t *>(c->d_res + 4);
   const uint64_t need = (n_tiles + block / 32 - 1) / (block / 32);
   const int grid = int(std::min<uint64_t>(uint64_t(c->sm_count) * bpsm, need));
+  a.one_pass = uint64_t(grid) * (block / 32) >= n_tiles;
   CU(cudaMemsetAsync(a.control, 0, kNoAllocCounterBytes, c->stream), "counter reset");
   CU(launch_price(a, grid, block, smem, c->stream), "price kernel");
   return PC_OK;
@@ -655,7 +689,11 @@ pc_status pc_create(pc_ctx **out, int device, void *cuda_stream) {
       cudaGetLastError();
     }
   }
-  if (e == cudaSuccess) e = cudaHostAlloc(reinterpret_cast<void **>(&c->h_res), 16 * sizeof(double), 0);
+  if (e == cudaSuccess) e = cudaHostAlloc(reinterpret_cast<void **>(&c->h_res), 64 * sizeof(double), 0);
+  if (e == cudaSuccess) {
+    c->h_done = reinterpret_cast<uint64_t *>(c->h_res + 48);
+    *c->h_done = 0;
+  }
   if (e == cudaSuccess) {
     c->stage_words = 16384;
     e = cudaHostAlloc(reinterpret_cast<void **>(&c->h_stage), 2 * c->stage_words * 4, 0);
@@ -1031,18 +1069,10 @@ pc_status pc_price(const pc_model *m, const pc_contract *k, uint64_t n_paths, ui
   if (n_paths < 2) return fail(PC_EINVAL, "n_paths must be >= 2 for a standard error");
   if (!m) return fail(PC_EINVAL, "null model");
   pc_ctx *c = m->ctx;
-  pc_status s = run_price(m, k, n_paths, 0, seed, 0, c->d_res, nullptr);
+  pc_status s = run_price(m, k, n_paths, 0, seed, 0, c->h_res, nullptr, true);
+  if (s == PC_OK) s = wait_report(c);
   if (s != PC_OK) return s;
-  // pinned read-back: the copy is queued and the bounded wait covers it
-  CU(cudaMemcpyAsync(c->h_res, c->d_res, 5 * sizeof(double), cudaMemcpyDeviceToHost, c->stream), "result copy");
-  s = wait_stream(c);
-  if (s != PC_OK) return s;
-  double h[5];
-  std::memcpy(h, c->h_res, sizeof(h));
-  int32_t status;
-  std::memcpy(&status, &h[4], 4);
-  s = check_status(c, status);
-  if (s != PC_OK) return s;
+  const double *h = c->h_res;
   const double n = double(n_paths), mean = h[0] / n;
   const double var = std::max(0.0, (h[1] - n * mean * mean) / (n - 1.0));
   *out_price = mean;
@@ -1119,19 +1149,12 @@ pc_status pc_greeks(const pc_model *m, const pc_contract *k, uint64_t n_paths, u
   pc_ctx *c = m->ctx;
   const int d = m->H.d;
   for (int l = 0; l < d; ++l) {
-    pc_status s = run_greeks(m, k, n_paths, 0, seed, l, c->d_gout + 8 * l, nullptr);
+    pc_status s = run_greeks(m, k, n_paths, 0, seed, l, c->h_res + 8 * l, nullptr, l == d - 1);
     if (s != PC_OK) return s;
   }
-  double h[PC_MAX_UNDERLYINGS * 8], st[5];
-  CU(cudaMemcpyAsync(h, c->d_gout, size_t(d) * 8 * sizeof(double), cudaMemcpyDeviceToHost, c->stream),
-     "result copy");
-  CU(cudaMemcpyAsync(st, c->d_res, 5 * sizeof(double), cudaMemcpyDeviceToHost, c->stream), "status copy");
-  pc_status s = wait_stream(c);
+  pc_status s = wait_report(c);
   if (s != PC_OK) return s;
-  int32_t status;
-  std::memcpy(&status, &st[4], 4);
-  s = check_status(c, status);
-  if (s != PC_OK) return s;
+  const double *h = c->h_res;
   const double n = double(n_paths);
   auto mean_se = [&](double sum, double sumsq, double &mean, double &se) {
     mean = sum / n;

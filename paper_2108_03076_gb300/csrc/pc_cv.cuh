@@ -199,7 +199,6 @@ __device__ __forceinline__ void cv_tiles(const PriceArgs &a, const CvArgs &c, EV
   constexpr bool WRITE = (MODE & kCvWrite) != 0, GAMMA = (MODE & kCvGamma) != 0,
                  PILOT = (MODE & kCvPilot) != 0;
   extern __shared__ __align__(16) uint32_t smem[];
-  __shared__ int last_block;
   const Staged st = stage_program(a, smem);
   const uint4 *P = st.P;
   const float *pool = st.pool;
@@ -207,13 +206,10 @@ __device__ __forceinline__ void cv_tiles(const PriceArgs &a, const CvArgs &c, EV
   const float(&Bm)[D * D] = *reinterpret_cast<const float(*)[D * D]>(a.m.Bv);
   const float(&S0)[D] = *reinterpret_cast<const float(*)[D]>(a.m.S0v);
   const int lane = threadIdx.x & 31;
-  unsigned long long *ctr = reinterpret_cast<unsigned long long *>(a.control);
   Rng2 g;
   rng_init(g, a.rk, a.stream, a.path_offset);
   for (;;) {
-    unsigned long long tile = 0;
-    if (lane == 0) tile = atomicAdd(ctr, 1ull);
-    tile = __shfl_sync(kFull, tile, 0);
+    const unsigned long long tile = next_unit(a, lane);
     if (tile >= a.n_tiles) break;
     const uint64_t i0 = tile * kTilePaths + lane, i1 = i0 + 32;
     const bool live0 = i0 < a.n_paths, live1 = i1 < a.n_paths;
@@ -241,44 +237,36 @@ __device__ __forceinline__ void cv_tiles(const PriceArgs &a, const CvArgs &c, EV
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         if (!live[q]) continue;
-        mo.add(0, xs[q]);
-        mo.add(1, Mv[q]);
-        mo.add(2, M2v[q]);
-        mo.add_prod(3, xs[q], Mv[q]);
-        mo.add_prod(4, xs[q], M2v[q]);
-        mo.add_prod(5, Mv[q], Mv[q]);
-        mo.add_prod(6, M2v[q], M2v[q]);
-        mo.add_prod(7, Mv[q], M2v[q]);
+        mo.add(0, xs[q], q == 0);
+        mo.add(1, Mv[q], q == 0);
+        mo.add(2, M2v[q], q == 0);
+        mo.add_prod(3, xs[q], Mv[q], q == 0);
+        mo.add_prod(4, xs[q], M2v[q], q == 0);
+        mo.add_prod(5, Mv[q], Mv[q], q == 0);
+        mo.add_prod(6, M2v[q], M2v[q], q == 0);
+        mo.add_prod(7, Mv[q], M2v[q], q == 0);
       }
-      double tp[8];
-      mo.warp_total(tp);
-      finish_tile<8>(a, tile, tp, lane);
+      int index;
+      const double tp = mo.warp_total(lane, index);
+      finish_tile<8>(a, tile, tp, index, lane);
     } else {
       Moments<4> mo;
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         if (!live[q]) continue;
         const float y = xs[q] - c.beta * Mv[q] - c.beta2 * M2v[q];
-        mo.add(0, xs[q]);
-        mo.add_prod(1, xs[q], xs[q]);
-        mo.add(2, y);
-        mo.add_prod(3, y, y);
+        mo.add(0, xs[q], q == 0);
+        mo.add_prod(1, xs[q], xs[q], q == 0);
+        mo.add(2, y, q == 0);
+        mo.add_prod(3, y, y, q == 0);
       }
-      double tp[4];
-      mo.warp_total(tp);
-      finish_tile<4>(a, tile, tp, lane);
+      int index;
+      const double tp = mo.warp_total(lane, index);
+      finish_tile<4>(a, tile, tp, index, lane);
     }
+    if (a.one_pass) break;
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    last_block = atomicAdd(ctr + 1, 1ull) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (last_block && threadIdx.x == 0) {
-    ctr[0] = 0;
-    ctr[1] = 0;
-  }
+  reset_units(a);
 }
 
 }  // namespace pc

@@ -84,7 +84,7 @@ CvArgs device_args(const pc_cv_desc *c, const float *tables, const ModelHost &H,
 // window of dates (in registers for a specialised kernel when that window is
 // one date).
 pc_status cv_launch(const pc_model *m, const pc_contract *k, const pc_cv_desc *c, const float *tables,
-                    uint64_t n_paths, uint64_t seed, double *d_out, float *d_xm, bool pilot) {
+                    uint64_t n_paths, uint64_t seed, double *d_out, float *d_xm, bool pilot, bool report = false) {
   pc_status s = check_desc(m, c);
   if (s != PC_OK) return s;
   if (!tables && c->n > 1) return fail(PC_EINVAL, "null tables");
@@ -114,6 +114,7 @@ pc_status cv_launch(const pc_model *m, const pc_contract *k, const pc_cv_desc *c
   a.control = ctx->d_control;
   a.out = d_out;
   a.out_paths = d_xm;
+  if (report) report_to_host(ctx, a);
   CU(cudaSetDevice(ctx->device), "cudaSetDevice");
   const CvArgs ca = device_args(c, tables, m->H, pilot);
   if (ctx->jit && jit_eligible(k)) {
@@ -145,6 +146,7 @@ pc_status cv_launch(const pc_model *m, const pc_contract *k, const pc_cv_desc *c
     const uint64_t jneed = (a.n_tiles + kBlock / 32 - 1) / (kBlock / 32);
     const int jgrid = int(std::min<uint64_t>(uint64_t(ctx->sm_count) * nb, jneed));
     CvArgs cv = ca;
+    a.one_pass = uint64_t(jgrid) * (kBlock / 32) >= a.n_tiles;
     void *args[] = {&a, &cv, &L.w->grid_all};
     CU(cudaLaunchKernel(kern, dim3(jgrid), dim3(kBlock), args, jsm, ctx->stream),
        "specialised control-variate kernel");
@@ -152,6 +154,7 @@ pc_status cv_launch(const pc_model *m, const pc_contract *k, const pc_cv_desc *c
   }
   const uint64_t need = (a.n_tiles + block / 32 - 1) / (block / 32);
   const int grid = int(std::min<uint64_t>(uint64_t(ctx->sm_count) * best / (block / 32), need));
+  a.one_pass = uint64_t(grid) * (block / 32) >= a.n_tiles;
   CU(launch_cv(a, ca, grid, block, smem, ctx->stream), "control-variate kernel");
   return PC_OK;
 }
@@ -342,30 +345,16 @@ pc_status pc_cv_tables_async(pc_mlp *net, const pc_model *m, pc_cv_desc *c, floa
   return cv_tables(net, m, c, d_tables, cap, true);
 }
 
-// Sums of the launch (width doubles) to the host, with the status check.
-pc_status cv_sums(pc_ctx *ctx, int width, double *h) {
-  double st[5];
-  CU(cudaMemcpyAsync(h, ctx->d_gout, size_t(width) * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream),
-     "result copy");
-  CU(cudaMemcpyAsync(st, ctx->d_res, 5 * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream), "status copy");
-  pc_status s = wait_stream(ctx);
-  if (s != PC_OK) return s;
-  int32_t status;
-  std::memcpy(&status, &st[4], 4);
-  return check_status(ctx, status);
-}
-
 pc_status pc_price_cv(const pc_model *m, const pc_contract *k, const pc_cv_desc *c, const float *d_tables,
                       uint64_t n_paths, uint64_t seed, double *out) {
   if (!out) return fail(PC_EINVAL, "null output");
   if (n_paths < 2) return fail(PC_EINVAL, "n_paths must be >= 2 for a standard error");
   if (!m) return fail(PC_EINVAL, "null model");
   pc_ctx *ctx = m->ctx;
-  pc_status s = cv_launch(m, k, c, d_tables, n_paths, seed, ctx->d_gout, nullptr, false);
+  pc_status s = cv_launch(m, k, c, d_tables, n_paths, seed, ctx->h_res, nullptr, false, true);
+  if (s == PC_OK) s = wait_report(ctx);
   if (s != PC_OK) return s;
-  double h[4];
-  s = cv_sums(ctx, 4, h);
-  if (s != PC_OK) return s;
+  const double *h = ctx->h_res;
   const double N = double(n_paths);
   const double mx = h[0] / N, my = h[2] / N;
   out[0] = my;
@@ -381,11 +370,10 @@ pc_status pc_cv_beta(const pc_model *m, const pc_contract *k, const pc_cv_desc *
   if (n_paths < 16) return fail(PC_EINVAL, "n_paths must be >= 16");
   if (!m) return fail(PC_EINVAL, "null model");
   pc_ctx *ctx = m->ctx;
-  pc_status s = cv_launch(m, k, c, d_tables, n_paths, seed, ctx->d_gout, nullptr, true);
+  pc_status s = cv_launch(m, k, c, d_tables, n_paths, seed, ctx->h_res, nullptr, true, true);
+  if (s == PC_OK) s = wait_report(ctx);
   if (s != PC_OK) return s;
-  double h[8];
-  s = cv_sums(ctx, 8, h);
-  if (s != PC_OK) return s;
+  const double *h = ctx->h_res;
   // moments: X, M, M2, XM, XM2, MM, M2M2, MM2
   const double N = double(n_paths);
   const double mx = h[0] / N, mm = h[1] / N, m2 = h[2] / N;

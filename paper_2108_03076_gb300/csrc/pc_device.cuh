@@ -993,31 +993,59 @@ struct Moments {
     add(v, p);
     lo[v] = __fadd_rn(lo[v], __fmaf_rn(x, y, -p));
   }
-  // warp totals (identical in every lane: the butterfly's additions are
-  // commutative) as doubles; two values at a time on packed pairs, each half
-  // rounding as the scalar two-sum
-  __device__ __forceinline__ void warp_total(double (&tp)[W]) {
-    static_assert(W % 2 == 0, "values in pairs");
+  // The values of the lane's first path: what add and add_prod leave from
+  // zero, without the two-sum.
+  __device__ __forceinline__ void set(int v, float x) {
+    hi[v] = x;
+    lo[v] = 0.f;
+  }
+  __device__ __forceinline__ void set_prod(int v, float x, float y) {
+    hi[v] = __fmul_rn(x, y);
+    lo[v] = __fmaf_rn(x, y, -hi[v]);
+  }
+  __device__ __forceinline__ void add(int v, float x, bool first) { first ? set(v, x) : add(v, x); }
+  __device__ __forceinline__ void add_prod(int v, float x, float y, bool first) {
+    first ? set_prod(v, x, y) : add_prod(v, x, y);
+  }
+  // Warp totals as doubles, the one value `index` per lane that this lane
+  // ends with (the same for several lanes; the total is identical in all).
+  // Each butterfly step halves the values a lane carries: a lane keeps one half
+  // of them and sends its partner the other, so W values take W - 1 + (5 -
+  // log2 W) two-sums and twice as many shuffles in place of 5 W and 10 W (14
+  // values: 15 instead of 70), and one conversion to double in place of W.
+  // The two-sum's operands may be swapped without changing a bit, so the
+  // totals are those of the full butterfly.
+  __device__ __forceinline__ double warp_total(int lane, int &index) {
+    index = 0;
+    halve<W, 16>(lane, index);
+    return double(hi[0]) + double(lo[0]);
+  }
+
+ private:
+  template <int N, int O>
+  __device__ __forceinline__ void halve(int lane, int &index) {
+    constexpr int K = (N + 1) / 2;  // values kept (of an odd N both lanes keep the middle one)
+    const bool up = (lane & O) != 0;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-      for (int v = 0; v < W; v += 2) {
-        const float2 a = make_float2(hi[v], hi[v + 1]), c = make_float2(lo[v], lo[v + 1]);
-        const float2 h = make_float2(__shfl_xor_sync(kFull, a.x, o), __shfl_xor_sync(kFull, a.y, o));
-        const float2 l = make_float2(__shfl_xor_sync(kFull, c.x, o), __shfl_xor_sync(kFull, c.y, o));
-        const float2 s = add_x2(a, h);
-        const float2 b = sub_x2(s, a);
-        const float2 e = add_x2(sub_x2(a, sub_x2(s, b)), sub_x2(h, b));
-        const float2 t = add_x2(add_x2(c, l), e);
-        hi[v] = s.x;
-        hi[v + 1] = s.y;
-        lo[v] = t.x;
-        lo[v + 1] = t.y;
-      }
+    for (int j = 0; j < K; ++j) {
+      const float kh = N > 1 && up ? hi[N - K + j] : hi[j], kl = N > 1 && up ? lo[N - K + j] : lo[j];
+      const float sh = N > 1 && up ? hi[j] : hi[N - K + j], sl = N > 1 && up ? lo[j] : lo[N - K + j];
+      const float h = __shfl_xor_sync(kFull, sh, O), l = __shfl_xor_sync(kFull, sl, O);
+      const float s = __fadd_rn(kh, h);
+      const float b = __fsub_rn(s, kh);
+      const float e = __fadd_rn(__fsub_rn(kh, __fsub_rn(s, b)), __fsub_rn(h, b));
+      nh[j] = s;
+      nl[j] = __fadd_rn(__fadd_rn(kl, l), e);
     }
 #pragma unroll
-    for (int v = 0; v < W; ++v) tp[v] = double(hi[v]) + double(lo[v]);
+    for (int j = 0; j < K; ++j) {
+      hi[j] = nh[j];
+      lo[j] = nl[j];
+    }
+    if (N > 1 && up) index += N - K;
+    if constexpr (O > 1) halve<K, O / 2>(lane, index);
   }
+  float nh[(W + 1) / 2], nl[(W + 1) / 2];
 };
 
 // Deterministic reduction.  Tile t's partials (sum, sum of squares, ...) are
@@ -1033,17 +1061,52 @@ __device__ __forceinline__ void warp_sum_strided(const double *src, uint32_t n, 
                                                  double (&acc)[W]) {
 #pragma unroll
   for (int v = 0; v < W; ++v) acc[v] = 0.0;
-  for (uint32_t i = lane; i < n; i += 32) {
+  if constexpr (W <= 4) {  // four tiles' loads in flight
+    uint32_t i = lane;
+    for (; i + 96 < n; i += 128) {
+      double x[4][W];
 #pragma unroll
-    for (int v = 0; v < W; ++v) acc[v] += __ldcg(src + size_t(i) * W + v);
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < W; ++v) x[u][v] = __ldcg(src + size_t(i + 32 * u) * W + v);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < W; ++v) acc[v] += x[u][v];
+    }
+    for (; i < n; i += 32)
+#pragma unroll
+      for (int v = 0; v < W; ++v) acc[v] += __ldcg(src + size_t(i) * W + v);
+  } else {
+    for (uint32_t i = lane; i < n; i += 32) {
+#pragma unroll
+      for (int v = 0; v < W; ++v) acc[v] += __ldcg(src + size_t(i) * W + v);
+    }
   }
 #pragma unroll
   for (int v = 0; v < W; ++v) acc[v] = warp_sum(acc[v]);
 }
 
+// The launch's totals: out, then (blocking calls) the ticket and the device
+// status to the host's pinned flag, which the host polls instead of waiting
+// for a copy and the stream.
 template <int W>
-__device__ __noinline__ void finish_tile(const PriceArgs &a, uint64_t tile, const double (&tp)[W],
-                                         int lane) {
+__device__ __forceinline__ void finish_launch(const PriceArgs &a, const double (&acc)[W], int lane) {
+  if (lane != 0) return;
+#pragma unroll
+  for (int v = 0; v < W; ++v) a.out[v] = acc[v];
+  a.out[W] = double(a.n_paths);
+  if (a.done) {
+    const uint32_t status = uint32_t(__ldcg(a.status));
+    __threadfence_system();
+    *reinterpret_cast<volatile unsigned long long *>(a.done) =
+        (static_cast<unsigned long long>(a.ticket) << 32) | status;
+  }
+}
+
+// Tile `tile`'s partials: value `index` is this lane's `tp` (Moments::warp_total).
+template <int W>
+__device__ __noinline__ void finish_tile(const PriceArgs &a, uint64_t tile, double tp, int index, int lane) {
   unsigned long long *ctr = reinterpret_cast<unsigned long long *>(a.control);
   uint32_t *chunk_cnt = reinterpret_cast<uint32_t *>(a.control + kChunkCountOff);
   double *chunk_part = reinterpret_cast<double *>(a.control + kChunkPartOff);
@@ -1051,10 +1114,10 @@ __device__ __noinline__ void finish_tile(const PriceArgs &a, uint64_t tile, cons
   const uint64_t first = uint64_t(chunk) * a.chunk_tiles;
   const uint64_t rest = a.n_tiles - first;
   const uint32_t size = rest < a.chunk_tiles ? uint32_t(rest) : a.chunk_tiles;
+  a.tile_partials[tile * W + index] = tp;  // lanes with the same value store the same bits
+  __syncwarp();
   uint32_t seen = 0;
   if (lane == 0) {
-#pragma unroll
-    for (int v = 0; v < W; ++v) a.tile_partials[tile * W + v] = tp[v];
     // release: the partials are visible before the count that reports them
     asm volatile("atom.release.gpu.global.add.u32 %0, [%1], 1;" : "=r"(seen) : "l"(chunk_cnt + chunk) : "memory");
   }
@@ -1064,11 +1127,15 @@ __device__ __noinline__ void finish_tile(const PriceArgs &a, uint64_t tile, cons
   __threadfence();
   double acc[W];
   warp_sum_strided<W>(a.tile_partials + first * W, size, lane, acc);
+  if (lane == 0) chunk_cnt[chunk] = 0;
+  if (a.n_chunks == 1) {
+    finish_launch<W>(a, acc, lane);
+    return;
+  }
   unsigned long long done = 0;
   if (lane == 0) {
 #pragma unroll
     for (int v = 0; v < W; ++v) chunk_part[size_t(chunk) * W + v] = acc[v];
-    chunk_cnt[chunk] = 0;
     asm volatile("atom.release.gpu.global.add.u64 %0, [%1], 1;" : "=l"(done) : "l"(ctr + 2) : "memory");
   }
   done = __shfl_sync(kFull, done, 0);
@@ -1076,11 +1143,35 @@ __device__ __noinline__ void finish_tile(const PriceArgs &a, uint64_t tile, cons
   // this warp completed the last chunk
   __threadfence();
   warp_sum_strided<W>(chunk_part, a.n_chunks, lane, acc);
-  if (lane == 0) {
-#pragma unroll
-    for (int v = 0; v < W; ++v) a.out[v] = acc[v];
-    a.out[W] = double(a.n_paths);
-    ctr[2] = 0;
+  if (lane == 0) ctr[2] = 0;
+  finish_launch<W>(a, acc, lane);
+}
+
+// The next unit of work (a tile, or a pair) of this warp from the launch's
+// counter; with one_pass (no more units than warps) the warp's own number,
+// once: no counter to read, none to reset at the end.
+__device__ __forceinline__ unsigned long long next_unit(const PriceArgs &a, int lane) {
+  if (a.one_pass) return (static_cast<unsigned long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+  unsigned long long u = 0;
+  if (lane == 0) u = atomicAdd(reinterpret_cast<unsigned long long *>(a.control), 1ull);
+  return __shfl_sync(kFull, u, 0);
+}
+
+// The last block to exit re-zeroes the unit counter: no warp takes units any
+// more once every block has left its loop.
+__device__ __forceinline__ void reset_units(const PriceArgs &a) {
+  if (a.one_pass) return;
+  __shared__ int last_block;
+  unsigned long long *ctr = reinterpret_cast<unsigned long long *>(a.control);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last_block = atomicAdd(ctr + 1, 1ull) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (last_block && threadIdx.x == 0) {
+    ctr[0] = 0;
+    ctr[1] = 0;
   }
 }
 

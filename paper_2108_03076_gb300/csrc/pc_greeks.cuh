@@ -142,7 +142,6 @@ __device__ TV eval_greeks(const uint4 *P, const float *pool, float2 *R, const Pr
 template <int D, bool WRITE, typename EVAL>
 __device__ __forceinline__ void greeks_tiles(const PriceArgs &a, EVAL eval) {
   extern __shared__ __align__(16) uint32_t smem[];
-  __shared__ int last_block;
   const Staged st = stage_program(a, smem);
   const uint4 *P = st.P;
   const float *pool = st.pool;
@@ -155,13 +154,10 @@ __device__ __forceinline__ void greeks_tiles(const PriceArgs &a, EVAL eval) {
   const int gl = a.greek_label;
   const float sig_g = __ldg(a.m.sig + gl);
   const int lane = threadIdx.x & 31;
-  unsigned long long *ctr = reinterpret_cast<unsigned long long *>(a.control);
   Rng2 g;
   rng_init(g, a.rk, a.stream, a.path_offset);
   for (;;) {
-    unsigned long long tile = 0;
-    if (lane == 0) tile = atomicAdd(ctr, 1ull);
-    tile = __shfl_sync(kFull, tile, 0);
+    const unsigned long long tile = next_unit(a, lane);
     if (tile >= a.n_tiles) break;
     const uint64_t i0 = tile * kTilePaths + lane, i1 = i0 + 32;
     const bool live0 = i0 < a.n_paths, live1 = i1 < a.n_paths;
@@ -174,8 +170,8 @@ __device__ __forceinline__ void greeks_tiles(const PriceArgs &a, EVAL eval) {
     if (live0) {
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
-        mo.add(2 * j, q0[j]);
-        mo.add_prod(2 * j + 1, q0[j], q0[j]);
+        mo.set(2 * j, q0[j]);
+        mo.set_prod(2 * j + 1, q0[j], q0[j]);
         if (WRITE) a.out_paths[i0 * 3 + j] = q0[j];
       }
     }
@@ -187,20 +183,12 @@ __device__ __forceinline__ void greeks_tiles(const PriceArgs &a, EVAL eval) {
         if (WRITE) a.out_paths[i1 * 3 + j] = q1[j];
       }
     }
-    double tp[6];
-    mo.warp_total(tp);
-    finish_tile<6>(a, tile, tp, lane);
+    int index;
+    const double tp = mo.warp_total(lane, index);
+    finish_tile<6>(a, tile, tp, index, lane);
+    if (a.one_pass) break;
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    last_block = atomicAdd(ctr + 1, 1ull) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (last_block && threadIdx.x == 0) {
-    ctr[0] = 0;
-    ctr[1] = 0;
-  }
+  reset_units(a);
 }
 
 }  // namespace pc

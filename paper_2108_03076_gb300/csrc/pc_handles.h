@@ -29,6 +29,9 @@ constexpr int kJitPrice = 0, kJitPriceWrite = 1, kJitHbm = 2, kJitWinRegs = 4, k
 // resident blocks per SM the specialised pricing kernel's register bound is
 // set for by default (<= 72 registers at 128 threads: the fastest measured)
 constexpr int kJitMinBlocks = 7;
+// one underlying needs fewer registers: 8 blocks (<= 64; 35-date average, 3e5 paths: 58.7 -> 45 us, where 7
+// blocks' 4,256 warps left a second round of 432 tiles)
+constexpr int kJitMinBlocks1 = 8;
 // the same with a static walk, whose bridge stack and normals are registers
 // (autocall, 3 underlyings, 5 dates, 2^20 paths: 5 / 6 / 7 / 8 blocks 52.5 / 51.4 / 52.1 / 52.1 us a call)
 constexpr int kWalkMinBlocks = 6;
@@ -95,7 +98,9 @@ struct pc_ctx {
   std::map<uint64_t, std::vector<std::vector<int32_t>>> jit_walks;  // program hash -> its static walks (admit_walk)
   std::map<std::pair<const void *, size_t>, int> jit_occ;  // (kernel, smem) -> resident blocks
   cudaMemPool_t pool = nullptr;  // stream-ordered allocations of contracts (null: cudaMalloc)
-  double *h_res = nullptr;       // pinned [16]: results read back by the blocking calls
+  double *h_res = nullptr;       // pinned [64]: the blocking calls' results, written by the kernel
+  uint64_t *h_done = nullptr;    // pinned: (ticket << 32) | device status, written after them
+  uint32_t ticket = 0;           // the last blocking call's
   // pinned staging of program uploads, two halves filled in turn: a half is
   // reused once the event recorded when it was left has completed
   uint32_t *h_stage = nullptr;
@@ -172,6 +177,14 @@ pc_status cuda_fail(cudaError_t e, const char *what);
 // Wait for the context's stream with its wall-clock limit.
 pc_status wait_stream(pc_ctx *c);
 
+// A blocking call's results: the launch writes its sums to pinned host memory
+// and then the call's ticket with the device status to a pinned word, which
+// the host polls (with the wall-clock limit; the stream is queried now and
+// then, for errors).  A copy back and a stream query took 4 us more, two
+// copies to pageable memory 15.
+void report_to_host(pc_ctx *c, PriceArgs &a);       // sets a.done and a.ticket (the call's last launch)
+pc_status wait_report(pc_ctx *c);                   // results in c->h_res; PC_EDEVICE for a raised status
+
 // cudaMalloc for the context's buffers, or a simulated out-of-memory
 // (cudaErrorMemoryAllocation, nothing allocated) while the context's
 // failure injection count is positive.
@@ -243,7 +256,7 @@ pc_status jit_compile_many(pc_ctx *c, const std::vector<JitRequest> &reqs);
 // memory; may re-choose the block) and the register bound it is compiled for.
 int jit_window_kind(const pc_ctx *c, const Launch &L);
 size_t jit_layout(const pc_ctx *c, Launch &L, int bits);
-int jit_min_blocks(const pc_ctx *c, size_t smem, int block);
+int jit_min_blocks(const pc_ctx *c, size_t smem, int block, int d);
 // What the contract's specialised kernel of `kind` is compiled for: the
 // launch's arguments (layout final) and a walk (may be empty).
 JitSpec jit_spec(const pc_contract *k, const PriceArgs &a, int kind, int min_blocks, const std::vector<int32_t> &walk);

@@ -70,16 +70,16 @@ __device__ __forceinline__ void batch_unit(const PriceArgs &a, const BatchUnit &
     const float2 x = eval_path<D>(P, pool, R, a, g, live0, live1, Bm, S0);
     Moments<2> mo;
     if (live0) {
-      mo.add(0, x.x);
-      mo.add_prod(1, x.x, x.x);
+      mo.set(0, x.x);
+      mo.set_prod(1, x.x, x.x);
     }
     if (live1) {
       mo.add(0, x.y);
       mo.add_prod(1, x.y, x.y);
     }
-    double tp[2];
-    mo.warp_total(tp);
-    finish_tile<2>(a, tile, tp, lane);
+    int index;
+    const double tp = mo.warp_total(lane, index);
+    finish_tile<2>(a, tile, tp, index, lane);
   }
 }
 

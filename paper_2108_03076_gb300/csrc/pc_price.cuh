@@ -12,7 +12,6 @@ namespace pc {
 template <int D, bool WRITE, typename EVAL>
 __device__ __forceinline__ void price_tiles(const PriceArgs &a, EVAL eval) {
   extern __shared__ __align__(16) uint32_t smem[];
-  __shared__ int last_block;
   const Staged st = stage_program(a, smem);
   const uint4 *P = st.P;
   const float *pool = st.pool;
@@ -20,13 +19,10 @@ __device__ __forceinline__ void price_tiles(const PriceArgs &a, EVAL eval) {
   const float(&Bm)[D * D] = *reinterpret_cast<const float(*)[D * D]>(a.m.Bv);
   const float(&S0)[D] = *reinterpret_cast<const float(*)[D]>(a.m.S0v);
   const int lane = threadIdx.x & 31;
-  unsigned long long *ctr = reinterpret_cast<unsigned long long *>(a.control);
   Rng2 g;
   rng_init(g, a.rk, a.stream, a.path_offset);
   for (;;) {
-    unsigned long long tile = 0;
-    if (lane == 0) tile = atomicAdd(ctr, 1ull);
-    tile = __shfl_sync(kFull, tile, 0);
+    const unsigned long long tile = next_unit(a, lane);
     if (tile >= a.n_tiles) break;
     const uint64_t i0 = tile * kTilePaths + lane, i1 = i0 + 32;
     const bool live0 = i0 < a.n_paths, live1 = i1 < a.n_paths;
@@ -36,8 +32,8 @@ __device__ __forceinline__ void price_tiles(const PriceArgs &a, EVAL eval) {
     const float2 x = eval(P, pool, R, g, live0, live1, Bm, S0);
     Moments<2> mo;
     if (live0) {
-      mo.add(0, x.x);
-      mo.add_prod(1, x.x, x.x);
+      mo.set(0, x.x);
+      mo.set_prod(1, x.x, x.x);
       if (WRITE) a.out_paths[i0] = x.x;
     }
     if (live1) {
@@ -45,22 +41,12 @@ __device__ __forceinline__ void price_tiles(const PriceArgs &a, EVAL eval) {
       mo.add_prod(1, x.y, x.y);
       if (WRITE) a.out_paths[i1] = x.y;
     }
-    double tp[2];
-    mo.warp_total(tp);
-    finish_tile<2>(a, tile, tp, lane);
+    int index;
+    const double tp = mo.warp_total(lane, index);
+    finish_tile<2>(a, tile, tp, index, lane);
+    if (a.one_pass) break;
   }
-  // the last block to exit re-zeroes the tile counter: no warp grabs tiles
-  // any more once every block has left its loop
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    last_block = atomicAdd(ctr + 1, 1ull) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (last_block && threadIdx.x == 0) {
-    ctr[0] = 0;
-    ctr[1] = 0;
-  }
+  reset_units(a);
 }
 
 #if PC_PAIRS == 2
@@ -73,7 +59,6 @@ __device__ __forceinline__ void price_tiles(const PriceArgs &a, EVAL eval) {
 template <int D, bool WRITE, typename EVAL>
 __device__ __forceinline__ void price_tiles2(const PriceArgs &a, EVAL eval) {
   extern __shared__ __align__(16) uint32_t smem[];
-  __shared__ int last_block;
   const Staged st = stage_program(a, smem);
   const uint4 *P = st.P;
   const float *pool = st.pool;
@@ -81,14 +66,11 @@ __device__ __forceinline__ void price_tiles2(const PriceArgs &a, EVAL eval) {
   const float(&Bm)[D * D] = *reinterpret_cast<const float(*)[D * D]>(a.m.Bv);
   const float(&S0)[D] = *reinterpret_cast<const float(*)[D]>(a.m.S0v);
   const int lane = threadIdx.x & 31;
-  unsigned long long *ctr = reinterpret_cast<unsigned long long *>(a.control);
   const uint64_t n_pairs = (a.n_tiles + 1) / 2;
   RngH<2> g;
   rng_init(g, a.rk, a.stream, a.path_offset);
   for (;;) {
-    unsigned long long u = 0;
-    if (lane == 0) u = atomicAdd(ctr, 1ull);
-    u = __shfl_sync(kFull, u, 0);
+    const unsigned long long u = next_unit(a, lane);
     if (u >= n_pairs) break;
     uint64_t idx[4];
     bool live[4];
@@ -106,8 +88,8 @@ __device__ __forceinline__ void price_tiles2(const PriceArgs &a, EVAL eval) {
       const float x0 = pv_get(x, 2 * h), x1 = pv_get(x, 2 * h + 1);
       Moments<2> mo;
       if (live[2 * h]) {
-        mo.add(0, x0);
-        mo.add_prod(1, x0, x0);
+        mo.set(0, x0);
+        mo.set_prod(1, x0, x0);
         if (WRITE) a.out_paths[idx[2 * h]] = x0;
       }
       if (live[2 * h + 1]) {
@@ -115,21 +97,13 @@ __device__ __forceinline__ void price_tiles2(const PriceArgs &a, EVAL eval) {
         mo.add_prod(1, x1, x1);
         if (WRITE) a.out_paths[idx[2 * h + 1]] = x1;
       }
-      double tp[2];
-      mo.warp_total(tp);
-      finish_tile<2>(a, tile, tp, lane);
+      int index;
+      const double tp = mo.warp_total(lane, index);
+      finish_tile<2>(a, tile, tp, index, lane);
     }
+    if (a.one_pass) break;
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    last_block = atomicAdd(ctr + 1, 1ull) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (last_block && threadIdx.x == 0) {
-    ctr[0] = 0;
-    ctr[1] = 0;
-  }
+  reset_units(a);
 }
 #endif
 

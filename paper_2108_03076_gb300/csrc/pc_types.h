@@ -229,6 +229,9 @@ struct PriceArgs {
   double *out;              // [width + 1]: sums over all paths, then n_paths
   float *out_paths;         // nullable: per-path payoffs (sensitivities: 3 floats per path)
   int32_t *status;          // device status word (nonzero = error)
+  int32_t one_pass;         // 1: the grid has a warp for every unit of work (tile or pair of tiles)
+  uint32_t ticket;          // blocking calls: written to *done with the status at the end
+  uint64_t *done;           // pinned host word (null: not reported)
   int32_t greek_label;      // sensitivity kernel: the underlying g of the tangents
 };
 
@@ -251,7 +254,7 @@ constexpr size_t kChunkPartOff = 2048;
 constexpr size_t kControlBytes = kChunkPartOff + size_t(kMaxChunks) * 8 * sizeof(double);
 inline void reduction_chunks(PriceArgs &a, uint32_t max_chunks = kMaxChunks) {
   uint64_t c = (a.n_tiles + kMaxChunks - 1) / kMaxChunks;
-  if (c < 64) c = 64;
+  if (c < 64) c = a.n_tiles <= 256 ? 256 : 64;  // up to 256 tiles: one chunk, one level fewer
   if ((a.n_tiles + c - 1) / c > max_chunks) c = (a.n_tiles + max_chunks - 1) / max_chunks;
   a.chunk_tiles = uint32_t(c);
   a.n_chunks = uint32_t((a.n_tiles + c - 1) / c);
