@@ -71,10 +71,11 @@ struct Tape {
 // for a constant (history).
 template <int D>
 __device__ __forceinline__ int adj_leaf(Tape &T, int o, int l, float2 s, float scale, const float2 *R,
-                                        const ModelDev &m, const Layout &lay, const float (&S0)[D]) {
+                                        const ModelDev &m, const Layout &lay, const float (&S0)[D],
+                                        const float2 (&w)[D], const float *Lm) {
   if (o < 0) return -1;
   if (o == 0) return T.put(-2 - l, -1, make_float2(scale, scale), make_float2(0.f, 0.f));
-  const float2 x = SL(lay.off_xwin + (o & (lay.win - 1)) * D + l);
+  const float2 x = read_x<D>(o, l, w, Lm, R, lay);
   const float st = __fmul_rn(__ldg(m.sig + l), __ldg(m.tau + o));
   const float r0 = __fdiv_rn(scale, S0[l]);
   return T.put(-2 - l, -1, make_float2(__fmul_rn(s.x, r0), __fmul_rn(s.y, r0)),
@@ -110,10 +111,17 @@ __device__ __forceinline__ void reverse_sweep(Tape &T, int res, float2 (&dS)[D],
   if (res < 0) return;
   const int lane = T.lane;
   T.adj[size_t(res) * 32 + lane] = make_float2(1.f, 1.f);
+  // the next entry's inputs and partials (written by the forward sweep only)
+  // are fetched ahead; its adjoint is final only when it is reached
+  int2 in_next = T.ids[T.n - 1];
+  float4 p_next = T.part[size_t(T.n - 1) * 32 + lane];
   for (int e = T.n - 1; e >= 0; --e) {
     const float2 ad = T.adj[size_t(e) * 32 + lane];
-    const int2 in = T.ids[e];
-    const float4 p = T.part[size_t(e) * 32 + lane];
+    const int2 in = in_next;
+    const float4 p = p_next;
+    const int q1 = e > 0 ? e - 1 : 0;
+    in_next = T.ids[q1];
+    p_next = T.part[size_t(q1) * 32 + lane];
     if (in.x <= -2) {
       const int l = -2 - in.x;
 #pragma unroll

@@ -46,12 +46,13 @@ pc_status run_adjoint(const pc_model *m, const pc_contract *k, uint64_t n_paths,
   const int64_t emax = std::max<int64_t>(walk.entries, 1);
   if (emax > (int64_t(1) << 24)) return fail(PC_ELIMIT, "adjoint tape bound above 2^24 entries per path");
   Layout lay = L.args.lay;
-  lay.stack = 2 * k->prog.frame_slots;
+  lay.ids = (k->prog.frame_slots + 63) / 64;  // a slot holds 64 ints of the warp
+  lay.stack = lay.ids + k->prog.frame_slots;
   lay.off_bstack = lay.stack;
   lay.off_cache = lay.off_bstack + H.bstack * d;
   lay.off_win = lay.off_cache;
   lay.off_xwin = lay.off_win + lay.win * d;
-  lay.words = lay.off_xwin + lay.win * d;
+  lay.words = lay.off_xwin + (lay.win > 1 ? lay.win * d : 0);
   int block = 0, best_warps = 0;
   size_t smem = 0;
   for (int b = kBlock; b >= 32; b /= 2) {

@@ -358,7 +358,7 @@ pc_status run_greeks(const pc_model *m, const pc_contract *k, uint64_t n_paths, 
   lay.off_cache = lay.off_bstack + m->H.bstack * d;
   lay.off_win = lay.off_cache;
   lay.off_xwin = lay.off_win + lay.win * d;
-  lay.words = lay.off_xwin + lay.win * d;
+  lay.words = lay.off_xwin + (lay.win > 1 ? lay.win * d : 0);
   int block = 0, best_warps = 0;
   size_t smem = 0;
   for (int b = kBlock; b >= 32; b /= 2) {

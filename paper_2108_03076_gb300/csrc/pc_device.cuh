@@ -235,6 +235,7 @@ __device__ __forceinline__ Layout layout_of(const PriceArgs &a) {
   l.off_xwin = v[4];
   l.words = v[5];
   l.win = v[6];
+  l.ids = v[7];
   return l;
 }
 #else
@@ -346,6 +347,28 @@ __device__ __forceinline__ void path_state_init(PathState<D, H> &ps, float2 *R, 
 #endif
 }
 
+// X_i = sum_k L_ik W_k.
+template <int D>
+__device__ __forceinline__ float2 correlated(int i, const float2 (&w)[D], const float *Lm) {
+  float2 x = mul_x2(dup2(Lm[i * D]), w[0]);
+#pragma unroll
+  for (int k = 1; k < D; ++k)
+    if (k <= i) x = fma_x2(dup2(Lm[i * D + k]), w[k], x);
+  return x;
+}
+// X_l of a read at ordinal o > 0: from the window, or of the frontier date
+// from W (a window of one date).
+template <int D>
+__device__ __forceinline__ float2 read_x(int o, int l, const float2 (&w)[D], const float *Lm, const float2 *R,
+                                         const Layout &lay) {
+  if (lay.win > 1) return SL(lay.off_xwin + (o & (lay.win - 1)) * D + l);
+  float2 x = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int i = 0; i < D; ++i)
+    if (i == l) x = correlated<D>(i, w, Lm);
+  return x;
+}
+
 // GBM at date t from W at the frontier into the window slot of t.  With XW
 // the correlated Brownian values X = L W of the date are also kept (window
 // at lay.off_xwin), which the pathwise sensitivities need.
@@ -372,13 +395,10 @@ __device__ __forceinline__ void date_values(int t, PathState<D, H> &ps, const La
     }
   }
   if constexpr (XW) {
-    const int xs = lay.off_xwin + (t & (lay.win - 1)) * D;
+    if (lay.win > 1) {  // (with a window of one date X is formed from W where it is read)
+      const int xs = lay.off_xwin + (t & (lay.win - 1)) * D;
 #pragma unroll
-    for (int i = 0; i < D; ++i) {
-      float2 x = mul_x2(dup2(Lm[i * D]), ps.w[0][0]);
-#pragma unroll
-      for (int k = 1; k <= i; ++k) x = fma_x2(dup2(Lm[i * D + k]), ps.w[0][k], x);
-      SL(xs + i) = x;
+      for (int i = 0; i < D; ++i) SL(xs + i) = correlated<D>(i, ps.w[0], Lm);
     }
   }
 }
@@ -924,6 +944,32 @@ __device__ __forceinline__ void fused_test_regs(const uint4 &I, int o, const flo
                                                 const ModelDev &m, bool &t0, bool &t1) {
   fused_test_rd<D>(I, o, pool, m, [&](int l) { return cur[l]; }, t0, t1);
 }
+
+// A whole-loop barrier's decoded test (LOOP_TEST, before the loop) and the
+// sensitivity evaluators' use of it (LOOP_VALUE: the test at ordinal o,
+// fresh_: the date was produced for it, its S is in registers).
+#ifdef PC_JIT
+#define LOOP_TEST(I_)
+#define LOOP_VALUE(I_, o_, fresh_, c0_, c1_)                         \
+  do {                                                               \
+    (void)(fresh_);                                                  \
+    const float2 v_ = fused_value<D>(I_, o_, pool, R, m, lay);       \
+    c0_ = bits(v_.x) != 0;                                           \
+    c1_ = bits(v_.y) != 0;                                           \
+  } while (0)
+#else
+#define LOOP_TEST(I_) const LoopTest<D> lt_(I_)
+#define LOOP_VALUE(I_, o_, fresh_, c0_, c1_)                         \
+  do {                                                               \
+    if (lt_.use && (fresh_)) {                                       \
+      lt_.test(ps.s[0], c0_, c1_);                                   \
+    } else {                                                         \
+      const float2 v_ = fused_value<D>(I_, o_, pool, R, m, lay);     \
+      c0_ = bits(v_.x) != 0;                                         \
+      c1_ = bits(v_.y) != 0;                                         \
+    }                                                                \
+  } while (0)
+#endif
 
 // Values of the stack machine: one per path of the lane, kPL = 2 PC_PAIRS of
 // them (PC_PAIRS pairs; a specialised kernel with four paths a lane defines

@@ -57,7 +57,6 @@ __device__ float2 eval_path(const uint4 *P, const float *pool, float2 *R, const 
 #undef EACH_DATE
 #undef FUSED_VALUE
 #undef FUSED_TEST
-#undef LOOP_TEST
 #undef LOOP_FUSED_TEST
 }
 

@@ -57,12 +57,13 @@ __device__ __forceinline__ void stv(float2 *R, int s, const TV &x) {
 // Model read of label l at ordinal o with tangents for underlying g.
 template <int D>
 __device__ __forceinline__ TV model_read(int o, int l, int g, const float2 *R, const ModelDev &m,
-                                         const Layout &lay, const float (&S0)[D], float sig_g) {
+                                         const Layout &lay, const float (&S0)[D], float sig_g,
+                                         const float2 (&w)[D], const float *Lm) {
   l = l < D ? l : 0;
   if (o > 0) {
     const float2 s = SL(lay.off_win + (o & (lay.win - 1)) * D + l);
     if (l != g) return tv(s);
-    const float2 x = SL(lay.off_xwin + (o & (lay.win - 1)) * D + l);
+    const float2 x = read_x<D>(o, l, w, Lm, R, lay);
     const float st = __fmul_rn(sig_g, __ldg(m.tau + o));
     return {s, scl2(s, __frcp_rn(S0[l])), f2(__fmul_rn(s.x, __fsub_rn(x.x, st)), __fmul_rn(s.y, __fsub_rn(x.y, st)))};
   }
@@ -77,7 +78,7 @@ __device__ __forceinline__ TV model_read(int o, int l, int g, const float2 *R, c
 template <int D>
 __device__ __forceinline__ TV fused_tv(const uint4 &I, int o, const float *pool, const float2 *R,
                                        const ModelDev &m, const Layout &lay, const float (&S0)[D],
-                                       int g, float sig_g) {
+                                       int g, float sig_g, const float2 (&w)[D], const float *Lm) {
   const uint32_t A = I.x >> 8;
   const int n = int((A >> 8) & 3u) + 1, kind = int((A >> 2) & 3u), code = int((A >> 4) & 7u);
   const bool any = (I.x & 0xffu) == X_LANY, conj = (A & 1u) != 0;
@@ -85,7 +86,7 @@ __device__ __forceinline__ TV fused_tv(const uint4 &I, int o, const float *pool,
   const float k = __uint_as_float(I.w);
   TV v = tv(f2(0.f, 0.f));
   for (int i = 0; i < n; ++i) {
-    TV s = model_read<D>(o, int(A >> (10 + 2 * i)) & 3, g, R, m, lay, S0, sig_g);
+    TV s = model_read<D>(o, int(A >> (10 + 2 * i)) & 3, g, R, m, lay, S0, sig_g, w, Lm);
     if (kind == 1) {
       const float c = pool[I.z + i];
       s = {scl2(s.v, c), scl2(s.a, c), scl2(s.b, c)};

@@ -597,7 +597,7 @@ JitSpec jit_spec(const pc_contract *k, const PriceArgs &a, int kind, int min_blo
   sp.one_phi = one_phi(a.path_offset, a.n_tiles);
   // constants by value, unless an out-of-line date generator takes them by reference
   if (kind >= kJitCv || !outlined_dates(k->prog))
-    sp.lay = {a.lay.stack, a.lay.off_bstack, a.lay.off_cache, a.lay.off_win, a.lay.off_xwin, a.lay.words, a.lay.win};
+    sp.lay = {a.lay.stack, a.lay.off_bstack, a.lay.off_cache, a.lay.off_win, a.lay.off_xwin, a.lay.words, a.lay.win, a.lay.ids};
   if (!walk.empty()) sp.grid = {a.m.n, a.m.n_hist, a.m.t_now};
   return sp;
 }

@@ -165,6 +165,8 @@ struct Layout {
   int32_t off_xwin;   // window of X = L W (win * d), sensitivity kernel only
   int32_t words;      // total words per thread in shared memory
   int32_t win;        // window size (power of two)
+  int32_t ids;        // adjoint kernel: leading slots that hold the stack's entry numbers, one int a value
+                      // for the whole warp
   int32_t skip;       // with a window of one date: the first date the program reads (else 0)
   // HBM window (programs whose lookback does not fit shared memory): the
   // window of thread t of the launch is column t of gwin, slot s at
