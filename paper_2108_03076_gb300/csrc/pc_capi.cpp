@@ -17,6 +17,7 @@
 
 #include "pc_handles.h"
 #include "pc_internal.h"
+#include "pc_screen.h"
 
 using namespace pc;
 
@@ -480,6 +481,36 @@ int jit_min_blocks(const pc_ctx *c, size_t smem, int block, int d) {
   return std::max(1, std::min(most, warps / (kBlock / 32)));
 }
 
+// A contract whose launches on the model are screened when they are large
+// enough (pc_screen.h); fills `s` but its buffers.
+bool screen_suits(const pc_model *m, const pc_contract *k, Screen &s) {
+  return screen_program(k->prog, m->H, s) && screen_fraction(m->H, s) >= kScreenFraction;
+}
+
+// Sets up a screened launch where it pays: the context's list and payoff
+// buffers (grown here; no memory for them: unscreened).  `payoffs`: the
+// caller's per-path payoffs, else the context's.
+bool screen_launch(pc_ctx *c, const pc_model *m, const pc_contract *k, const PriceArgs &a, float *payoffs, Screen &s) {
+  if (a.n_paths > kScreenPaths || double(a.n_paths) * m->H.n * m->H.d < kScreenWork) return false;
+  if (!screen_suits(m, k, s)) return false;
+  const size_t words = 64 + size_t(a.n_paths) * (payoffs ? 1 : 2);
+  if (words > c->screen_cap) {
+    if (cudaStreamSynchronize(c->stream) != cudaSuccess) return false;
+    if (c->d_screen) cudaFree(c->d_screen);
+    c->d_screen = nullptr;
+    c->screen_cap = 0;
+    if (ctx_malloc(c, reinterpret_cast<void **>(&c->d_screen), words * 4) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    c->screen_cap = words;
+  }
+  s.count = c->d_screen;
+  s.list = c->d_screen + 64;
+  s.payoffs = payoffs ? payoffs : reinterpret_cast<float *>(c->d_screen + 64 + a.n_paths);
+  return true;
+}
+
 pc_status run_price(const pc_model *m, const pc_contract *k, uint64_t n_paths, uint64_t offset,
                     uint64_t seed, uint32_t stream, double *d_out, float *d_payoffs, bool report = false) {
   Launch L;
@@ -496,12 +527,22 @@ pc_status run_price(const pc_model *m, const pc_contract *k, uint64_t n_paths, u
   L.args.out_paths = d_payoffs;
   if (report) report_to_host(c, L.args);
   CU(cudaSetDevice(c->device), "cudaSetDevice");
+  Screen sc;
+  const bool screened = screen_launch(c, m, k, L.args, d_payoffs, sc);
+  const PriceArgs all = L.args;  // the screen's and the totals' launch
+  if (screened) {
+    CU(cudaMemsetAsync(sc.count, 0, sizeof(uint32_t), c->stream), "screen count");
+    CU(launch_screen(all, sc, c->sm_count, c->stream), "screen kernel");
+    L.args.list = sc.list;
+    L.args.list_n = sc.count;
+    L.args.out_paths = sc.payoffs;
+  }
   if (c->jit && jit_eligible(k)) {
     // the contract's run-time specialised kernel (same arguments and shape)
     cudaKernel_t jk = nullptr;
     const int wk = jit_window_kind(c, L);
     const size_t smem = jit_layout(c, L, wk);
-    s = jit_pair_kernel(k, L.w, L.args, (d_payoffs != nullptr ? kJitPriceWrite : kJitPrice) | wk,
+    s = jit_pair_kernel(k, L.w, L.args, (d_payoffs || screened ? kJitPriceWrite : kJitPrice) | wk,
                         jit_price_bound(c, L, smem), L.w->walk, jk);
     if (s != PC_OK) return s;
     const void *kern = reinterpret_cast<const void *>(jk);
@@ -512,7 +553,7 @@ pc_status run_price(const pc_model *m, const pc_contract *k, uint64_t n_paths, u
     // a warp takes a tile, or a pair of tiles with two path pairs a lane
     const uint64_t units = (wk & kJitPairs2) ? (L.args.n_tiles + 1) / 2 : L.args.n_tiles;
     const int grid = int(std::min<uint64_t>(uint64_t(c->sm_count) * nb, (units + wpb - 1) / wpb));
-    L.args.one_pass = uint64_t(grid) * wpb >= units;
+    L.args.one_pass = !screened && uint64_t(grid) * wpb >= units;
     if (L.hbm_window) {
       // the HBM window holds a column per thread of this launch's grid
       L.grid = grid;
@@ -521,14 +562,15 @@ pc_status run_price(const pc_model *m, const pc_contract *k, uint64_t n_paths, u
     }
     void *args[] = {&L.args, &L.w->grid};
     CU(cudaLaunchKernel(kern, dim3(grid), dim3(L.block), args, smem, c->stream), "specialised price kernel");
-    return PC_OK;
+  } else {
+    if (L.hbm_window) {
+      s = bind_hbm_window(c, L, m->H.d);
+      if (s != PC_OK) return s;
+    }
+    L.args.one_pass = !screened && uint64_t(L.grid) * (L.block / 32) >= L.args.n_tiles;
+    CU(launch_price(L.args, L.grid, L.block, L.smem, c->stream), "price kernel");
   }
-  if (L.hbm_window) {
-    s = bind_hbm_window(c, L, m->H.d);
-    if (s != PC_OK) return s;
-  }
-  L.args.one_pass = uint64_t(L.grid) * (L.block / 32) >= L.args.n_tiles;
-  CU(launch_price(L.args, L.grid, L.block, L.smem, c->stream), "price kernel");
+  if (screened) CU(launch_totals(all, sc.payoffs, c->sm_count, c->stream), "totals kernel");
   return PC_OK;
 }
 
@@ -739,6 +781,7 @@ pc_status pc_destroy(pc_ctx *c) {
   if (c->d_control) cudaFree(c->d_control);
   if (c->d_gwin) cudaFree(c->d_gwin);
   if (c->d_tape) cudaFree(c->d_tape);
+  if (c->d_screen) cudaFree(c->d_screen);
   jit_release(c);
   if (c->d_gout) cudaFree(c->d_gout);
   if (c->d_res) cudaFree(c->d_res);
@@ -1122,6 +1165,11 @@ pc_status pc_jit_compile(const pc_model *m, const pc_contract *k) {
   cudaKernel_t jk = nullptr;
   const int wk = jit_window_kind(m->ctx, L);
   const size_t smem = jit_layout(m->ctx, L, wk);
+  Screen sc;
+  if (screen_suits(m, k, sc)) {  // large launches walk the listed paths with the per-path kernel
+    s = jit_kernel(k, jit_price_spec(m->ctx, k, L, kJitPriceWrite | wk, smem), jk);
+    if (s != PC_OK) return s;
+  }
   return jit_kernel(k, jit_price_spec(m->ctx, k, L, kJitPrice | wk, smem), jk);
 }
 

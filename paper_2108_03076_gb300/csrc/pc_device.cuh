@@ -623,6 +623,24 @@ __device__ __forceinline__ void gen_date(int t, PathState<D, H> &ps, const Model
 #endif
 
 #ifndef PC_JIT
+// The normals of op j on their own: its Philox blocks anew, one or two.
+template <int D>
+__device__ __forceinline__ void op_normals(uint32_t j, const Rng2 &g, float2 (&z)[1][D]) {
+  const uint32_t first = D * j;  // normals first .. first + D - 1
+  uint32_t blk = first >> 2;
+  float2 e[1][4];
+  block_normals_h<1>(blk, g, e);
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    if (((first + i) >> 2) != blk) {
+      blk = (first + i) >> 2;
+      block_normals_h<1>(blk, g, e);
+    }
+    const uint32_t w = (first + i) & 3;
+    z[0][i] = w == 0 ? e[0][0] : w == 1 ? e[0][1] : w == 2 ? e[0][2] : e[0][3];
+  }
+}
+
 // A path's start for an interpreted program that reads no date before t
 // (Layout::skip): the frontier straight to t.  From the interval that the
 // frontier opens (its right end from the by-date table) bisect while t lies
@@ -651,19 +669,8 @@ __device__ __noinline__ void skip_to(int t, PathState<D, 1> &ps, const PriceArgs
     while (t < r) {
       r = (ps.f + r) >> 1;
       const OpRegs op = load_op(m.nodes + r);
-      const uint32_t first = D * op.j;  // normals first .. first + D - 1
-      float2 z[1][D], e[1][4];
-      uint32_t blk = first >> 2;
-      block_normals_h<1>(blk, g, e);
-#pragma unroll
-      for (int i = 0; i < D; ++i) {
-        if (((first + i) >> 2) != blk) {
-          blk = (first + i) >> 2;
-          block_normals_h<1>(blk, g, e);
-        }
-        const uint32_t w = (first + i) & 3;
-        z[0][i] = w == 0 ? e[0][0] : w == 1 ? e[0][1] : w == 2 ? e[0][2] : e[0][3];
-      }
+      float2 z[1][D];
+      op_normals<D>(op.j, g, z);
       push_node<D, 1>(op, z, ps, lay, R);
     }
     pop_date<D, 1>(ps, lay, R);
@@ -1201,6 +1208,18 @@ __device__ __forceinline__ unsigned long long next_unit(const PriceArgs &a, int 
   unsigned long long u = 0;
   if (lane == 0) u = atomicAdd(reinterpret_cast<unsigned long long *>(a.control), 1ull);
   return __shfl_sync(kFull, u, 0);
+}
+
+// Paths to walk: all of the launch, or (per-path kernels only) the listed
+// ones of a screened launch.
+template <bool LIST>
+__device__ __forceinline__ uint64_t walk_paths(const PriceArgs &a) {
+  return LIST && a.list ? __ldcg(a.list_n) : a.n_paths;
+}
+// The i-th of them (i below their number, else any).
+template <bool LIST>
+__device__ __forceinline__ uint64_t walk_path(const PriceArgs &a, uint64_t i, bool live) {
+  return !(LIST && a.list) ? i : live ? __ldcg(a.list + i) : 0;
 }
 
 // The last block to exit re-zeroes the unit counter: no warp takes units any

@@ -84,6 +84,8 @@ struct pc_ctx {
   size_t tape_cap = 0;           // bytes
   float2 *d_gwin = nullptr;      // HBM windows of simulated dates (grow-only)
   size_t gwin_cap = 0;           // float2 slots
+  uint32_t *d_screen = nullptr;  // screened launches: count, list and payoffs (grow-only)
+  size_t screen_cap = 0;         // 4-byte words
   int32_t window_mode = 0;       // PC_WINDOW_AUTO / _SHARED / _HBM
   int32_t jit = 0;               // 1: price with run-time specialised kernels
   // streams and events of one-shot portfolio launches (pc_price_batch),

@@ -21,15 +21,20 @@ __device__ __forceinline__ void price_tiles(const PriceArgs &a, EVAL eval) {
   const int lane = threadIdx.x & 31;
   Rng2 g;
   rng_init(g, a.rk, a.stream, a.path_offset);
+  const uint64_t n = walk_paths<WRITE>(a), n_tiles = (n + kTilePaths - 1) / kTilePaths;
   for (;;) {
     const unsigned long long tile = next_unit(a, lane);
-    if (tile >= a.n_tiles) break;
+    if (tile >= n_tiles) break;
     const uint64_t i0 = tile * kTilePaths + lane, i1 = i0 + 32;
-    const bool live0 = i0 < a.n_paths, live1 = i1 < a.n_paths;
-    const uint64_t p0 = a.path_offset + i0, p1 = a.path_offset + i1;
-    rng_path(g, 0, p0, a.path_offset);
-    rng_path(g, 1, p1, a.path_offset);
+    const bool live0 = i0 < n, live1 = i1 < n;
+    rng_path(g, 0, a.path_offset + walk_path<WRITE>(a, i0, live0), a.path_offset);
+    rng_path(g, 1, a.path_offset + walk_path<WRITE>(a, i1, live1), a.path_offset);
     const float2 x = eval(P, pool, R, g, live0, live1, Bm, S0);
+    if (WRITE && a.list) {
+      if (live0) a.out_paths[walk_path<WRITE>(a, i0, true)] = x.x;
+      if (live1) a.out_paths[walk_path<WRITE>(a, i1, true)] = x.y;
+      continue;
+    }
     Moments<2> mo;
     if (live0) {
       mo.set(0, x.x);
@@ -66,7 +71,7 @@ __device__ __forceinline__ void price_tiles2(const PriceArgs &a, EVAL eval) {
   const float(&Bm)[D * D] = *reinterpret_cast<const float(*)[D * D]>(a.m.Bv);
   const float(&S0)[D] = *reinterpret_cast<const float(*)[D]>(a.m.S0v);
   const int lane = threadIdx.x & 31;
-  const uint64_t n_pairs = (a.n_tiles + 1) / 2;
+  const uint64_t n = walk_paths<WRITE>(a), n_tiles = (n + kTilePaths - 1) / kTilePaths, n_pairs = (n_tiles + 1) / 2;
   RngH<2> g;
   rng_init(g, a.rk, a.stream, a.path_offset);
   for (;;) {
@@ -77,14 +82,20 @@ __device__ __forceinline__ void price_tiles2(const PriceArgs &a, EVAL eval) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       idx[q] = (2 * u + (q >> 1)) * kTilePaths + lane + 32 * (q & 1);
-      live[q] = idx[q] < a.n_paths;
-      rng_path(g, q, a.path_offset + idx[q], a.path_offset);
+      live[q] = idx[q] < n;
+      rng_path(g, q, a.path_offset + walk_path<WRITE>(a, idx[q], live[q]), a.path_offset);
     }
     const PV x = eval(P, pool, R, g, live, Bm, S0);
+    if (WRITE && a.list) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (live[q]) a.out_paths[walk_path<WRITE>(a, idx[q], true)] = pv_get(x, q);
+      continue;
+    }
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const uint64_t tile = 2 * u + h;
-      if (tile >= a.n_tiles) break;  // warp-uniform
+      if (tile >= n_tiles) break;  // warp-uniform
       const float x0 = pv_get(x, 2 * h), x1 = pv_get(x, 2 * h + 1);
       Moments<2> mo;
       if (live[2 * h]) {

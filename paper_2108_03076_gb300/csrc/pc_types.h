@@ -231,6 +231,9 @@ struct PriceArgs {
   double *out;              // [width + 1]: sums over all paths, then n_paths
   float *out_paths;         // nullable: per-path payoffs (sensitivities: 3 floats per path)
   int32_t *status;          // device status word (nonzero = error)
+  // a screened launch (pc_screen.h): path numbers to walk and how many;
+  // their payoffs go to out_paths, the sums are left to the totals kernel
+  const uint32_t *list, *list_n;
   int32_t one_pass;         // 1: the grid has a warp for every unit of work (tile or pair of tiles)
   uint32_t ticket;          // blocking calls: written to *done with the status at the end
   uint64_t *done;           // pinned host word (null: not reported)
