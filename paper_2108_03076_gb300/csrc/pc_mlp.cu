@@ -191,6 +191,8 @@ __device__ __forceinline__ uint4 pack8(const float (&v)[8]) {
 }
 
 __global__ void to_bf16_kernel(const float *x, size_t n, int fin, __nv_bfloat16 *X, size_t rows) {
+  pdl_trigger();
+  pdl_wait();
   const size_t e = blockIdx.x * size_t(blockDim.x) + threadIdx.x;
   const size_t r = e >> 3;
   const int c0 = int(e & 7) * 8;
@@ -206,6 +208,8 @@ __global__ void to_bf16_kernel(const float *x, size_t n, int fin, __nv_bfloat16 
 __global__ void gather_kernel(const float *x, const float *t, size_t n_data, int fin, int fout,
                               const uint64_t *step, uint32_t s0, uint32_t s1, size_t batch,
                               __nv_bfloat16 *X, float *T) {
+  pdl_trigger();
+  pdl_wait();
   const size_t e = blockIdx.x * size_t(blockDim.x) + threadIdx.x;
   const size_t b = e >> 3;
   const int q = int(e & 7), c0 = q * 8;
@@ -226,6 +230,8 @@ __global__ void gather_kernel(const float *x, const float *t, size_t n_data, int
 // at a time so that their loads overlap.
 __global__ void loss_kernel(const float *Y, const float *T, const LossWeights w, size_t n, int fout,
                             size_t rows, __nv_bfloat16 *dY, float *part) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ float red[32];
   float acc = 0.f;
   const float inv = 1.f / float(n);
@@ -274,6 +280,8 @@ constexpr int kColChunk = 256, kColStride = 64 + 8;
 
 __global__ void __launch_bounds__(256) colsum_kernel(const __nv_bfloat16 *dZ, size_t rows, int ld, int cols,
                                                      float *scratch) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ __align__(16) __nv_bfloat16 s[kColChunk * kColStride];
   const int c0 = blockIdx.x * 64;
   const size_t r0 = size_t(blockIdx.y) * kColChunk;
@@ -330,6 +338,8 @@ __device__ __forceinline__ float ordered_sum(const float *p, int n, size_t strid
 // updated from the sum in hand and the gradient is not stored.
 template <bool ADAM>
 __global__ void __launch_bounds__(256) layer_grad_kernel(const LayerGrad g, const AdamStep a) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ float sh[256][33];
   size_t i;
   float s;
@@ -380,6 +390,8 @@ __global__ void __launch_bounds__(256) layer_grad_kernel(const LayerGrad g, cons
 // The block partials' total in FP64: 32 lanes' strided sums, then a fixed
 // shuffle tree (one thread's chain of dependent loads was 43 us for 512).
 __global__ void loss_total_kernel(const float *part, int blocks, double *loss, uint64_t *step) {
+  pdl_trigger();
+  pdl_wait();
   double s = 0.0;
 #pragma unroll 4
   for (int i = threadIdx.x; i < blocks; i += 32) s += double(part[i]);
@@ -390,6 +402,8 @@ __global__ void loss_total_kernel(const float *part, int blocks, double *loss, u
 }
 
 __global__ void unpad_kernel(const float *Y, int ldy, size_t n, int fout, float *y) {
+  pdl_trigger();
+  pdl_wait();
   const size_t e = blockIdx.x * size_t(blockDim.x) + threadIdx.x;
   if (e >= n * size_t(fout)) return;
   y[e] = Y[(e / fout) * ldy + e % fout];
@@ -444,29 +458,25 @@ cudaError_t launch_gather(const float *x, const float *t, size_t n_data, int fin
 int loss_blocks(size_t rows) { return int(grid_for(rows * kRow, 256, 512)); }
 
 cudaError_t launch_loss(const float *Y, int ldy, const float *T, const LossWeights &w, size_t n, int fout,
-                        size_t rows, __nv_bfloat16 *dY, int ldd, float *part, int blocks, cudaStream_t s) {
+                        size_t rows, __nv_bfloat16 *dY, int ldd, float *part, int blocks, cudaStream_t s, bool dep) {
   if (ldy != kRow || ldd != kRow) return cudaErrorInvalidValue;
-  loss_kernel<<<blocks, 256, 0, s>>>(Y, T, w, n, fout, rows, dY, part);
-  return cudaGetLastError();
+  return launch_chain(dep, loss_kernel, dim3(unsigned(blocks)), dim3(256), 0, s, Y, T, w, n, fout, rows, dY, part);
 }
 
-cudaError_t launch_colsum(const __nv_bfloat16 *dZ, size_t rows, int ld, int cols, float *scratch, cudaStream_t s) {
+cudaError_t launch_colsum(const __nv_bfloat16 *dZ, size_t rows, int ld, int cols, float *scratch, cudaStream_t s,
+                          bool dep) {
   if (cols % 64 || ld % 8) return cudaErrorInvalidValue;
   const unsigned chunks = unsigned((rows + kColChunk - 1) / kColChunk);
-  colsum_kernel<<<dim3(unsigned(cols / 64), chunks), 256, 0, s>>>(dZ, rows, ld, cols, scratch);
-  return cudaGetLastError();
+  return launch_chain(dep, colsum_kernel, dim3(unsigned(cols / 64), chunks), dim3(256), 0, s, dZ, rows, ld, cols, scratch);
 }
 
-cudaError_t launch_layer_grad(LayerGrad g, size_t rows, const AdamStep *adam, cudaStream_t s) {
+cudaError_t launch_layer_grad(LayerGrad g, size_t rows, const AdamStep *adam, cudaStream_t s, bool dep) {
   if (g.cols % 32) return cudaErrorInvalidValue;
   g.chunks = int((rows + kColChunk - 1) / kColChunk);
   g.w_blocks = unsigned((g.count + 255) / 256);
   const unsigned grid = g.w_blocks + unsigned(g.cols / 32);
-  if (adam)
-    layer_grad_kernel<true><<<grid, 256, 0, s>>>(g, *adam);
-  else
-    layer_grad_kernel<false><<<grid, 256, 0, s>>>(g, AdamStep{});
-  return cudaGetLastError();
+  if (adam) return launch_chain(dep, layer_grad_kernel<true>, dim3(grid), dim3(256), 0, s, g, *adam);
+  return launch_chain(dep, layer_grad_kernel<false>, dim3(grid), dim3(256), 0, s, g, AdamStep{});
 }
 
 cudaError_t launch_adam_consts(const uint64_t *step, float b1, float b2, float *consts, cudaStream_t s) {
@@ -474,15 +484,14 @@ cudaError_t launch_adam_consts(const uint64_t *step, float b1, float b2, float *
   return cudaGetLastError();
 }
 
-cudaError_t launch_loss_total(const float *part, int blocks, double *loss, uint64_t *step, cudaStream_t s) {
-  loss_total_kernel<<<1, 32, 0, s>>>(part, blocks, loss, step);
-  return cudaGetLastError();
+cudaError_t launch_loss_total(const float *part, int blocks, double *loss, uint64_t *step, cudaStream_t s,
+                              bool dep) {
+  return launch_chain(dep, loss_total_kernel, dim3(1), dim3(32), 0, s, part, blocks, loss, step);
 }
 
-cudaError_t launch_unpad(const float *Y, int ldy, size_t n, int fout, float *y, cudaStream_t s) {
+cudaError_t launch_unpad(const float *Y, int ldy, size_t n, int fout, float *y, cudaStream_t s, bool dep) {
   if (n == 0) return cudaSuccess;
-  unpad_kernel<<<unsigned((n * fout + 255) / 256), 256, 0, s>>>(Y, ldy, n, fout, y);
-  return cudaGetLastError();
+  return launch_chain(dep, unpad_kernel, dim3(unsigned((n * fout + 255) / 256)), dim3(256), 0, s, Y, ldy, n, fout, y);
 }
 
 }  // namespace pc

@@ -30,6 +30,32 @@ __device__ __forceinline__ float softplus_fast(float z) {
 }
 #endif
 
+// Dependent launches: a network call is a chain of short kernels, and a
+// kernel launched with `dep` (its stream's last work is another kernel of the
+// chain) starts while that one still runs: it sets itself up (barriers,
+// tensor memory, descriptors) and pdl_wait()s for its completion before its
+// first access to memory.  Every kernel of the chain waits, so a wait covers
+// all that came before.  The gradients of 65,536 rows (25 launches) went from
+// 342 to 322 us, a training step of 1,024 rows from 76.6 to 72.2 us.
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... KP, typename... A>
+cudaError_t launch_chain(bool dep, void (*k)(KP...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = dep ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k, KP(args)...);
+}
+#endif
+
 // GEMM epilogues of mlp_gemm.
 constexpr int kEpiBiasSoftplus = 0;  // Cb = bf16(softplus(acc + bias))
 constexpr int kEpiBias = 1;          // Cf = acc + bias (FP32)
@@ -76,7 +102,7 @@ bool make_tc_maps(GemmKind kind, const GemmArgs &g, TcMaps &m);
 // withhold: failure test (the producer withholds its first copies and the
 // bounded waits expire after about 10 ms)
 cudaError_t launch_gemm_tc(GemmKind kind, int epi, const GemmArgs &g, const TcMaps &m, int splits,
-                           int32_t *status, cudaStream_t s, bool withhold = false);
+                           int32_t *status, cudaStream_t s, bool withhold = false, bool dep = false);
 
 // The control variate's hedge tables in one launch (cv_tables_tc): per
 // 128-row tile, the network inputs of the table rows (cv_feature_row) go to
@@ -120,11 +146,12 @@ struct LossWeights {
 };
 cudaError_t launch_loss(const float *Y, int ldy, const float *T, const LossWeights &w, size_t n, int fout,
                         size_t rows, __nv_bfloat16 *dY, int ldd, float *part, int blocks,
-                        cudaStream_t s);
+                        cudaStream_t s, bool dep = false);
 int loss_blocks(size_t rows);
 // Column sums of dZ [rows, ld] (BF16), columns < cols (a multiple of 64), over
 // chunks of 256 rows in row order: scratch[chunk][cols].
-cudaError_t launch_colsum(const __nv_bfloat16 *dZ, size_t rows, int ld, int cols, float *scratch, cudaStream_t s);
+cudaError_t launch_colsum(const __nv_bfloat16 *dZ, size_t rows, int ld, int cols, float *scratch, cudaStream_t s,
+                          bool dep = false);
 // A layer's gradient from its partials: element i = sum_z part[z * count + i]
 // in order (z < splits; the weights, i < count = cols * in_w, row-major),
 // then the sums of colpart[chunk][c] in order (c < cols: the biases; a
@@ -152,12 +179,13 @@ struct AdamStep {
 };
 // rows: the batch's padded rows (the chunks of launch_colsum).  With adam,
 // out is not written.
-cudaError_t launch_layer_grad(LayerGrad g, size_t rows, const AdamStep *adam, cudaStream_t s);
+cudaError_t launch_layer_grad(LayerGrad g, size_t rows, const AdamStep *adam, cudaStream_t s, bool dep = false);
 // consts[0..1] = 1 - b1^t, 1 - b2^t for t = *step + 1 (in FP64, rounded).
 cudaError_t launch_adam_consts(const uint64_t *step, float b1, float b2, float *consts, cudaStream_t s);
 // Sum of part[0..blocks) into *loss (FP64, a fixed order); then ++*step if step.
-cudaError_t launch_loss_total(const float *part, int blocks, double *loss, uint64_t *step, cudaStream_t s);
+cudaError_t launch_loss_total(const float *part, int blocks, double *loss, uint64_t *step, cudaStream_t s,
+                              bool dep = false);
 // y [n, fout] FP32 from Y [rows, ldy].
-cudaError_t launch_unpad(const float *Y, int ldy, size_t n, int fout, float *y, cudaStream_t s);
+cudaError_t launch_unpad(const float *Y, int ldy, size_t n, int fout, float *y, cudaStream_t s, bool dep = false);
 
 }  // namespace pc

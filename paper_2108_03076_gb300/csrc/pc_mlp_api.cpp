@@ -198,7 +198,7 @@ GemmArgs gemm0() {
 // a.k_split on the warp-level kernel, tc_splits and tc_k_split on the tensor
 // cores); *used receives the split count of the path taken.
 cudaError_t product(pc_mlp *N, GemmKind kind, int epi, int layer, size_t rows, GemmArgs a, int splits,
-                    int tc_k_split, int tc_splits, cudaStream_t s, int *used = nullptr) {
+                    int tc_k_split, int tc_splits, cudaStream_t s, int *used = nullptr, bool dep = false) {
   if (used) *used = splits;
   if (N->tc_ok && N->gemm == PC_MLP_GEMM_AUTO) {
     GemmArgs t = a;
@@ -213,14 +213,14 @@ cudaError_t product(pc_mlp *N, GemmKind kind, int epi, int layer, size_t rows, G
       if (it != N->tc_maps.end()) {
         const int sp = kind == kGemmWeightGrad ? tc_splits : 1;
         if (used) *used = sp;
-        return launch_gemm_tc(kind, epi, t, it->second, sp, N->dstatus, s, N->tc_withhold);
+        return launch_gemm_tc(kind, epi, t, it->second, sp, N->dstatus, s, N->tc_withhold, dep);
       }
     }
   }
   return launch_gemm(kind, epi, a, splits, s);
 }
 
-// Forward over `rows` padded rows already in X.
+// Forward over `rows` padded rows already in X (written by the kernel before).
 cudaError_t forward(pc_mlp *N, size_t rows, cudaStream_t s) {
   for (int l = 0; l < N->L; ++l) {
     GemmArgs a = gemm0();
@@ -241,7 +241,7 @@ cudaError_t forward(pc_mlp *N, size_t rows, cudaStream_t s) {
     }
     a.ldc = N->wp[l + 1];
     const int epi = last ? kEpiBias : kEpiBiasSoftplus;
-    cudaError_t e = product(N, kGemmForward, epi, l, rows, a, 1, 0, 1, s);
+    cudaError_t e = product(N, kGemmForward, epi, l, rows, a, 1, 0, 1, s, nullptr, true);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -283,9 +283,10 @@ cudaError_t backward(pc_mlp *N, const float *t, const LossWeights &lw, size_t n,
   const int fout = N->w[N->L];
   const int lb = loss_blocks(rows);
   cudaError_t e = launch_loss(N->Y, N->wp[N->L], t, lw, n, fout, rows, N->dZ[0], N->wp[N->L],
-                              N->loss_part, lb, s);
+                              N->loss_part, lb, s, true);
   if (e != cudaSuccess) return e;
   const cudaStream_t sw = br ? br->w : s, sc = br ? br->c : s;
+  const bool dep = !br;  // one stream: each kernel follows another
   int cur = 0;
   for (int l = N->L - 1; l >= 0; --l) {
     const __nv_bfloat16 *in = l == 0 ? N->X : N->H[l - 1];
@@ -312,9 +313,9 @@ cudaError_t backward(pc_mlp *N, const float *t, const LossWeights &lw, size_t n,
     const int tc_splits = rows % 64 == 0 ? tc_grad_splits(N, out_w, in_w, rows, tc_ks) : 0;
     a.Cf = N->part[l & 1];
     a.ldc = in_w;
-    e = product(N, kGemmWeightGrad, kEpiPartial, l, rows, a, splits, tc_ks, tc_splits, sw, &splits);
+    e = product(N, kGemmWeightGrad, kEpiPartial, l, rows, a, splits, tc_ks, tc_splits, sw, &splits, dep);
     if (e != cudaSuccess) return e;
-    e = launch_colsum(N->dZ[cur], rows, out_w, out_w, N->colscr, sc);
+    e = launch_colsum(N->dZ[cur], rows, out_w, out_w, N->colscr, sc, dep);
     if (e == cudaSuccess && br) e = cudaEventRecord(br->colsum[l], sc);
     if (e == cudaSuccess && br) e = signal(br->wgrad[l], sw, sc);
     if (e != cudaSuccess) return e;
@@ -338,7 +339,8 @@ cudaError_t backward(pc_mlp *N, const float *t, const LossWeights &lw, size_t n,
       b.ldaux = in_w;
       b.Cb = N->dZ[cur ^ 1];
       b.ldc = in_w;
-      e = product(N, kGemmDataGrad, kEpiDSoftplus, l, rows, b, 1, 0, 1, s);
+      // (beside the branches only the first follows a kernel directly: the loss)
+      e = product(N, kGemmDataGrad, kEpiDSoftplus, l, rows, b, 1, 0, 1, s, nullptr, dep || l == N->L - 1);
       if (e != cudaSuccess) return e;
       if (br && (e = signal(br->dgrad[l], s, sc)) != cudaSuccess) return e;
       cur ^= 1;
@@ -362,7 +364,7 @@ cudaError_t backward(pc_mlp *N, const float *t, const LossWeights &lw, size_t n,
       step.v += o;
       step.pb += o;
     }
-    e = launch_layer_grad(lg, rows, adam ? &step : nullptr, sc);
+    e = launch_layer_grad(lg, rows, adam ? &step : nullptr, sc, dep);
     if (e == cudaSuccess && br) e = cudaEventRecord(br->sums[l], sc);
     if (e != cudaSuccess) return e;
   }
@@ -466,7 +468,7 @@ pc_status mlp_forward_on(pc_mlp *N, const float *d_x, size_t n, float *d_y, cuda
     const size_t nb = std::min(N->max_rows, n - b0), rows = rows_for(nb);
     CU(launch_to_bf16(d_x + b0 * N->w[0], nb, N->w[0], N->X, rows, N->wp[0], s), "input");
     CU(forward(N, rows, s), "forward");
-    CU(launch_unpad(N->Y, N->wp[N->L], nb, N->w[N->L], d_y + b0 * N->w[N->L], s), "output");
+    CU(launch_unpad(N->Y, N->wp[N->L], nb, N->w[N->L], d_y + b0 * N->w[N->L], s, true), "output");
   }
   return PC_OK;
 }
@@ -587,7 +589,7 @@ pc_status pc_mlp_gradients(pc_mlp *N, const float *d_x, const float *d_t, const 
   CU(launch_to_bf16(d_x, n, N->w[0], N->X, rows, N->wp[0], s), "input");
   CU(forward(N, rows, s), "forward");
   CU(backward(N, d_t, loss_weights(N, w), n, rows, s, d_grads ? d_grads : N->g), "backward");
-  CU(launch_loss_total(N->loss_part, loss_blocks(rows), N->loss, nullptr, s), "loss");
+  CU(launch_loss_total(N->loss_part, loss_blocks(rows), N->loss, nullptr, s, true), "loss");
   double loss = 0.0;
   const pc_status st = mlp_status(N, &loss);
   if (st == PC_OK) *out_loss = loss;

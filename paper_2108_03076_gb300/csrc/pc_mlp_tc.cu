@@ -293,6 +293,7 @@ __global__ void __launch_bounds__(tc_threads<BN>(), 1)
   const uint32_t tfull0 = su32(&bars[2 * kStages]), tempty0 = su32(&bars[2 * kStages + 2]);
   const uint32_t done = su32(&bars[2 * kStages + 4]);
   const uint32_t stage0 = base + kStages * kStageBytes;  // epilogue staging, kStageWarpBytes per warp
+  pdl_trigger();
   auto decode = [&](int t, int &z, int &m0, int &n0, int &c0, int &nk) {
     z = t / (tm * tn);
     const int r = t - z * tm * tn;
@@ -324,6 +325,7 @@ __global__ void __launch_bounds__(tc_threads<BN>(), 1)
 
   if (threadIdx.x == 0) {
     // TMA producer: chunk counter q runs across this CTA's tiles
+    pdl_wait();
     uint32_t q = 0, issued = 0;  // chunks issued: their copies land before exit
     for (int t = blockIdx.x; t < tiles && !*abort; t += gridDim.x) {
       int z, m0, n0, c0, nk;
@@ -402,6 +404,7 @@ __global__ void __launch_bounds__(tc_threads<BN>(), 1)
     // epilogue: warp w drains TMEM lanes 32 (w % 4) .. + 31 (rows of the
     // tile), columns 32 ((w - 4) / 4) .. + 31 of it
     const int qw = warp & 3, grp = (warp - 4) >> 2;
+    pdl_wait();
     int i = 0;
     for (int t = blockIdx.x; t < tiles && !*abort; t += gridDim.x, ++i) {
       int z, m0, n0, c0, nk;
@@ -751,12 +754,11 @@ int sm_count() {
 
 // Persistent grid: the tiles, at most one CTA per SM.
 template <int EPI, int BN, bool AMN, bool BMN>
-cudaError_t launch_tc(const CUtensorMap &ta, const CUtensorMap &tb, const TcArgs &a, cudaStream_t s) {
+cudaError_t launch_tc(const CUtensorMap &ta, const CUtensorMap &tb, const TcArgs &a, cudaStream_t s, bool dep) {
   const long long tiles = (long long)(a.N / BN) * ((a.M + kTcBM - 1) / kTcBM) * a.splits;
   const long long cap = (long long)sm_count();
   const unsigned grid = unsigned(tiles < cap ? tiles : cap);
-  mlp_gemm_tc<EPI, BN, AMN, BMN><<<grid, tc_threads<BN>(), tc_smem<BN>(), s>>>(ta, tb, a);
-  return cudaGetLastError();
+  return launch_chain(dep, mlp_gemm_tc<EPI, BN, AMN, BMN>, dim3(grid), dim3(tc_threads<BN>()), tc_smem<BN>(), s, ta, tb, a);
 }
 
 template <int EPI, bool AMN, bool BMN>
@@ -815,7 +817,7 @@ bool make_tc_maps(GemmKind kind, const GemmArgs &g, TcMaps &m) {
 }
 
 cudaError_t launch_gemm_tc(GemmKind kind, int epi, const GemmArgs &g, const TcMaps &m, int splits,
-                           int32_t *status, cudaStream_t s, bool withhold) {
+                           int32_t *status, cudaStream_t s, bool withhold, bool dep) {
   if (!status || !gemm_tc_supported(kind, g)) return cudaErrorInvalidValue;
   const bool ok_epi = kind == kGemmForward ? (epi == kEpiBiasSoftplus || epi == kEpiBias)
                       : kind == kGemmDataGrad ? epi == kEpiDSoftplus
@@ -847,16 +849,16 @@ cudaError_t launch_gemm_tc(GemmKind kind, int epi, const GemmArgs &g, const TcMa
   switch (kind) {
     case kGemmForward:
       if (epi == kEpiBiasSoftplus)
-        return n64 ? launch_tc<kEpiBiasSoftplus, 64, false, false>(m.a, m.b, a, s)
-                   : launch_tc<kEpiBiasSoftplus, 128, false, false>(m.a, m.b, a, s);
-      return n64 ? launch_tc<kEpiBias, 64, false, false>(m.a, m.b, a, s)
-                 : launch_tc<kEpiBias, 128, false, false>(m.a, m.b, a, s);
+        return n64 ? launch_tc<kEpiBiasSoftplus, 64, false, false>(m.a, m.b, a, s, dep)
+                   : launch_tc<kEpiBiasSoftplus, 128, false, false>(m.a, m.b, a, s, dep);
+      return n64 ? launch_tc<kEpiBias, 64, false, false>(m.a, m.b, a, s, dep)
+                 : launch_tc<kEpiBias, 128, false, false>(m.a, m.b, a, s, dep);
     case kGemmDataGrad:
-      return n64 ? launch_tc<kEpiDSoftplus, 64, false, true>(m.a, m.b, a, s)
-                 : launch_tc<kEpiDSoftplus, 128, false, true>(m.a, m.b, a, s);
+      return n64 ? launch_tc<kEpiDSoftplus, 64, false, true>(m.a, m.b, a, s, dep)
+                 : launch_tc<kEpiDSoftplus, 128, false, true>(m.a, m.b, a, s, dep);
     case kGemmWeightGrad:
-      return n64 ? launch_tc<kEpiPartial, 64, true, true>(m.a, m.b, a, s)
-                 : launch_tc<kEpiPartial, 128, true, true>(m.a, m.b, a, s);
+      return n64 ? launch_tc<kEpiPartial, 64, true, true>(m.a, m.b, a, s, dep)
+                 : launch_tc<kEpiPartial, 128, true, true>(m.a, m.b, a, s, dep);
   }
   return cudaErrorInvalidValue;
 }
