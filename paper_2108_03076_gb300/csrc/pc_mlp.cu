@@ -176,8 +176,7 @@ namespace {
 
 // Rows are padded to kRow = 64 columns (network inputs and outputs); a thread
 // takes eight columns of a row and stores them as 16 bytes.  (Indexing by
-// 64-bit division over single elements: 12.5 us for 65,536 rows; this: see
-// the launch list in profiles/.)
+// 64-bit division over single elements: 12.5 us for 65,536 rows; this 4.5.)
 constexpr int kRow = 64;
 
 __device__ __forceinline__ uint4 pack8(const float (&v)[8]) {
@@ -226,8 +225,10 @@ __global__ void gather_kernel(const float *x, const float *t, size_t n_data, int
 }
 
 // Weighted squared error; rows of kRow columns, thread (tid / 64, tid % 64)
-// of block k takes rows 4 k + tid / 64, + 4 gridDim, ... of its column, four
-// at a time so that their loads overlap.
+// of block k takes rows 4 k + tid / 64, + 4 gridDim, ... of its column, eight
+// at a time so that their loads overlap (65,536 rows: four at a time in 512
+// blocks 13.4 us, eight in kLossBlocks 10.6).
+constexpr int kLossAhead = 8;
 __global__ void loss_kernel(const float *Y, const float *T, const LossWeights w, size_t n, int fout,
                             size_t rows, __nv_bfloat16 *dY, float *part) {
   pdl_trigger();
@@ -239,17 +240,17 @@ __global__ void loss_kernel(const float *Y, const float *T, const LossWeights w,
   const size_t step = size_t(gridDim.x) * (blockDim.x / kRow);
   const bool col = c < fout;
   const float wc = w.w[c];
-  for (size_t r0 = blockIdx.x * size_t(blockDim.x / kRow) + threadIdx.x / kRow; r0 < rows; r0 += 4 * step) {
-    float y[4], t[4];
+  for (size_t r0 = blockIdx.x * size_t(blockDim.x / kRow) + threadIdx.x / kRow; r0 < rows; r0 += kLossAhead * step) {
+    float y[kLossAhead], t[kLossAhead];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < kLossAhead; ++i) {
       const size_t r = r0 + size_t(i) * step;
       const bool in = col && r < n;
       y[i] = in ? Y[r * kRow + c] : 0.f;
       t[i] = in ? T[r * fout + c] : 0.f;
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < kLossAhead; ++i) {
       const size_t r = r0 + size_t(i) * step;
       if (r >= rows) break;
       float g = 0.f;
@@ -274,9 +275,10 @@ __global__ void loss_kernel(const float *Y, const float *T, const LossWeights w,
 // Column sums of dZ over chunks of kColChunk rows, in row order: a block
 // brings its chunk's 64 columns to shared memory with every load in flight,
 // then one thread a column adds the rows (a thread a column straight from
-// memory waited on each of its 256 loads: 24 us whatever the row count; the
-// chunk's chain of 256 additions is the floor, about 0.6 us).
-constexpr int kColChunk = 256, kColStride = 64 + 8;
+// memory waited on each of its 256 loads: 24 us whatever the row count; this
+// 4.6 us for 1,024 rows of 256 columns and 11 for 65,536.  The chunk's chain
+// of 256 additions takes about 0.6).
+constexpr int kColChunk = 256, kColStride = 64;
 
 __global__ void __launch_bounds__(256) colsum_kernel(const __nv_bfloat16 *dZ, size_t rows, int ld, int cols,
                                                      float *scratch) {
@@ -393,8 +395,13 @@ __global__ void loss_total_kernel(const float *part, int blocks, double *loss, u
   pdl_trigger();
   pdl_wait();
   double s = 0.0;
-#pragma unroll 4
-  for (int i = threadIdx.x; i < blocks; i += 32) s += double(part[i]);
+  for (int i = threadIdx.x; i < blocks; i += 32 * 8) {
+    float v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = i + 32 * u < blocks ? part[i + 32 * u] : 0.f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) s += double(v[u]);
+  }
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (threadIdx.x != 0) return;
   *loss = s;
@@ -455,7 +462,7 @@ cudaError_t launch_gather(const float *x, const float *t, size_t n_data, int fin
   return cudaGetLastError();
 }
 
-int loss_blocks(size_t rows) { return int(grid_for(rows * kRow, 256, 512)); }
+int loss_blocks(size_t rows) { return int(grid_for(rows * kRow, 256, kLossBlocks)); }
 
 cudaError_t launch_loss(const float *Y, int ldy, const float *T, const LossWeights &w, size_t n, int fout,
                         size_t rows, __nv_bfloat16 *dY, int ldd, float *part, int blocks, cudaStream_t s, bool dep) {

@@ -28,6 +28,53 @@ __device__ __forceinline__ float softplus_fast(float z) {
   p = fmaf(p, u, 0.9999987483024597f);
   return fmaxf(z, 0.f) + u * p;
 }
+
+// Two FP32 values a register pair and their packed operations (each half
+// rounded as the scalar operation): half the issue slots of an epilogue.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pair(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpair(f32x2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 both(float a) { return pair(a, a); }
+
+// softplus_fast of z.x and z.y (the same operations and roundings).
+__device__ __forceinline__ float2 softplus_pair(f32x2 z2) {
+  const float2 z = unpair(z2);
+  float u0, u1;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(u0) : "f"(-1.4426950408889634f * fabsf(z.x)));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(u1) : "f"(-1.4426950408889634f * fabsf(z.y)));
+  const f32x2 u = pair(u0, u1);
+  f32x2 p = both(0.014202825725078583f);
+  p = fma2(p, u, both(-0.06658805161714554f));
+  p = fma2(p, u, both(0.14943458139896393f));
+  p = fma2(p, u, both(-0.23514863848686218f));
+  p = fma2(p, u, both(0.3311205208301544f));
+  p = fma2(p, u, both(-0.4998719096183777f));
+  p = fma2(p, u, both(0.9999987483024597f));
+  return unpair(fma2(u, p, pair(fmaxf(z.x, 0.f), fmaxf(z.y, 0.f))));
+}
 #endif
 
 // Dependent launches: a network call is a chain of short kernels, and a
@@ -147,6 +194,7 @@ struct LossWeights {
 cudaError_t launch_loss(const float *Y, int ldy, const float *T, const LossWeights &w, size_t n, int fout,
                         size_t rows, __nv_bfloat16 *dY, int ldd, float *part, int blocks,
                         cudaStream_t s, bool dep = false);
+constexpr int kLossBlocks = 1024;  // most loss partials
 int loss_blocks(size_t rows);
 // Column sums of dZ [rows, ld] (BF16), columns < cols (a multiple of 64), over
 // chunks of 256 rows in row order: scratch[chunk][cols].

@@ -179,7 +179,7 @@ size_t layout(pc_mlp *N, size_t rows) {
   for (float *&q : N->part) q = c.take<float>(part);
   N->colscr = c.take<float>(chunks * widest);
   N->adam_c = c.take<float>(2);
-  N->loss_part = c.take<float>(512);
+  N->loss_part = c.take<float>(kLossBlocks);
   N->loss = c.take<double>(2);  // the loss, then the products' status word
   N->step = c.take<uint64_t>(1);
   N->dstatus = reinterpret_cast<int32_t *>(N->loss + 1);
