@@ -240,7 +240,7 @@ int pick_block(const Program &p, int words, int max_smem, int d, size_t &smem, b
   for (int b = kBlock; b >= 32; b /= 2) {
     const size_t sm = price_smem_bytes(p.code.size(), pool_padded(p), words, b);
     if (sm + kStaticSmemReserve > size_t(max_smem)) continue;
-    const int warps = price_blocks_per_sm(d, b, sm, false, memoise) * (b / 32);
+    const int warps = price_blocks_per_sm(d, b, sm, kPriceShared, memoise) * (b / 32);
     if (warps > best_warps) {
       best = b;
       best_warps = warps;
@@ -269,7 +269,7 @@ pc_status prepare(const pc_model *m, const pc_contract *k, uint64_t n_paths, uin
   bool hbm = mode == PC_WINDOW_HBM;
   if (!hbm) {
     L.block = win <= PC_MAX_WINDOW ? pick_block(k->prog, lay.words, c->max_smem, m->H.d, L.smem) : 0;
-    bpsm = L.block ? price_blocks_per_sm(m->H.d, L.block, L.smem, false) : 0;
+    bpsm = L.block ? price_blocks_per_sm(m->H.d, L.block, L.smem, kPriceShared) : 0;
     const int warps = bpsm * L.block / 32;
     if (mode == PC_WINDOW_AUTO && (!L.block || warps < 8)) hbm = true;
   }
@@ -284,7 +284,7 @@ pc_status prepare(const pc_model *m, const pc_contract *k, uint64_t n_paths, uin
       L.block = 32;
       L.smem = price_smem_bytes(k->prog.code.size(), pool_padded(k->prog), lay.words, L.block);
     }
-    bpsm = price_blocks_per_sm(m->H.d, L.block, L.smem, true);
+    bpsm = price_blocks_per_sm(m->H.d, L.block, L.smem, kPriceHbm);
     L.hbm_window = true;
   } else if (!L.block) {
     if (win > PC_MAX_WINDOW)
@@ -313,6 +313,13 @@ pc_status prepare(const pc_model *m, const pc_contract *k, uint64_t n_paths, uin
   const uint64_t warps_per_block = uint64_t(L.block) / 32;
   const uint64_t need = (n_tiles + warps_per_block - 1) / warps_per_block;
   L.grid = int(std::min<uint64_t>(uint64_t(c->sm_count) * bpsm, need));
+  if (L.hbm_window && m->H.d == 2) {
+    const int dense = price_blocks_per_sm(2, L.block, L.smem, kPriceHbmDense);
+    if (need > uint64_t(L.grid) && need <= uint64_t(c->sm_count) * dense) {
+      L.sparse_grid = L.grid;
+      L.grid = int(need);
+    }
+  }
   return PC_OK;
 }
 
@@ -565,10 +572,16 @@ pc_status run_price(const pc_model *m, const pc_contract *k, uint64_t n_paths, u
   } else {
     if (L.hbm_window) {
       s = bind_hbm_window(c, L, m->H.d);
+      if (s == PC_ENOMEM && L.sparse_grid) {  // no memory for the dense variant's window
+        cudaGetLastError();
+        L.grid = L.sparse_grid;
+        L.sparse_grid = 0;
+        s = bind_hbm_window(c, L, m->H.d);
+      }
       if (s != PC_OK) return s;
     }
     L.args.one_pass = !screened && uint64_t(L.grid) * (L.block / 32) >= L.args.n_tiles;
-    CU(launch_price(L.args, L.grid, L.block, L.smem, c->stream), "price kernel");
+    CU(launch_price(L.args, L.grid, L.block, L.smem, c->stream, L.sparse_grid != 0), "price kernel");
   }
   if (screened) CU(launch_totals(all, sc.payoffs, c->sm_count, c->stream), "totals kernel");
   return PC_OK;
@@ -635,7 +648,7 @@ pc_status pc_price_noalloc(const pc_model *m, const pc_contract *k, uint64_t n_p
   const uint64_t n_tiles = (n_paths + kTilePaths - 1) / kTilePaths;
   if (kNoAllocCounterBytes + n_tiles * 2 * sizeof(double) > scratch_bytes)
     return fail(PC_ELIMIT, "request exceeds the fixed scratch array");
-  const int bpsm = price_blocks_per_sm(H.d, block, smem, false, false);
+  const int bpsm = price_blocks_per_sm(H.d, block, smem, kPriceShared, false);
   if (bpsm < 1) return fail(PC_ELIMIT, "kernel cannot be resident with this shared-memory footprint");
   PriceArgs a{};
   a.prog = k->d_code;

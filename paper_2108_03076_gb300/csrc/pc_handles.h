@@ -207,6 +207,7 @@ struct Launch {
   size_t smem = 0;
   pc_contract::Window *w = nullptr;  // the contract on the model: its static walks and kernels
   bool hbm_window = false;  // window in HBM (args.lay.gwin set by the launcher)
+  int sparse_grid = 0;      // the dense variant's launch (PriceKind): the grid without it, else 0
 };
 
 // Validate (model, contract, n_paths), resolve the contract's date window for

@@ -14,7 +14,15 @@
 
 namespace pc {
 // Kernel launchers (pc_kernels.cu).  All return a cudaError_t.
-cudaError_t launch_price(const PriceArgs &a, int grid, int block, size_t smem_bytes, cudaStream_t s);
+// The interpreting kernel's variants: the window of dates in shared memory or
+// in HBM, and for two underlyings the latter at seven blocks an SM (72
+// registers) instead of six.  Seven cost 2-9 % a tile (300 dates newest
+// first, 1,024 tiles: 417 -> 455 us; 4,688 tiles of 200: 608 -> 625; 16,384
+// of 30: 233 -> 243), and are taken where they hold every tile at once and
+// six do not: 4,096 tiles of 300 dates, 1.12 rounds of six blocks, 867 -> 680
+// us; of 50 dates 149 -> 124.
+enum PriceKind { kPriceShared = 0, kPriceHbm = 1, kPriceHbmDense = 2 };
+cudaError_t launch_price(const PriceArgs &a, int grid, int block, size_t smem_bytes, cudaStream_t s, bool dense = false);
 cudaError_t launch_greeks(const PriceArgs &a, int grid, int block, size_t smem_bytes, cudaStream_t s);
 int greeks_blocks_per_sm(int d, int block, size_t smem_bytes);
 cudaError_t launch_debug_philox(const uint32_t *ctr, uint32_t k0, uint32_t k1, uint32_t *out,
@@ -22,7 +30,7 @@ cudaError_t launch_debug_philox(const uint32_t *ctr, uint32_t k0, uint32_t k1, u
 cudaError_t launch_debug_paths(const ModelDev &m, const Layout &lay, uint64_t n_paths,
                                uint64_t offset, uint32_t k0, uint32_t k1, uint32_t stream,
                                float *out, cudaStream_t s);
-int price_blocks_per_sm(int d, int block, size_t smem_bytes, bool hbm_window, bool memoise = true);
+int price_blocks_per_sm(int d, int block, size_t smem_bytes, PriceKind kind, bool memoise = true);
 
 // Portfolio pricing (one persistent launch per group of contracts with the
 // same underlying count and a similar per-path footprint).  A work unit is a

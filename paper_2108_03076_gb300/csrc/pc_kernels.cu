@@ -31,8 +31,8 @@ namespace {
 // (price_tiles, pc_price.cuh).  GW: the window of simulated dates lives in
 // HBM (lay.gwin) instead of shared memory, for programs that look back
 // further than shared memory holds.
-template <int D, bool WRITE, bool GW = false>
-__global__ void __launch_bounds__(kBlock, D == 1 ? 7 : D == 2 ? 6 : 5) price_kernel(const __grid_constant__ PriceArgs a) {
+template <int D, bool WRITE, bool GW = false, bool DENSE = false>
+__global__ void __launch_bounds__(kBlock, D == 1 ? 7 : D == 2 ? (DENSE ? 7 : 6) : 5) price_kernel(const __grid_constant__ PriceArgs a) {
   price_tiles<D, WRITE>(a, [&](const uint4 *P, const float *pool, float2 *R, const Rng2 &g, bool live0,
                                bool live1, const float(&Bm)[D * D], const float(&S0)[D]) {
     return eval_path<D, GW>(P, pool, R, a, g, live0, live1, Bm, S0);
@@ -178,11 +178,11 @@ cudaError_t set_smem(K kern, size_t smem) {
 
 }  // namespace
 
-cudaError_t launch_price(const PriceArgs &a, int grid, int block, size_t smem, cudaStream_t s) {
+cudaError_t launch_price(const PriceArgs &a, int grid, int block, size_t smem, cudaStream_t s, bool dense) {
   const bool w = a.out_paths != nullptr, gw = a.lay.gwin != nullptr;
-#define LAUNCH(DD, WW, GG)                                                         \
+#define LAUNCH(DD, WW, ...)                                                        \
   do {                                                                             \
-    auto k = price_kernel<DD, WW, GG>;                                             \
+    auto k = price_kernel<DD, WW, __VA_ARGS__>;                                    \
     cudaError_t e = set_smem(k, smem);                                             \
     if (e != cudaSuccess) return e;                                                \
     k<<<grid, block, smem, s>>>(a);                                                \
@@ -195,7 +195,9 @@ cudaError_t launch_price(const PriceArgs &a, int grid, int block, size_t smem, c
   } while (0)
   switch (a.m.d) {
     case 1: LAUNCH_D(1);
-    case 2: LAUNCH_D(2);
+    case 2:
+      if (gw && dense) { if (w) LAUNCH(2, true, true, true); else LAUNCH(2, false, true, true); }
+      LAUNCH_D(2);
     case 3: LAUNCH_D(3);
     case 4: LAUNCH_D(4);
     default: return cudaErrorInvalidValue;
@@ -207,18 +209,20 @@ cudaError_t launch_price(const PriceArgs &a, int grid, int block, size_t smem, c
 namespace {
 int price_occupancy(uint64_t v, int block, size_t smem) {
   const int d = int(v & 0xff);
-  const bool hbm_window = (v >> 8) & 1;
+  const PriceKind kind = PriceKind((v >> 8) & 3);
   int nb = 0;
   cudaError_t e = cudaSuccess;
+#define OCC_K(...)                                                                                   \
+  do {                                                                                               \
+    auto k = price_kernel<__VA_ARGS__>;                                                              \
+    set_smem(k, smem);                                                                               \
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, block, smem);                          \
+  } while (0)
 #define OCC(DD)                                                                                      \
   do {                                                                                               \
-    if (hbm_window) {                                                                                \
-      set_smem(price_kernel<DD, false, true>, smem);                                                 \
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, price_kernel<DD, false, true>, block, smem); \
-    } else {                                                                                         \
-      set_smem(price_kernel<DD, false, false>, smem);                                                \
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, price_kernel<DD, false, false>, block, smem); \
-    }                                                                                                \
+    if (kind == kPriceHbmDense) OCC_K(DD, false, true, DD == 2);                                     \
+    else if (kind == kPriceHbm) OCC_K(DD, false, true);                                              \
+    else OCC_K(DD, false, false);                                                                    \
   } while (0)
   switch (d) {
     case 0:
@@ -232,12 +236,13 @@ int price_occupancy(uint64_t v, int block, size_t smem) {
     default: return 0;
   }
 #undef OCC
+#undef OCC_K
   return e == cudaSuccess ? nb : 0;
 }
 }  // namespace
 
-int price_blocks_per_sm(int d, int block, size_t smem, bool hbm_window, bool memoise) {
-  return occupancy_memo((uint64_t(1) << 32) | (uint64_t(hbm_window) << 8) | uint64_t(d), block, smem,
+int price_blocks_per_sm(int d, int block, size_t smem, PriceKind kind, bool memoise) {
+  return occupancy_memo((uint64_t(1) << 32) | (uint64_t(kind) << 8) | uint64_t(d), block, smem,
                         price_occupancy, memoise);
 }
 
