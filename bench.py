@@ -514,7 +514,7 @@ def main():
             "contracts_per_sec_at_1e-4_rel_se": contracts_per_s,
             "price": mean, "stderr": math.sqrt(var / w.n_paths),
             "paths_for_1e-4_rel_se": paths_needed,
-            "gpu_launches": args.steps,
+            "gpu_launches": args.steps * pc.pc_debug_price_kernels(model, contract, w.n_paths),
             "e2e": {"value": e2e_value, "unit": UNIT,
                     "h2d_bytes_per_step": int(words.nbytes + consts.nbytes + 4 * len(w.tparams)),
                     "d2h_bytes_per_step": 40,

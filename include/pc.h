@@ -367,9 +367,11 @@ pc_status pc_price_info(const pc_model *model, const pc_contract *contract, uint
 /* The paper compiles each contract into its own payoff function (Sec. 6).
  * With pc_set_jit(ctx, 1), pc_price / pc_price_async / pc_price_paths run a
  * kernel specialised to the contract's executable program (compiled at run
- * time by NVRTC on first use for each underlying count, cached on the
- * context by program content -- reloading the same program reuses it --
- * and freed by pc_destroy): the same operations in the same order as the
+ * time by NVRTC on first use, cached on the context by program content --
+ * reloading the same program reuses it -- and freed by pc_destroy; one
+ * kernel per underlying count, or, where the bridge has few nodes that the
+ * program needs (at most 16), one per date grid's walk, up to 8 walks a
+ * program, the rest sharing the general kernel): the same operations in the same order as the
  * interpreting kernel, without the per-instruction dispatch, with the
  * window of dates in shared memory or in HBM as the launch places it.
  * pc_price_cv and pc_greeks likewise run specialised control-variate and
@@ -380,7 +382,8 @@ pc_status pc_price_info(const pc_model *model, const pc_contract *contract, uint
 #define PC_JIT_MAX_INSNS 384
 pc_status pc_set_jit(pc_ctx *ctx, int32_t enabled);
 /* Compile (now) the contract's specialised kernel for the model's
- * underlying count (shared-memory window, pooled sums); does nothing for a
+ * underlying count and walk, and for a program whose large launches are
+ * screened the per-path kernel that walks the remaining paths; does nothing for a
  * program beyond PC_JIT_MAX_INSNS instructions.  Blocks; typically tens
  * of milliseconds to a few seconds.
  * Errors: PC_EINVAL, PC_ECUDA (the compiler's log in pc_last_error). */
@@ -736,6 +739,13 @@ pc_status pc_debug_set_status(pc_ctx *ctx, int32_t value);
  * per-path values and sums are the same either way; the kernels are cached
  * per choice.  Errors: PC_EINVAL. */
 pc_status pc_debug_set_jit_pairs(pc_ctx *ctx, int32_t pairs);
+
+/* Kernels that one pc_price / pc_price_async / pc_price_paths call of n_paths
+ * launches: 1, or 3 where a daily barrier's decided paths are screened out
+ * before the walk (the screen, the walk over the paths left, the totals).
+ * Errors: PC_EINVAL, those of pc_price_info. */
+pc_status pc_debug_price_kernels(const pc_model *model, const pc_contract *contract, uint64_t n_paths,
+                                 int32_t *out_kernels);
 
 /* Resident 128-thread blocks per SM the register bound of the context's
  * specialised control-variate kernels is set for (1..16), or 0 for the

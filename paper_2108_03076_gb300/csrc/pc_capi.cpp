@@ -323,19 +323,40 @@ pc_status prepare(const pc_model *m, const pc_contract *k, uint64_t n_paths, uin
   return PC_OK;
 }
 
+// The caller is capturing the context's stream.
+bool capturing(const pc_ctx *c) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(c->stream, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone;
+}
+
+// Frees a buffer about to grow, or keeps it for the graphs that hold it.
+void drop_buffer(pc_ctx *c, void *p, bool &held) {
+  if (held && p)
+    c->captured.push_back(p);
+  else if (p)
+    cudaFree(p);
+  held = false;
+}
+
 // Point the launch's window at the context's HBM window buffer (grown to
 // grid * block threads x win * d slots).
 pc_status bind_hbm_window(pc_ctx *c, Launch &L, int d) {
-  const size_t threads = size_t(L.grid) * size_t(L.block);
-  const size_t slots = threads * size_t(L.args.lay.win) * size_t(d);
+  const bool cap = capturing(c);
+  const auto slots_of = [&](int grid) { return size_t(grid) * size_t(L.block) * size_t(L.args.lay.win) * size_t(d); };
+  if (cap && L.sparse_grid && slots_of(L.grid) > c->gwin_cap) {  // no growing under capture
+    L.grid = L.sparse_grid;
+    L.sparse_grid = 0;
+  }
+  const size_t threads = size_t(L.grid) * size_t(L.block), slots = slots_of(L.grid);
   if (slots > c->gwin_cap) {
     CU(cudaStreamSynchronize(c->stream), "sync");
-    if (c->d_gwin) cudaFree(c->d_gwin);
+    drop_buffer(c, c->d_gwin, c->gwin_captured);
     c->d_gwin = nullptr;
     c->gwin_cap = 0;
     CU(ctx_malloc(c, reinterpret_cast<void **>(&c->d_gwin), slots * sizeof(float2)), "HBM window");
     c->gwin_cap = slots;
   }
+  if (cap) c->gwin_captured = true;
   L.args.lay.gwin = c->d_gwin;
   L.args.lay.gstride = int64_t(threads);
   return PC_OK;
@@ -494,16 +515,21 @@ bool screen_suits(const pc_model *m, const pc_contract *k, Screen &s) {
   return screen_program(k->prog, m->H, s) && screen_fraction(m->H, s) >= kScreenFraction;
 }
 
+bool screen_large(const pc_model *m, uint64_t n_paths) {
+  return n_paths <= kScreenPaths && double(n_paths) * m->H.n * m->H.d >= kScreenWork;
+}
+
 // Sets up a screened launch where it pays: the context's list and payoff
-// buffers (grown here; no memory for them: unscreened).  `payoffs`: the
+// buffers (grown here; no memory for them, or the stream is being captured:
+// unscreened).  `payoffs`: the
 // caller's per-path payoffs, else the context's.
 bool screen_launch(pc_ctx *c, const pc_model *m, const pc_contract *k, const PriceArgs &a, float *payoffs, Screen &s) {
-  if (a.n_paths > kScreenPaths || double(a.n_paths) * m->H.n * m->H.d < kScreenWork) return false;
-  if (!screen_suits(m, k, s)) return false;
+  if (!screen_large(m, a.n_paths) || !screen_suits(m, k, s)) return false;
   const size_t words = 64 + size_t(a.n_paths) * (payoffs ? 1 : 2);
+  const bool cap = capturing(c);
   if (words > c->screen_cap) {
-    if (cudaStreamSynchronize(c->stream) != cudaSuccess) return false;
-    if (c->d_screen) cudaFree(c->d_screen);
+    if (cap || cudaStreamSynchronize(c->stream) != cudaSuccess) return false;
+    drop_buffer(c, c->d_screen, c->screen_captured);
     c->d_screen = nullptr;
     c->screen_cap = 0;
     if (ctx_malloc(c, reinterpret_cast<void **>(&c->d_screen), words * 4) != cudaSuccess) {
@@ -512,6 +538,7 @@ bool screen_launch(pc_ctx *c, const pc_model *m, const pc_contract *k, const Pri
     }
     c->screen_cap = words;
   }
+  if (cap) c->screen_captured = true;
   s.count = c->d_screen;
   s.list = c->d_screen + 64;
   s.payoffs = payoffs ? payoffs : reinterpret_cast<float *>(c->d_screen + 64 + a.n_paths);
@@ -795,6 +822,7 @@ pc_status pc_destroy(pc_ctx *c) {
   if (c->d_gwin) cudaFree(c->d_gwin);
   if (c->d_tape) cudaFree(c->d_tape);
   if (c->d_screen) cudaFree(c->d_screen);
+  for (void *p : c->captured) cudaFree(p);
   jit_release(c);
   if (c->d_gout) cudaFree(c->d_gout);
   if (c->d_res) cudaFree(c->d_res);
@@ -1141,6 +1169,16 @@ pc_status pc_set_window_mode(pc_ctx *c, int32_t mode) {
   if (mode != PC_WINDOW_AUTO && mode != PC_WINDOW_SHARED && mode != PC_WINDOW_HBM)
     return fail(PC_EINVAL, "window mode must be PC_WINDOW_AUTO, _SHARED or _HBM");
   c->window_mode = mode;
+  return PC_OK;
+}
+
+pc_status pc_debug_price_kernels(const pc_model *m, const pc_contract *k, uint64_t n_paths, int32_t *out_kernels) {
+  if (!out_kernels) return fail(PC_EINVAL, "null output");
+  Launch L;
+  pc_status s = prepare(m, k, n_paths, 0, 0, 0, L, true);
+  if (s != PC_OK) return s;
+  Screen sc;
+  *out_kernels = screen_large(m, n_paths) && screen_suits(m, k, sc) ? 3 : 1;
   return PC_OK;
 }
 

@@ -86,6 +86,10 @@ struct pc_ctx {
   size_t gwin_cap = 0;           // float2 slots
   uint32_t *d_screen = nullptr;  // screened launches: count, list and payoffs (grow-only)
   size_t screen_cap = 0;         // 4-byte words
+  // a caller's stream capture holds the buffer's address: when it grows, the
+  // old one is kept until the context goes
+  bool screen_captured = false, gwin_captured = false;
+  std::vector<void *> captured;
   int32_t window_mode = 0;       // PC_WINDOW_AUTO / _SHARED / _HBM
   int32_t jit = 0;               // 1: price with run-time specialised kernels
   // streams and events of one-shot portfolio launches (pc_price_batch),

@@ -7,10 +7,10 @@
 //   -> the payoff expression (IL of Sec. 3, semantics of Fig. 3) run by a
 //   warp-uniform stack machine -> per-tile FP64 sums.
 // No path value is written to global memory.  Per-thread state (operand
-// stack, loop frames, bridge stack, per-level Philox block caches, the
-// window of recent dates) lives in shared memory as word-interleaved slots:
-// word w of thread t is at region[w * kBlock + t], so the warp-uniform slot
-// indices of the interpreter give conflict-free accesses.
+// stack, loop frames, bridge stack, the window of recent dates) lives in
+// shared memory in a region per warp: slot s of lane l is at region[32 s + l],
+// so the warp-uniform slot indices of the interpreter give conflict-free
+// accesses at a constant stride.
 #include <cstdint>
 #include <map>
 #include <mutex>

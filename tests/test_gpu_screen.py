@@ -78,3 +78,38 @@ def test_screened_equals_unscreened(ctx, case):
         pc.pc_contract_destroy(k)
         pc.pc_model_destroy(m)
 
+
+
+def test_captured_launches_keep_their_buffers(ctx):
+    """A screened launch captured on the caller's stream replays right after a
+    larger call has grown the context's screen buffers; a capture that would
+    have to grow them runs unscreened."""
+    text, tp, n, _ = CASES["knock_out_either"]
+    m = pc.pc_model_create(ctx, [1.0, 1.02], [0.28, 0.2], [[1.0, 0.4], [0.4, 1.0]], 0.02, list(range(1, n + 1)), 0, None, None)
+    w, c = pc.pc_assemble(text)
+    k = pc.pc_load_payoff(ctx, w, c, tp)
+    small, large = 300_000, 600_000  # both screened, the partials of either fit from the start
+    try:
+        out = torch.zeros(3, 4, dtype=torch.float64, device="cuda")
+        ref = torch.zeros(2, 4, dtype=torch.float64, device="cuda")
+        for i, paths in enumerate((small, large)):
+            pc.pc_price_noalloc(m, k, paths, 0, 99, 0, ref[i].data_ptr())
+        pc.pc_price_async(m, k, 100, 0, 99, 0, out[0].data_ptr())     # (the unscreened kernel is loaded)
+        pc.pc_price_async(m, k, small, 0, 99, 0, out[0].data_ptr())
+        torch.cuda.synchronize()
+        graphs = []
+        for i, paths in enumerate((small, large)):
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=torch.cuda.current_stream()):
+                pc.pc_price_async(m, k, paths, 0, 99, 0, out[i].data_ptr())
+            graphs.append(g)
+        pc.pc_price_async(m, k, large, 0, 99, 0, out[2].data_ptr())   # grows the buffers
+        out[:2].zero_()
+        for g in graphs:
+            g.replay()
+        torch.cuda.synchronize()
+        np.testing.assert_array_equal(out[:2, :3].cpu().numpy(), ref[:, :3].cpu().numpy())
+        np.testing.assert_array_equal(out[2, :3].cpu().numpy(), ref[1, :3].cpu().numpy())
+    finally:
+        pc.pc_contract_destroy(k)
+        pc.pc_model_destroy(m)
