@@ -482,6 +482,7 @@ def main():
     ops = alg_ops_per_path(minfo)
     launch_s = t_dev / args.steps
     achieved = ops["ops"] * w.n_paths / launch_s
+    n_kernels = pc.pc_debug_price_kernels(model, contract, w.n_paths)
     kind = "interpreter" if args.interpret or info.n_insn > pc.JIT_MAX_INSNS else "specialised"
     traffic = profile_traffic(w, kind)
     prof = profile_record(w, kind)
@@ -498,7 +499,11 @@ def main():
                                   if info.n_insn <= pc.JIT_MAX_INSNS else
                                   f"interpreter ({info.n_insn} instructions: above the "
                                   f"{pc.JIT_MAX_INSNS} that are specialised)")
-                                 + (", window of dates in HBM" if linfo.hbm_window else "")},
+                                 + (", window of dates in HBM" if linfo.hbm_window else "")
+                                 + (f", {n_kernels} launches a step: paths knocked out at the last, middle or "
+                                    "quarter dates are settled first and not walked (payoffs and sums "
+                                    "bit-equal; value and roofline count every path's dates)"
+                                    if n_kernels > 1 else "")},
             # where the window of simulated dates lives (a program that looks
             # far back keeps it in HBM: bytes of the launch's buffer, bytes
             # each path writes per simulated date)
@@ -514,7 +519,7 @@ def main():
             "contracts_per_sec_at_1e-4_rel_se": contracts_per_s,
             "price": mean, "stderr": math.sqrt(var / w.n_paths),
             "paths_for_1e-4_rel_se": paths_needed,
-            "gpu_launches": args.steps * pc.pc_debug_price_kernels(model, contract, w.n_paths),
+            "gpu_launches": args.steps * n_kernels,
             "e2e": {"value": e2e_value, "unit": UNIT,
                     "h2d_bytes_per_step": int(words.nbytes + consts.nbytes + 4 * len(w.tparams)),
                     "d2h_bytes_per_step": 40,
