@@ -764,6 +764,13 @@ pc_status pc_debug_set_cv_min_blocks(pc_ctx *ctx, int32_t blocks);
  * network's captured graphs. */
 pc_status pc_debug_mlp_withhold_tma(pc_mlp *net, int32_t on);
 
+/* Host-side sizes of a network's weight-gradient partials (no GPU): the
+ * floats that one layer's product over `batch` rows writes at most on a GPU
+ * of sm_count SMs, and the floats of the buffer that a network created with
+ * these widths and max_batch holds for it.  Errors: PC_EINVAL. */
+pc_status pc_debug_mlp_partials(const int32_t *widths, int32_t n_widths, uint64_t max_batch, uint64_t batch,
+                                int32_t sm_count, uint64_t *written, uint64_t *held);
+
 /* Per-path probe of pc_greeks for one underlying: writes (payoff,
  * d payoff / d S0[underlying], d payoff / d sigma[underlying]) of path
  * path_offset+i to d_paths[3i..3i+2] (device floats) and the six sums

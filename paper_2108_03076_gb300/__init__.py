@@ -125,6 +125,7 @@ _SIGS = {
     "pc_debug_fail_allocations": [VP, I32],
     "pc_debug_set_status": [VP, I32],
     "pc_debug_mlp_withhold_tma": [VP, I32],
+    "pc_debug_mlp_partials": [C.POINTER(C.c_int32), C.c_int32, U64, U64, C.c_int32, C.POINTER(U64), C.POINTER(U64)],
     "pc_greeks_adjoint": [VP, VP, U64, U64, PD, PD, PD, PD],
     "pc_greeks_adjoint_async": [VP, VP, U64, U64, U64, U32, VP],
     "pc_debug_adjoint_paths": [VP, VP, U64, U64, U64, VP, VP],
@@ -391,6 +392,15 @@ def pc_debug_set_status(ctx: int, value: int) -> None:
 
 def pc_debug_mlp_withhold_tma(net: int, on: bool) -> None:
     _check(lib().pc_debug_mlp_withhold_tma(VP(net), int(bool(on))))
+
+
+def pc_debug_mlp_partials(widths, max_batch: int, batch: int, sm_count: int):
+    """(floats a batch's weight-gradient partials take, floats of the network's buffer); host only."""
+    w = _arr(widths, np.int32)
+    a, b = U64(), U64()
+    _check(lib().pc_debug_mlp_partials(_ptr(w, C.c_int32), w.size, int(max_batch), int(batch), int(sm_count),
+                                       C.byref(a), C.byref(b)))
+    return a.value, b.value
 
 
 def pc_debug_set_jit_pairs(ctx: int, pairs: int) -> None:

@@ -114,26 +114,52 @@ struct Carve {
   }
 };
 
-// Splits of the weight-gradient product over `rows`: enough blocks to cover
-// the GPU, k ranges in whole 32-row steps.
-int grad_splits(const pc_mlp *N, int M, int Nn, size_t rows, int &k_split) {
-  const int tiles = (M / 64) * (Nn / 64);
-  int want = std::max(1, (2 * N->ctx->sm_count + tiles - 1) / tiles);
-  const int steps32 = int(rows / 32);
-  want = std::min(want, steps32);
+// Splits of the weight-gradient product over `rows` on a GPU of `sms` SMs:
+// enough blocks to cover it (most_splits, at most one a 32-row step), k
+// ranges in whole 32-row steps.  A range is rounded up to whole steps, so the
+// count may be well below most_splits, and is not monotonic in the rows.
+int most_splits(int sms, int tiles, size_t steps) {
+  return int(std::max<size_t>(1, std::min(size_t(2 * sms + tiles - 1) / tiles, steps)));
+}
+int grad_tiles(int M, int Nn) { return (M / 64) * (Nn / 64); }
+int grad_splits(int sms, int M, int Nn, size_t rows, int &k_split) {
+  const int steps32 = int(rows / 32), want = most_splits(sms, grad_tiles(M, Nn), rows / 32);
   k_split = ((steps32 + want - 1) / want) * 32;
   return int((rows + k_split - 1) / k_split);
 }
 
 // The same for the tensor-core weight gradient: 128 x (64 or 128) output
 // tiles, k ranges in whole 64-row chunks.
-int tc_grad_splits(const pc_mlp *N, int M, int Nn, size_t rows, int &k_split) {
-  const int tiles = ((M + 127) / 128) * (Nn == 64 ? 1 : Nn / 128);
-  int want = std::max(1, (2 * N->ctx->sm_count + tiles - 1) / tiles);
-  const int steps64 = int(rows / 64);
-  want = std::max(1, std::min(want, steps64));
+int tc_grad_tiles(int M, int Nn) { return ((M + 127) / 128) * (Nn == 64 ? 1 : Nn / 128); }
+int tc_grad_splits(int sms, int M, int Nn, size_t rows, int &k_split) {
+  const int steps64 = int(rows / 64), want = most_splits(sms, tc_grad_tiles(M, Nn), rows / 64);
   k_split = ((steps64 + want - 1) / want) * 64;
   return int((rows + k_split - 1) / k_split);
+}
+
+// Floats of split-k partials that the largest layer of padded widths wp
+// writes in a product over `rows`, on either kernel.
+size_t partials_written(const std::vector<int> &wp, size_t rows, int sms) {
+  size_t part = 0;
+  for (size_t l = 0; l + 1 < wp.size(); ++l) {
+    int ks = 0;
+    const size_t layer = size_t(wp[l + 1]) * wp[l];
+    part = std::max(part, size_t(grad_splits(sms, wp[l + 1], wp[l], rows, ks)) * layer);
+    if (rows % 64 == 0) part = std::max(part, size_t(tc_grad_splits(sms, wp[l + 1], wp[l], rows, ks)) * layer);
+  }
+  return part;
+}
+
+// Floats of a partials buffer for calls of up to `rows` rows: the most splits
+// that any number of rows up to that can take.
+size_t partials_held(const std::vector<int> &wp, size_t rows, int sms) {
+  size_t part = 0;
+  for (size_t l = 0; l + 1 < wp.size(); ++l) {
+    const int M = wp[l + 1], Nn = wp[l];
+    const int most = std::max(most_splits(sms, grad_tiles(M, Nn), rows / 32), most_splits(sms, tc_grad_tiles(M, Nn), rows / 64));
+    part = std::max(part, size_t(most) * M * Nn);
+  }
+  return part;
 }
 
 // Parameter offsets and the device buffers for `rows` padded rows, carved
@@ -151,17 +177,7 @@ size_t layout(pc_mlp *N, size_t rows) {
   N->n_flat = flat;
   int widest = 0;
   for (int x : N->wp) widest = std::max(widest, x);
-  size_t part = 0;  // split-k partials: the largest layer at its split count
-  for (int l = 0; l < N->L; ++l) {
-    int ks = 0;
-    const int sp = grad_splits(N, N->wp[l + 1], N->wp[l], rows, ks);
-    part = std::max(part, size_t(sp) * N->wp[l + 1] * N->wp[l]);
-    if (rows % 64 == 0) {
-      const int tsp = tc_grad_splits(N, N->wp[l + 1], N->wp[l], rows, ks);
-      part = std::max(part, size_t(tsp) * N->wp[l + 1] * N->wp[l]);
-    }
-  }
-  N->part_cap = part;
+  const size_t part = N->part_cap = partials_held(N->wp, rows, N->ctx->sm_count);
   const size_t chunks = (rows + 255) / 256;
   Carve c{static_cast<char *>(N->mem)};
   N->p = c.take<float>(flat);
@@ -199,6 +215,9 @@ GemmArgs gemm0() {
 // cores); *used receives the split count of the path taken.
 cudaError_t product(pc_mlp *N, GemmKind kind, int epi, int layer, size_t rows, GemmArgs a, int splits,
                     int tc_k_split, int tc_splits, cudaStream_t s, int *used = nullptr, bool dep = false) {
+  const size_t layer_size = size_t(N->wp[layer + 1]) * N->wp[layer];
+  if (kind == kGemmWeightGrad && size_t(std::max(splits, tc_splits)) * layer_size > N->part_cap)
+    return cudaErrorInvalidValue;  // (partials_held holds the splits of every call)
   if (used) *used = splits;
   if (N->tc_ok && N->gemm == PC_MLP_GEMM_AUTO) {
     GemmArgs t = a;
@@ -308,9 +327,9 @@ cudaError_t backward(pc_mlp *N, const float *t, const LossWeights &lw, size_t n,
     a.M = out_w;
     a.N = in_w;
     a.K = int(rows);
-    int splits = grad_splits(N, out_w, in_w, rows, a.k_split);
+    int splits = grad_splits(N->ctx->sm_count, out_w, in_w, rows, a.k_split);
     int tc_ks = 0;
-    const int tc_splits = rows % 64 == 0 ? tc_grad_splits(N, out_w, in_w, rows, tc_ks) : 0;
+    const int tc_splits = rows % 64 == 0 ? tc_grad_splits(N->ctx->sm_count, out_w, in_w, rows, tc_ks) : 0;
     a.Cf = N->part[l & 1];
     a.ldc = in_w;
     e = product(N, kGemmWeightGrad, kEpiPartial, l, rows, a, splits, tc_ks, tc_splits, sw, &splits, dep);
@@ -408,6 +427,18 @@ pc_status copy_unpadded(pc_mlp *N, const float *src, float *dst, cudaMemcpyKind 
   return PC_OK;
 }
 
+// The widths and rows that a network is created for.
+pc_status check_widths(const int32_t *widths, int32_t n_widths, uint64_t max_batch) {
+  if (n_widths < 2 || n_widths > kMaxLayers + 1) return fail(PC_EINVAL, "n_widths must be 2..9");
+  if (max_batch < 1 || max_batch > (uint64_t(1) << 24)) return fail(PC_EINVAL, "max_batch must be 1..2^24");
+  for (int i = 0; i < n_widths; ++i) {
+    const bool edge = i == 0 || i == n_widths - 1;
+    if (widths[i] < 1 || (edge && widths[i] > kPad) || (!edge && (widths[i] % kPad || widths[i] > 1024)))
+      return fail(PC_EINVAL, "widths: input/output 1..64, hidden multiples of 64 up to 1024");
+  }
+  return PC_OK;
+}
+
 LossWeights loss_weights(const pc_mlp *N, const float *w) {
   LossWeights lw{};
   for (int j = 0; j < N->w[N->L]; ++j) lw.w[j] = w[j];
@@ -479,13 +510,8 @@ extern "C" {
 pc_status pc_mlp_create(pc_ctx *c, const int32_t *widths, int32_t n_widths, uint64_t max_batch,
                         uint64_t seed, pc_mlp **out) {
   if (!c || !widths || !out) return fail(PC_EINVAL, "null argument");
-  if (n_widths < 2 || n_widths > kMaxLayers + 1) return fail(PC_EINVAL, "n_widths must be 2..9");
-  if (max_batch < 1 || max_batch > (uint64_t(1) << 24)) return fail(PC_EINVAL, "max_batch must be 1..2^24");
-  for (int i = 0; i < n_widths; ++i) {
-    const bool edge = i == 0 || i == n_widths - 1;
-    if (widths[i] < 1 || (edge && widths[i] > kPad) || (!edge && (widths[i] % kPad || widths[i] > 1024)))
-      return fail(PC_EINVAL, "widths: input/output 1..64, hidden multiples of 64 up to 1024");
-  }
+  pc_status ws = check_widths(widths, n_widths, max_batch);
+  if (ws != PC_OK) return ws;
   pc_mlp *N = new (std::nothrow) pc_mlp;
   if (!N) return fail(PC_ENOMEM, "network");
   N->ctx = c;
@@ -529,6 +555,19 @@ pc_status pc_mlp_create(pc_ctx *c, const int32_t *widths, int32_t n_widths, uint
     return s;
   }
   *out = N;
+  return PC_OK;
+}
+
+pc_status pc_debug_mlp_partials(const int32_t *widths, int32_t n_widths, uint64_t max_batch, uint64_t batch,
+                                int32_t sm_count, uint64_t *written, uint64_t *held) {
+  if (!widths || !written || !held) return fail(PC_EINVAL, "null argument");
+  const pc_status s = check_widths(widths, n_widths, max_batch);
+  if (s != PC_OK) return s;
+  if (batch < 1 || batch > max_batch || sm_count < 1) return fail(PC_EINVAL, "batch must be 1..max_batch, sm_count >= 1");
+  std::vector<int> wp;
+  for (int32_t i = 0; i < n_widths; ++i) wp.push_back(pad64(widths[i]));
+  *written = partials_written(wp, rows_for(batch), sm_count);
+  *held = partials_held(wp, rows_for(max_batch), sm_count);
   return PC_OK;
 }
 
