@@ -338,17 +338,17 @@ void drop_buffer(pc_ctx *c, void *p, bool &held) {
   held = false;
 }
 
-// Point the launch's window at the context's HBM window buffer (grown to
-// grid * block threads x win * d slots).
-pc_status bind_hbm_window(pc_ctx *c, Launch &L, int d) {
+// Point the window of a launch of grid blocks of `block` threads at the
+// context's HBM window buffer, a column per thread of that launch (grown to
+// grid * block threads x win * d slots).  A capture that would have to grow
+// it is refused, the buffer and the capture unharmed.
+pc_status bind_hbm_window(pc_ctx *c, Layout &lay, int grid, int block, int d) {
+  const size_t threads = size_t(grid) * size_t(block), slots = threads * size_t(lay.win) * size_t(d);
   const bool cap = capturing(c);
-  const auto slots_of = [&](int grid) { return size_t(grid) * size_t(L.block) * size_t(L.args.lay.win) * size_t(d); };
-  if (cap && L.sparse_grid && slots_of(L.grid) > c->gwin_cap) {  // no growing under capture
-    L.grid = L.sparse_grid;
-    L.sparse_grid = 0;
-  }
-  const size_t threads = size_t(L.grid) * size_t(L.block), slots = slots_of(L.grid);
   if (slots > c->gwin_cap) {
+    if (cap)
+      return fail(PC_ECUDA, "the window of dates in HBM would have to grow while the stream is being captured: "
+                            "make the call once before the capture");
     CU(cudaStreamSynchronize(c->stream), "sync");
     drop_buffer(c, c->d_gwin, c->gwin_captured);
     c->d_gwin = nullptr;
@@ -357,8 +357,8 @@ pc_status bind_hbm_window(pc_ctx *c, Launch &L, int d) {
     c->gwin_cap = slots;
   }
   if (cap) c->gwin_captured = true;
-  L.args.lay.gwin = c->d_gwin;
-  L.args.lay.gstride = int64_t(threads);
+  lay.gwin = c->d_gwin;
+  lay.gstride = int64_t(threads);
   return PC_OK;
 }
 
@@ -589,21 +589,19 @@ pc_status run_price(const pc_model *m, const pc_contract *k, uint64_t n_paths, u
     const int grid = int(std::min<uint64_t>(uint64_t(c->sm_count) * nb, (units + wpb - 1) / wpb));
     L.args.one_pass = !screened && uint64_t(grid) * wpb >= units;
     if (L.hbm_window) {
-      // the HBM window holds a column per thread of this launch's grid
-      L.grid = grid;
-      s = bind_hbm_window(c, L, m->H.d);
+      s = bind_hbm_window(c, L.args.lay, grid, L.block, m->H.d);
       if (s != PC_OK) return s;
     }
     void *args[] = {&L.args, &L.w->grid};
     CU(cudaLaunchKernel(kern, dim3(grid), dim3(L.block), args, smem, c->stream), "specialised price kernel");
   } else {
     if (L.hbm_window) {
-      s = bind_hbm_window(c, L, m->H.d);
-      if (s == PC_ENOMEM && L.sparse_grid) {  // no memory for the dense variant's window
+      s = bind_hbm_window(c, L.args.lay, L.grid, L.block, m->H.d);
+      if (s != PC_OK && L.sparse_grid) {  // no room for the dense variant's window
         cudaGetLastError();
         L.grid = L.sparse_grid;
         L.sparse_grid = 0;
-        s = bind_hbm_window(c, L, m->H.d);
+        s = bind_hbm_window(c, L.args.lay, L.grid, L.block, m->H.d);
       }
       if (s != PC_OK) return s;
     }

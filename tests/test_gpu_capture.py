@@ -1,0 +1,102 @@
+"""Calls captured on the caller's stream: a graph's replay equals the same
+call made eagerly, bit for bit, whatever the calls between capture and replay
+do with the context's scratch; a capture that would need more scratch than
+the context holds runs without it or is refused."""
+import numpy as np
+import pytest
+
+from gpu_common import torch
+import paper_2108_03076_gb300 as pc
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+TILE, WARPS = 64, 4  # paths a tile, warps a block
+
+
+@pytest.fixture(params=[False, True], ids=["interpreted", "specialised"])
+def ctx(request):
+    """A context of its own per test: its scratch starts small."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2108_03076_gb300 import build
+    build.build()
+    st = torch.cuda.Stream()
+    torch.cuda.set_stream(st)
+    c = pc.pc_create(0, st.cuda_stream)
+    pc.pc_set_jit(c, request.param)
+    yield c
+    torch.cuda.synchronize()
+    pc.pc_destroy(c)
+
+
+def capture(call):
+    """(graph, None) of `call` captured on the current stream, or (None, the
+    refusal)."""
+    g, refused = torch.cuda.CUDAGraph(), None
+    mark = torch.zeros(1, device="cuda")
+    with torch.cuda.graph(g, stream=torch.cuda.current_stream()):
+        mark.add_(1)
+        try:
+            call()
+        except pc.PcError as e:
+            refused = e
+    return (None if refused else g), refused
+
+
+def market(ctx, spec):
+    return pc.pc_model_create(ctx, spec.S0, spec.sigma, spec.corr, spec.r, spec.days)
+
+
+def contract(ctx, text, tp=()):
+    w, k = pc.pc_assemble(text)
+    return pc.pc_load_payoff(ctx, w, k, tp)
+
+
+def newest_first(n):
+    s = "(add (model 0 $0) (model 1 $0))"
+    for j in range(1, n):
+        s = f"(add {s} (add (model 0 (tplus $0 {-j})) (model 1 (tplus $0 {-j}))))"
+    return f"(max (sub (div {s} {2.0 * n}) 1.1) 0.0)"
+
+
+def test_hbm_window_never_smaller_than_its_launch(ctx, request):
+    """A window buffer of six blocks an SM, then a captured call of one path
+    more: the interpreter keeps to six blocks, a specialised launch that holds
+    more is refused.  Captured after an eager call of that size, it runs."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    spec = W.MarketSpec([1.0, 1.2], [0.25, 0.3], W.const_corr(2, 0.4), 0.02, list(range(1, 13)))
+    m, k = market(ctx, spec), contract(ctx, newest_first(12), [12])
+    pc.pc_set_window_mode(ctx, pc.WINDOW_HBM)
+    n = 6 * sms * WARPS * TILE
+    out = torch.zeros(5, 4, dtype=torch.float64, device="cuda")
+
+    def price(paths, row):
+        return lambda: pc.pc_price_async(m, k, paths, 0, 7, 0, out[row].data_ptr())
+    try:
+        price(n, 0)()
+        small, refused = capture(price(n, 1))
+        assert refused is None
+        first, refused = capture(price(n + 1, 2))
+        assert first is not None or refused.name == "PC_ECUDA"
+        if first is not None:
+            first.replay()
+            torch.cuda.synchronize()
+        price(n + 1, 3)()  # grows the buffer; the captured one is kept
+        second, again = capture(price(n + 1, 4))
+        assert again is None
+        small.replay()
+        second.replay()
+        torch.cuda.synchronize()
+        o = out[:, :3].cpu().numpy()
+        np.testing.assert_array_equal(o[1], o[0])
+        np.testing.assert_array_equal(o[4], o[3])
+        if first is not None:
+            np.testing.assert_array_equal(o[2], o[3])
+        pc.pc_set_window_mode(ctx, pc.WINDOW_SHARED)
+        price(n + 1, 0)()
+        torch.cuda.synchronize()
+        np.testing.assert_array_equal(out[0, :3].cpu().numpy(), o[3])
+    finally:
+        pc.pc_contract_destroy(k)
+        pc.pc_model_destroy(m)
