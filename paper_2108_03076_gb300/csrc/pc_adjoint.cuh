@@ -41,6 +41,18 @@ __device__ __forceinline__ float2 adsel(float2 c, float2 p, float2 q) {
   return make_float2(bits(c.x) ? p.x : q.x, bits(c.y) ? p.y : q.y);
 }
 
+// Ints shared by the warp: every lane writes the same value and reads it
+// later, at the same places of a warp-uniform program.  The barrier before a
+// write lets no lane overwrite what another has still to read.
+struct WarpInts {
+  int *p;
+  __device__ __forceinline__ int get(int s) const { return p[s]; }
+  __device__ __forceinline__ void set(int s, int v) const {
+    __syncwarp();
+    p[s] = v;
+  }
+};
+
 // The adjoint launch's per-warp tape cursor and recording.
 struct Tape {
   float4 *part;
