@@ -113,13 +113,13 @@ pc_status run_adjoint(const pc_model *m, const pc_contract *k, uint64_t n_paths,
     if (s != PC_OK) return s;
     const void *kern = reinterpret_cast<const void *>(jk);
     int nb = 0;
-    smem = price_smem_bytes(0, 0, ja.lay.words, block);
-    CU(jit_occupancy(c, kern, block, smem, nb), "jit occupancy");
+    const size_t jsmem = price_smem_bytes(0, 0, ja.lay.words, block);
+    CU(jit_occupancy(c, kern, block, jsmem, nb), "jit occupancy");
     if (nb >= 1) {
       const int jgrid = std::min(grid, c->sm_count * nb);
       ja.one_pass = uint64_t(jgrid) * wpb >= a.n_tiles;
       void *args[] = {&ja, &t, &L.w->grid};
-      CU(cudaLaunchKernel(kern, dim3(jgrid), dim3(block), args, smem, c->stream), "specialised adjoint kernel");
+      CU(cudaLaunchKernel(kern, dim3(jgrid), dim3(block), args, jsmem, c->stream), "specialised adjoint kernel");
       return PC_OK;
     }
   }
