@@ -73,18 +73,12 @@ pc_status run_adjoint(const pc_model *m, const pc_contract *k, uint64_t n_paths,
   if (size_t(grid) * wpb * region > kTapeCapBytes)
     grid = int(std::max<size_t>(1, kTapeCapBytes / (size_t(wpb) * region)));
   const size_t bytes = size_t(grid) * wpb * region;
-  if (bytes > c->tape_cap) {
-    CU(cudaStreamSynchronize(c->stream), "sync");
-    if (c->d_tape) cudaFree(c->d_tape);
-    c->d_tape = nullptr;
-    c->tape_cap = 0;
-    CU(ctx_malloc(c, &c->d_tape, bytes), "adjoint tape");
-    c->tape_cap = bytes;
-  }
+  s = grow_scratch(c, c->tape, bytes, "adjoint tape");
+  if (s != PC_OK) return s;
   const size_t regions = size_t(grid) * wpb;
   TapeArgs t;
   t.emax = int32_t(emax);
-  char *base = static_cast<char *>(c->d_tape);
+  char *base = c->tape.as<char>();
   t.part = reinterpret_cast<float4 *>(base);
   t.adj = reinterpret_cast<float2 *>(base + regions * size_t(emax) * 32 * sizeof(float4));
   t.ids = reinterpret_cast<int2 *>(base + regions * size_t(emax) * 32 * (sizeof(float4) + sizeof(float2)));
@@ -97,7 +91,7 @@ pc_status run_adjoint(const pc_model *m, const pc_contract *k, uint64_t n_paths,
   reduction_chunks(a, uint32_t(kMaxChunks * 8 / width));
   s = ensure_partials(c, size_t(a.n_tiles) * size_t(width));
   if (s != PC_OK) return s;
-  a.tile_partials = c->d_partials;
+  a.tile_partials = c->partials.as<double>();
   a.control = c->d_control;
   a.out = d_out;
   a.out_paths = d_paths;

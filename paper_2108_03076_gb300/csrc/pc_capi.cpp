@@ -149,16 +149,31 @@ Layout make_layout(const Program &p, const ModelHost &H, int32_t win, int32_t sk
   return L;
 }
 
-pc_status ensure_partials(pc_ctx *c, size_t doubles) {
-  if (doubles <= c->partial_cap) return PC_OK;
-  CU(cudaStreamSynchronize(c->stream), "sync");
-  if (c->d_partials) cudaFree(c->d_partials);
-  c->d_partials = nullptr;
-  c->partial_cap = 0;
-  size_t cap = std::max<size_t>(doubles, 1 << 16);
-  CU(ctx_malloc(c, reinterpret_cast<void **>(&c->d_partials), cap * sizeof(double)), "partials");
-  c->partial_cap = cap;
+bool capturing(const pc_ctx *c) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(c->stream, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone;
+}
+
+pc_status grow_scratch(pc_ctx *c, Scratch &b, size_t bytes, const char *what) {
+  const bool cap = capturing(c);
+  if (bytes > b.bytes) {
+    if (cap)
+      return fail(PC_ECUDA, std::string(what) + " would have to grow while the stream is being captured: make the "
+                            "call once before the capture");
+    CU(cudaStreamSynchronize(c->stream), "sync");
+    if (b.captured) c->captured.push_back(b.p);
+    else if (b.p) cudaFree(b.p);
+    b = Scratch{};
+    CU(ctx_malloc(c, &b.p, bytes), what);
+    b.bytes = bytes;
+  }
+  if (cap) b.captured = true;
   return PC_OK;
+}
+
+pc_status ensure_partials(pc_ctx *c, size_t doubles) {
+  if (doubles * sizeof(double) > c->partials.bytes) doubles = std::max<size_t>(doubles, 1 << 16);
+  return grow_scratch(c, c->partials, doubles * sizeof(double), "partials");
 }
 
 // Constant-pool floats of a program, rounded up to whole 16-byte words.
@@ -323,41 +338,14 @@ pc_status prepare(const pc_model *m, const pc_contract *k, uint64_t n_paths, uin
   return PC_OK;
 }
 
-// The caller is capturing the context's stream.
-bool capturing(const pc_ctx *c) {
-  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(c->stream, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone;
-}
-
-// Frees a buffer about to grow, or keeps it for the graphs that hold it.
-void drop_buffer(pc_ctx *c, void *p, bool &held) {
-  if (held && p)
-    c->captured.push_back(p);
-  else if (p)
-    cudaFree(p);
-  held = false;
-}
-
 // Point the window of a launch of grid blocks of `block` threads at the
-// context's HBM window buffer, a column per thread of that launch (grown to
-// grid * block threads x win * d slots).  A capture that would have to grow
-// it is refused, the buffer and the capture unharmed.
+// context's HBM window buffer, a column per thread of that launch (grid *
+// block threads x win * d slots).
 pc_status bind_hbm_window(pc_ctx *c, Layout &lay, int grid, int block, int d) {
   const size_t threads = size_t(grid) * size_t(block), slots = threads * size_t(lay.win) * size_t(d);
-  const bool cap = capturing(c);
-  if (slots > c->gwin_cap) {
-    if (cap)
-      return fail(PC_ECUDA, "the window of dates in HBM would have to grow while the stream is being captured: "
-                            "make the call once before the capture");
-    CU(cudaStreamSynchronize(c->stream), "sync");
-    drop_buffer(c, c->d_gwin, c->gwin_captured);
-    c->d_gwin = nullptr;
-    c->gwin_cap = 0;
-    CU(ctx_malloc(c, reinterpret_cast<void **>(&c->d_gwin), slots * sizeof(float2)), "HBM window");
-    c->gwin_cap = slots;
-  }
-  if (cap) c->gwin_captured = true;
-  lay.gwin = c->d_gwin;
+  const pc_status s = grow_scratch(c, c->gwin, slots * sizeof(float2), "the HBM window");
+  if (s != PC_OK) return s;
+  lay.gwin = c->gwin.as<float2>();
   lay.gstride = int64_t(threads);
   return PC_OK;
 }
@@ -403,7 +391,7 @@ pc_status run_greeks(const pc_model *m, const pc_contract *k, uint64_t n_paths, 
   a.lay = lay;
   a.width = 6;
   reduction_chunks(a);
-  a.tile_partials = c->d_partials;
+  a.tile_partials = c->partials.as<double>();
   a.control = c->d_control;
   a.out = d_out;
   a.out_paths = d_paths;
@@ -526,22 +514,13 @@ bool screen_large(const pc_model *m, uint64_t n_paths) {
 bool screen_launch(pc_ctx *c, const pc_model *m, const pc_contract *k, const PriceArgs &a, float *payoffs, Screen &s) {
   if (!screen_large(m, a.n_paths) || !screen_suits(m, k, s)) return false;
   const size_t words = 64 + size_t(a.n_paths) * (payoffs ? 1 : 2);
-  const bool cap = capturing(c);
-  if (words > c->screen_cap) {
-    if (cap || cudaStreamSynchronize(c->stream) != cudaSuccess) return false;
-    drop_buffer(c, c->d_screen, c->screen_captured);
-    c->d_screen = nullptr;
-    c->screen_cap = 0;
-    if (ctx_malloc(c, reinterpret_cast<void **>(&c->d_screen), words * 4) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    c->screen_cap = words;
+  if (grow_scratch(c, c->screen, words * 4, "screen") != PC_OK) {
+    cudaGetLastError();
+    return false;
   }
-  if (cap) c->screen_captured = true;
-  s.count = c->d_screen;
-  s.list = c->d_screen + 64;
-  s.payoffs = payoffs ? payoffs : reinterpret_cast<float *>(c->d_screen + 64 + a.n_paths);
+  s.count = c->screen.as<uint32_t>();
+  s.list = s.count + 64;
+  s.payoffs = payoffs ? payoffs : reinterpret_cast<float *>(s.list + a.n_paths);
   return true;
 }
 
@@ -555,7 +534,7 @@ pc_status run_price(const pc_model *m, const pc_contract *k, uint64_t n_paths, u
   if (s != PC_OK) return s;
   L.args.width = 2;
   reduction_chunks(L.args);
-  L.args.tile_partials = c->d_partials;
+  L.args.tile_partials = c->partials.as<double>();
   L.args.control = c->d_control;
   L.args.out = d_out;
   L.args.out_paths = d_payoffs;
@@ -815,11 +794,9 @@ pc_status pc_destroy(pc_ctx *c) {
   if (c->live_objects) return fail(PC_EINVAL, "destroy the context's models and contracts first");
   cudaSetDevice(c->device);
   cudaStreamSynchronize(c->stream);
-  if (c->d_partials) cudaFree(c->d_partials);
   if (c->d_control) cudaFree(c->d_control);
-  if (c->d_gwin) cudaFree(c->d_gwin);
-  if (c->d_tape) cudaFree(c->d_tape);
-  if (c->d_screen) cudaFree(c->d_screen);
+  for (const Scratch *b : {&c->partials, &c->gwin, &c->tape, &c->screen})
+    if (b->p) cudaFree(b->p);
   for (void *p : c->captured) cudaFree(p);
   jit_release(c);
   if (c->d_gout) cudaFree(c->d_gout);

@@ -110,7 +110,7 @@ pc_status cv_launch(const pc_model *m, const pc_contract *k, const pc_cv_desc *c
   reduction_chunks(a);
   s = ensure_partials(ctx, size_t(a.n_tiles) * size_t(a.width));
   if (s != PC_OK) return s;
-  a.tile_partials = ctx->d_partials;
+  a.tile_partials = ctx->partials.as<double>();
   a.control = ctx->d_control;
   a.out = d_out;
   a.out_paths = d_xm;

@@ -67,6 +67,15 @@ struct JitEntry {
   cudaKernel_t kernel = nullptr;
 };
 
+// Device scratch, grown on demand (grow_scratch) and shared by the calls.
+struct Scratch {
+  void *p = nullptr;
+  size_t bytes = 0;
+  bool captured = false;  // a caller's graph holds the address
+  template <typename T>
+  T *as() const { return static_cast<T *>(p); }
+};
+
 struct pc_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
@@ -77,19 +86,12 @@ struct pc_ctx {
   int smem_reserve = 0;  // shared memory the system reserves per resident block (bytes)
   double *d_res = nullptr;       // [8]: sum, sumsq, n, -, status word (int32 at d_res+4)
   double *d_gout = nullptr;      // [PC_MAX_UNDERLYINGS * 8]: sensitivity sums per underlying
-  double *d_partials = nullptr;  // tile partials (scratch)
-  size_t partial_cap = 0;        // doubles
+  Scratch partials;              // tile partials (doubles)
   unsigned char *d_control = nullptr;  // reduction control block (kControlBytes, zero between launches)
-  void *d_tape = nullptr;        // adjoint tapes, one region per resident warp (grow-only)
-  size_t tape_cap = 0;           // bytes
-  float2 *d_gwin = nullptr;      // HBM windows of simulated dates (grow-only)
-  size_t gwin_cap = 0;           // float2 slots
-  uint32_t *d_screen = nullptr;  // screened launches: count, list and payoffs (grow-only)
-  size_t screen_cap = 0;         // 4-byte words
-  // a caller's stream capture holds the buffer's address: when it grows, the
-  // old one is kept until the context goes
-  bool screen_captured = false, gwin_captured = false;
-  std::vector<void *> captured;
+  Scratch tape;                  // adjoint tapes, one region per resident warp
+  Scratch gwin;                  // HBM windows of simulated dates (float2 slots)
+  Scratch screen;                // screened launches: count, list and payoffs (4-byte words)
+  std::vector<void *> captured;  // scratch that grew after a caller's graph took its address: kept until the context goes
   int32_t window_mode = 0;       // PC_WINDOW_AUTO / _SHARED / _HBM
   int32_t jit = 0;               // 1: price with run-time specialised kernels
   // streams and events of one-shot portfolio launches (pc_price_batch),
@@ -223,7 +225,14 @@ struct Launch {
 pc_status prepare(const pc_model *m, const pc_contract *k, uint64_t n_paths, uint64_t offset,
                   uint64_t seed, uint32_t stream, Launch &L, bool allow_hbm = false);
 
-// Grow the context's tile-partial scratch to at least `doubles`.
+// Whether the caller is capturing the context's stream.
+bool capturing(const pc_ctx *c);
+// A scratch buffer of at least `bytes`.  Under a caller's capture its address
+// goes into the caller's graph: nothing is grown then (PC_ECUDA, the capture
+// unharmed), and when the buffer grows later the captured one is kept until
+// the context goes, so that the graph may be replayed after any call.
+pc_status grow_scratch(pc_ctx *c, Scratch &b, size_t bytes, const char *what);
+// The context's tile-partial scratch for at least `doubles`.
 pc_status ensure_partials(pc_ctx *c, size_t doubles);
 
 // The run-time specialised kernel of the contract's program for d

@@ -57,8 +57,7 @@ struct pc_mlp {
   float g_lr = 0.f;
   uint64_t g_seed = 0;
   std::vector<float> g_w;
-  float *scratch = nullptr;         // caller scratch (mlp_scratch), grow-only
-  size_t scratch_cap = 0;
+  Scratch scratch;                  // caller scratch (mlp_scratch)
   int32_t *dstatus = nullptr;       // device status of the tensor-core products
   int32_t gemm = PC_MLP_GEMM_AUTO;  // product kernel choice (pc_mlp_set_gemm)
   bool tc_ok = false;               // tcgen05 products available on this device
@@ -71,15 +70,12 @@ namespace pc {
 void mlp_drop_graphs(pc_mlp *N);
 
 float *mlp_scratch(pc_mlp *N, size_t floats) {
-  if (floats <= N->scratch_cap) return N->scratch;
-  if (wait_stream(N->ctx) != PC_OK) return nullptr;
-  mlp_drop_graphs(N);
-  if (N->scratch) cudaFree(N->scratch);
-  N->scratch = nullptr;
-  N->scratch_cap = 0;
-  if (cudaMalloc(&N->scratch, floats * sizeof(float)) != cudaSuccess) return nullptr;
-  N->scratch_cap = floats;
-  return N->scratch;
+  if (floats * sizeof(float) > N->scratch.bytes && !capturing(N->ctx)) {
+    if (wait_stream(N->ctx) != PC_OK) return nullptr;
+    mlp_drop_graphs(N);  // they hold the address
+  }
+  return grow_scratch(N->ctx, N->scratch, floats * sizeof(float), "network scratch") == PC_OK ? N->scratch.as<float>()
+                                                                                              : nullptr;
 }
 
 // Waits for the stream's work; the loss (when wanted) and the products'
@@ -579,7 +575,7 @@ pc_status pc_mlp_destroy(pc_mlp *N) {
   mlp_drop_graphs(N);
   if (N->h_pin) cudaFreeHost(N->h_pin);
   if (N->mem) cudaFree(N->mem);
-  if (N->scratch) cudaFree(N->scratch);
+  if (N->scratch.p) cudaFree(N->scratch.p);
   delete N;
   return PC_OK;
 }

@@ -100,3 +100,37 @@ def test_hbm_window_never_smaller_than_its_launch(ctx, request):
     finally:
         pc.pc_contract_destroy(k)
         pc.pc_model_destroy(m)
+
+
+def test_captured_scratch_is_kept(ctx):
+    """Pricing and sensitivity graphs replayed after calls that outgrow the
+    tile partials and the tapes they hold."""
+    spec = W.MarketSpec([1.0, 1.2], [0.25, 0.3], W.const_corr(2, 0.4), 0.02, list(range(1, 31)))
+    m = market(ctx, spec)
+    k = contract(ctx, "(mult (max (sub (max (model 0 15) (model 1 30)) 1.1) 0.0) (payoff 30 0 1))")
+    small, large = 20_000, 2_400_000
+    out = torch.zeros(2, 16, dtype=torch.float64, device="cuda")
+    sens = torch.zeros(2, 16, dtype=torch.float64, device="cuda")
+    big = torch.zeros(16, dtype=torch.float64, device="cuda")
+    try:
+        pc.pc_price_async(m, k, small, 0, 7, 0, out[0].data_ptr())
+        pc.pc_greeks_adjoint_async(m, k, small, 0, 7, 0, sens[0].data_ptr())
+        price, refused = capture(lambda: pc.pc_price_async(m, k, small, 0, 7, 0, out[1].data_ptr()))
+        assert refused is None
+        greeks, refused = capture(lambda: pc.pc_greeks_adjoint_async(m, k, small, 0, 7, 0, sens[1].data_ptr()))
+        assert refused is None
+        # a capture that would have to grow them is refused
+        for call in (pc.pc_price_async, pc.pc_greeks_adjoint_async):
+            _, refused = capture(lambda: call(m, k, large, 0, 7, 0, big.data_ptr()))
+            assert refused is not None and refused.name == "PC_ECUDA"
+        pc.pc_price_async(m, k, large, 0, 7, 0, big.data_ptr())
+        pc.pc_greeks_adjoint_async(m, k, large, 0, 7, 0, big.data_ptr())
+        for g in (price, greeks):
+            g.replay()
+        torch.cuda.synchronize()
+        np.testing.assert_array_equal(out[1].cpu().numpy(), out[0].cpu().numpy())
+        np.testing.assert_array_equal(sens[1].cpu().numpy(), sens[0].cpu().numpy())
+        assert out[0, 2].item() == small and out[0, 0].item() > 0
+    finally:
+        pc.pc_contract_destroy(k)
+        pc.pc_model_destroy(m)
