@@ -543,36 +543,30 @@ pc_status run_price(const pc_model *m, const pc_contract *k, uint64_t n_paths, u
   Screen sc;
   const bool screened = screen_launch(c, m, k, L.args, d_payoffs, sc);
   const PriceArgs all = L.args;  // the screen's and the totals' launch
-  if (screened) {
-    CU(cudaMemsetAsync(sc.count, 0, sizeof(uint32_t), c->stream), "screen count");
-    CU(launch_screen(all, sc, c->sm_count, c->stream), "screen kernel");
-    L.args.list = sc.list;
-    L.args.list_n = sc.count;
-    L.args.out_paths = sc.payoffs;
-  }
+  // everything that can fail, then the launches: a failed call writes nothing
+  const void *kern = nullptr;  // the contract's run-time specialised kernel (same arguments and shape), if any
+  int grid = 0;
+  size_t smem = 0;
   if (c->jit && jit_eligible(k)) {
-    // the contract's run-time specialised kernel (same arguments and shape)
     cudaKernel_t jk = nullptr;
     const int wk = jit_window_kind(c, L);
-    const size_t smem = jit_layout(c, L, wk);
+    smem = jit_layout(c, L, wk);
     s = jit_pair_kernel(k, L.w, L.args, (d_payoffs || screened ? kJitPriceWrite : kJitPrice) | wk,
                         jit_price_bound(c, L, smem), L.w->walk, jk);
     if (s != PC_OK) return s;
-    const void *kern = reinterpret_cast<const void *>(jk);
+    kern = reinterpret_cast<const void *>(jk);
     int nb = 0;
     CU(jit_occupancy(c, kern, L.block, smem, nb), "jit occupancy");
     if (nb < 1) return fail(PC_ELIMIT, "specialised kernel cannot be resident");
     const uint64_t wpb = uint64_t(L.block) / 32;
     // a warp takes a tile, or a pair of tiles with two path pairs a lane
     const uint64_t units = (wk & kJitPairs2) ? (L.args.n_tiles + 1) / 2 : L.args.n_tiles;
-    const int grid = int(std::min<uint64_t>(uint64_t(c->sm_count) * nb, (units + wpb - 1) / wpb));
+    grid = int(std::min<uint64_t>(uint64_t(c->sm_count) * nb, (units + wpb - 1) / wpb));
     L.args.one_pass = !screened && uint64_t(grid) * wpb >= units;
     if (L.hbm_window) {
       s = bind_hbm_window(c, L.args.lay, grid, L.block, m->H.d);
       if (s != PC_OK) return s;
     }
-    void *args[] = {&L.args, &L.w->grid};
-    CU(cudaLaunchKernel(kern, dim3(grid), dim3(L.block), args, smem, c->stream), "specialised price kernel");
   } else {
     if (L.hbm_window) {
       s = bind_hbm_window(c, L.args.lay, L.grid, L.block, m->H.d);
@@ -585,6 +579,18 @@ pc_status run_price(const pc_model *m, const pc_contract *k, uint64_t n_paths, u
       if (s != PC_OK) return s;
     }
     L.args.one_pass = !screened && uint64_t(L.grid) * (L.block / 32) >= L.args.n_tiles;
+  }
+  if (screened) {
+    CU(cudaMemsetAsync(sc.count, 0, sizeof(uint32_t), c->stream), "screen count");
+    CU(launch_screen(all, sc, c->sm_count, c->stream), "screen kernel");
+    L.args.list = sc.list;
+    L.args.list_n = sc.count;
+    L.args.out_paths = sc.payoffs;
+  }
+  if (kern) {
+    void *args[] = {&L.args, &L.w->grid};
+    CU(cudaLaunchKernel(kern, dim3(grid), dim3(L.block), args, smem, c->stream), "specialised price kernel");
+  } else {
     CU(launch_price(L.args, L.grid, L.block, L.smem, c->stream, L.sparse_grid != 0), "price kernel");
   }
   if (screened) CU(launch_totals(all, sc.payoffs, c->sm_count, c->stream), "totals kernel");

@@ -134,3 +134,36 @@ def test_captured_scratch_is_kept(ctx):
     finally:
         pc.pc_contract_destroy(k)
         pc.pc_model_destroy(m)
+
+
+BARRIER = ("(loopif (or (le (model 0 0) 0.75) (le (model 1 0) 0.75)) 0.0 "
+           "(mult (max (sub (min (model 0 0) (model 1 0)) {K}) 0.0) (payoff 0 0 1)) 240)")
+
+
+def daily(ctx):
+    return pc.pc_model_create(ctx, [1.0, 1.02], [0.28, 0.2], [[1.0, 0.4], [0.4, 1.0]], 0.02, list(range(1, 241)))
+
+
+def test_a_failed_screened_call_writes_no_payoffs(ctx):
+    """A call that finds no memory for the window of dates leaves the payoffs
+    as they were, the screened paths' too."""
+    m, k = daily(ctx), contract(ctx, BARRIER.format(K=0.9))
+    n = 300_000
+    out = torch.zeros(4, dtype=torch.float64, device="cuda")
+    x = torch.full((n,), float("nan"), device="cuda")
+    try:
+        pc.pc_price_paths(m, k, n, 0, 99, 0, out.data_ptr(), x.data_ptr())  # (the screen's buffers are there)
+        torch.cuda.synchronize()
+        assert not torch.isnan(x).any()
+        x.fill_(float("nan"))
+        pc.pc_set_window_mode(ctx, pc.WINDOW_HBM)
+        pc.pc_debug_fail_allocations(ctx, 1)
+        with pytest.raises(pc.PcError) as e:
+            pc.pc_price_paths(m, k, n, 0, 99, 0, out.data_ptr(), x.data_ptr())
+        assert e.value.name == "PC_ENOMEM"
+        torch.cuda.synchronize()
+        assert torch.isnan(x).all()
+    finally:
+        pc.pc_debug_fail_allocations(ctx, 0)
+        pc.pc_contract_destroy(k)
+        pc.pc_model_destroy(m)
