@@ -369,9 +369,12 @@ pc_status pc_price_info(const pc_model *model, const pc_contract *contract, uint
  * kernel specialised to the contract's executable program (compiled at run
  * time by NVRTC on first use, cached on the context by program content --
  * reloading the same program reuses it -- and freed by pc_destroy; one
- * kernel per underlying count, or, where the bridge has few nodes that the
- * program needs (at most 16), one per date grid's walk, up to 8 walks a
- * program, the rest sharing the general kernel): the same operations in the same order as the
+ * general kernel per underlying count serves the models of every date grid
+ * (per placement of the window, paths a lane and register bound, which the
+ * grid's size decides); where the bridge has few nodes that the program needs
+ * (at most 16), one per date grid instead, for the first 8 grids that the
+ * context meets a program on, the later ones sharing the general kernel): the
+ * same operations in the same order as the
  * interpreting kernel, without the per-instruction dispatch, with the
  * window of dates in shared memory or in HBM as the launch places it.
  * pc_price_cv and pc_greeks likewise run specialised control-variate and
@@ -746,6 +749,9 @@ pc_status pc_debug_set_jit_pairs(pc_ctx *ctx, int32_t pairs);
  * Errors: PC_EINVAL, those of pc_price_info. */
 pc_status pc_debug_price_kernels(const pc_model *model, const pc_contract *contract, uint64_t n_paths,
                                  int32_t *out_kernels);
+
+/* Specialised kernels that the context has compiled so far.  Errors: PC_EINVAL. */
+pc_status pc_debug_jit_kernels(pc_ctx *ctx, uint64_t *out_kernels);
 
 /* Resident 128-thread blocks per SM the register bound of the context's
  * specialised control-variate kernels is set for (1..16), or 0 for the

@@ -116,7 +116,10 @@ cudaError_t jit_occupancy(pc_ctx *c, const void *kern, int block, size_t smem, i
     blocks = it->second;
     return cudaSuccess;
   }
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  cudaError_t e = cudaSuccess;
+  size_t &most = c->jit_smem[kern];  // models of different grids share a kernel: the limit is never lowered
+  if (smem > most) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  if (e == cudaSuccess) most = std::max(most, smem);
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, block, smem);
   if (e == cudaSuccess) c->jit_occ.emplace(key, blocks);
   return e;
@@ -1203,6 +1206,13 @@ pc_status pc_jit_compile(const pc_model *m, const pc_contract *k) {
     if (s != PC_OK) return s;
   }
   return jit_kernel(k, jit_price_spec(m->ctx, k, L, kJitPrice | wk, smem), jk);
+}
+
+pc_status pc_debug_jit_kernels(pc_ctx *c, uint64_t *out_kernels) {
+  if (!c || !out_kernels) return fail(PC_EINVAL, "null argument");
+  std::lock_guard<std::mutex> g(c->jit_mu);
+  *out_kernels = c->jit_cache.size();
+  return PC_OK;
 }
 
 pc_status pc_price_info(const pc_model *m, const pc_contract *k, uint64_t n_paths, pc_launch_info *info) {

@@ -221,21 +221,22 @@ __device__ __forceinline__ void block_normals_h(uint32_t b, const RngH<H> &g, fl
 // Slot s of this lane in its warp's region (warp_region).
 #define SL(s) R[(s) * 32]
 
-// A specialised kernel's layout is a constant (PC_LAYOUT), and with a static
-// walk the model's grid too (PC_GRID): slot addresses become immediate
-// offsets, and grid checks and ordinals fold.
+// A specialised kernel's layout is a constant (PC_LAYOUT; a field of -1 comes
+// from the arguments: jit_spec), and with a static walk the model's grid too
+// (PC_GRID): slot addresses become immediate offsets, and grid checks and
+// ordinals fold.
 #if defined(PC_LAYOUT)
 __device__ __forceinline__ Layout layout_of(const PriceArgs &a) {
   constexpr int32_t v[] = {PC_LAYOUT};
   Layout l = a.lay;
-  l.stack = v[0];
-  l.off_bstack = v[1];
-  l.off_cache = v[2];
-  l.off_win = v[3];
-  l.off_xwin = v[4];
-  l.words = v[5];
-  l.win = v[6];
-  l.ids = v[7];
+  if (v[0] >= 0) l.stack = v[0];
+  if (v[1] >= 0) l.off_bstack = v[1];
+  if (v[2] >= 0) l.off_cache = v[2];
+  if (v[3] >= 0) l.off_win = v[3];
+  if (v[4] >= 0) l.off_xwin = v[4];
+  if (v[5] >= 0) l.words = v[5];
+  if (v[6] >= 0) l.win = v[6];
+  if (v[7] >= 0) l.ids = v[7];
   return l;
 }
 #else

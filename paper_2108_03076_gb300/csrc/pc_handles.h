@@ -50,8 +50,8 @@ struct JitSpec {
   // pc_capi.cpp): per step the date, 1 if it is read, the number of bridge
   // ops and their numbers; empty: the general walk
   std::vector<int32_t> walk;
-  // the launch's layout as constants (jit_layout_constants; empty: read from
-  // the arguments) and with a walk the model's n, n_hist and t_now
+  // the launch's layout as constants (empty, or a field of -1: read from the
+  // arguments; see jit_spec) and with a walk the model's n, n_hist and t_now
   std::vector<int32_t> lay, grid;
   bool one_phi = false;  // every path of the launch has the same upper 32 index bits
   bool operator==(const JitSpec &o) const {
@@ -105,6 +105,7 @@ struct pc_ctx {
   std::multimap<uint64_t, JitEntry> jit_cache;  // program hash -> compiled kernels
   std::map<uint64_t, std::vector<std::vector<int32_t>>> jit_walks;  // program hash -> its static walks (admit_walk)
   std::map<std::pair<const void *, size_t>, int> jit_occ;  // (kernel, smem) -> resident blocks
+  std::map<const void *, size_t> jit_smem;                 // kernel -> the most dynamic shared memory it was set for
   cudaMemPool_t pool = nullptr;  // stream-ordered allocations of contracts (null: cudaMalloc)
   double *h_res = nullptr;       // pinned [64]: the blocking calls' results, written by the kernel
   uint64_t *h_done = nullptr;    // pinned: (ticket << 32) | device status, written after them

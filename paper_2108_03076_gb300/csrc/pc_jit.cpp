@@ -596,8 +596,16 @@ JitSpec jit_spec(const pc_contract *k, const PriceArgs &a, int kind, int min_blo
   sp.walk = walk;
   sp.one_phi = one_phi(a.path_offset, a.n_tiles);
   // constants by value, unless an out-of-line date generator takes them by reference
-  if (kind >= kJitCv || !outlined_dates(k->prog))
+  if (kind >= kJitCv || !outlined_dates(k->prog)) {
     sp.lay = {a.lay.stack, a.lay.off_bstack, a.lay.off_cache, a.lay.off_win, a.lay.off_xwin, a.lay.words, a.lay.win, a.lay.ids};
+    if (walk.empty()) {
+      // the general kernel serves every model: what follows the bridge stack
+      // (its depth is the grid's) and the window's size come from the
+      // arguments, but for a window of one date
+      for (int i : {2, 3, 4, 5}) sp.lay[size_t(i)] = -1;
+      if (a.lay.win > 1) sp.lay[6] = -1;
+    }
+  }
   if (!walk.empty()) sp.grid = {a.m.n, a.m.n_hist, a.m.t_now};
   return sp;
 }
