@@ -1197,15 +1197,13 @@ pc_status pc_jit_compile(const pc_model *m, const pc_contract *k) {
   pc_status s = prepare(m, k, 1u << 20, 0, 0, 0, L, true);
   if (s != PC_OK) return s;
   CU(cudaSetDevice(m->ctx->device), "cudaSetDevice");
-  cudaKernel_t jk = nullptr;
   const int wk = jit_window_kind(m->ctx, L);
   const size_t smem = jit_layout(m->ctx, L, wk);
+  std::vector<JitRequest> reqs = {{k, jit_price_spec(m->ctx, k, L, kJitPrice | wk, smem)}};
   Screen sc;
-  if (screen_suits(m, k, sc)) {  // large launches walk the listed paths with the per-path kernel
-    s = jit_kernel(k, jit_price_spec(m->ctx, k, L, kJitPriceWrite | wk, smem), jk);
-    if (s != PC_OK) return s;
-  }
-  return jit_kernel(k, jit_price_spec(m->ctx, k, L, kJitPrice | wk, smem), jk);
+  if (screen_suits(m, k, sc))  // large launches walk the listed paths with the per-path kernel
+    reqs.push_back({k, jit_price_spec(m->ctx, k, L, kJitPriceWrite | wk, smem)});
+  return jit_compile_many(m->ctx, reqs);
 }
 
 pc_status pc_debug_jit_kernels(pc_ctx *c, uint64_t *out_kernels) {

@@ -62,3 +62,17 @@ def test_one_general_kernel_for_all_grids(eng, text, grid_param, what):
         seen[n] = got[True][0]
     if not grid_param:  # (the barrier's instructions hold its number of dates)
         assert kernels == [kernels[0]] * len(GRIDS)
+
+
+def test_compile_leaves_nothing_to_the_first_large_call(eng):
+    """A screened barrier has two kernels, for its small launches and for the
+    paths left by the screen: pc_jit_compile makes both."""
+    m, k = eng.model(spec(240)), eng.contract(BARRIER, [240])
+    assert pc.pc_debug_price_kernels(m, k, 1 << 20) == 3 and pc.pc_debug_price_kernels(m, k, 1 << 12) == 1
+    pc.pc_set_jit(eng.ctx, True)
+    pc.pc_jit_compile(m, k)
+    assert pc.pc_debug_jit_kernels(eng.ctx) == 2
+    large, small = pc.pc_price(m, k, 1 << 20, 5), pc.pc_price(m, k, 1 << 12, 5)
+    assert pc.pc_debug_jit_kernels(eng.ctx) == 2
+    pc.pc_set_jit(eng.ctx, False)
+    assert (large, small) == (pc.pc_price(m, k, 1 << 20, 5), pc.pc_price(m, k, 1 << 12, 5))
