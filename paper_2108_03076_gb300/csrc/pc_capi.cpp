@@ -197,13 +197,13 @@ int32_t max_label(const Program &p) {
   return top;
 }
 
-// The contract's window and static walks on the model (kept by the contract;
-// `out` stays valid as long as it does).
-pc_status window_for(const pc_model *m, const pc_contract *k, pc_contract::Window *&out) {
+// The contract's window and, where specialised kernels are to be used, static
+// walks on the model (kept by the contract; `out` stays valid as long as it does).
+pc_status window_for(const pc_model *m, const pc_contract *k, bool walks, pc_contract::Window *&out) {
   auto *kc = const_cast<pc_contract *>(k);
   std::lock_guard<std::mutex> g(kc->mu);
   auto it = kc->win_cache.find(m->id);
-  if (it != kc->win_cache.end() && (it->second.with_walks || !k->ctx->jit)) {
+  if (it != kc->win_cache.end() && (it->second.with_walks || !walks)) {
     out = &it->second;
     return PC_OK;
   }
@@ -217,7 +217,7 @@ pc_status window_for(const pc_model *m, const pc_contract *k, pc_contract::Windo
   std::vector<uint8_t> reads;
   pc_status s = analyse_program(k->prog, m->H.t_now, m->H.n, m->H.n_hist, w.win, w.skip, reads, err);
   if (s != PC_OK) return fail(s, err);
-  if (k->ctx->jit && walk_jit_eligible(k->prog)) {
+  if (walks && walk_jit_eligible(k->prog)) {
     w.walk = static_walk(m->H, reads);
     if (m->H.n <= kStaticOps) w.walk_all = static_walk(m->H, std::vector<uint8_t>(size_t(m->H.n) + 1, 1));
     if (!w.walk.empty() && !admit_walk(k->ctx, k->prog, m->H, w.walk)) {
@@ -225,7 +225,7 @@ pc_status window_for(const pc_model *m, const pc_contract *k, pc_contract::Windo
       w.walk_all.clear();
     }
   }
-  w.with_walks = k->ctx->jit != 0;
+  w.with_walks = walks;
   w.grid = static_grid(m->H, w.walk);
   w.grid_all = static_grid(m->H, w.walk_all);
   out = &(kc->win_cache[m->id] = std::move(w));
@@ -270,13 +270,13 @@ int pick_block(const Program &p, int words, int max_smem, int d, size_t &smem, b
 }
 
 pc_status prepare(const pc_model *m, const pc_contract *k, uint64_t n_paths, uint64_t offset,
-                  uint64_t seed, uint32_t stream, Launch &L, bool allow_hbm) {
+                  uint64_t seed, uint32_t stream, Launch &L, bool allow_hbm, bool specialised) {
   if (!m || !k) return fail(PC_EINVAL, "null model or contract");
   if (m->ctx != k->ctx) return fail(PC_EINVAL, "model and contract belong to different contexts");
   if (n_paths == 0) return fail(PC_EINVAL, "n_paths must be >= 1");
   if (n_paths > (uint64_t(1) << 40)) return fail(PC_ELIMIT, "n_paths exceeds 2^40");
   pc_contract::Window *w = nullptr;
-  pc_status s = window_for(m, k, w);
+  pc_status s = window_for(m, k, specialised || m->ctx->jit, w);
   if (s != PC_OK) return s;
   const int32_t win = w->win;
   L.w = w;
@@ -1194,7 +1194,7 @@ pc_status pc_jit_compile(const pc_model *m, const pc_contract *k) {
   // the block a pricing launch of this pair uses (it does not depend on
   // the path count)
   Launch L;
-  pc_status s = prepare(m, k, 1u << 20, 0, 0, 0, L, true);
+  pc_status s = prepare(m, k, 1u << 20, 0, 0, 0, L, true, true);
   if (s != PC_OK) return s;
   CU(cudaSetDevice(m->ctx->device), "cudaSetDevice");
   const int wk = jit_window_kind(m->ctx, L);

@@ -145,7 +145,7 @@ struct pc_contract {
   std::mutex mu;
   struct Window {
     int32_t win = 1, skip = 0;
-    bool with_walks = false;  // computed with the context's specialised kernels on
+    bool with_walks = false;  // computed for specialised kernels
     // static walks over the dates the program reads, and over every date
     // of the model (a per-date hook); empty where they are too long; and
     // their launch arguments
@@ -223,8 +223,9 @@ struct Launch {
 // allow_hbm the window may be placed in HBM (pricing kernel only): when the
 // context asks for it, or (automatic mode) when the shared window would
 // leave fewer than 8 resident warps per SM or exceeds PC_MAX_WINDOW.
+// specialised: for a specialised kernel although the context interprets.
 pc_status prepare(const pc_model *m, const pc_contract *k, uint64_t n_paths, uint64_t offset,
-                  uint64_t seed, uint32_t stream, Launch &L, bool allow_hbm = false);
+                  uint64_t seed, uint32_t stream, Launch &L, bool allow_hbm = false, bool specialised = false);
 
 // Whether the caller is capturing the context's stream.
 bool capturing(const pc_ctx *c);

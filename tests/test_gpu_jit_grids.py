@@ -76,3 +76,16 @@ def test_compile_leaves_nothing_to_the_first_large_call(eng):
     assert pc.pc_debug_jit_kernels(eng.ctx) == 2
     pc.pc_set_jit(eng.ctx, False)
     assert (large, small) == (pc.pc_price(m, k, 1 << 20, 5), pc.pc_price(m, k, 1 << 12, 5))
+
+
+def test_compile_before_the_context_is_switched(eng):
+    """pc_jit_compile while the context still interprets compiles the kernel
+    that the first specialised call runs."""
+    text = "(mult (max (sub (max (model 0 2) (model 1 5)) 1.0) 0.0) (payoff 5 0 1))"
+    m, k = eng.model(spec(5)), eng.contract(text)
+    plain = pc.pc_price(m, k, 1 << 12, 5)
+    pc.pc_jit_compile(m, k)
+    compiled = pc.pc_debug_jit_kernels(eng.ctx)
+    pc.pc_set_jit(eng.ctx, True)
+    assert pc.pc_price(m, k, 1 << 12, 5) == plain
+    assert pc.pc_debug_jit_kernels(eng.ctx) == compiled == 1
