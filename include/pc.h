@@ -750,6 +750,10 @@ pc_status pc_debug_set_jit_pairs(pc_ctx *ctx, int32_t pairs);
 pc_status pc_debug_price_kernels(const pc_model *model, const pc_contract *contract, uint64_t n_paths,
                                  int32_t *out_kernels);
 
+/* Models that the contract keeps its analysis of (those it was priced on that
+ * have not been destroyed).  Errors: PC_EINVAL. */
+pc_status pc_debug_contract_models(const pc_contract *contract, uint64_t *out_models);
+
 /* Specialised kernels that the context has compiled so far.  Errors: PC_EINVAL. */
 pc_status pc_debug_jit_kernels(pc_ctx *ctx, uint64_t *out_kernels);
 

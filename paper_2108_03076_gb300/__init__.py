@@ -133,6 +133,7 @@ _SIGS = {
     "pc_set_window_mode": [VP, C.c_int32],
     "pc_set_jit": [VP, C.c_int32],
     "pc_debug_set_jit_pairs": [VP, C.c_int32],
+    "pc_debug_contract_models": [VP, C.POINTER(U64)],
     "pc_debug_jit_kernels": [VP, C.POINTER(U64)],
     "pc_debug_price_kernels": [VP, VP, U64, PI32],
     "pc_debug_set_cv_min_blocks": [VP, C.c_int32],
@@ -406,6 +407,12 @@ def pc_debug_mlp_partials(widths, max_batch: int, batch: int, sm_count: int):
 
 def pc_debug_set_jit_pairs(ctx: int, pairs: int) -> None:
     _check(lib().pc_debug_set_jit_pairs(VP(ctx), int(pairs)))
+
+
+def pc_debug_contract_models(contract: int) -> int:
+    n = U64()
+    _check(lib().pc_debug_contract_models(VP(contract), C.byref(n)))
+    return n.value
 
 
 def pc_debug_jit_kernels(ctx: int) -> int:

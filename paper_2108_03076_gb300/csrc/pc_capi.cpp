@@ -225,9 +225,11 @@ pc_status window_for(const pc_model *m, const pc_contract *k, bool walks, pc_con
       w.walk_all.clear();
     }
   }
+  w.model = m;
   w.with_walks = walks;
   w.grid = static_grid(m->H, w.walk);
   w.grid_all = static_grid(m->H, w.walk_all);
+  m->users.insert(kc);
   out = &(kc->win_cache[m->id] = std::move(w));
   return PC_OK;
 }
@@ -907,6 +909,10 @@ pc_status pc_model_destroy(pc_model *m) {
   cudaSetDevice(m->ctx->device);
   cudaStreamSynchronize(m->ctx->stream);
   cudaFree(m->d_mem);
+  for (pc_contract *k : m->users) {
+    std::lock_guard<std::mutex> g(k->mu);
+    k->win_cache.erase(m->id);
+  }
   --m->ctx->live_objects;
   delete m;
   return PC_OK;
@@ -1063,6 +1069,7 @@ pc_status pc_contract_destroy(pc_contract *k) {
   cudaSetDevice(k->ctx->device);
   ctx_free(k->ctx, k->d_code, k->pooled);  // after the stream's launches that read it
   --k->ctx->live_objects;
+  for (const auto &w : k->win_cache) w.second.model->users.erase(k);
   delete k;
   return PC_OK;
 }
@@ -1204,6 +1211,12 @@ pc_status pc_jit_compile(const pc_model *m, const pc_contract *k) {
   if (screen_suits(m, k, sc))  // large launches walk the listed paths with the per-path kernel
     reqs.push_back({k, jit_price_spec(m->ctx, k, L, kJitPriceWrite | wk, smem)});
   return jit_compile_many(m->ctx, reqs);
+}
+
+pc_status pc_debug_contract_models(const pc_contract *k, uint64_t *out_models) {
+  if (!k || !out_models) return fail(PC_EINVAL, "null argument");
+  *out_models = k->win_cache.size();
+  return PC_OK;
 }
 
 pc_status pc_debug_jit_kernels(pc_ctx *c, uint64_t *out_kernels) {

@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <map>
 #include <mutex>
+#include <set>
 #include <string>
 #include <utility>
 #include <vector>
@@ -127,12 +128,15 @@ struct pc_ctx {
   int live_objects = 0;
 };
 
+struct pc_contract;
+
 struct pc_model {
   pc_ctx *ctx = nullptr;
   pc::ModelHost H;
   void *d_mem = nullptr;
   pc::ModelDev dev{};
   uint64_t id = 0;
+  mutable std::set<pc_contract *> users;  // contracts that keep a Window of this model
 };
 
 
@@ -143,7 +147,9 @@ struct pc_contract {
   bool pooled = false;            // d_code came from the context's memory pool
   std::vector<uint32_t> image;    // program then padded pool: the uploaded words
   std::mutex mu;
+  // (an entry goes with its model: pc_model_destroy)
   struct Window {
+    const pc_model *model = nullptr;
     int32_t win = 1, skip = 0;
     bool with_walks = false;  // computed for specialised kernels
     // static walks over the dates the program reads, and over every date
