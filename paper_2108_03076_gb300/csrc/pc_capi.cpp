@@ -333,9 +333,9 @@ pc_status prepare(const pc_model *m, const pc_contract *k, uint64_t n_paths, uin
   const uint64_t warps_per_block = uint64_t(L.block) / 32;
   const uint64_t need = (n_tiles + warps_per_block - 1) / warps_per_block;
   L.grid = int(std::min<uint64_t>(uint64_t(c->sm_count) * bpsm, need));
-  if (L.hbm_window && m->H.d == 2) {
-    const int dense = price_blocks_per_sm(2, L.block, L.smem, kPriceHbmDense);
-    if (need > uint64_t(L.grid) && need <= uint64_t(c->sm_count) * dense) {
+  if (L.hbm_window && need > uint64_t(L.grid)) {
+    const int dense = price_blocks_per_sm(m->H.d, L.block, L.smem, kPriceHbmDense);
+    if (need <= uint64_t(c->sm_count) * dense) {
       L.sparse_grid = L.grid;
       L.grid = int(need);
     }

@@ -15,12 +15,20 @@
 namespace pc {
 // Kernel launchers (pc_kernels.cu).  All return a cudaError_t.
 // The interpreting kernel's variants: the window of dates in shared memory or
-// in HBM, and for two underlyings the latter at seven blocks an SM (72
-// registers) instead of six.  Seven cost 2-9 % a tile (300 dates newest
-// first, 1,024 tiles: 417 -> 455 us; 4,688 tiles of 200: 608 -> 625; 16,384
-// of 30: 233 -> 243), and are taken where they hold every tile at once and
-// six do not: 4,096 tiles of 300 dates, 1.12 rounds of six blocks, 867 -> 680
-// us; of 50 dates 149 -> 124.
+// in HBM, the latter at its usual register bound or at one block an SM more
+// (dense).  Dense launches are taken where they hold every tile at once and
+// the usual ones do not, which saves the second round of tiles; elsewhere the
+// tighter bound costs more than it gives (spills).  Newest-first averages, us,
+// usual / dense, in that band and below it, by underlyings:
+//   1 (7 / 8 blocks): 300 dates 676 / 510, 446 / 474; 50 dates 115 / 84, 74 / 76
+//   2 (6 / 7):        300 dates 881 / 671, 575 / 604; 50 dates 141 / 115, 96 / 101
+//   3 (5 / 6):        50 dates 163 / 142, 111 / 125
+//   4 (5 / 6):        50 dates 171 / 158, 121 / 142
+// (300 dates of three or four: the program leaves no shared memory for
+// another block, and the rule takes none.)  Past the band the third round
+// that dense launches of one or two underlyings save is worth 2 to 13 %, for
+// three or four they lose 1 to 20 %; by 40 blocks an SM all are within 4 % or
+// lose.
 enum PriceKind { kPriceShared = 0, kPriceHbm = 1, kPriceHbmDense = 2 };
 cudaError_t launch_price(const PriceArgs &a, int grid, int block, size_t smem_bytes, cudaStream_t s, bool dense = false);
 cudaError_t launch_greeks(const PriceArgs &a, int grid, int block, size_t smem_bytes, cudaStream_t s);

@@ -32,7 +32,7 @@ namespace {
 // HBM (lay.gwin) instead of shared memory, for programs that look back
 // further than shared memory holds.
 template <int D, bool WRITE, bool GW = false, bool DENSE = false>
-__global__ void __launch_bounds__(kBlock, D == 1 ? 7 : D == 2 ? (DENSE ? 7 : 6) : 5) price_kernel(const __grid_constant__ PriceArgs a) {
+__global__ void __launch_bounds__(kBlock, (D == 1 ? 7 : D == 2 ? 6 : 5) + (DENSE ? 1 : 0)) price_kernel(const __grid_constant__ PriceArgs a) {
   price_tiles<D, WRITE>(a, [&](const uint4 *P, const float *pool, float2 *R, const Rng2 &g, bool live0,
                                bool live1, const float(&Bm)[D * D], const float(&S0)[D]) {
     return eval_path<D, GW>(P, pool, R, a, g, live0, live1, Bm, S0);
@@ -188,16 +188,19 @@ cudaError_t launch_price(const PriceArgs &a, int grid, int block, size_t smem, c
     k<<<grid, block, smem, s>>>(a);                                                \
     return cudaGetLastError();                                                     \
   } while (0)
+#define LAUNCH_W(DD, ...)                                                          \
+  do {                                                                             \
+    if (w) LAUNCH(DD, true, __VA_ARGS__); else LAUNCH(DD, false, __VA_ARGS__);     \
+  } while (0)
 #define LAUNCH_D(DD)                                                               \
   do {                                                                             \
-    if (gw) { if (w) LAUNCH(DD, true, true); else LAUNCH(DD, false, true); }       \
-    else { if (w) LAUNCH(DD, true, false); else LAUNCH(DD, false, false); }        \
+    if (gw && dense) LAUNCH_W(DD, true, true);                                     \
+    else if (gw) LAUNCH_W(DD, true);                                               \
+    else LAUNCH_W(DD, false);                                                      \
   } while (0)
   switch (a.m.d) {
     case 1: LAUNCH_D(1);
-    case 2:
-      if (gw && dense) { if (w) LAUNCH(2, true, true, true); else LAUNCH(2, false, true, true); }
-      LAUNCH_D(2);
+    case 2: LAUNCH_D(2);
     case 3: LAUNCH_D(3);
     case 4: LAUNCH_D(4);
     default: return cudaErrorInvalidValue;
@@ -220,7 +223,7 @@ int price_occupancy(uint64_t v, int block, size_t smem) {
   } while (0)
 #define OCC(DD)                                                                                      \
   do {                                                                                               \
-    if (kind == kPriceHbmDense) OCC_K(DD, false, true, DD == 2);                                     \
+    if (kind == kPriceHbmDense) OCC_K(DD, false, true, true);                                     \
     else if (kind == kPriceHbm) OCC_K(DD, false, true);                                              \
     else OCC_K(DD, false, false);                                                                    \
   } while (0)
