@@ -30,8 +30,12 @@ constexpr int kJitPrice = 0, kJitPriceWrite = 1, kJitHbm = 2, kJitWinRegs = 4, k
 // resident blocks per SM the specialised pricing kernel's register bound is
 // set for by default (<= 72 registers at 128 threads: the fastest measured)
 constexpr int kJitMinBlocks = 7;
-// one underlying needs fewer registers: 8 blocks (<= 64; 35-date average, 3e5 paths: 58.7 -> 45 us, where 7
-// blocks' 4,256 warps left a second round of 432 tiles)
+// one underlying needs fewer registers: 8 blocks (<= 64).  Averages over 20,
+// 35 and 60 dates and barriers over 20 to 60, us at 7 / 8 blocks: 3e5 paths,
+// where 7 leave a second round, 38.9 / 27.0, 58.6 / 40.8, 94.8 / 63.6 and
+// 35.0 / 24.7 to 77.9 / 53.4; 5e5 and 1e6 paths up to 7 % faster (20 dates,
+// 5e5: 43.8 / 44.1); 2^14 to 1.5e5 within 3 %, most equal (20 dates, 5e4: 21.3
+// / 22.6).  Four paths a lane (100 and 252 dates): within 2 %, 4 % faster at 1e6.
 constexpr int kJitMinBlocks1 = 8;
 // the same with a static walk, whose bridge stack and normals are registers
 // (autocall, 3 underlyings, 5 dates, 2^20 paths: 5 / 6 / 7 / 8 blocks 52.5 / 51.4 / 52.1 / 52.1 us a call)
@@ -250,8 +254,8 @@ pc_status jit_kernel(const pc_contract *k, const JitSpec &spec, cudaKernel_t &ou
 // Programs of at most PC_JIT_MAX_INSNS instructions are specialised; the
 // launches of longer ones interpret them.
 bool jit_eligible(const pc_contract *k);
-// A program the specialised adjoint kernel takes (at most the reading
-// instructions that the shared date generator's re-entry switch is kept to).
+// A program the specialised adjoint kernel takes: one of at most
+// kAdjointDateSites reading instructions (pc_jit.cpp).
 bool adjoint_jit_eligible(const pc_contract *k);
 // A program whose evaluator can take a static walk: one copy of it, or two.
 bool walk_jit_eligible(const pc::Program &p);
