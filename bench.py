@@ -401,6 +401,9 @@ def main():
     kernel_ms = [a.elapsed_time(b) for a, b in evs]
     t_dev = sum(kernel_ms) / 1e3
     sums = out.cpu().numpy()
+    n_kernels = pc.pc_debug_price_kernels(model, contract, w.n_paths)
+    # a screened launch walks the paths that four nodes have not settled
+    walked = pc.pc_debug_walked_paths(ctx) if n_kernels > 1 else w.n_paths
     interp_ms = None
     if not args.interpret:
         # the interpreting kernel on the same inputs, for comparison
@@ -481,8 +484,12 @@ def main():
     peak_mufu = props.multi_processor_count * 16 * clock_hz
     ops = alg_ops_per_path(minfo)
     launch_s = t_dev / args.steps
-    achieved = ops["ops"] * w.n_paths / launch_s
-    n_kernels = pc.pc_debug_price_kernels(model, contract, w.n_paths)
+    every_date = ops["ops"] * w.n_paths / launch_s
+    # the operations done: all dates of the walked paths, and where a launch
+    # is screened the four screened dates of every path
+    screened = 4.0 / spec.n if n_kernels > 1 else 0.0
+    done = walked / w.n_paths + screened
+    achieved = done * every_date
     kind = "interpreter" if args.interpret or info.n_insn > pc.JIT_MAX_INSNS else "specialised"
     traffic = profile_traffic(w, kind)
     prof = profile_record(w, kind)
@@ -502,7 +509,7 @@ def main():
                                  + (", window of dates in HBM" if linfo.hbm_window else "")
                                  + (f", {n_kernels} launches a step: paths knocked out at the last, middle or "
                                     "quarter dates are settled first and not walked (payoffs and sums "
-                                    "bit-equal; value and roofline count every path's dates)"
+                                    "bit-equal; value counts every path's dates, roofline the operations done)"
                                     if n_kernels > 1 else "")},
             # where the window of simulated dates lives (a program that looks
             # far back keeps it in HBM: bytes of the launch's buffer, bytes
@@ -527,7 +534,9 @@ def main():
                             "(a reloaded program finds its compiled kernel in the context's cache)"},
             "roofline": {"bound": "alu", "achieved": achieved / 1e12, "peak": peak_ops / 1e12,
                          "unit": "Tops/s", "frac": achieved / peak_ops, "traffic": traffic,
-                         "mufu_frac": ops["mufu"] * w.n_paths / launch_s / peak_mufu,
+                         "mufu_frac": done * ops["mufu"] * w.n_paths / launch_s / peak_mufu,
+                         # every path's dates counted, settled paths' too (not work done)
+                         "frac_every_date": every_date / peak_ops, "paths_walked": walked / w.n_paths,
                          # the busiest pipe's issue rate and the issue-active fraction from the
                          # committed ncu capture of this kernel source (null if none)
                          "ncu_max_pipe": prof.get("ncu_max_pipe"),

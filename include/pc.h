@@ -746,9 +746,15 @@ pc_status pc_debug_set_jit_pairs(pc_ctx *ctx, int32_t pairs);
 /* Kernels that one pc_price / pc_price_async / pc_price_paths call of n_paths
  * launches: 1, or 3 where a daily barrier's decided paths are screened out
  * before the walk (the screen, the walk over the paths left, the totals).
+ * (A call that finds no memory for the screen, or a captured one whose screen
+ * would have to grow, launches 1 all the same.)
  * Errors: PC_EINVAL, those of pc_price_info. */
 pc_status pc_debug_price_kernels(const pc_model *model, const pc_contract *contract, uint64_t n_paths,
                                  int32_t *out_kernels);
+/* Paths that the context's latest screened launch walked, the others being
+ * settled by the screen (0: none was screened yet).  Blocks.
+ * Errors: PC_EINVAL, PC_ECUDA, PC_ETIMEOUT. */
+pc_status pc_debug_walked_paths(pc_ctx *ctx, uint64_t *out_paths);
 
 /* Models that the contract keeps its analysis of (those it was priced on that
  * have not been destroyed).  Errors: PC_EINVAL. */

@@ -135,6 +135,7 @@ _SIGS = {
     "pc_debug_set_jit_pairs": [VP, C.c_int32],
     "pc_debug_contract_models": [VP, C.POINTER(U64)],
     "pc_debug_jit_kernels": [VP, C.POINTER(U64)],
+    "pc_debug_walked_paths": [VP, C.POINTER(U64)],
     "pc_debug_price_kernels": [VP, VP, U64, PI32],
     "pc_debug_set_cv_min_blocks": [VP, C.c_int32],
     "pc_jit_compile": [VP, VP],
@@ -403,6 +404,12 @@ def pc_debug_mlp_partials(widths, max_batch: int, batch: int, sm_count: int):
     _check(lib().pc_debug_mlp_partials(_ptr(w, C.c_int32), w.size, int(max_batch), int(batch), int(sm_count),
                                        C.byref(a), C.byref(b)))
     return a.value, b.value
+
+
+def pc_debug_walked_paths(ctx: int) -> int:
+    n = U64()
+    _check(lib().pc_debug_walked_paths(VP(ctx), C.byref(n)))
+    return n.value
 
 
 def pc_debug_set_jit_pairs(ctx: int, pairs: int) -> None:

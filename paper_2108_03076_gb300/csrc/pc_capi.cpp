@@ -1173,6 +1173,17 @@ pc_status pc_debug_price_kernels(const pc_model *m, const pc_contract *k, uint64
   return PC_OK;
 }
 
+pc_status pc_debug_walked_paths(pc_ctx *c, uint64_t *out_paths) {
+  if (!c || !out_paths) return fail(PC_EINVAL, "null argument");
+  uint32_t n = 0;
+  CU(cudaSetDevice(c->device), "cudaSetDevice");
+  if (c->screen.p) CU(cudaMemcpyAsync(&n, c->screen.p, sizeof(n), cudaMemcpyDeviceToHost, c->stream), "count copy");
+  const pc_status s = wait_stream(c);
+  if (s != PC_OK) return s;
+  *out_paths = n;
+  return PC_OK;
+}
+
 pc_status pc_debug_set_jit_pairs(pc_ctx *c, int32_t pairs) {
   if (!c) return fail(PC_EINVAL, "null context");
   if (pairs < 0 || pairs > 2) return fail(PC_EINVAL, "pairs must be 0 (automatic), 1 or 2");

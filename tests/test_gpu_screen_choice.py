@@ -69,6 +69,9 @@ def test_ranges_that_hold_some_of_the_screened_dates(ctx, name):
     try:
         assert kernels(m, k) == (3 if dates else 1, 1)
         x, sums = run(ctx, m, k, PIECE * PIECES, OFFSET)
+        if dates:  # every other path is settled, and has the literal as its payoff
+            walked = pc.pc_debug_walked_paths(ctx)
+            assert np.count_nonzero(x != np.float32(0.25)) <= walked < 0.98 * x.size
         parts = [run(ctx, m, k, PIECE, OFFSET + i * PIECE)[0] for i in range(PIECES)]
         np.testing.assert_array_equal(x, np.concatenate(parts))
         assert 0.02 < np.mean(x == np.float32(0.25)) < 0.98
