@@ -14,7 +14,7 @@ namespace {
 // (optional) receives the last generated date ordinal: the window holds the
 // simulated dates up to it.
 // `hook_` (optional, type PcHook) is called after each generated date.
-template <int D, bool GW = false, class PcHook = NoDateHook>
+template <int D, bool GW = false, class PcHook = NoDateHook, bool SKIP = true>
 __device__ float2 eval_path(const uint4 *P, const float *pool, float2 *R, const PriceArgs &a,
                             const Rng2 &g, bool live0, bool live1, const float (&Bm)[D * D],
                             const float (&S0)[D], int *frontier = nullptr, PcHook *hook_ = nullptr) {
@@ -57,7 +57,6 @@ __device__ float2 eval_path(const uint4 *P, const float *pool, float2 *R, const 
 #undef EACH_DATE
 #undef FUSED_VALUE
 #undef FUSED_TEST
-#undef LOOP_FUSED_TEST
 }
 
 }  // namespace
