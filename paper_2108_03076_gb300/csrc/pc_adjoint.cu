@@ -8,12 +8,13 @@
 namespace pc {
 namespace {
 
-template <int D, bool WRITE>
+// SKIP: programs that start at a later date than the first (as price_kernel).
+template <int D, bool WRITE, bool SKIP>
 __global__ void __launch_bounds__(kBlock, D == 4 ? 4 : 5) adjoint_kernel(const __grid_constant__ PriceArgs a, const TapeArgs t) {
   adjoint_tiles<D, WRITE>(a, t, [&](const uint4 *P, const float *pool, float2 *R, const Rng2 &g, bool live0,
                                    bool live1, const float (&Bm)[D * D], const float (&S0)[D],
                                    const float (&Lm)[D * D], Tape &T, int &res) {
-    return eval_adjoint<D>(P, pool, R, a, g, live0, live1, Bm, S0, Lm, T, res);
+    return eval_adjoint<D, SKIP>(P, pool, R, a, g, live0, live1, Bm, S0, Lm, T, res);
   });
 }
 
@@ -27,21 +28,27 @@ cudaError_t set_smem_a(K kern, size_t smem) {
 cudaError_t launch_adjoint(const PriceArgs &a, const TapeArgs &t, int grid, int block, size_t smem,
                            cudaStream_t s) {
   const bool w = a.out_paths != nullptr;
-#define ALAUNCH(DD, WW)                                                            \
+#define ALAUNCH(DD, WW, SS)                                                        \
   do {                                                                             \
-    auto k = adjoint_kernel<DD, WW>;                                               \
+    auto k = adjoint_kernel<DD, WW, SS>;                                           \
     cudaError_t e = set_smem_a(k, smem);                                           \
     if (e != cudaSuccess) return e;                                                \
     k<<<grid, block, smem, s>>>(a, t);                                             \
     return cudaGetLastError();                                                     \
   } while (0)
+#define ALAUNCH_D(DD)                                                              \
+  do {                                                                             \
+    if (a.lay.skip > 1) { if (w) ALAUNCH(DD, true, true); else ALAUNCH(DD, false, true); } \
+    else { if (w) ALAUNCH(DD, true, false); else ALAUNCH(DD, false, false); }                  \
+  } while (0)
   switch (a.m.d) {
-    case 1: if (w) ALAUNCH(1, true); else ALAUNCH(1, false);
-    case 2: if (w) ALAUNCH(2, true); else ALAUNCH(2, false);
-    case 3: if (w) ALAUNCH(3, true); else ALAUNCH(3, false);
-    case 4: if (w) ALAUNCH(4, true); else ALAUNCH(4, false);
+    case 1: ALAUNCH_D(1);
+    case 2: ALAUNCH_D(2);
+    case 3: ALAUNCH_D(3);
+    case 4: ALAUNCH_D(4);
     default: return cudaErrorInvalidValue;
   }
+#undef ALAUNCH_D
 #undef ALAUNCH
 }
 
@@ -52,9 +59,9 @@ int adjoint_occupancy(uint64_t v, int block, size_t smem) {
   cudaError_t e = cudaErrorInvalidValue;
 #define AOCC(DD)                                                                                 \
   do {                                                                                           \
-    e = set_smem_a(adjoint_kernel<DD, false>, smem);                                             \
+    e = set_smem_a(adjoint_kernel<DD, false, false>, smem);                                             \
     if (e == cudaSuccess)                                                                        \
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, adjoint_kernel<DD, false>, block, smem); \
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, adjoint_kernel<DD, false, false>, block, smem); \
   } while (0)
   switch (d) {
     case 1: AOCC(1); break;

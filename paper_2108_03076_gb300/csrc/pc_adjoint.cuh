@@ -97,7 +97,7 @@ __device__ __forceinline__ int adj_leaf(Tape &T, int o, int l, float2 s, float s
 
 // The payoff program of two paths per lane with its tape (forward sweep);
 // returns the result and sets `res` to its entry number.
-template <int D>
+template <int D, bool SKIP>
 __device__ float2 eval_adjoint(const uint4 *P, const float *pool, float2 *R, const PriceArgs &a,
                                const Rng2 &g, bool live0, bool live1, const float (&Bm)[D * D],
                                const float (&S0)[D], const float (&Lm)[D * D], Tape &T, int &res) {

@@ -953,30 +953,58 @@ __device__ __forceinline__ void fused_test_regs(const uint4 &I, int o, const flo
   fused_test_rd<D>(I, o, pool, m, [&](int l) { return cur[l]; }, t0, t1);
 }
 
-// A whole-loop barrier's decoded test (LOOP_TEST, before the loop) and the
-// sensitivity evaluators' use of it (LOOP_VALUE: the test at ordinal o,
-// fresh_: the date was produced for it, its S is in registers).
+// The sensitivity evaluators' whole-loop barrier: the descriptor Dsc tested at
+// n + 1 dates, ordinal ORDINAL_ at the k-th, the walk brought there by the
+// evaluator's LOOP_ADVANCE.  The interpreter decodes a plain test once and
+// takes a date just produced from the registers, in a loop of its own (as in
+// pc_ops.inc).
+#define LOOP_DATES_(ORDINAL_, TEST_)        \
+  for (int k = 0;; ++k) {                   \
+    int o = ORDINAL_;                       \
+    bool c0, c1;                            \
+    TEST_                                   \
+    if (c0 && !d0) { d0 = true; r0 = lit; } \
+    if (c1 && !d1) { d1 = true; r1 = lit; } \
+    all = __all_sync(kFull, d0 && d1);      \
+    if (all || k == n) break;               \
+  }
+#define LOOP_GENERAL_                                          \
+  {                                                            \
+    LOOP_ADVANCE                                               \
+    const float2 v_ = fused_value<D>(Dsc, o, pool, R, m, lay); \
+    c0 = bits(v_.x) != 0;                                      \
+    c1 = bits(v_.y) != 0;                                      \
+  }
 #ifdef PC_JIT
-#define LOOP_TEST(I_)
-#define LOOP_VALUE(I_, o_, fresh_, c0_, c1_)                         \
-  do {                                                               \
-    (void)(fresh_);                                                  \
-    const float2 v_ = fused_value<D>(I_, o_, pool, R, m, lay);       \
-    c0_ = bits(v_.x) != 0;                                           \
-    c1_ = bits(v_.y) != 0;                                           \
-  } while (0)
+#define LOOP_TESTS(ORDINAL_) LOOP_DATES_(ORDINAL_, LOOP_GENERAL_)
 #else
-#define LOOP_TEST(I_) const LoopTest<D> lt_(I_)
-#define LOOP_VALUE(I_, o_, fresh_, c0_, c1_)                         \
-  do {                                                               \
-    if (lt_.use && (fresh_)) {                                       \
-      lt_.test(ps.s[0], c0_, c1_);                                   \
-    } else {                                                         \
-      const float2 v_ = fused_value<D>(I_, o_, pool, R, m, lay);     \
-      c0_ = bits(v_.x) != 0;                                         \
-      c1_ = bits(v_.y) != 0;                                         \
-    }                                                                \
-  } while (0)
+// S at ordinal o, produced before (in the window) or history.
+template <int D>
+__device__ __forceinline__ void past_values(int o, const float2 *R, const ModelDev &m, const Layout &lay,
+                                            float2 (&s)[D]) {
+#pragma unroll
+  for (int i = 0; i < D; ++i)
+    s[i] = o > 0 ? SL(lay.off_win + (o & (lay.win - 1)) * D + i) : dup2(__ldg(m.sval + (o + m.n_hist) * D + i));
+}
+#define LOOP_PLAIN_                     \
+  {                                     \
+    if (ps.f < o) {                     \
+      LOOP_ADVANCE                      \
+      lt_.test(ps.s[0], c0, c1);        \
+    } else {                            \
+      LOOP_ADVANCE                      \
+      float2 s_[D];                     \
+      past_values<D>(o, R, m, lay, s_); \
+      lt_.test(s_, c0, c1);             \
+    }                                   \
+  }
+#define LOOP_TESTS(ORDINAL_)               \
+  const LoopTest<D> lt_(Dsc);              \
+  if (!lt_.use) {                          \
+    LOOP_DATES_(ORDINAL_, LOOP_GENERAL_)   \
+  } else {                                 \
+    LOOP_DATES_(ORDINAL_, LOOP_PLAIN_)     \
+  }
 #endif
 
 // Values of the stack machine: one per path of the lane, kPL = 2 PC_PAIRS of

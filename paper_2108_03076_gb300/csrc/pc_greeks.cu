@@ -9,12 +9,13 @@
 namespace pc {
 namespace {
 
-template <int D, bool WRITE>
+// SKIP: programs that start at a later date than the first (as price_kernel).
+template <int D, bool WRITE, bool SKIP>
 __global__ void __launch_bounds__(kBlock, D == 4 ? 4 : 5) greeks_kernel(const __grid_constant__ PriceArgs a) {
   greeks_tiles<D, WRITE>(a, [&](const uint4 *P, const float *pool, float2 *R, const Rng2 &g, bool live0,
                                 bool live1, const float (&Bm)[D * D], const float (&S0)[D],
                                 const float (&Lm)[D * D], int gl, float sig_g) {
-    return eval_greeks<D>(P, pool, R, a, g, live0, live1, Bm, S0, Lm, gl, sig_g);
+    return eval_greeks<D, SKIP>(P, pool, R, a, g, live0, live1, Bm, S0, Lm, gl, sig_g);
   });
 }
 
@@ -27,21 +28,27 @@ cudaError_t set_smem_g(K kern, size_t smem) {
 
 cudaError_t launch_greeks(const PriceArgs &a, int grid, int block, size_t smem, cudaStream_t s) {
   const bool w = a.out_paths != nullptr;
-#define GLAUNCH(DD, WW)                                                            \
+#define GLAUNCH(DD, WW, SS)                                                        \
   do {                                                                             \
-    auto k = greeks_kernel<DD, WW>;                                                \
+    auto k = greeks_kernel<DD, WW, SS>;                                            \
     cudaError_t e = set_smem_g(k, smem);                                           \
     if (e != cudaSuccess) return e;                                                \
     k<<<grid, block, smem, s>>>(a);                                                \
     return cudaGetLastError();                                                     \
   } while (0)
+#define GLAUNCH_D(DD)                                                              \
+  do {                                                                             \
+    if (a.lay.skip > 1) { if (w) GLAUNCH(DD, true, true); else GLAUNCH(DD, false, true); } \
+    else { if (w) GLAUNCH(DD, true, false); else GLAUNCH(DD, false, false); }                  \
+  } while (0)
   switch (a.m.d) {
-    case 1: if (w) GLAUNCH(1, true); else GLAUNCH(1, false);
-    case 2: if (w) GLAUNCH(2, true); else GLAUNCH(2, false);
-    case 3: if (w) GLAUNCH(3, true); else GLAUNCH(3, false);
-    case 4: if (w) GLAUNCH(4, true); else GLAUNCH(4, false);
+    case 1: GLAUNCH_D(1);
+    case 2: GLAUNCH_D(2);
+    case 3: GLAUNCH_D(3);
+    case 4: GLAUNCH_D(4);
     default: return cudaErrorInvalidValue;
   }
+#undef GLAUNCH_D
 #undef GLAUNCH
 }
 
@@ -49,8 +56,8 @@ int greeks_blocks_per_sm(int d, int block, size_t smem) {
   int nb = 0;
   cudaError_t e = cudaErrorInvalidValue;
 #define GOCC(DD)                                                                             \
-  set_smem_g(greeks_kernel<DD, false>, smem);                                                \
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, greeks_kernel<DD, false>, block, smem)
+  set_smem_g(greeks_kernel<DD, false, false>, smem);                                                \
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, greeks_kernel<DD, false, false>, block, smem)
   switch (d) {
     case 1: GOCC(1); break;
     case 2: GOCC(2); break;

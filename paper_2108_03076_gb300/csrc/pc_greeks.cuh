@@ -117,7 +117,7 @@ __device__ __forceinline__ TV fused_tv(const uint4 &I, int o, const float *pool,
 }
 
 // The payoff program with tangents, two paths per lane, warp in step.
-template <int D>
+template <int D, bool SKIP>
 __device__ TV eval_greeks(const uint4 *P, const float *pool, float2 *R, const PriceArgs &a,
                           const Rng2 &g, bool live0, bool live1, const float (&Bm)[D * D],
                           const float (&S0)[D], const float (&Lm)[D * D], int gl, float sig_g) {

@@ -48,6 +48,24 @@ def paths(ctx, m, text):
     return x.cpu().numpy()
 
 
+def sensitivities(ctx, m, d, text):
+    """Per-path tangents of every underlying and adjoints, with their sums."""
+    w, c = pc.pc_assemble(text)
+    k = pc.pc_load_payoff(ctx, w, c)
+    res = []
+    for l in range(d):
+        out = torch.zeros(8, dtype=torch.float64, device="cuda")
+        x = torch.full((3 * N,), float("nan"), device="cuda")
+        pc.pc_debug_greeks_paths(m, k, N, 3, 99, l, out.data_ptr(), x.data_ptr())
+        res += [out, x]
+    out = torch.zeros(20, dtype=torch.float64, device="cuda")
+    x = torch.full(((1 + 2 * d) * N,), float("nan"), device="cuda")
+    pc.pc_debug_adjoint_paths(m, k, N, 3, 99, out.data_ptr(), x.data_ptr())
+    torch.cuda.synchronize()
+    pc.pc_contract_destroy(k)
+    return [r.cpu().numpy() for r in res + [out, x]]
+
+
 def chain(op, xs):
     s = xs[0]
     for x in xs[1:]:
@@ -91,5 +109,22 @@ def test_sums_of_walks_that_start_later(ctx, d, n, first):
     try:
         x = paths(ctx, m, f"(max (sub (model {d - 1} {first}) (model 0 {n})) 0.0)")
         assert np.all(np.isfinite(x)) and (first == n and d == 1 or x.max() > 0)
+    finally:
+        pc.pc_model_destroy(m)
+
+
+@pytest.mark.parametrize("test", list(TESTS))
+@pytest.mark.parametrize("d,n,now", [(1, 40, 3), (2, 9, 0), (3, 30, 2), (4, 12, 1)])
+def test_sensitivities_of_plain_tests_equal_scaled_ones(ctx, test, d, n, now):
+    m = model(ctx, d, n, now)
+    plain = TESTS[test](lambda i: f"(model {i} 0)", d, lambda k: k)
+    scaled = TESTS[test](lambda i: f"(mult (model {i} 0) 2.0)", d, lambda k: 2.0 * k)
+    top = n + now
+    try:
+        for form in ("{}", "(add (mult 0.0 (model 0 %d)) {})" % top):
+            a, b = (sensitivities(ctx, m, d, form.format(f"(loopif {t} 0.25 (model {d - 1} 0) {top})"))
+                    for t in (plain, scaled))
+            for x, y in zip(a, b):
+                np.testing.assert_array_equal(x, y)
     finally:
         pc.pc_model_destroy(m)
